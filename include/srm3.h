@@ -76,7 +76,10 @@ typedef struct srm3_spectrum {
  * A separable g turns the pair sum of every lattice point into a
  * self-convolution: plans with it sample through a zero-padded 2-D FFT
  * instead of the O(N^2) pair sum (Sec. 4.3 FFT form; any storage setting is
- * ignored). */
+ * ignored).  The Gaussian envelope factors on the pairs of k as well, since
+ * (i-j)^2 = 2 (i-c)^2 + 2 (j-c)^2 - (k-2c)^2: with W recomputed it takes the
+ * same form, in an arithmetic that leaves FP32 plans FP32 accuracy, unless
+ * sigma_g is so small (below about 0.22) that the factors' range is too wide. */
 enum srm3_bispectrum_kind {
     SRM3_BISPECTRUM_GAUSS_ENVELOPE = 0,
     SRM3_BISPECTRUM_SEPARABLE = 1
@@ -127,7 +130,9 @@ enum srm3_precision {
     SRM3_FP64 = 1  /* plain FP64 pair sum (one warp per k and sheet-sample), FP64 FFT */
 };
 enum srm3_storage {
-    SRM3_STORAGE_AUTO = 0,     /* table if it fits the budget, else recompute */
+    SRM3_STORAGE_AUTO = 0,     /* the fastest: recompute where the pair sum is a
+                                  self-convolution (below), else the table if
+                                  it fits the budget, else recompute */
     SRM3_STORAGE_TABLE = 1,    /* W streamed from an HBM table (FP32 only) */
     SRM3_STORAGE_RECOMPUTE = 2, /* W rebuilt from envelope factors in-kernel */
     SRM3_STORAGE_TUNED = 3      /* the storage srm3_autotune chose for this lattice
@@ -233,9 +238,9 @@ typedef struct srm3_info {
                                 of the FP64 pass at the FP32 root estimate, moved to
                                 the final eps to first order (FP32 plans);
                                 bit 2 (SRM3_PAIRSUM_SEPARABLE): the FP32 pair sum
-                                runs in separable form, g = a_i a_j b_k with the
-                                omega factor folded into the phasor rows (W
-                                recomputed, Gaussian envelope, Sec. 4.3);
+                                runs in separable form, g = a_i a_j b_k, as a
+                                self-convolution of a y (W recomputed, Gaussian
+                                envelope, Sec. 4.3);
                                 bit 3 (SRM3_REC_COARSE_START): the eps search
                                 started from the root of the same search on a
                                 coarser lattice (coarse_fk, coarse_fw below) and

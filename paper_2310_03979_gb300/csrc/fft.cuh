@@ -8,6 +8,7 @@
 
 #include <utility>
 
+#include "df.cuh"
 #include "srm3_internal.cuh"
 
 namespace srm3 {
@@ -173,9 +174,10 @@ __device__ __forceinline__ T2 rot16(T2 b, int e) {
     default: {
       const T c = e == 1 ? (T)c1 : e == 3 ? (T)s1 : e == 5 ? (T)-s1 : (T)-c1;
       const T s = (e == 1 || e == 7) ? (T)s1 : (T)c1;
-      r.x = b.x * c - b.y * s;
-      r.y = b.x * s + b.y * c;
-      return r;
+      T2 w;
+      w.x = c;
+      w.y = s;
+      return cmul(b, w);
     }
   }
 }
@@ -340,17 +342,23 @@ __device__ __forceinline__ void load_tw(const T2 *__restrict__ p, T2 (&w)[R]) {
       w[2 * i + 1].y = t.w;
     }
   } else {
+    const float4 *q = reinterpret_cast<const float4 *>(p);  // one 16-byte entry each
 #pragma unroll
-    for (int i = 0; i < R; ++i) w[i] = __ldg(p + i);
+    for (int i = 0; i < R; ++i) {
+      const float4 t = __ldg(q + i);
+      w[i] = *reinterpret_cast<const T2 *>(&t);
+    }
   }
 }
 
 // One Stockham pass of radix R (see above).  tpt threads per transform, jt
 // this thread's index among them; items jt, jt + tpt, ... < L/R.  twp: this
-// pass's run of the pass-twiddle table.  FIRST: inputs from src(i) (global);
-// else from sm (shared, padded positions).  LAST: outputs to dst(i, v)
-// (global); else to sm.
-template <int R, bool FIRST, bool LAST, unsigned VMASK, typename T2, class Src, class Dst>
+// pass's run of the pass-twiddle table.  FIRST: inputs from src(i) (global,
+// or with SRCSM from sm itself, in place); else from sm (shared, padded
+// positions).  LAST: outputs to dst(i, v) (global), the upper half of the
+// outputs left out with HALFOUT; with DSTSM, and on every other pass, to sm.
+template <int R, bool FIRST, bool LAST, unsigned VMASK, bool SRCSM, bool DSTSM, bool HALFOUT,
+          typename T2, class Src, class Dst>
 __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
                                               const T2 *__restrict__ twp, T2 *sm, Src &src,
                                               Dst &dst) {
@@ -391,16 +399,17 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
         dft_inv<R>(v[it]);
     }
   }
-  if constexpr (!FIRST && !LAST) __syncthreads();  // in place: all reads before any write
+  if constexpr ((!FIRST || SRCSM) && (!LAST || DSTSM))
+    __syncthreads();  // in place: all reads before any write
 #pragma unroll
   for (int it = 0; it < NI; ++it) {
     const int j = jt + it * tpt;
     if (j < LR) {
       const int k = j & (Ns - 1);
       const int b = (j - k) * R + k;
-      if constexpr (LAST) {
+      if constexpr (LAST && !DSTSM) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) dst(b + r * Ns, v[it][r]);
+        for (int r = 0; r < (HALFOUT ? R / 2 : R); ++r) dst(b + r * Ns, v[it][r]);
       } else if (Ns % 16 == 0) {
         const int a = sp16(b), st = Ns + (Ns >> 4);
 #pragma unroll
@@ -411,7 +420,7 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
       }
     }
   }
-  if constexpr (!LAST) __syncthreads();
+  if constexpr (!LAST || DSTSM) __syncthreads();
 }
 
 // Passes p, p + 1, ... of the inverse DFT of length 2^l (1 <= l <= 13),
@@ -419,18 +428,20 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
 // live; Ns is the length transformed by the passes before p, toff the
 // offset of pass p's run in the pass-twiddle table tw.
 // VM0: the inputs of the first pass that can be nonzero (bit r: the block
-// r of L/R inputs, R the first radix; 0 = all).
-template <int l, int p, unsigned VM0, typename T2, class Src, class Dst>
+// r of L/R inputs, R the first radix; 0 = all).  SRCSM, DSTSM, HALFOUT: see
+// stockham_pass (the first pass's source, the last pass's destination).
+template <int l, int p, unsigned VM0, bool SRCSM = false, bool DSTSM = false,
+          bool HALFOUT = false, typename T2, class Src, class Dst>
 __device__ __forceinline__ void stockham_passes(int Ns, int toff, int tpt, int jt,
                                                 const T2 *__restrict__ tw, T2 *sm, Src &src,
                                                 Dst &dst) {
   if constexpr (p < tx_npass(l)) {
     constexpr int lr = tx_lr(l, p);
     constexpr unsigned vm = (p == 0 && VM0 != 0u) ? VM0 : tx_in_mask(1 << lr, 0);
-    stockham_pass<(1 << lr), p == 0, p == tx_npass(l) - 1, vm>(1 << l, Ns, tpt, jt, tw + toff,
-                                                               sm, src, dst);
-    stockham_passes<l, p + 1, VM0>(Ns << lr, p == 0 ? 0 : toff + (Ns << lr), tpt, jt, tw, sm,
-                                   src, dst);
+    stockham_pass<(1 << lr), p == 0, p == tx_npass(l) - 1, vm, SRCSM, DSTSM, HALFOUT>(
+        1 << l, Ns, tpt, jt, tw + toff, sm, src, dst);
+    stockham_passes<l, p + 1, VM0, SRCSM, DSTSM, HALFOUT>(
+        Ns << lr, p == 0 ? 0 : toff + (Ns << lr), tpt, jt, tw, sm, src, dst);
   }
 }
 

@@ -290,12 +290,6 @@ struct PsDesc {  // aligned as CUtensorMap
   // half-warps then take two row pairs of a work item (a = 2i and 2i + 1),
   // reading 256-byte rows through a tensor map with 64-float boxes
   int half;
-  // sep = 1: W recomputed in separable form, g(i, j) = a_i a_j b_k on the
-  // pairs of k -- the omega factor a_w is in y, the kappa factor aK[row]
-  // weights each row pair, b_k is in ck: the register blocks multiply y
-  // rows alone and no envelope window is staged
-  int sep;
-  const float *aK;
   float cb, sb;          // cos / sin of the biphase
 };
 
@@ -324,7 +318,7 @@ __device__ __forceinline__ int4 ps_get_unit(int u, const PsDesc &d0,
 
 // One staged chunk for one compute warp: all register blocks of the chunk.
 // RS: float4 per staged row (32, or 16 in half mode).
-template <bool TABLE, int RS, bool SEPW = false>
+template <bool TABLE, int RS>
 __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
                                          const float4 *__restrict__ pb,
                                          const float2 *__restrict__ pw,
@@ -348,25 +342,7 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
       Bc[m0 + vv] = lds_pair(pb + (m0 + vv - U * (NB - 1)) * RS);
     }
     const ulonglong2 *B = Bc + m0;
-    if constexpr (SEPW) {
-      // separable form: the weights are in the rows, four packed FMAs per
-      // product of two sheet-samples; omega outermost and the two updates
-      // of Ty[r] in separate sweeps over the outputs, so that no FMA waits
-      // on the one before it (every accumulator's terms keep their order)
-#pragma unroll
-      for (int uu = 0; uu < U; ++uu) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const int v = r - uu + U - 1;
-          Txp[r] = f2_fma(A[uu].x, B[v].x, Txp[r]);
-          Txm[r] = f2_fma(A[uu].y, B[v].y, Txm[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) Ty[r] = f2_fma(A[uu].x, B[r - uu + U - 1].y, Ty[r]);
-#pragma unroll
-        for (int r = 0; r < R; ++r) Ty[r] = f2_fma(A[uu].y, B[r - uu + U - 1].x, Ty[r]);
-      }
-    } else if (TABLE) {
+    if (TABLE) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const float4 w4 =
@@ -419,12 +395,7 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
 // sorted by decreasing cost).  MIXED = false compiles the full-group path
 // alone (every descriptor has half = 0); MIXED = true also takes half-mode
 // descriptors.
-// FORM: kPsSeparable when every descriptor of the launch has W recomputed in
-// separable form (the kernel holds those register blocks alone), else
-// kPsAnyForm (each descriptor's form decided at run time).
-constexpr int kPsAnyForm = 0, kPsSeparable = 2;
-
-template <bool MIXED, int NCW, int FORM = kPsAnyForm>
+template <bool MIXED, int NCW>
 __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CTAS_PER_SM)
     k_pairsum_f32p(const __grid_constant__ PsDesc d0, const PsDesc *__restrict__ descs,
                    const int4 *__restrict__ units, int nunits, int *__restrict__ err) {
@@ -462,8 +433,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
       const int kk = un.y, kws0 = un.z, nch = (kws0 + SW + CH - 1) / CH;
       const int half = MIXED ? d.half : 0;
       const int nitems = ps_nitems(kk, kws0, half, SW), rs = d.rowstride;
-      const bool tab = FORM == kPsAnyForm && d.table != 0;
-      const bool sepf = FORM == kPsSeparable || d.sep != 0;
+      const bool tab = d.table != 0;
       const int x = un.w * LANES * 4;  // first float of the group in a row of y
       int a = 0, c = 0;
       for (int item = 0; item < nitems; ++item, ++q) {
@@ -484,7 +454,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
             }
           const unsigned tx = YROWS * ROW_BYTES +
                               (tab ? ntile * R * CH * (unsigned)sizeof(float)
-                                   : (sepf ? 0u : EWIN * (unsigned)sizeof(float)));
+                                   : EWIN * (unsigned)sizeof(float));
           mbar_expect_tx(&full[stage], tx);
           // one row pair (full rows), or two in half mode (half rows each; a
           // second row pair past the centre repeats the first and is
@@ -501,9 +471,8 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
                           &full[stage]);
           }
           if (!tab) {
-            if (!sepf)
-              bulk_g2s(sw + stage * STAGE_W, d.Ew + d.ew_off + 2 * i0 - kws0 - (SW - 1),
-                       EWIN * sizeof(float), &full[stage]);
+            bulk_g2s(sw + stage * STAGE_W, d.Ew + d.ew_off + 2 * i0 - kws0 - (SW - 1),
+                     EWIN * sizeof(float), &full[stage]);
           } else {
             for (int t = 0; t < NC; ++t) {  // the tiles counted above
               const int k0 = kws0 + R * t;
@@ -542,8 +511,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
     const int4 un = ps_get_unit(u, d0, units);
     const PsDesc &d = descs ? descs[un.x] : d0;
     const int kk = un.y, kws0 = un.z, grp = un.w, nw = d.nw;
-    const bool tab = FORM == kPsAnyForm && d.table != 0;
-    const bool sepf = FORM == kPsSeparable || d.sep != 0;
+    const bool tab = d.table != 0;
     const int kw0 = kws0 + R * warp, nch = (kws0 + SW + CH - 1) / CH;
     const int half = MIXED ? d.half : 0;
     const int nitems = ps_nitems(kk, kws0, half, SW);
@@ -569,17 +537,12 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
         if (half) {
           const float4 *pa = sy + stage * STAGE_Y + hl * YROWS * (LANES / 2) + ln;
           const float4 *pb = pa + (CH + R * warp + CH - U) * (LANES / 2);
-          if (sepf)
-            ps_chunk<false, LANES / 2, true>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
-          else
-            ps_chunk<false, LANES / 2>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
+          ps_chunk<false, LANES / 2>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
         } else {
           const float4 *pa = sy + stage * STAGE_Y + lane;
           const float4 *pb = pa + (CH + R * warp + CH - U) * LANES;
           if (tab)
             ps_chunk<true, LANES>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
-          else if (sepf)
-            ps_chunk<false, LANES, true>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
           else
             ps_chunk<false, LANES>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
         }
@@ -593,14 +556,9 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
         const int ah = half ? 2 * a + hl : a;  // this lane's row pair
         const bool live = ah <= kk / 2;
         const int b = kk - (live ? ah : a);
-        // the row pair's kappa weight: none for the table (in W), the
-        // envelope at kk - 2a, or in separable form aK[a] aK[kk - a]
-        // (the merge and the epilogue round every operation explicitly, so
-        // that the kernel compiled for one weight form gives the bits of the
-        // general one: a sample's result does not depend on the launch)
-        auto rw = [&](int a_) {
-          return sepf ? __fmul_rn(d.aK[a_], d.aK[kk - a_]) : d.Ek[kk - 2 * a_];
-        };
+        // the row pair's kappa weight: none for the table (in W), else the
+        // envelope at kk - 2a
+        auto rw = [&](int a_) { return d.Ek[kk - 2 * a_]; };
         const float rowfac = tab ? 1.0f : (live ? rw(ah) : 0.0f);
         const bool odd_live = half && 2 * a + 1 <= kk / 2;
         const float rowfac_odd = odd_live ? rw(2 * a + 1) : 0.0f;
@@ -620,7 +578,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
                   tab ? d.W[d.toff[kk * d.ntw + kw0 / R] +
                             (((long long)ah * (my_L / CH) + ((kw >> 1) / CH)) * R + r) * CH +
                             ((kw >> 1) % CH)]
-                      : (sepf ? 1.0f : d.Ew[d.ew_off]);
+                      : d.Ew[d.ew_off];
               const float t[4] = {__fsub_rn(__fmul_rn(h.x, h.x), __fmul_rn(h.z, h.z)),
                                   __fsub_rn(__fmul_rn(h.y, h.y), __fmul_rn(h.w, h.w)),
                                   __fmul_rn(__fmul_rn(2.f, h.x), h.z),

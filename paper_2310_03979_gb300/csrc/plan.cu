@@ -263,31 +263,26 @@ __global__ void k_sampling_tables(int n, double dkdw, double eps,
   ck[k] = (T)(pos ? 2.0 * eps * dkdw * sqrt(s) : 0.0);
 }
 
-// The separable form of the FP32 pair sum (Gaussian envelope): on the pairs
-// of k, (i - j)^2 = 2 (i - c)^2 + 2 (j - c)^2 - (k - 2c)^2 per axis (c =
-// (n - 1)/2), so g(i, j) = exp(-1/2 ((ik - jk)/sk)^2 - 1/2 ((iw - jw)/sw)^2)
-// = a_i a_j b_k with a = exp(-((ik - ck)/sk)^2 - ((iw - cw)/sw)^2) and b =
-// exp(1/2 ((kk - 2ck)/sk)^2 + 1/2 ((kw - 2cw)/sw)^2).  The pair sum then
-// multiplies scaled phasor rows, sum (a_w y)_i (a_w y)_j per lattice row
-// pair, weighted by aK[a] aK[kk - a] and at the end by c_k b_k; the pure term
-// P_k y_k = (P_k / a_w) (a_w y)_k.  Factor ranges within [exp(-E/2), 1] and
-// [1, exp(E)] (E <= 40), as the recursion's (k_gauss_sep).
-__global__ void k_sep_sampling(int nk, int nw, double sk, double sw, const float *__restrict__ sqq,
-                               const float *__restrict__ Pk, const float *__restrict__ ck,
-                               float *__restrict__ sqq_s, float *__restrict__ Pk_s,
-                               float *__restrict__ ck_s, float *__restrict__ aK) {
+// The factors of the Gaussian envelope for the self-convolution (conv.cuh):
+// per axis a = exp(-((i - c)/s)^2) and b = exp(1/2 ((k - 2c)/s)^2), c = (n -
+// 1)/4, the omega axis of a over the signed indices -(nw - 1) .. nw - 1.
+template <typename F>
+__global__ void k_conv_factors(int nk, int nw, double sk, double sw, F *__restrict__ fac) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nk * nw) return;
-  const int kk = i / nw, kw = i - kk * nw;
-  const double ck0 = 0.5 * (nk - 1), cw0 = 0.5 * (nw - 1);
-  const double uw = (kw - cw0) / sw, vk = (kk - 2.0 * ck0) / sk, vw = (kw - 2.0 * cw0) / sw;
-  const double aw = exp(-uw * uw), b = exp(0.5 * (vk * vk + vw * vw));
-  sqq_s[i] = (float)((double)sqq[i] * aw);
-  Pk_s[i] = (float)((double)Pk[i] / aw);
-  ck_s[i] = (float)((double)ck[i] * b);
-  if (kw == 0) {
-    const double uk = (kk - ck0) / sk;
-    aK[kk] = (float)exp(-uk * uk);
+  F *aK = fac, *bK = fac + nk, *aW = fac + 2 * nk, *bW = aW + 2 * nw - 1;
+  const double ck = 0.25 * (nk - 1), cw = 0.25 * (nw - 1);
+  if (i < nk) {
+    const double u = (i - ck) / sk, v = (i - 2.0 * ck) / sk;
+    aK[i] = (F)exp(-u * u);
+    bK[i] = (F)exp(0.5 * v * v);
+  }
+  if (i < 2 * nw - 1) {
+    const double u = (i - (nw - 1) - cw) / sw;
+    aW[i] = (F)exp(-u * u);
+  }
+  if (i < nw) {
+    const double v = (i - 2.0 * cw) / sw;
+    bW[i] = (F)exp(0.5 * v * v);
   }
 }
 
@@ -1742,7 +1737,11 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     if (p->storage == SRM3_STORAGE_TUNED)  // the autotuner's storage for this lattice
       p->storage = tuned >= 0 ? tuned : SRM3_STORAGE_AUTO;
     if (p->storage == SRM3_STORAGE_AUTO) {
-      p->storage = bytes <= p->table_budget ? SRM3_STORAGE_TABLE : SRM3_STORAGE_RECOMPUTE;
+      // W recomputed by the self-convolution is the faster one at every size
+      // (conv_launch.cuh; 256 x 512, 64 samples: 2.2 ms against 69 ms with the
+      // stored table, whose build and memory it saves too)
+      p->storage = !p->conv && bytes <= p->table_budget ? SRM3_STORAGE_TABLE
+                                                        : SRM3_STORAGE_RECOMPUTE;
     }
     if (p->mixed) p->storage = SRM3_STORAGE_RECOMPUTE;  // the table holds sum pairs only
     if (p->storage == SRM3_STORAGE_TABLE) {
@@ -1856,13 +1855,30 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
   // boundaries; the table reaches d = 2 nw + 127, past the last window.
   p->ew_off = ((nw + 32 + 7) / 8) * 8 + 7;
   p->ew_len = p->ew_off + 2 * nw + 128;  // difference pairs reach d = 2 nw - 2
-  if (p->sep) {  // zero-padded self-convolution grid
+  if (p->conv) {  // zero-padded self-convolution grid
     p->log2cNk = 1;
     while ((1 << p->log2cNk) < 2 * nk - 1) ++p->log2cNk;
     p->log2cNw = 1;
-    while ((1 << p->log2cNw) < 2 * nw - 1) ++p->log2cNw;
+    while ((1 << p->log2cNw) < (p->mixed ? 3 * nw - 2 : 2 * nw - 1)) ++p->log2cNw;
     p->cNk = 1 << p->log2cNk;
     p->cNw = 1 << p->log2cNw;
+    const int lk = p->log2cNk, lw = p->log2cNw;
+    const int ntwc = tx_twlen(lk) + tx_twlen(lw) + (1 << lw);
+    const int nfac = 2 * nk + 3 * nw - 1, m = std::max(nk, 2 * nw - 1);
+    const double sk = p->sigma_g * nk, sw = p->sigma_g * nw;
+    SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(double2), st));
+    if (!p->sep) SRM3_CUDA(dev_alloc(&p->conv_fac, (size_t)nfac * sizeof(double), st));
+    if (!f32) {
+      k_tx_twiddles<double2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (double2 *)p->tw_conv);
+      if (!p->sep)
+        k_conv_factors<double><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw,
+                                                             (double *)p->conv_fac);
+    } else if (p->sep) {
+      k_tx_twiddles<float2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (float2 *)p->tw_conv);
+    } else {
+      k_tx_twiddles<df2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (df2 *)p->tw_conv);
+      k_conv_factors<df><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw, (df *)p->conv_fac);
+    }
   }
   p->rowstride = nw + 2 * kPad;  // y row length, workspace or batch buffers
   SRM3_CUDA(dev_alloc(&p->Ek, nk * es, st));
@@ -1883,26 +1899,12 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
     }
     k_tx_twiddles<float2><<<cdiv(tw_n, 256), 256, 0, st>>>(p->log2nx, p->log2nt - 1,
                                                             (float2 *)p->tw);
-    if (p->sep) {
-      // pass twiddles of the self-convolution's lengths Nk, then Nw
-      const int ntwc = tx_twlen(p->log2cNk) + tx_twlen(p->log2cNw) + (1 << p->log2cNw);
-      SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(float2), st));
-      k_tx_twiddles<float2><<<cdiv(ntwc, 256), 256, 0, st>>>(p->log2cNk, p->log2cNw,
-                                                            (float2 *)p->tw_conv);
-    }
   } else {
     k_env<double><<<cdiv(nk, 256), 256, 0, st>>>(nk, 0, p->sigma_g * nk, (double *)p->Ek);
     k_env<double><<<cdiv(p->ew_len, 256), 256, 0, st>>>(p->ew_len, p->ew_off,
                                                        p->sigma_g * nw, (double *)p->Ews);
     k_tx_twiddles<double2><<<cdiv(tw_n, 256), 256, 0, st>>>(p->log2nx, p->log2nt - 1,
                                                              (double2 *)p->tw);
-    if (p->sep) {
-      // pass twiddles of the self-convolution's lengths Nk, then Nw
-      const int ntwc = tx_twlen(p->log2cNk) + tx_twlen(p->log2cNw) + (1 << p->log2cNw);
-      SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(double2), st));
-      k_tx_twiddles<double2><<<cdiv(ntwc, 256), 256, 0, st>>>(p->log2cNk, p->log2cNw,
-                                                            (double2 *)p->tw_conv);
-    }
   }
   SRM3_CUDA(cudaGetLastError());
   return SRM3_OK;
@@ -1922,15 +1924,6 @@ int prepare_sampling_tables(srm3_plan *p, cudaStream_t st) {
     k_sampling_tables<float><<<cdiv(nl, 256), 256, 0, st>>>(
         (int)nl, p->dkdw, p->eps, p->S, p->qm, p->sb2, (float *)p->sqq, (float *)p->Pk,
         (float *)p->ck);
-    if (pairsum_sep_capable(p)) {
-      SRM3_CUDA(dev_alloc(&p->sqq_s, nl * sizeof(float), st));
-      SRM3_CUDA(dev_alloc(&p->Pk_s, nl * sizeof(float), st));
-      SRM3_CUDA(dev_alloc(&p->ck_s, nl * sizeof(float), st));
-      SRM3_CUDA(dev_alloc(&p->aK, p->nk * sizeof(float), st));
-      k_sep_sampling<<<cdiv(nl, 256), 256, 0, st>>>(
-          p->nk, p->nw, p->sigma_g * p->nk, p->sigma_g * p->nw, (const float *)p->sqq,
-          (const float *)p->Pk, (const float *)p->ck, p->sqq_s, p->Pk_s, p->ck_s, p->aK);
-    }
   }
   else
     k_sampling_tables<double><<<cdiv(nl, 256), 256, 0, st>>>(
@@ -2004,12 +1997,11 @@ void free_plan(srm3_plan *p) {
                  p->rec_bar, p->rec_max,
                  p->rec_pairs, p->rec_pair_off,
                  p->ps_err,  p->env_e,    p->env_e2,     p->env_e32, p->qh,
-                 p->tw_conv, p->Zc, p->rec_z, p->tw_rec32, p->tw_rec64,
+                 p->tw_conv, p->rec_z, p->tw_rec32, p->tw_rec64,
                  p->sep_b ? p->env_b : nullptr, p->sep_b ? p->env_b2 : nullptr,
                  p->sep_b ? (void *)p->env_b32 : nullptr,
                  p->Dsum, p->qprev, p->qlo, p->fp_change, p->Ewd, p->ys, p->super_order_d,
-                 p->rs_a2, p->rs_b2, p->dsb2, p->red_part, p->sqq_s, p->Pk_s, p->ck_s, p->aK,
-                 p->qo3};
+                 p->rs_a2, p->rs_b2, p->dsb2, p->red_part, p->conv_fac, p->qo3};
   // no plan work may be in flight; the blocks go back to the pool
   cudaDeviceSynchronize();
   for (void *d : dev)
@@ -2122,6 +2114,12 @@ SRM3_API int srm3_plan_create(const srm3_spectrum *spectrum, const srm3_bispectr
     const double E = (g.n_kappa - 1) * (g.n_kappa - 1) / (sk * sk) +
                      (g.n_omega - 1) * (g.n_omega - 1) / (sw * sw);
     p->rec_sep = p->sep || (!p->mixed && E <= kSepExpMax);
+    // the pair sum as a self-convolution: its factors centred at a quarter
+    // of the lattice, b reaches exp(E / 8), which the transform's rounding is
+    // multiplied by (e^5 at the limit: 1e-12 of an output in double-float);
+    // one padded row and column of the grid have to fit in shared memory
+    const int padw = p->mixed ? 3 * g.n_omega - 2 : 2 * g.n_omega - 1;
+    p->conv = p->sep || (E <= kSepExpMax && 2 * g.n_kappa - 1 <= kMaxFft && padw <= kMaxFft);
   }
   p->beta = bispectrum->beta;
   p->table_budget = g.table_budget_bytes > 0 ? g.table_budget_bytes : 64.0 * (1ull << 30);
@@ -2177,7 +2175,8 @@ SRM3_API int srm3_plan_info(const srm3_plan *plan, srm3_info *info) {
   info->recursion_flags = (plan->rec_sep ? SRM3_REC_SEPARABLE : 0) |
                           (plan->eps_shifted ? SRM3_REC_TABLES_MOVED : 0) |
                           (plan->eps_interp ? SRM3_REC_TABLES_INTERPOLATED : 0) |
-                          (pairsum_sep_now(plan) ? SRM3_PAIRSUM_SEPARABLE : 0) |
+                          (conv_now(plan) && !plan->sep && plan->precision == SRM3_FP32
+                               ? SRM3_PAIRSUM_SEPARABLE : 0) |
                           (plan->coarse_start ? SRM3_REC_COARSE_START : 0);
   info->coarse_fk = plan->coarse_fk;
   info->coarse_fw = plan->coarse_fw;

@@ -10,8 +10,8 @@
 
 #include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 
-#include "fft.cuh"
 #include "pairsum.cuh"
+#include "philox.cuh"
 #include "srm3_internal.cuh"
 
 namespace srm3 {
@@ -19,37 +19,6 @@ namespace srm3 {
 static int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 // ---------------------------------------------------------------------------
-// Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of
-// (hi, lo) = M * x on words 0 and 2, mixed with words 1 and 3 and the key;
-// the key advances by the Weyl constants between rounds.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
-    uint32_t hi0 = __umulhi(m0, c.x), lo0 = m0 * c.x;
-    uint32_t hi1 = __umulhi(m1, c.z), lo1 = m1 * c.z;
-    c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-    k.x += 0x9E3779B9u;
-    k.y += 0xBB67AE85u;
-  }
-  return c;
-}
-
-
-// Unit phasor e^{i 2 pi (w + 1/2) 2^-32}.
-__device__ __forceinline__ float2 phasor(uint32_t w, float) {
-  float v = fmaf(__uint2float_rn(w), 0x1p-31f, 0x1p-32f);  // 2 (w + 1/2) 2^-32
-  float s, c;
-  sincospif(v, &s, &c);
-  return make_float2(c, s);
-}
-__device__ __forceinline__ double2 phasor(uint32_t w, double) {
-  double v = ((double)w + 0.5) * 0x1p-31;
-  double s, c;
-  sincospi(v, &s, &c);
-  return make_double2(c, s);
-}
-
 // a3: phases.  Thread per (Philox counter, sample), sample index fastest.
 // Counter c covers lattice entries e = 4c .. 4c+3 of e = (s nk + kk) nw + kw.
 // Writes y^s_k = sqrt(q_k) z^s_k (0 where S = 0) into the padded layout
@@ -139,18 +108,12 @@ int ensure_workspace(srm3_plan *p, int chunk) {
   const size_t e2 = elem2(p);
   p->rowstride = p->nw + 2 * kPad;
   const int sp = sspad_for(cap);
-  SRM3_CUDA(dev_alloc(&p->y, (size_t)p->nk * p->rowstride * sp * e2, p->stream));
+  SRM3_CUDA(dev_alloc(&p->y, y_bytes(p, sp), p->stream));
   SRM3_CUDA(dev_alloc(&p->y0, (size_t)sp * e2, p->stream));
   SRM3_CUDA(dev_alloc(&p->C, (size_t)2 * cap * p->nk * p->nw * e2, p->stream));
   SRM3_CUDA(dev_alloc(&p->H, (size_t)cap * transform_elems(p) * e2, p->stream));
-  if (p->mixed && p->precision == SRM3_FP32)
-    SRM3_CUDA(dev_alloc(&p->ys, (size_t)p->nk * p->rowstride * sp * e2, p->stream));
-  if (p->sep) {  // the self-convolution grid's n_kappa rows, every sheet-sample of a chunk
-    if (p->Zc) dev_free(p->Zc, p->stream);
-    p->Zc = nullptr;
-    SRM3_CUDA(dev_alloc(&p->Zc, (size_t)2 * cap * p->nk * p->cNw * e2, p->stream));
-    p->zc_ss = 2LL * cap;
-  }
+  if (p->mixed && p->precision == SRM3_FP32 && !p->conv)
+    SRM3_CUDA(dev_alloc(&p->ys, y_bytes(p, sp), p->stream));
   // stream-ordered blocks: usable from any stream (batches) once this passes
   SRM3_CUDA(cudaStreamSynchronize(p->stream));
   p->ws_chunk = cap;
@@ -172,12 +135,9 @@ static int phases_into(srm3_plan *p, cudaStream_t st, const uint64_t *seeds,
   const int blocks = cdiv(nc * n, 256);
   // the swapped copy of the mixed FP32 pair sum (plan workspace only)
   float *ys = (p->mixed && p->precision == SRM3_FP32 && y == p->y) ? (float *)p->ys : nullptr;
-  // the separable pair sum takes the rows with the omega factor folded in
-  // (not the raw Philox words, which do not depend on the table)
-  const float *sq32 = pairsum_sep_now(p) ? p->sqq_s : (const float *)p->sqq;
   if (p->precision == SRM3_FP32)
-    k_phases<float><<<blocks, 256, 0, st>>>(p->nk, p->nw, n, sc, dseeds, ss_off, sq32,
-                                            (float2 *)y, (float2 *)y0, sp, p->rowstride,
+    k_phases<float><<<blocks, 256, 0, st>>>(p->nk, p->nw, n, sc, dseeds, ss_off,
+                                            (const float *)p->sqq, (float2 *)y, (float2 *)y0, sp, p->rowstride,
                                             words_out, ys);
   else
     k_phases<double><<<blocks, 256, 0, st>>>(p->nk, p->nw, n, sc, dseeds, ss_off,
@@ -258,11 +218,8 @@ static int fill_pairsum_desc_into(srm3_plan *p, int n, void *y, void *y0, void *
   d->Ew = (const float *)p->Ews;
   d->W = table ? p->W : nullptr;
   d->toff = table ? p->tile_off : nullptr;
-  const bool sepf = pairsum_sep_now(p);
-  d->Pk = sepf ? p->Pk_s : (const float *)p->Pk;
-  d->ck = sepf ? p->ck_s : (const float *)p->ck;
-  d->sep = sepf ? 1 : 0;
-  d->aK = sepf ? p->aK : nullptr;
+  d->Pk = (const float *)p->Pk;
+  d->ck = (const float *)p->ck;
   d->C = (float2 *)C_out;
   d->order = p->super_order[tile_index(p->ps_nc)];
   d->nk = p->nk;
@@ -287,14 +244,11 @@ static int fill_pairsum_desc_into(srm3_plan *p, int n, void *y, void *y0, void *
 template <int NC>
 static int launch_pairsum_f32_nc(srm3_plan *p, cudaStream_t st, const PsDesc &d0,
                                  const PsDesc *descs, const int4 *units, int nunits, int max_ctas,
-                                 bool mixed, int form) {
+                                 bool mixed) {
   const size_t smem = pairsum_f32p_smem<NC>();
   constexpr int NT = packed::Shape<NC>::NT;
-  // every instantiation: the general form and the separable form alone
-  const void *kf[4] = {(const void *)k_pairsum_f32p<false, NC>,
-                       (const void *)k_pairsum_f32p<true, NC>,
-                       (const void *)k_pairsum_f32p<false, NC, kPsSeparable>,
-                       (const void *)k_pairsum_f32p<true, NC, kPsSeparable>};
+  const void *kf[2] = {(const void *)k_pairsum_f32p<false, NC>,
+                       (const void *)k_pairsum_f32p<true, NC>};
   for (const void *f : kf) {
     SRM3_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     SRM3_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
@@ -314,13 +268,7 @@ static int launch_pairsum_f32_nc(srm3_plan *p, cudaStream_t st, const PsDesc &d0
   int grid = std::min(nunits, ctas);
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
   if (grid == 0) return SRM3_OK;
-  if (form == kPsSeparable && mixed)
-    k_pairsum_f32p<true, NC, kPsSeparable><<<grid, NT, smem, st>>>(d0, descs, units, nunits,
-                                                                   p->ps_err);
-  else if (form == kPsSeparable)
-    k_pairsum_f32p<false, NC, kPsSeparable><<<grid, NT, smem, st>>>(d0, descs, units, nunits,
-                                                                    p->ps_err);
-  else if (mixed)
+  if (mixed)
     k_pairsum_f32p<true, NC><<<grid, NT, smem, st>>>(d0, descs, units, nunits, p->ps_err);
   else
     k_pairsum_f32p<false, NC><<<grid, NT, smem, st>>>(d0, descs, units, nunits, p->ps_err);
@@ -328,25 +276,11 @@ static int launch_pairsum_f32_nc(srm3_plan *p, cudaStream_t st, const PsDesc &d0
   return SRM3_OK;
 }
 
-// The instantiation for a descriptor's weight form: the separable form has
-// one of its own (its register blocks alone: 166 registers and no spills
-// against 168 and spills, 6 % faster on the bridge lattice); the stored
-// table and the weighted recompute form take the general kernel (compiled
-// for the table alone it spilled more and ran 0.3 % slower).
-static int ps_form_of(const PsDesc &d) {
-  return !d.table && d.sep ? kPsSeparable : kPsAnyForm;
-}
-
-// form: kPsSeparable when every descriptor of the launch has the separable
-// weight form, else kPsAnyForm; -1: that of d0 for a single-plan launch
-// (descs == NULL).
 int launch_pairsum_f32(srm3_plan *p, cudaStream_t st, const PsDesc &d0, const PsDesc *descs,
-                       const int4 *units, int nunits, int max_ctas, bool mixed, int nc,
-                       int form = -1) {
-  if (form < 0) form = descs ? kPsAnyForm : ps_form_of(d0);
+                       const int4 *units, int nunits, int max_ctas, bool mixed, int nc) {
   if (nc == 2)
-    return launch_pairsum_f32_nc<2>(p, st, d0, descs, units, nunits, max_ctas, mixed, form);
-  return launch_pairsum_f32_nc<4>(p, st, d0, descs, units, nunits, max_ctas, mixed, form);
+    return launch_pairsum_f32_nc<2>(p, st, d0, descs, units, nunits, max_ctas, mixed);
+  return launch_pairsum_f32_nc<4>(p, st, d0, descs, units, nunits, max_ctas, mixed);
 }
 
 // The difference-pair launch of a mixed FP32 plan over n samples whose rows
@@ -416,7 +350,6 @@ static int pairsum_f64_on(srm3_plan *p, cudaStream_t st, int n, void *C_out) {
 }
 
 int run_pairsum(srm3_plan *p, int n, void *C_out) {
-  if (p->sep) return conv_pairsum_on(p, p->stream, n, p->y, p->y0, C_out);
   if (p->precision == SRM3_FP64) return pairsum_f64_on(p, p->stream, n, C_out);
   PsDesc d;
   int rc = fill_pairsum_desc(p, n, C_out, &d);
@@ -425,6 +358,22 @@ int run_pairsum(srm3_plan *p, int n, void *C_out) {
                           p->nsuper[tile_index(p->ps_nc)] * d.G, 0, d.half != 0, p->ps_nc);
   if (rc || !p->mixed) return rc;
   return launch_pairsum_f32_diff(p, p->stream, n, C_out);
+}
+
+// The self-convolution of n samples in the plan's workspace.
+static int conv_on(srm3_plan *p, cudaStream_t st, const uint64_t *seeds, const uint64_t *dseeds,
+                   int n, void *C_out) {
+  ConvJob j;
+  std::memset(&j, 0, sizeof(j));
+  j.plan = p;
+  j.stream = st;
+  j.n = n;
+  j.seeds = seeds;
+  j.dseeds = dseeds;
+  j.work = p->y;
+  j.work_bytes = y_bytes(p, sspad_for(p->ws_chunk));
+  j.C = C_out;
+  return conv_sample(j);
 }
 
 int run_transform(srm3_plan *p, const void *C, int n, void *out) {
@@ -483,11 +432,14 @@ int collect_timings(srm3_plan *p) {
 // One chunk of samples through the three sampling stages.
 static int run_chunk(srm3_plan *p, const uint64_t *seeds, int m, void *C, void *out) {
   int rc, rec;
-  if ((rc = stage_begin(p, 0, 0, &rec))) return rc;
-  if ((rc = run_phases(p, seeds, m, nullptr))) return rc;
-  if ((rc = stage_end(p, rec))) return rc;
+  const bool conv = conv_now(p);  // the phases are then part of the pair sum's first pass
+  if (!conv) {
+    if ((rc = stage_begin(p, 0, 0, &rec))) return rc;
+    if ((rc = run_phases(p, seeds, m, nullptr))) return rc;
+    if ((rc = stage_end(p, rec))) return rc;
+  }
   if ((rc = stage_begin(p, 1, 2LL * m * (p->pairs + p->diffpairs), &rec))) return rc;
-  if ((rc = run_pairsum(p, m, C))) return rc;
+  if ((rc = conv ? conv_on(p, p->stream, seeds, nullptr, m, C) : run_pairsum(p, m, C))) return rc;
   if ((rc = stage_end(p, rec))) return rc;
   if (!out) return SRM3_OK;
   if ((rc = stage_begin(p, 2, 0, &rec))) return rc;
@@ -538,10 +490,14 @@ struct srm3_batch {
     int total = 0, sp = 0, nmax = 0;
     void *y = nullptr, *y0 = nullptr, *C = nullptr, *H = nullptr;
     size_t ybytes = 0;
-    const float **pk_of = nullptr, **ck_of = nullptr;  // device, [total]
+    // per sample, device, [total] each, one block
+    const float **sqq_of = nullptr, **pk_of = nullptr, **ck_of = nullptr;
   };
   std::vector<srm3_plan *> plans;
-  std::vector<int> counts, seed_off, group_of;  // group_of[i]: group index or -1
+  std::vector<int> counts, group_of;  // group_of[i]: group index or -1
+  // first seed of each plan in the caller's order and in device memory,
+  // where the members of a shape group follow one another
+  std::vector<int> seed_off, dev_off;
   std::vector<void *> outs;
   std::vector<Group> groups;
   int total = 0;
@@ -557,7 +513,6 @@ struct srm3_batch {
   int nunits = 0;                 // both shapes
   int nunits_v[2] = {0, 0};
   bool mixed_v[2] = {false, false};  // some descriptor of the shape takes the half-group mode
-  int ps_form = 0;                   // the weight form common to every descriptor (kPsAnyForm: none)
   srm3_plan *lead = nullptr;      // first FP32 plan: CTA count and error word of the launch
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -575,45 +530,63 @@ using namespace srm3;
 // The launch sequence of one batch run on the batch stream.
 static int batch_launch(srm3_batch *b) {
   int rc;
+  const unsigned evf = b->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
   for (auto &g : b->groups) {
+    if (conv_now(b->plans[g.members[0]])) continue;
     SRM3_CUDA(cudaMemsetAsync(g.y, 0, g.ybytes, b->stream));
     for (size_t m = 0; m < g.members.size(); ++m) {
       const int i = g.members[m];
-      if ((rc = phases_into(b->plans[i], b->stream, nullptr, b->dseeds + b->seed_off[i],
+      if ((rc = phases_into(b->plans[i], b->stream, nullptr, b->dseeds + b->dev_off[i],
                             b->counts[i], g.y, g.y0, g.sp, 2 * g.sample_off[m], nullptr)))
         return rc;
     }
   }
   for (size_t i = 0; i < b->plans.size(); ++i)
-    if (b->group_of[i] < 0 &&
-        (rc = phases_on(b->plans[i], b->stream, nullptr, b->dseeds + b->seed_off[i],
+    if (b->group_of[i] < 0 && !conv_now(b->plans[i]) &&
+        (rc = phases_on(b->plans[i], b->stream, nullptr, b->dseeds + b->dev_off[i],
                         b->counts[i], nullptr)))
       return rc;
+  // in a capture the events must be external nodes of the graph
+  if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[0], b->stream, evf));
+  for (auto &g : b->groups) {  // phases, self-convolution and coefficients of a shape group
+    if (!conv_now(b->plans[g.members[0]])) continue;
+    ConvJob j;
+    std::memset(&j, 0, sizeof(j));
+    j.plan = b->plans[g.members[0]];
+    j.stream = b->stream;
+    j.n = g.total;
+    j.dseeds = b->dseeds + b->dev_off[g.members[0]];
+    j.sqq_of = (const void *const *)g.sqq_of;
+    j.pk_of = (const void *const *)g.pk_of;
+    j.ck_of = (const void *const *)g.ck_of;
+    j.work = g.y;
+    j.work_bytes = g.ybytes;
+    j.C = g.C;
+    if ((rc = conv_sample(j))) return rc;
+  }
   if (b->nunits > 0) {
     PsDesc none;
     std::memset(static_cast<void *>(&none), 0, sizeof(none));
-    // in a capture the events must be external nodes of the graph
-    const unsigned evf = b->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-    if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[0], b->stream, evf));
     for (int v = 0, off = 0; v < 2; off += b->nunits_v[v], ++v)
       if (b->nunits_v[v] > 0 &&
           (rc = launch_pairsum_f32(b->lead, b->stream, none, b->ddesc, b->dunits + off,
-                                   b->nunits_v[v], b->max_ctas, b->mixed_v[v], v == 0 ? 4 : 2,
-                                   b->ps_form)))
+                                   b->nunits_v[v], b->max_ctas, b->mixed_v[v], v == 0 ? 4 : 2)))
         return rc;
-    if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[1], b->stream, evf));
   }
   for (size_t i = 0; i < b->plans.size(); ++i) {
     srm3_plan *p = b->plans[i];
-    if (p->mixed && p->precision == SRM3_FP32) {  // its difference pairs, after its sum pairs
+    if (b->group_of[i] >= 0) continue;
+    if (conv_now(p)) {
+      if ((rc = conv_on(p, b->stream, nullptr, b->dseeds + b->dev_off[i], b->counts[i], p->C)))
+        return rc;
+    } else if (p->mixed && p->precision == SRM3_FP32) {  // its difference pairs, after its sum pairs
       if ((rc = launch_pairsum_f32_diff(p, b->stream, b->counts[i], p->C))) return rc;
-    } else if (p->sep) {
-      if ((rc = conv_pairsum_on(p, b->stream, b->counts[i], p->y, p->y0, p->C))) return rc;
     } else if (p->precision == SRM3_FP64 &&
                (rc = pairsum_f64_on(p, b->stream, b->counts[i], p->C))) {
       return rc;
     }
   }
+  if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[1], b->stream, evf));
   for (auto &g : b->groups)
     for (size_t m = 0; m < g.members.size(); ++m) {
       const int i = g.members[m];
@@ -642,7 +615,7 @@ static void batch_free(srm3_batch *b) {
   for (cudaEvent_t e : b->ps_ev)
     if (e) cudaEventDestroy(e);
   for (auto &g : b->groups)
-    for (void *q : {g.y, g.y0, g.C, g.H, (void *)g.pk_of, (void *)g.ck_of})
+    for (void *q : {g.y, g.y0, g.C, g.H, (void *)g.sqq_of})
       if (q) cudaFreeAsync(q, b->stream);
   for (void *q : {(void *)b->dseeds, (void *)b->ddesc, (void *)b->dunits})
     if (q) cudaFreeAsync(q, b->stream);
@@ -797,7 +770,6 @@ SRM3_API int srm3_autotune(srm3_plan *plan, int n, srm3_tune_result *res) {
   if (rc) return rc;
   std::vector<uint64_t> seeds(n);
   for (int j = 0; j < n; ++j) seeds[j] = (uint64_t)j + 1;
-  if ((rc = run_phases(plan, seeds.data(), n, nullptr))) return rc;
   const bool can_table = (double)plan->table_entries * sizeof(float) <= plan->table_budget;
   if (can_table && !plan->W) {
     if ((rc = build_w_table(plan, plan->stream))) return rc;
@@ -808,19 +780,18 @@ SRM3_API int srm3_autotune(srm3_plan *plan, int n, srm3_tune_result *res) {
   auto time_one = [&](int storage, int nc, double *ms) -> int {
     plan->storage = storage;
     plan->ps_nc = nc;
-    PsDesc d;
-    int r = fill_pairsum_desc(plan, n, plan->C, &d);
+    auto once = [&]() {  // with the phases, which the self-convolution's first pass draws
+      int r1 = SRM3_OK;
+      if (conv_now(plan)) return conv_on(plan, plan->stream, seeds.data(), nullptr, n, plan->C);
+      if ((r1 = run_phases(plan, seeds.data(), n, nullptr))) return r1;
+      return run_pairsum(plan, n, plan->C);
+    };
+    int r = once();
     if (r) return r;
-    const int nunits = plan->nsuper[tile_index(nc)] * d.G;
-    if ((r = launch_pairsum_f32(plan, plan->stream, d, nullptr, nullptr, nunits, 0, d.half != 0,
-                                nc)))
-      return r;
     float best = 1e30f;
     for (int rep = 0; rep < 3; ++rep) {
       SRM3_CUDA(cudaEventRecord(ev[0], plan->stream));
-      if ((r = launch_pairsum_f32(plan, plan->stream, d, nullptr, nullptr, nunits, 0,
-                                  d.half != 0, nc)))
-        return r;
+      if ((r = once())) return r;
       SRM3_CUDA(cudaEventRecord(ev[1], plan->stream));
       SRM3_CUDA(cudaEventSynchronize(ev[1]));
       float t = 0.f;
@@ -919,7 +890,7 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
   // launch, no tail of a second
   long long terms_v[2] = {0, 0};
   for (int i = 0; i < m; ++i)
-    if (plans[i]->precision == SRM3_FP32 && !plans[i]->sep)
+    if (plans[i]->precision == SRM3_FP32 && !conv_now(plans[i]))
       terms_v[tile_index(plans[i]->ps_nc)] += (plans[i]->pairs + plans[i]->diffpairs) * counts[i];
   const int batch_nc = terms_v[1] > terms_v[0] ? 2 : 4;
   auto add_units = [&](srm3_plan *p, int j, const PsDesc &d) {
@@ -964,8 +935,20 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
       return bail(rc);
     }
     b->group_of.push_back(gi);
-    if (p->precision == SRM3_FP32 && !p->sep && !b->lead) b->lead = p;
+    if (p->precision == SRM3_FP32 && !conv_now(p) && !b->lead) b->lead = p;
   }
+  b->dev_off.assign(m, 0);
+  int doff = 0;
+  for (const auto &g : b->groups)
+    for (int i : g.members) {
+      b->dev_off[i] = doff;
+      doff += b->counts[i];
+    }
+  for (int i = 0; i < m; ++i)
+    if (b->group_of[i] < 0) {
+      b->dev_off[i] = doff;
+      doff += b->counts[i];
+    }
   cudaError_t e;
   for (auto &g : b->groups) {  // batch-owned buffers of each shape group
     srm3_plan *p = b->plans[g.members[0]];
@@ -977,29 +960,30 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
     const size_t hb = (size_t)g.nmax * transform_elems(p) * sizeof(float2);
     cudaStream_t st = b->stream;
     b->dev_bytes += (long long)(g.ybytes + (size_t)g.sp * sizeof(float2) + cb + hb +
-                                2 * sizeof(float *) * g.total);
+                                3 * sizeof(float *) * g.total);
     if ((e = cudaMallocAsync(&g.y, g.ybytes, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&g.y0, (size_t)g.sp * sizeof(float2), st)) != cudaSuccess ||
         (e = cudaMallocAsync(&g.C, cb, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&g.H, hb, st)) != cudaSuccess ||
-        (e = cudaMallocAsync((void **)&g.pk_of, sizeof(float *) * g.total, st)) != cudaSuccess ||
-        (e = cudaMallocAsync((void **)&g.ck_of, sizeof(float *) * g.total, st)) != cudaSuccess)
+        (e = cudaMallocAsync((void **)&g.sqq_of, 3 * sizeof(float *) * g.total, st)) != cudaSuccess)
       return bail(cuda_fail(e, "cudaMallocAsync(batch shape group)"));
-    std::vector<const float *> pk(g.total), ck(g.total);
+    g.pk_of = g.sqq_of + g.total;
+    g.ck_of = g.pk_of + g.total;
+    std::vector<const float *> fac(3 * (size_t)g.total);
     for (size_t mm = 0; mm < g.members.size(); ++mm) {
       srm3_plan *q = b->plans[g.members[mm]];
-      const bool sepf = pairsum_sep_now(q);  // as the group's descriptor (same shape and storage)
       for (int j = 0; j < b->counts[g.members[mm]]; ++j) {
-        pk[g.sample_off[mm] + j] = sepf ? q->Pk_s : (const float *)q->Pk;
-        ck[g.sample_off[mm] + j] = sepf ? q->ck_s : (const float *)q->ck;
+        const int o = g.sample_off[mm] + j;
+        fac[o] = (const float *)q->sqq;
+        fac[g.total + o] = (const float *)q->Pk;
+        fac[2 * g.total + o] = (const float *)q->ck;
       }
     }
-    if ((e = cudaMemcpyAsync(g.pk_of, pk.data(), sizeof(float *) * g.total,
-                             cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(g.ck_of, ck.data(), sizeof(float *) * g.total,
+    if ((e = cudaMemcpyAsync(g.sqq_of, fac.data(), sizeof(float *) * fac.size(),
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
       return bail(cuda_fail(e, "cudaMemcpy(batch factor tables)"));
+    if (conv_now(p)) continue;
     PsDesc d;
     if ((rc = fill_pairsum_desc_into(p, g.total, g.y, g.y0, g.C, &d))) return bail(rc);
     d.pk_of = g.pk_of;
@@ -1010,7 +994,7 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
   }
   for (int i = 0; i < m; ++i) {  // FP32 plans with a stored W table, on their workspace
     srm3_plan *p = b->plans[i];
-    if (b->group_of[i] >= 0 || p->precision != SRM3_FP32 || p->sep) continue;
+    if (b->group_of[i] >= 0 || p->precision != SRM3_FP32 || conv_now(p)) continue;
     PsDesc d;
     if ((rc = fill_pairsum_desc(p, counts[i], p->C, &d))) return bail(rc);
     const int j = (int)descs.size();
@@ -1029,9 +1013,6 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
   b->nunits = (int)u.size();
   if (!descs.empty()) {
     b->dev_bytes += (long long)(sizeof(PsDesc) * descs.size() + sizeof(int4) * u.size());
-    b->ps_form = ps_form_of(descs[0]);
-    for (const PsDesc &dd : descs)
-      if (ps_form_of(dd) != b->ps_form) b->ps_form = kPsAnyForm;
     e = cudaMallocAsync(&b->ddesc, sizeof(PsDesc) * descs.size(), b->stream);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMallocAsync(batch descriptors)"));
     e = cudaMemcpyAsync(b->ddesc, descs.data(), sizeof(PsDesc) * descs.size(),
@@ -1048,7 +1029,7 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
     std::memset(static_cast<void *>(&none), 0, sizeof(none));
     for (int v = 0; v < 2; ++v)
       if ((rc = launch_pairsum_f32(b->lead, b->stream, none, b->ddesc, b->dunits, 0, 0,
-                                   b->mixed_v[v], v == 0 ? 4 : 2, b->ps_form)))
+                                   b->mixed_v[v], v == 0 ? 4 : 2)))
         return bail(rc);
   }
   b->dev_bytes += (long long)(sizeof(uint64_t) * b->total);
@@ -1066,7 +1047,9 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
 SRM3_API int srm3_batch_run(srm3_batch *b, const uint64_t *seeds) {
   if (!b || !seeds) return fail(SRM3_ERR_INVALID_ARG, "batch and seeds must be non-NULL");
   // from pageable memory the copy has read the host buffer when it returns
-  std::memcpy(b->hseeds.data(), seeds, sizeof(uint64_t) * b->total);
+  for (size_t i = 0; i < b->plans.size(); ++i)
+    std::memcpy(b->hseeds.data() + b->dev_off[i], seeds + b->seed_off[i],
+                sizeof(uint64_t) * b->counts[i]);
   SRM3_CUDA(cudaMemcpyAsync(b->dseeds, b->hseeds.data(), sizeof(uint64_t) * b->total,
                             cudaMemcpyHostToDevice, b->stream));
   if (b->exec) {
@@ -1125,7 +1108,7 @@ SRM3_API int srm3_batch_enable_timing(srm3_batch *b, int on) {
     SRM3_CUDA(cudaEventCreate(&b->ps_ev[0]));
     SRM3_CUDA(cudaEventCreate(&b->ps_ev[1]));
   }
-  b->timing = on != 0 && b->nunits > 0;
+  b->timing = on != 0;
   return SRM3_OK;
 }
 

@@ -106,13 +106,16 @@ struct srm3_plan {
   // envelope split on i + j = k (a^2 per point in rs_a2, b^2 in rs_b2)
   bool rec_sep = false;
   double *rs_a2 = nullptr, *rs_b2 = nullptr;
-  // FFT self-convolution grid of the separable pair sum (powers of two,
-  // cNk >= 2 nk - 1, cNw >= 2 nw - 1), its twiddles e^{+2 pi i j / ntwc},
-  // and the workspace of zc_ss sheet-samples (complex, plan precision)
+  // the pair sum as an FFT self-convolution (conv.cuh): separable envelopes,
+  // and the Gaussian one where its factors' range allows; its grid (powers of
+  // two, cNk >= 2 nk - 1, cNw >= 2 nw - 1, or 3 nw - 2 with mixed
+  // interactions), the pass twiddles of both lengths, and the Gaussian
+  // envelope's factors (aK, bK [nk], aW [2 nw - 1], bW [nw], in the
+  // transform's real type)
+  bool conv = false;
   int cNk = 0, cNw = 0, log2cNk = 0, log2cNw = 0;
   void *tw_conv = nullptr;
-  void *Zc = nullptr;
-  long long zc_ss = 0;
+  void *conv_fac = nullptr;
   // mixed-sign interactions: opposite-sheet pairs as well; Eq. pure then
   // a fixed point solved by iterations of (difference sums at the previous
   // iterate, level pass)
@@ -169,12 +172,6 @@ struct srm3_plan {
   void *sqq = nullptr;    // sqrt(q) masked by S > 0, [nk*nw]
   void *Pk = nullptr;     // pure factor 2 sqrt(dk dw S) (1 - sb2), [nk*nw]
   void *ck = nullptr;     // pair factor 2 eps dk dw sqrt(S), [nk*nw]
-  // the FP32 pair sum in separable form (Gaussian envelope, W recomputed):
-  // g(i, j) = a_i a_j b_k on the pairs of k, the omega factor a_w folded
-  // into y (sqq_s = sqrt(q) a_w), the kappa factor a_k per lattice row
-  // (aK, applied per row pair), b_k into the pair factor (ck_s = ck b_k) and
-  // 1/a_w into the pure factor (Pk_s = Pk / a_w); FP32, [nk*nw] (aK [nk])
-  float *sqq_s = nullptr, *Pk_s = nullptr, *ck_s = nullptr, *aK = nullptr;
   void *Ek = nullptr;     // envelope factor along kappa, |d| < nk
   void *Ews = nullptr;    // envelope factor along omega, signed d, offset ew_off
   int ew_off = 0, ew_len = 0;
@@ -267,10 +264,25 @@ int stage_end(srm3_plan *p, int rec);
 int collect_timings(srm3_plan *p);
 int check_pairsum_error(srm3_plan *p);
 int sspad_for(int chunk);
-// The separable pair sum (FFT self-convolution, conv.cu) of n samples whose
-// phasor rows y / y0 are laid out for sspad_for(n), on stream st.
-int conv_pairsum_on(srm3_plan *p, cudaStream_t st, int n, const void *y, const void *y0,
-                    void *C_out);
+// The pair sum of n samples as an FFT self-convolution (conv_launch.cuh):
+// phases, convolution and coefficients into C ([2 n][nk][nw], the rows of the
+// plan), on a stream.  Seeds from the host array (passed by value) or from
+// device memory; with sqq_of, pk_of, ck_of (device, per sample) the samples
+// take those factors instead of the plan's.  work: device scratch, at least
+// one sample's grid rows and phasors.
+struct ConvJob {
+  const srm3_plan *plan;
+  cudaStream_t stream;
+  int n;
+  const uint64_t *seeds, *dseeds;
+  const void *const *sqq_of, *const *pk_of, *const *ck_of;
+  void *work;
+  size_t work_bytes;
+  void *C;
+};
+int conv_run_f32(const ConvJob &j);
+int conv_run_f64(const ConvJob &j);
+int conv_run_df(const ConvJob &j);
 int build_w_table(srm3_plan *p, cudaStream_t st);
 // autotuner choices per lattice shape (process-wide): storage (or -1 when
 // the shape was never tuned) and the pair-sum tile's compute warps
@@ -286,13 +298,20 @@ static inline int ilog2_exact(int v) {
   return ((1 << l) == v) ? l : -1;
 }
 
-// The FP32 pair sum may take the separable form (plan tables sqq_s, Pk_s,
-// ck_s, aK): a Gaussian envelope whose factors' exponent range fits (the
-// recursion's separable form), sum interactions only; it does take it while
-// the plan's W is recomputed.
-inline bool pairsum_sep_capable(const srm3_plan *p) {
-  return p->precision == SRM3_FP32 && p->rec_sep && !p->sep && !p->mixed;
+// The plan's pair sum is the self-convolution: separable envelopes always,
+// the Gaussian one unless its W table is stored.
+inline bool conv_now(const srm3_plan *p) {
+  return p->conv && (p->sep || p->storage == SRM3_STORAGE_RECOMPUTE);
 }
-inline bool pairsum_sep_now(const srm3_plan *p) {
-  return pairsum_sep_capable(p) && p->sqq_s && p->storage == SRM3_STORAGE_RECOMPUTE;
+// Device bytes of y rows for sp sheet-samples, the layout of the O(N^2) pair
+// sum; the self-convolution takes the same block as its scratch (room for at
+// least one sample: 64 sheet-samples of rows against the grid rows of two).
+inline size_t y_bytes(const srm3_plan *p, int sp) {
+  return (size_t)p->nk * p->rowstride * sp *
+         (p->precision == SRM3_FP32 ? sizeof(float2) : sizeof(double2));
+}
+inline int conv_sample(const srm3::ConvJob &j) {
+  const srm3_plan *p = j.plan;
+  if (p->precision == SRM3_FP64) return srm3::conv_run_f64(j);
+  return p->sep ? srm3::conv_run_f32(j) : srm3::conv_run_df(j);
 }

@@ -1,0 +1,71 @@
+"""The pair sum as an FFT self-convolution (Gaussian envelope with W recomputed,
+FP32 plans in double-float and FP64 plans in FP64) where it can go wrong: grids
+just below, at and past a power of two, one-row and one-column lattices, more
+samples than the scratch holds at a time, the widest range of the envelope's
+factors that takes this form, a biphase, and mixed-sign interactions with
+power at omega = 0.  Coefficients against the FP64 oracle at the tolerances
+of the O(N^2) forms (tests/test_gpu_parity.py): 2e-6 of max|C| in FP32, whose
+phasors are FP32, 1e-11 in FP64."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2310_03979_gb300 import srm3
+from paper_2310_03979_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 2e-6, "fp64": 1e-11}
+pow2 = lambda n: 1 << max(1, (n - 1).bit_length())  # noqa: E731
+
+
+def _case(nk, nw, precision, sigma_g=0.25, beta=0.0, interactions="sum"):
+    return replace(W.small_case(nk=nk, nw=nw, nx=pow2(max(2, nk)), nt=pow2(max(2, 2 * nw)),
+                                precision=precision, sigma_g=sigma_g, beta=beta),
+                   interactions=interactions)
+
+
+def _cplx(C):
+    C = C.cpu().numpy()
+    return C[..., 0] + 1j * C[..., 1]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("nk,nw,sigma_g,beta,interactions", [
+    (1, 9, 0.25, 0.0, "sum"), (9, 1, 0.25, 0.0, "sum"), (2, 2, 0.25, 0.3, "sum"),
+    (16, 16, 0.25, 0.0, "sum"), (17, 33, 0.25, 1.1, "sum"), (33, 17, 0.6, 0.0, "sum"),
+    (8, 129, 0.25, 0.0, "sum"), (64, 32, 0.225, 0.0, "sum"), (40, 64, 0.225, 2.0, "sum"),
+    (1, 9, 0.25, 0.0, "mixed"), (9, 2, 0.25, 0.5, "mixed"), (11, 22, 0.25, 0.0, "mixed"),
+    (12, 43, 0.225, 0.7, "mixed"),
+])
+def test_coefficients_against_oracle(oracle_lib, precision, nk, nw, sigma_g, beta, interactions):
+    wl = _case(nk, nw, precision, sigma_g, beta, interactions)
+    S = oracle.kaimal_lorentzian(nk, nw, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    S[:, 0] = 0.4 * S.max() / (1.0 + np.arange(nk))  # power at omega = 0 as well
+    S[nk // 2, nw // 2] = 0.0
+    mixed = interactions == "mixed"
+    eps = 0.1
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=eps, beta=beta, mixed=mixed,
+                          env=oracle.Envelope("gauss", sigma_g))
+    with srm3.Plan.create(wl, table=S, eps=eps) as p:
+        C = _cplx(p.coeffs([3, 11]))
+        info = p.info()
+        assert bool(info.recursion_flags & srm3.SRM3_PAIRSUM_SEPARABLE) == (precision == "fp32")
+    for i, s in enumerate((3, 11)):
+        ref = op.coeffs(s)
+        assert np.abs(C[i] - ref).max() <= TOL[precision] * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision,interactions,n", [("fp32", "sum", 100), ("fp32", "mixed", 100),
+                                                      ("fp64", "sum", 100)])
+def test_samples_do_not_depend_on_the_scratch(precision, interactions, n):
+    """A lattice one past a power of two, whose padded rows are four times as
+    long: the scratch takes fewer samples at a time than the call has."""
+    wl = _case(24, 65, precision, interactions=interactions)
+    with srm3.Plan.create(wl, eps=0.4) as p:
+        C = p.coeffs(list(range(1, n + 1)))
+        for j in (0, 41, 42, n - 1):
+            assert torch.equal(C[j], p.coeffs([j + 1])[0])
