@@ -303,19 +303,20 @@ __host__ __device__ constexpr unsigned tx_in_mask(int R, int nz) {
                                    : ((1u << nz) - 1u) | (((1u << nz) - 1u) << (R - nz));
 }
 
-// Pass plan of a length-2^l transform: ceil(l / 4) passes, pass p of radix
-// 2^tx_lr(l, p) (larger radices first).
-__host__ __device__ constexpr int tx_npass(int l) { return (l + 3) >> 2; }
-__host__ __device__ constexpr int tx_lr(int l, int p) {
-  return l / tx_npass(l) + (p < l - (l / tx_npass(l)) * tx_npass(l) ? 1 : 0);
+// Pass plan of a length-2^l transform with 2^lv values per thread (16 unless
+// said otherwise): ceil(l / lv) passes, pass p of radix 2^tx_lr(l, p) (larger
+// radices first).
+__host__ __device__ constexpr int tx_npass(int l, int lv = 4) { return (l + lv - 1) / lv; }
+__host__ __device__ constexpr int tx_lr(int l, int p, int lv = 4) {
+  return l / tx_npass(l, lv) + (p < l - (l / tx_npass(l, lv)) * tx_npass(l, lv) ? 1 : 0);
 }
 // Entries of the pass-twiddle table: passes p >= 1 in order, pass p holding
 // w_{Ns R}^{k r} at k R + r (k < Ns, r < R; Ns = the length its earlier
 // passes transformed), so that an item's R twiddles are one contiguous run.
-__host__ __device__ constexpr int tx_twlen(int l) {
+__host__ __device__ constexpr int tx_twlen(int l, int lv = 4) {
   int n = 0, ns = 1;
-  for (int p = 0; p < tx_npass(l); ++p) {
-    ns <<= tx_lr(l, p);
+  for (int p = 0; p < tx_npass(l, lv); ++p) {
+    ns <<= tx_lr(l, p, lv);
     if (p >= 1) n += ns;
   }
   return n;
@@ -325,7 +326,7 @@ __host__ __device__ constexpr int tx_twlen(int l) {
 // which spreads the first pass's stride-R writes over the banks.
 __device__ __forceinline__ int sp16(int i) { return i + (i >> 4); }
 __host__ __device__ constexpr int tx_len(int L) { return L + (L >> 4); }
-__host__ __device__ constexpr int tx_tpt(int L) { return L >= 16 ? L >> 4 : 1; }
+__host__ __device__ constexpr int tx_tpt(int L, int lv = 4) { return L >> lv > 0 ? L >> lv : 1; }
 
 // The R twiddles of one item (16-byte loads; the tables start 16-byte aligned
 // and every run is an even number of entries).
@@ -357,12 +358,12 @@ __device__ __forceinline__ void load_tw(const T2 *__restrict__ p, T2 (&w)[R]) {
 // or with SRCSM from sm itself, in place); else from sm (shared, padded
 // positions).  LAST: outputs to dst(i, v) (global), the upper half of the
 // outputs left out with HALFOUT; with DSTSM, and on every other pass, to sm.
-template <int R, bool FIRST, bool LAST, unsigned VMASK, bool SRCSM, bool DSTSM, bool HALFOUT,
-          typename T2, class Src, class Dst>
+template <int R, int LV, bool FIRST, bool LAST, unsigned VMASK, bool SRCSM, bool DSTSM,
+          bool HALFOUT, typename T2, class Src, class Dst>
 __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
                                               const T2 *__restrict__ twp, T2 *sm, Src &src,
                                               Dst &dst) {
-  constexpr int NI = 16 / R;
+  constexpr int NI = (1 << LV) / R;
   const int LR = L / R;
   T2 v[NI][R];
 #pragma unroll
@@ -431,16 +432,16 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
 // r of L/R inputs, R the first radix; 0 = all).  SRCSM, DSTSM, HALFOUT: see
 // stockham_pass (the first pass's source, the last pass's destination).
 template <int l, int p, unsigned VM0, bool SRCSM = false, bool DSTSM = false,
-          bool HALFOUT = false, typename T2, class Src, class Dst>
+          bool HALFOUT = false, int LV = 4, typename T2, class Src, class Dst>
 __device__ __forceinline__ void stockham_passes(int Ns, int toff, int tpt, int jt,
                                                 const T2 *__restrict__ tw, T2 *sm, Src &src,
                                                 Dst &dst) {
-  if constexpr (p < tx_npass(l)) {
-    constexpr int lr = tx_lr(l, p);
+  if constexpr (p < tx_npass(l, LV)) {
+    constexpr int lr = tx_lr(l, p, LV);
     constexpr unsigned vm = (p == 0 && VM0 != 0u) ? VM0 : tx_in_mask(1 << lr, 0);
-    stockham_pass<(1 << lr), p == 0, p == tx_npass(l) - 1, vm, SRCSM, DSTSM, HALFOUT>(
+    stockham_pass<(1 << lr), LV, p == 0, p == tx_npass(l, LV) - 1, vm, SRCSM, DSTSM, HALFOUT>(
         1 << l, Ns, tpt, jt, tw + toff, sm, src, dst);
-    stockham_passes<l, p + 1, VM0, SRCSM, DSTSM, HALFOUT>(
+    stockham_passes<l, p + 1, VM0, SRCSM, DSTSM, HALFOUT, LV>(
         Ns << lr, p == 0 ? 0 : toff + (Ns << lr), tpt, jt, tw, sm, src, dst);
   }
 }
@@ -452,9 +453,9 @@ template <int l>
 __host__ __device__ constexpr unsigned tx_mask_ends(int nz) {
   return tx_in_mask(1 << tx_lr(l, 0), nz);
 }
-template <int l>
+template <int l, int lv = 4>
 __host__ __device__ constexpr unsigned tx_mask_low_half() {
-  return (1u << ((1 << tx_lr(l, 0)) / 2)) - 1u;
+  return (1u << ((1 << tx_lr(l, 0, lv)) / 2)) - 1u;
 }
 
 // Stage 1: TC columns m0 + c of one coefficient set per CTA (blockIdx.y =

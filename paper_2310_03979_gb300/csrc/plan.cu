@@ -6,13 +6,16 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <cstdlib>
+#include <functional>
 #include <mutex>
 #include <numeric>
 #include <unordered_map>
 
 #include "recursion.cuh"
+#include "solve.cuh"
 #include "srm3_internal.cuh"
 
 namespace srm3 {
@@ -36,23 +39,27 @@ int cuda_fail(cudaError_t e, const char *what) {
 // Discretisation: Kaimal S(omega) (Eq. kaimal_spectrum) times the normalised
 // Lorentzian a/(pi (a^2 + kappa^2)), a = lam omega / (2 pi U); S := 0 where
 // omega = 0 (Sec. 5).
+// A thread takes an omega and every gridDim.y-th kappa row: the factors of omega
+// (a logarithm and a power in FP64) are formed once per thread, not per point
+// (256 x 512: 55 -> 8 us).
 __global__ void k_discretise_kaimal(int nk, int nw, double dk, double dw, double U,
                                     double z, double z0, double kvk, double lam,
                                     double *S) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nk * nw) return;
-  int kk = idx / nw, kw = idx - kk * nw;
-  double val = 0.0;
+  const int kw = blockIdx.x * blockDim.x + threadIdx.x;
+  if (kw >= nw) return;
+  const double pi = 3.14159265358979323846;
+  double kaimal = 0.0, a = 0.0;
   if (kw > 0) {
-    const double pi = 3.14159265358979323846;
-    double kappa = kk * dk, omega = kw * dw;
-    double ustar = kvk * U / log(z / z0);
-    double kaimal = 0.5 * (200.0 / (2.0 * pi)) * ustar * ustar * (z / U) /
-                    pow(1.0 + 50.0 * omega * z / (2.0 * pi * U), 5.0 / 3.0);
-    double a = lam * omega / (2.0 * pi * U);
-    val = kaimal * (a / (pi * (a * a + kappa * kappa)));
+    const double omega = kw * dw;
+    const double ustar = kvk * U / log(z / z0);
+    kaimal = 0.5 * (200.0 / (2.0 * pi)) * ustar * ustar * (z / U) /
+             pow(1.0 + 50.0 * omega * z / (2.0 * pi * U), 5.0 / 3.0);
+    a = lam * omega / (2.0 * pi * U);
   }
-  S[idx] = val;
+  for (int kk = blockIdx.y; kk < nk; kk += gridDim.y) {
+    const double kappa = kk * dk;
+    S[(size_t)kk * nw + kw] = kw > 0 ? kaimal * (a / (pi * (a * a + kappa * kappa))) : 0.0;
+  }
 }
 
 // Squared envelope factors for the recursion: g^2 = EkSq[|ik-jk|] EwSq[|iw-jw|]
@@ -302,19 +309,19 @@ __global__ void k_env(int len, int off, double sigma_n, T *out) {
 // and nt / 2 (tx_twlen entries each: pass p >= 1 of the length-2^l transform
 // holds w_{Ns R}^{k r} at k R + r), then e^{2 pi i m / nt}, m < nt / 2.
 template <typename T2>
-__global__ void k_tx_twiddles(int lx, int lm, T2 *tw) {
+__global__ void k_tx_twiddles(int lx, int lm, T2 *tw, int vx = 4, int vm = 4) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n1 = tx_twlen(lx), n2 = tx_twlen(lm), M = 1 << lm;
+  const int n1 = tx_twlen(lx, vx), n2 = tx_twlen(lm, vm), M = 1 << lm;
   if (e >= n1 + n2 + M) return;
   long long num = 0, den = 1;  // angle 2 pi num / den
   if (e >= n1 + n2) {
     num = e - n1 - n2;
     den = 2 * M;
   } else {
-    const int l = e < n1 ? lx : lm;
-    int q = e < n1 ? e : e - n1, ns = 1 << tx_lr(l, 0);
-    for (int p = 1; p < tx_npass(l); ++p) {
-      const int R = 1 << tx_lr(l, p);
+    const int l = e < n1 ? lx : lm, lv = e < n1 ? vx : vm;
+    int q = e < n1 ? e : e - n1, ns = 1 << tx_lr(l, 0, lv);
+    for (int p = 1; p < tx_npass(l, lv); ++p) {
+      const int R = 1 << tx_lr(l, p, lv);
       if (q < ns * R) {
         num = (long long)(q / R) * (q % R);
         den = (long long)ns * R;
@@ -424,7 +431,8 @@ static constexpr int kSumSlot = 8 + 4 * kPlanes - 1;
 // reuse when the plan is destroyed: page-locking costs ~0.1 ms, a tenth of
 // the build of a small plan.
 static constexpr size_t kPinErrOff = (8 + 4 * kPlanes) * sizeof(double);
-static constexpr size_t kPinBytes = kPinErrOff + (kPlanes + 1) * sizeof(int);
+static constexpr size_t kPinCtlOff = (kPinErrOff + (kPlanes + 1) * sizeof(int) + 15) / 16 * 16;
+static constexpr size_t kPinBytes = kPinCtlOff + sizeof(SolveCtl);
 static std::mutex g_pin_mu;
 static std::vector<void *> g_pin_free;
 
@@ -537,9 +545,38 @@ static int rec_occupancy(int dev, RecOccupancy *out) {
   return SRM3_OK;
 }
 
-// Device state of the persistent recursion pass.
+// Sum of S (the exact variance) into the pinned scalars, read after the next
+// synchronisation of the stream; the plane-0 results of this reduction are
+// not used.
+static int start_sum_S(srm3_plan *p, cudaStream_t st) {
+  SRM3_CUDA(cudaMemsetAsync(p->sb2, 0, (size_t)p->nk * p->nw * sizeof(double), st));
+  if (int rc = reduce_plane0(p, st)) return rc;
+  SRM3_CUDA(cudaMemcpyAsync(p->h_pinned + kSumSlot, p->scal + 11, sizeof(double),
+                            cudaMemcpyDeviceToHost, st));
+  p->sumS = -1.0;  // not read yet
+  return SRM3_OK;
+}
+
+// Device state of the persistent recursion pass, built when a plan first
+// runs one (the whole-lattice solve does without).
 static int setup_recursion(srm3_plan *p, cudaStream_t st) {
+  if (p->rec_bar) return SRM3_OK;
   const int nk = p->nk, nw = p->nw;
+  const size_t nl = (size_t)nk * nw;
+  SRM3_CUDA(dev_alloc(&p->qm32, kPlanes * nl * sizeof(float), st));
+  SRM3_CUDA(cudaMemsetAsync(p->qm32, 0, kPlanes * nl * sizeof(float), st));
+  if (p->rec_sep) {  // h = a^2 q of the FP64 passes
+    SRM3_CUDA(dev_alloc(&p->qh, nl * sizeof(double), st));
+    SRM3_CUDA(cudaMemsetAsync(p->qh, 0, nl * sizeof(double), st));
+  }
+  if (p->rec_sep && !p->sep && !p->rs_a2) {
+    // the Gaussian envelope's factors for the pass
+    SRM3_CUDA(dev_alloc(&p->rs_a2, nl * sizeof(double), st));
+    SRM3_CUDA(dev_alloc(&p->rs_b2, nl * sizeof(double), st));
+    k_gauss_sep<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, p->sigma_g * nk, p->sigma_g * nw, p->rs_a2,
+                                               p->rs_b2);
+    p->n_launch += 1;
+  }
   const int nlev = nk + nw - 1;
   // first point of each level, and the first bulk pair of each (phase, row)
   std::vector<int> lev_off(nlev + 1, 0);
@@ -611,14 +648,6 @@ static int setup_recursion(srm3_plan *p, cudaStream_t st) {
       p->n_launch += 2;
     }
   }
-  // sum of S (the exact variance), once, read after the next synchronisation
-  // of the stream (run_pass_multi); the plane-0 results of this reduction
-  // are not used
-  SRM3_CUDA(cudaMemsetAsync(p->sb2, 0, (size_t)nk * nw * sizeof(double), st));
-  if (int rc0 = reduce_plane0(p, st)) return rc0;
-  SRM3_CUDA(cudaMemcpyAsync(p->h_pinned + kSumSlot, p->scal + 11, sizeof(double),
-                            cudaMemcpyDeviceToHost, st));
-  p->sumS = -1.0;  // not read yet
   // barrier counter, two tickets per bulk phase (its points of the next
   // fringe block, then the others), and the fringe progress of every
   // lattice row
@@ -646,6 +675,7 @@ static int start_w_table(srm3_plan *p, cudaStream_t st);
 
 static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M, bool fp64,
                           PassResult *r) {
+  if (int rc0 = setup_recursion(p, st)) return rc0;
   for (int m = 0; m < M; ++m) p->h_pinned[m] = x[m] * p->dkdw;
   SRM3_CUDA(cudaMemcpyAsync(p->scal, p->h_pinned, M * sizeof(double), cudaMemcpyHostToDevice, st));
   SRM3_CUDA(cudaMemsetAsync(p->err, 0, (kPlanes + 1) * sizeof(int), st));
@@ -739,6 +769,336 @@ static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M,
 
 static int run_pass(srm3_plan *p, cudaStream_t st, double x, bool fp64, PassResult *r) {
   return run_pass_multi(p, st, &x, 1, fp64, r);
+}
+
+// ---------------------------------------------------------------------------
+// Eq. pure on the whole lattice at once (solve.cuh).
+
+// The squared envelope factors per axis, centred at a quarter of the lattice
+// (k_conv_factors, squared), in FP64 and in the transform's type.
+template <typename F>
+__global__ void k_solve_factors(int nk, int nw, double sk, double sw, double *__restrict__ fac,
+                                F *__restrict__ ffac) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int oa = 2 * nk, ob = 2 * nk + 2 * nw - 1;  // aK, bK, aW, bW
+  const double ck = 0.25 * (nk - 1), cw = 0.25 * (nw - 1);
+  auto put = [&](int j, double v) {
+    fac[j] = v;
+    ffac[j] = F(v);
+  };
+  if (i < nk) {
+    const double u = (i - ck) / sk, v = (i - 2.0 * ck) / sk;
+    put(i, exp(-2.0 * u * u));
+    put(nk + i, exp(v * v));
+  }
+  if (i < 2 * nw - 1) {
+    const double u = (i - (nw - 1) - cw) / sw;
+    put(oa + i, exp(-2.0 * u * u));
+  }
+  if (i < nw) {
+    const double v = (i - 2.0 * cw) / sw;
+    put(ob + i, exp(v * v));
+  }
+}
+
+// n doubles in the transform's type.
+template <typename F>
+__global__ void k_solve_convert(long long n, const double *__restrict__ in, F *__restrict__ out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = F(in[i]);
+}
+
+// sum_b2 = X g and q = 1/(1 - sum_b2) (0 where S = 0 or sum_b2 >= 1, which
+// also sets ctl->err) from the last g of a solve of nit launched iterations,
+// with the maximum and the solve's outcome in ctl.  Stage 1: g from the
+// iterations (F), kept in FP64 in g64, X theirs; gmax over the points that
+// k_solve_low leaves.  Stage 2: g64, X from gmax where the target is given.
+constexpr int kSolveLow = 2048;
+
+template <typename F>
+__global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArgs A, int nit,
+                                                     int stage, int low, double *__restrict__ g64,
+                                                     double *__restrict__ sb2,
+                                                     double *__restrict__ q) {
+  __shared__ double sX;
+  if (threadIdx.x < 32) {  // the first iteration whose change is within tol
+    int first = nit;
+    for (int j = 1 + A.hold + threadIdx.x; j < nit; j += 32)
+      if (as_double(A.ctl->chg[j]) <= A.tol) {
+        first = j;
+        break;
+      }
+    for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
+    if (threadIdx.x == 0) {
+      const int last = min(first, nit - 1);
+      sX = solve_X(A, last);
+      const double gm = as_double(A.ctl->gmax);
+      if (stage == 2 && A.target > 0.0) sX = gm > 0.0 ? A.target / gm : 0.0;
+      if (blockIdx.x == 0) {
+        A.ctl->X = sX;
+        A.ctl->last = last;
+        A.ctl->converged = first < nit;
+      }
+    }
+  }
+  __syncthreads();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  double v = 0.0, g = 0.0;
+  bool direct = false;
+  if (i < n) {
+    const bool pos = A.S[i] > 0.0;
+    if (stage == 1) {
+      const int kk = (int)(i / A.nw), kw = (int)(i - (long long)kk * A.nw);
+      direct = low && (long long)(kk + 1) * (kw + 1) <= kSolveLow;
+      g64[i] = g = solve_real(static_cast<const F *>(A.g)[i]);
+    } else {
+      g = g64[i];
+    }
+    v = pos ? sX * g : 0.0;
+    sb2[i] = v;
+    q[i] = pos && v < 1.0 ? 1.0 / (1.0 - v) : 0.0;
+    if (stage == 2 && !(v < 1.0)) atomicOr(&A.ctl->err, 1);
+  }
+  if (stage == 1)
+    warp_atomic_max(&A.ctl->gmax, direct ? 0.0 : g);
+  else
+    warp_atomic_max(&A.ctl->max_sb2, v);
+}
+
+// g of the points with few pairs, (kk + 1)(kw + 1) <= kSolveLow, summed
+// directly in FP64 from the solve's q: their sums are small, and a
+// transform's rounding is not relative to them.  One warp per point, up to 8
+// points of a lattice row per CTA (solve_low_ctas); e2, b2: the separable tables
+// in FP64, or NULL and fac the Gaussian envelope's.  256 x 512: 20 M products.
+__host__ __device__ inline int solve_low_ctas(int kk, int nw) {
+  const int n = kSolveLow / (kk + 1) < nw ? kSolveLow / (kk + 1) : nw;
+  return (n + 7) / 8;
+}
+
+__global__ void __launch_bounds__(256) k_solve_low(const SolveArgs A,
+                                                   const double *__restrict__ e2,
+                                                   const double *__restrict__ b2,
+                                                   const double *__restrict__ fac,
+                                                   const double *__restrict__ q,
+                                                   double *__restrict__ g64) {
+  const int lane = threadIdx.x & 31, nw = A.nw;
+  // CTA -> (row, chunk of 8 omega): rows in order, solve_low_ctas(row) each
+  int kk = 0, j = blockIdx.x;
+  for (int c; j >= (c = solve_low_ctas(kk, nw)); ++kk) j -= c;
+  const int kw = j * 8 + (threadIdx.x >> 5);
+  if (kw >= min(nw, kSolveLow / (kk + 1))) return;
+  const double *aK = fac, *bK = fac + A.nk, *aW = fac + 2 * A.nk + nw - 1, *bW = aW + nw;
+  const int W = kw + 1, rows = kk / 2 + 1, da = 32 / W, dw = 32 % W;
+  double t = 0.0;
+  int a = lane / W, iw = lane % W;
+  while (a < rows) {
+    const int b = kk - a, jw = kw - iw;
+    if (!((a == 0 && iw == 0) || iw > ((a == b) ? kw / 2 : kw))) {
+      const size_t i = (size_t)a * nw + iw, jj = (size_t)b * nw + jw;
+      const double w = e2 ? e2[i] * e2[jj] : (aK[a] * aW[iw]) * (aK[b] * aW[jw]);
+      t = fma(w, q[i] * q[jj], t);
+    }
+    a += da;
+    iw += dw;
+    if (iw >= W) {
+      iw -= W;
+      ++a;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const size_t k = (size_t)kk * nw + kw;
+  const double g = A.S[k] > 0.0 ? (b2 ? b2[k] : bK[kk] * bW[kw]) * t : 0.0;
+  if (lane == 0) {
+    g64[k] = g;
+    if (g > 0.0) atomicMax(&A.ctl->gmax, (unsigned long long)__double_as_longlong(g));
+  }
+}
+
+// The first iterate from a solve on the lattice of every fk-th kappa and
+// fw-th omega point: its sum_b2, linear between the points.
+__global__ void k_solve_prolong(int nk, int nw, int fk, int fw, int nkc, int nwc,
+                                const double *__restrict__ sc, double *__restrict__ s) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nk * nw) return;
+  const int kk = i / nw, kw = i - kk * nw;
+  const int k0 = min(kk / fk, nkc - 1), w0 = min(kw / fw, nwc - 1);
+  const int k1 = min(k0 + 1, nkc - 1), w1 = min(w0 + 1, nwc - 1);
+  const double tk = (double)(kk - k0 * fk) / fk, tw = (double)(kw - w0 * fw) / fw;
+  const double uk = fmin(tk, 1.0), uw = fmin(tw, 1.0);
+  const double lo = sc[k0 * nwc + w0] + uw * (sc[k0 * nwc + w1] - sc[k0 * nwc + w0]);
+  const double hi = sc[k1 * nwc + w0] + uw * (sc[k1 * nwc + w1] - sc[k1 * nwc + w0]);
+  s[i] = lo + uk * (hi - lo);
+}
+
+int solve_iterate_df(const SolveArgs &A, int it, int device, int nsm, cudaStream_t st);
+int solve_iterate_f64(const SolveArgs &A, int it, int device, int nsm, cudaStream_t st);
+
+struct SolveResult {
+  bool converged;
+  double x, max_sb2;  // eps^2, max_k sum_b2
+  int its, err;
+  bool no_pairs;
+};
+
+// Iterations launched per further look of the host.
+static constexpr int kSolveMore = 5;
+// largest change of s at which the solve stops: the coarse
+// lattice's, and the root estimate the FP64 passes of FP64 plans start from
+// (their reach is 1e-5); the tables of FP32 plans (target met to 1e-9), in
+// double-float; those of separable bispectra, in FP64
+static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-11, kSolveF64 = 1e-12;
+
+// The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
+// target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
+// widths in lattice units.  from: a solved coarser plan (every fk-th, fw-th
+// point) to start from, or NULL.
+static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x, double sk,
+                         double sw, bool fp64, double tol, const srm3_plan *from, int fk, int fw,
+                         SolveResult *r) {
+  const int hold = 3;
+  const int nk = p->nk, nw = p->nw;
+  const long long nl = (long long)nk * nw;
+  int lk = 1, lw = 2;
+  while ((1 << lk) < 2 * nk - 1) ++lk;
+  while ((1 << lw) < (p->mixed ? 3 * nw - 2 : 2 * nw - 1)) ++lw;
+  const int lm = lw - 1, M = 1 << lm, nfac = 2 * nk + 3 * nw - 1;
+  const int vk = solve_lv(lk), vm = solve_lv(lm);
+  const int ntw = tx_twlen(lk, vk) + tx_twlen(lm, vm) + M;
+  auto up = [](size_t b) { return (b + 15) / 16 * 16; };
+  const size_t zb = (size_t)nk * M * 16, lb = up((size_t)nl * 8), tb = (size_t)ntw * 16;
+  const size_t fb = up((size_t)nfac * 8);
+  char *blk = nullptr, *at = nullptr;
+  SRM3_CUDA(dev_alloc((void **)&blk, zb + (p->sep ? 6 : 4) * lb + tb + 2 * fb + sizeof(SolveCtl), st));
+  struct Guard {
+    char *b;
+    cudaStream_t st;
+    ~Guard() { dev_free(b, st); }
+  } guard{blk, st};
+  at = blk;
+  auto take = [&](size_t b) {
+    char *q = at;
+    at += b;
+    return q;
+  };
+  SolveArgs A;
+  std::memset(static_cast<void *>(&A), 0, sizeof(A));
+  A.nk = nk;
+  A.nw = nw;
+  A.Nk = 1 << lk;
+  A.M = M;
+  A.mixed = p->mixed ? 1 : 0;
+  A.S = p->S;
+  A.Z = take(zb);
+  A.g = take(lb);
+  double *g64 = reinterpret_cast<double *>(take(lb));
+  char *s[2] = {take(lb), take(lb)};
+  char *tw = take(tb);
+  A.ctl = reinterpret_cast<SolveCtl *>(take(sizeof(SolveCtl)));
+  A.twk = tw;
+  A.twm = tw + (size_t)tx_twlen(lk, vk) * 16;
+  A.twz = tw + (size_t)(tx_twlen(lk, vk) + tx_twlen(lm, vm)) * 16;
+  SRM3_CUDA(cudaMemsetAsync(A.ctl, 0, sizeof(SolveCtl), st));
+  double *fac = nullptr;
+  if (p->sep) {
+    const double *t[2] = {p->env_e2, p->env_b2};
+    const void *c[2];
+    for (int j = 0; j < 2; ++j) {
+      char *o = take(lb);
+      if (fp64) {
+        c[j] = t[j];
+      } else {
+        k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, t[j], reinterpret_cast<df *>(o));
+        c[j] = o;
+        p->n_launch += 1;
+      }
+    }
+    A.e2 = c[0];
+    A.b2 = c[1];
+  } else {
+    fac = reinterpret_cast<double *>(take(fb));
+    char *f = fp64 ? reinterpret_cast<char *>(fac) : take(fb);
+    const int m = cdiv(std::max(nk, 2 * nw - 1), 256);
+    if (fp64)
+      k_solve_factors<double><<<m, 256, 0, st>>>(nk, nw, sk, sw, fac, fac);
+    else
+      k_solve_factors<df><<<m, 256, 0, st>>>(nk, nw, sk, sw, fac, reinterpret_cast<df *>(f));
+    p->n_launch += 1;
+    A.aK = f;
+    A.bK = f + (size_t)nk * 8;
+    A.aW = f + (size_t)2 * nk * 8;
+    A.bW = f + (size_t)(2 * nk + 2 * nw - 1) * 8;
+  }
+  if (fp64)
+    k_tx_twiddles<double2><<<cdiv(ntw, 256), 256, 0, st>>>(lk, lm, (double2 *)tw, vk, vm);
+  else
+    k_tx_twiddles<df2><<<cdiv(ntw, 256), 256, 0, st>>>(lk, lm, (df2 *)tw, vk, vm);
+  A.target = target;
+  A.X = x * p->dkdw;
+  A.w = target > 0.0 ? 0.75 : 1.0;
+  A.tol = tol;
+  if (from) {
+    k_solve_prolong<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, fk, fw, from->nk, from->nw, from->sb2,
+                                                   g64);
+    if (fp64)
+      k_solve_convert<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (double *)s[0]);
+    else
+      k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (df *)s[0]);
+    A.warm = 1;
+    A.hold = from == p ? 0 : hold;
+    p->n_launch += 2;
+  }
+  SRM3_CUDA(cudaGetLastError());
+  RecOccupancy occ;
+  if (int rc = rec_occupancy(p->device, &occ)) return rc;
+  SolveCtl *h = reinterpret_cast<SolveCtl *>(reinterpret_cast<char *>(p->h_pinned) + kPinCtlOff);
+  const int low = p->mixed ? 0 : 1;  // (with difference pairs no point has few)
+  auto final = [&](int nit, int stage) {
+    if (fp64)
+      k_solve_final<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, nit, stage, low, g64, p->sb2, p->qm);
+    else
+      k_solve_final<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, nit, stage, low, g64, p->sb2, p->qm);
+  };
+  int nlow = 0, nit = 0;
+  for (int kk = 0; kk < std::min(nk, kSolveLow); ++kk) nlow += solve_low_ctas(kk, nw);
+  // iterations launched before the host looks, from how long they take (a
+  // converged solve's later launches return at once): the damped ones from
+  // scratch, from a coarser lattice's solution or from this lattice's own
+  const int first = from == p ? 6 : tol >= kSolveLoose ? 16 : from ? 19 : 20;
+  do {
+    const int upto = std::min(kSolveMaxIt, nit + (nit == 0 ? first : kSolveMore));
+    for (; nit < upto; ++nit) {
+      A.s_in = s[nit & 1];
+      A.s_out = s[(nit + 1) & 1];
+      const int rc = fp64 ? solve_iterate_f64(A, nit, p->device, occ.nsm, st)
+                          : solve_iterate_df(A, nit, p->device, occ.nsm, st);
+      if (rc) return rc;
+    }
+    // (again after a further look: the results of the first one are overwritten)
+    SRM3_CUDA(cudaMemsetAsync(&A.ctl->X, 0, sizeof(SolveCtl) - offsetof(SolveCtl, X), st));
+    final(nit, 1);
+    if (low)
+      k_solve_low<<<nlow, 256, 0, st>>>(
+          A, p->sep ? p->env_e2 : nullptr, p->sep ? p->env_b2 : nullptr, fac, p->qm, g64);
+    final(nit, 2);
+    SRM3_CUDA(cudaGetLastError());
+    SRM3_CUDA(cudaMemcpyAsync(h, A.ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
+    SRM3_CUDA(cudaStreamSynchronize(st));
+    if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];  // copied by start_sum_S
+  } while (!h->converged && nit < kSolveMaxIt);
+  p->n_launch += 1 + 3 * nit + 2 + low;
+  r->converged = h->converged != 0 && h->X >= 0.0 && std::isfinite(h->X);
+  r->x = h->X / p->dkdw;
+  std::memcpy(&r->max_sb2, &h->max_sb2, sizeof(double));
+  r->its = h->last;
+  r->err = h->err;
+  r->no_pairs = h->maxg[0] == 0 && target > 0.0;
+#ifdef SRM3_SOLVE_DEBUG
+  fprintf(stderr, "solve %dx%d mixed %d sep %d fp64 %d target %g warm %d: conv %d its %d x %.15g max %.17g\n", nk, nw,
+          A.mixed, p->sep, fp64, target, A.warm, h->converged, h->last, r->x, r->max_sb2);
+  for (int j = 1; j <= h->last; ++j) { double c; std::memcpy(&c, &h->chg[j], 8); fprintf(stderr, " %.1e", c); }
+  fprintf(stderr, "\n");
+#endif
+  return SRM3_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1004,6 +1364,7 @@ static int linear_bound(srm3_plan *p, cudaStream_t st, double *Lmax) {
     *Lmax = r0[0].max_sb2 / xt;
     return SRM3_OK;
   }
+  if (int rc0 = setup_recursion(p, st)) return rc0;
   const int nblk = cdiv(p->nw, kLinOut);
   const size_t smem = (size_t)3 * p->nw * sizeof(float);
   const long long nl = (long long)p->nk * p->nw;
@@ -1161,14 +1522,18 @@ __global__ void k_subsample(int nw, int fk, int fw, int nkc, int nwc, const doub
 // The root of the FP32 search on the coarse lattice into *xc (-1: the
 // lattice is too small for a coarse start).  The coarse plan borrows the
 // plan's pinned host scalars; its device state is freed in stream order.
-static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc) {
+// For plans that take the whole-lattice solve (warm != NULL) it is that solve
+// on the coarse lattice, and its tables start the one on this lattice, which
+// *warm receives.
+static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc,
+                       const std::function<int(const srm3_plan *, int, int)> *warm) {
   *xc = -1.0;
   int fk = 1, fw = 1;
   while (p->nk / (2 * fk) >= kCoarseMinDim) fk *= 2;
   while (p->nw / (2 * fw) >= kCoarseMinDim) fw *= 2;
   if ((long long)p->nk * p->nw < kCoarsePoints || fk * fw < 4) return SRM3_OK;
   // the sum of S of this plan, copied to the shared pinned slot by
-  // setup_recursion, is read before the coarse plan reuses the slot
+  // start_sum_S, is read before the coarse plan reuses the slot
   SRM3_CUDA(cudaStreamSynchronize(st));
   if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];
   srm3_plan c;
@@ -1182,6 +1547,7 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
   c.rec_sep = p->rec_sep;
   c.sep = p->sep;
   c.sigma_g = p->sigma_g;
+  c.solve = p->solve;
   c.h_pinned = p->h_pinned;
   c.h_err = p->h_err;
   struct Cleanup {
@@ -1193,7 +1559,7 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
                      c->G2_32,    c->rs_a2,     c->rs_b2,   c->qm3,          c->rec_items,
                      c->rec_lev_off, c->rec_pairs, c->rec_pair_off, c->rec_partial,
                      c->rec_max,  c->rec_bar,   c->red_part, c->env_e2,      c->env_b2,
-                     c->rec_z,    c->tw_rec32,  c->tw_rec64};
+                     c->qh,       c->rec_z,    c->tw_rec32,  c->tw_rec64,  c->qm};
       for (void *d : dev)
         if (d) dev_free(d, st);
     }
@@ -1215,8 +1581,6 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
   SRM3_CUDA(dev_alloc(&c.sb2, kPlanes * nlc * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.scal, (8 + 4 * kPlanes) * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.err, (kPlanes + 1) * sizeof(int), st));
-  SRM3_CUDA(dev_alloc(&c.qm32, kPlanes * nlc * sizeof(float), st));
-  SRM3_CUDA(cudaMemsetAsync(c.qm32, 0, kPlanes * nlc * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&c.EkSq, nkc * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.EkSq32, nkc * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&c.EwSq, 2 * nwc * sizeof(double), st));
@@ -1233,12 +1597,12 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
     k_subsample<<<cdiv(nlc, 256), 256, 0, st>>>(p->nw, fk, fw, nkc, nwc, p->env_e2, c.env_e2);
     k_subsample<<<cdiv(nlc, 256), 256, 0, st>>>(p->nw, fk, fw, nkc, nwc, p->env_b2, c.env_b2);
     c.n_launch += 2;
-  } else {
+  } else if (!warm) {
     k_env_sq<<<cdiv(nkc, 256), 256, 0, st>>>(nkc, sk, c.EkSq, c.EkSq32);
     k_env_sq<<<cdiv(2 * nwc, 256), 256, 0, st>>>(2 * nwc, sw, c.EwSq, c.EwSq32);
     c.n_launch += 2;
   }
-  if (c.sep) {
+  if (c.sep || warm) {
     // no g^2 table: the separable recursion takes the pair factor from a^2
   } else if (c.rec_sep) {
     SRM3_CUDA(dev_alloc(&c.rs_a2, nlc * sizeof(double), st));
@@ -1249,9 +1613,30 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
     SRM3_CUDA(dev_alloc(&c.G2_32, nlc * sizeof(float), st));
     k_g2<<<cdiv(nlc, 256), 256, 0, st>>>(nkc, nwc, c.EkSq, c.EwSq, c.G2, c.G2_32);
   }
-  c.n_launch += c.sep ? 0 : 1;
+  c.n_launch += c.sep || warm ? 0 : 1;
   SRM3_CUDA(cudaGetLastError());
-  int rc = setup_recursion(&c, st);
+  p->coarse_fk = fk;
+  p->coarse_fw = fw;
+  if (warm) {
+    SRM3_CUDA(dev_alloc(&c.qm, nlc * sizeof(double), st));
+    c.sumS = 0.0;  // not needed here
+    SolveResult r;
+    if (int rc = solve_lattice(&c, st, target, 0.0, sk, sw, false, kSolveLoose, nullptr, 1, 1, &r))
+      return rc;
+    SRM3_CUDA(cudaEventRecord(e1, st));
+    SRM3_CUDA(cudaEventSynchronize(e1));
+    float ms = 0.f;
+    SRM3_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+    p->t_coarse_ms = ms;
+    p->coarse_passes = r.no_pairs ? 0 : 1;
+    p->coarse_launches = c.n_launch;
+    if (r.no_pairs || !r.converged || r.err) return SRM3_OK;
+    *xc = r.x;
+    c.eps = std::sqrt(r.x);
+    return (*warm)(&c, fk, fw);
+  }
+  int rc = start_sum_S(&c, st);
+  if (!rc) rc = setup_recursion(&c, st);
   if (rc) return rc;
   Search32 s;
   s.pts.push_back({0.0, -target});
@@ -1269,8 +1654,6 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc)
   p->t_recursion_ms += c.t_recursion_ms;
   p->coarse_passes = c.root_passes32;
   p->coarse_launches = c.n_launch;
-  p->coarse_fk = fk;
-  p->coarse_fw = fw;
   if (ok) *xc = x;
   return SRM3_OK;
 }
@@ -1280,9 +1663,58 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
   Search32 s;
   s.pts.push_back({0.0, -target});
   p->coarse_start = false;
-  {
+  double xs = -1.0;  // the root, from the whole-lattice solve
+  if (p->solve) {
+    if (p->w_deferred) {  // the W table beside it
+      p->w_deferred = false;
+      if ((rc = start_w_table(p, p->w_stream))) return rc;
+    }
+    const bool tables = p->precision == SRM3_FP32 || p->sep;  // not only the root
+    SolveResult r;
+    std::memset(&r, 0, sizeof(r));
+    auto run = [&](const srm3_plan *from, int fk, int fw) {
+      const double sk = p->sigma_g * p->nk, sw = p->sigma_g * p->nw;
+      const bool f64 = p->sep;  // separable bispectra: finished in FP64
+      int rc1 = solve_lattice(p, st, target, from ? from->eps * from->eps : 0.0, sk, sw, false,
+                              tables && !f64 ? kSolveDf : kSolveLoose, from, fk, fw, &r);
+      if (!rc1 && f64 && r.converged)
+        rc1 = solve_lattice(p, st, target, 0.0, sk, sw, true, kSolveF64, p, 1, 1, &r);
+      return rc1;
+    };
+    const std::function<int(const srm3_plan *, int, int)> warm = run;
     double xc = -1.0;
-    rc = coarse_root(p, st, target, &xc);
+    SRM3_CUDA(cudaEventRecord(t_ev[0], st));
+    if ((rc = coarse_root(p, st, target, &xc, &warm))) return rc;
+    if (!r.converged && (rc = run(nullptr, 1, 1))) return rc;
+    SRM3_CUDA(cudaEventRecord(t_ev[1], st));
+    SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
+    float ms = 0.f;
+    SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
+    if (r.no_pairs)
+      return fail(SRM3_ERR_BISECTION_FAILED, "no bispectral pairs: max_k sum_b2 is 0 for every eps");
+    if (r.converged && !r.err) {
+      p->t_recursion_ms += ms;
+      p->t_rec32_ms += ms - p->t_coarse_ms;
+      p->coarse_start = xc > 0.0 && std::fabs(xc - r.x) <= kCoarseWindow * r.x;
+      if (tables) {
+        p->root_passes32 += 1;  // the solve, and its tables in FP64
+        p->root_passes += 1;
+        p->eps = std::sqrt(r.x);
+        p->max_sb2 = r.max_sb2;
+        p->min_pure = 1.0 - r.max_sb2;
+        p->variance = 4.0 * p->dkdw * p->sumS;
+        p->eps_shifted = !p->sep;
+        return SRM3_OK;
+      }
+      xs = r.x;
+    } else {
+      p->coarse_launches = p->coarse_passes = 0;
+    }
+  }
+  if (xs < 0.0) {
+    if ((rc = setup_recursion(p, st))) return rc;  // which also decides on the bulk's form
+    double xc = -1.0;
+    rc = coarse_root(p, st, target, &xc, nullptr);
     if (rc) return rc;
     if (xc > 0.0) {
       // four planes over the window (its spacing of 1 % still leaves x32
@@ -1300,12 +1732,12 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
       p->coarse_start = j >= 2 && j < s.pts.size() && std::isfinite(s.pts[j].second);
     }
   }
-  if (!p->coarse_start) {
+  if (!p->coarse_start && xs < 0.0) {
     rc = wide_search(p, st, target, s);
     if (rc) return rc;
   }
-  double x32 = 0.0, slope32 = 0.0;
-  const bool hi_ok = root_fp32(s, &x32, &slope32);
+  double x32 = xs, slope32 = 0.0;
+  const bool hi_ok = xs > 0.0 || root_fp32(s, &x32, &slope32);
 
   // Loose targets (FP32 plans, tol >= kShiftTol): the slope in x of every
   // point's sum_b2 at x32, the derivative of the quadratic through the three
@@ -1366,7 +1798,8 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
   // x above the root serves (the linear bound x0, else four times the FP32
   // bracket's upper end).
   const size_t jb = first_above(s);
-  const double xup = s.x0 > 0.0 ? s.x0 : s.pts[std::min(jb, s.pts.size() - 1)].first;
+  const double xup = xs > 0.0 ? xs : s.x0 > 0.0 ? s.x0
+                                                 : s.pts[std::min(jb, s.pts.size() - 1)].first;
   Bracket b{0.0, -target, 4.0 * xup, 1.0, true};
   double xbest = -1.0;
   PassResult best{};
@@ -1568,7 +2001,7 @@ int build_w_table(srm3_plan *p, cudaStream_t st) {
 // Tiles of the FP32 pair sum.  A plan restricted to lattice rows [row_lo,
 // row_hi) (a shard of a k-sharded job) gets W-table space and work units for
 // those rows only.
-static int build_tiles(srm3_plan *p, cudaStream_t st, bool want_table, long long *table_entries) {
+static int build_tiles(srm3_plan *p, cudaStream_t st) {
   const int nk = p->nk;
   p->ntw = cdiv(p->nw, kTileR);
   p->ntiles = nk * p->ntw;
@@ -1610,13 +2043,21 @@ static int build_tiles(srm3_plan *p, cudaStream_t st, bool want_table, long long
     SRM3_CUDA(cudaMemcpyAsync(p->super_order_d, supd.data(), sizeof(int2) * n,
                               cudaMemcpyHostToDevice, st));
   }
-  *table_entries = off[p->ntiles];
-  (void)want_table;  // offsets are kept either way: the autotuner may build W later
+  p->table_entries = off[p->ntiles];
   SRM3_CUDA(dev_alloc(&p->tile_off, sizeof(long long) * p->ntiles, st));
   SRM3_CUDA(cudaMemcpyAsync(p->tile_off, off.data(), sizeof(long long) * p->ntiles,
                             cudaMemcpyHostToDevice, st));
   SRM3_CUDA(cudaStreamSynchronize(st));
   return SRM3_OK;
+}
+
+// The tiles where they are needed: the O(N^2) pair sum and the autotuner
+// (plans whose pair sum is the self-convolution do without: sorting the work
+// units of 512 x 1024 took 1 ms of the host).
+int ensure_tiles(srm3_plan *p, cudaStream_t st) {
+  if (p->tile_off) return SRM3_OK;
+  AllocOwner owner(p);
+  return build_tiles(p, st);
 }
 
 int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs) {
@@ -1652,14 +2093,12 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
   SRM3_CUDA(dev_alloc(&p->scal, (8 + 4 * kPlanes) * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&p->err, (kPlanes + 1) * sizeof(int), st));
   SRM3_CUDA(cudaMemsetAsync(p->qm, 0, nl * sizeof(double), st));
-  SRM3_CUDA(dev_alloc(&p->qm32, kPlanes * nl * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&p->EkSq32, nk * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&p->EwSq32, 2 * nw * sizeof(float), st));
-  SRM3_CUDA(cudaMemsetAsync(p->qm32, 0, kPlanes * nl * sizeof(float), st));
 
   // a1: spectrum on the lattice
   if (sp->kind == SRM3_SPECTRUM_KAIMAL_LORENTZIAN) {
-    k_discretise_kaimal<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, p->dk, p->dw, sp->U, sp->z,
+    k_discretise_kaimal<<<dim3(cdiv(nw, 64), std::min(nk, 64)), 64, 0, st>>>(nk, nw, p->dk, p->dw, sp->U, sp->z,
                                                        sp->z0, sp->k_vk, sp->lam, p->S);
     SRM3_CUDA(cudaGetLastError());
   } else {
@@ -1675,8 +2114,6 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     SRM3_CUDA(dev_alloc(&p->env_e, nl * sizeof(double), st));
     SRM3_CUDA(dev_alloc(&p->env_e2, nl * sizeof(double), st));
     SRM3_CUDA(dev_alloc(&p->env_e32, nl * sizeof(float), st));
-    SRM3_CUDA(dev_alloc(&p->qh, nl * sizeof(double), st));
-    SRM3_CUDA(cudaMemsetAsync(p->qh, 0, nl * sizeof(double), st));
     SRM3_CUDA(cudaMemcpyAsync(p->env_e, bs->env_table, nl * sizeof(double),
                               cudaMemcpyHostToDevice, st));
     k_sep_tables<<<cdiv(nl, 256), 256, 0, st>>>((int)nl, p->env_e, p->env_e2, p->env_e32,
@@ -1697,16 +2134,6 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     }
   } else {
     k_g2<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, p->EkSq, p->EwSq, p->G2, p->G2_32);
-    if (p->rec_sep) {
-      // Gaussian envelope in separable form for the recursion (the sampling
-      // path keeps W = c_k g(i, j))
-      SRM3_CUDA(dev_alloc(&p->rs_a2, nl * sizeof(double), st));
-      SRM3_CUDA(dev_alloc(&p->rs_b2, nl * sizeof(double), st));
-      SRM3_CUDA(dev_alloc(&p->qh, nl * sizeof(double), st));
-      SRM3_CUDA(cudaMemsetAsync(p->qh, 0, nl * sizeof(double), st));
-      k_gauss_sep<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, p->sigma_g * nk, p->sigma_g * nw,
-                                                 p->rs_a2, p->rs_b2);
-    }
   }
   SRM3_CUDA(cudaGetLastError());
 
@@ -1725,25 +2152,22 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     }
   } wguard{&wst};
   if (p->precision == SRM3_FP32 && !p->sep) {
-    long long entries = 0;
-    bool maybe_table = p->storage != SRM3_STORAGE_RECOMPUTE;
-    rc = build_tiles(p, st, maybe_table, &entries);
-    if (rc) return rc;
-    p->table_entries = entries;
-    const double bytes = (double)entries * sizeof(float);
     int tuned_nc = 4;
     const int tuned = tune_cache_lookup(nk, nw, &tuned_nc);
     if (tuned >= 0) p->ps_nc = tuned_nc;  // the tuned tile (results do not depend on it)
     if (p->storage == SRM3_STORAGE_TUNED)  // the autotuner's storage for this lattice
       p->storage = tuned >= 0 ? tuned : SRM3_STORAGE_AUTO;
-    if (p->storage == SRM3_STORAGE_AUTO) {
+    if (p->mixed) p->storage = SRM3_STORAGE_RECOMPUTE;  // the table holds sum pairs only
+    if (p->storage == SRM3_STORAGE_AUTO && p->conv) {
       // W recomputed by the self-convolution is the faster one at every size
       // (conv_launch.cuh; 256 x 512, 64 samples: 2.2 ms against 69 ms with the
       // stored table, whose build and memory it saves too)
-      p->storage = !p->conv && bytes <= p->table_budget ? SRM3_STORAGE_TABLE
-                                                        : SRM3_STORAGE_RECOMPUTE;
+      p->storage = SRM3_STORAGE_RECOMPUTE;
     }
-    if (p->mixed) p->storage = SRM3_STORAGE_RECOMPUTE;  // the table holds sum pairs only
+    if (!conv_now(p) && (rc = ensure_tiles(p, st))) return rc;
+    if (p->storage == SRM3_STORAGE_AUTO)
+      p->storage = (double)p->table_entries * sizeof(float) <= p->table_budget
+                       ? SRM3_STORAGE_TABLE : SRM3_STORAGE_RECOMPUTE;
     if (p->storage == SRM3_STORAGE_TABLE) {
       cudaEvent_t ready;
       SRM3_CUDA(cudaStreamCreateWithFlags(&wst, cudaStreamNonBlocking));
@@ -1764,9 +2188,8 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     p->table_bytes = 0.0;
   }
 
-  // a2: recursion, one graph node per anti-diagonal level
-  rc = setup_recursion(p, st);
-  if (rc) return rc;
+  // a2: Eq. pure
+  if ((rc = start_sum_S(p, st))) return rc;
   if (p->mixed) {
     SRM3_CUDA(dev_alloc(&p->Dsum, nl * sizeof(double), st));
     SRM3_CUDA(dev_alloc(&p->qprev, nl * sizeof(double), st));
@@ -1798,8 +2221,24 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     if (rc) return rc;
   } else {
     PassResult r;
-    rc = run_pass(p, st, bs->eps * bs->eps, true, &r);
-    if (rc) return rc;
+    bool done = false;
+    if (p->sep && p->solve) {
+      SolveResult sr;
+      const double x = bs->eps * bs->eps;
+      rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, false, kSolveLoose, nullptr, 1, 1, &sr);
+      if (!rc && sr.converged && !sr.err)
+        rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr);
+      if (rc) return rc;
+      // a solve that met sum_b2 >= 1 leaves the verdict to the level pass
+      if ((done = sr.converged && !sr.err)) {
+        r.max_sb2 = sr.max_sb2;
+        r.min_pure = 1.0 - sr.max_sb2;
+        r.sumS = p->sumS;
+        r.err = 0;
+        p->root_passes += 1;
+      }
+    }
+    if (!done && (rc = run_pass(p, st, bs->eps * bs->eps, true, &r))) return rc;
     if (r.err)
       return fail(SRM3_ERR_NONPOSITIVE_PURE,
                   "sum_b2 >= 1 at some lattice point: the pure spectrum is not positive");
@@ -2119,6 +2558,7 @@ SRM3_API int srm3_plan_create(const srm3_spectrum *spectrum, const srm3_bispectr
     // multiplied by (e^5 at the limit: 1e-12 of an output in double-float);
     // one padded row and column of the grid have to fit in shared memory
     const int padw = p->mixed ? 3 * g.n_omega - 2 : 2 * g.n_omega - 1;
+    p->solve = (p->sep || E <= kSepExpMax) && 2 * g.n_kappa - 1 <= kMaxFft / 2 && padw <= kMaxFft;
     p->conv = p->sep || (E <= kSepExpMax && 2 * g.n_kappa - 1 <= kMaxFft && padw <= kMaxFft);
   }
   p->beta = bispectrum->beta;

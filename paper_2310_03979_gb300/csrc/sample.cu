@@ -767,6 +767,7 @@ SRM3_API int srm3_autotune(srm3_plan *plan, int n, srm3_tune_result *res) {
     return fail(SRM3_ERR_NOT_SUPPORTED,
                 "mixed plans recompute W: there is no storage to choose");
   int rc = ensure_workspace(plan, n);
+  if (!rc) rc = ensure_tiles(plan, plan->stream);
   if (rc) return rc;
   std::vector<uint64_t> seeds(n);
   for (int j = 0; j < n; ++j) seeds[j] = (uint64_t)j + 1;

@@ -116,6 +116,9 @@ struct srm3_plan {
   int cNk = 0, cNw = 0, log2cNk = 0, log2cNw = 0;
   void *tw_conv = nullptr;
   void *conv_fac = nullptr;
+  // Eq. pure on the whole lattice by self-convolutions (solve.cuh) where the
+  // envelope factors and the grid fits; the plan's tables come from it
+  bool solve = false;
   // mixed-sign interactions: opposite-sheet pairs as well; Eq. pure then
   // a fixed point solved by iterations of (difference sums at the previous
   // iterate, level pass)
@@ -284,6 +287,7 @@ int conv_run_f32(const ConvJob &j);
 int conv_run_f64(const ConvJob &j);
 int conv_run_df(const ConvJob &j);
 int build_w_table(srm3_plan *p, cudaStream_t st);
+int ensure_tiles(srm3_plan *p, cudaStream_t st);
 // autotuner choices per lattice shape (process-wide): storage (or -1 when
 // the shape was never tuned) and the pair-sum tile's compute warps
 int tune_cache_lookup(int nk, int nw, int *nc = nullptr);
