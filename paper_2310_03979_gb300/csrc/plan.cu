@@ -432,7 +432,16 @@ static constexpr int kSumSlot = 8 + 4 * kPlanes - 1;
 // the build of a small plan.
 static constexpr size_t kPinErrOff = (8 + 4 * kPlanes) * sizeof(double);
 static constexpr size_t kPinCtlOff = (kPinErrOff + (kPlanes + 1) * sizeof(int) + 15) / 16 * 16;
-static constexpr size_t kPinBytes = kPinCtlOff + sizeof(SolveCtl);
+// control words of the direct iterations (run_pass_iter): per iteration the
+// bits of the largest relative change of q and of max sum_b2 per plane
+constexpr int kIterMax = 96;
+struct IterCtl {
+  unsigned long long chg[kIterMax];
+  unsigned long long maxb[kIterMax][3];
+  int err[3];
+};
+static constexpr size_t kPinIterOff = (kPinCtlOff + sizeof(SolveCtl) + 15) / 16 * 16;
+static constexpr size_t kPinBytes = kPinIterOff + sizeof(IterCtl);
 static std::mutex g_pin_mu;
 static std::vector<void *> g_pin_free;
 
@@ -621,7 +630,6 @@ static int setup_recursion(srm3_plan *p, cudaStream_t st) {
   SRM3_CUDA(dev_free(d_seg, st));
   // running bulk sums: up to 32 bytes per point (8 FP32 planes or 3 FP64)
   SRM3_CUDA(dev_alloc(&p->rec_partial, (size_t)nk * nw * 32, st));
-  SRM3_CUDA(dev_alloc(&p->rec_max, kPlanes * sizeof(unsigned long long), st));
   // separable envelope: the FFT form of the bulk when its grids fit the
   // pass's shared memory (else the direct bulk, as for any envelope)
   if (p->sep) {
@@ -673,8 +681,238 @@ static int setup_recursion(srm3_plan *p, cudaStream_t st) {
 // or kWindowPlanes without the FFT form of the bulk; writes qm32).
 static int start_w_table(srm3_plan *p, cudaStream_t st);
 
+// fixed point of mixed plans: largest relative change of q, iterations
+constexpr double kFpTol = 4e-16;
+constexpr int kFpMaxIters = 400;
+
+// ---------------------------------------------------------------------------
+// FP64 passes of small lattices: Eq. pure at M given x by iterations over all
+// points at once, every pair summed directly.  A point's sum takes lower
+// points only, so the iterations reach the level pass's fixed point to the
+// last bit or so in about ten steps from q = 1 (six from a solution at a
+// nearby x), each one launch of a few microseconds, where the level pass
+// hands n_kappa + n_omega levels on one after the other (32 x 32: 330 -> 50 us
+// for the three planes).  Taken while the products of ten such steps cost
+// less than the levels (kIterPairs; 4 us a level, 0.35e12 products/s).
+// Mixed interactions add their difference pairs (whose q are not lower
+// points': the iterations then converge geometrically, as the alternating
+// ones do).
+constexpr double kIterPairs = 4e7;
+
+enum { kIterTable = 0, kIterSep = 1, kIterMixed = 2 };
+
+struct IterArgs {
+  int nk, nw;
+  const double *S, *a2, *b2, *G2, *EkSq, *EwSq, *scal;
+  double *sb2, *q;   // [M][nl], and for M = 1 q itself
+  IterCtl *ctl;
+  double tol;
+};
+
+// The first iterate: q of a nearby solution (or NULL: 1 where S > 0), as h =
+// a^2 q in the separable form.
+template <int M, int FORM>
+__global__ void k_iter_init(long long n, const IterArgs A, const double *__restrict__ q0,
+                            double *__restrict__ h) {
+  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  double v = A.S[k] > 0.0 ? (q0 ? q0[k] : 1.0) : 0.0;
+  if (FORM == kIterSep) v = k == 0 ? 0.0 : A.a2[k] * v;
+#pragma unroll
+  for (int m = 0; m < M; ++m) h[k * M + m] = v;
+}
+
+// One warp per point: rows a <= kk/2 laid end to end as a (kw + 1) + iw, the
+// centre row to iw <= kw/2, i = 0 skipped; then the difference pairs.
+template <int M, int FORM>
+__global__ void __launch_bounds__(256) k_iter(const IterArgs A, int it, const double *__restrict__ in,
+                                              double *__restrict__ out) {
+  if (it >= 2 && as_double(A.ctl->chg[it - 1]) <= A.tol) return;
+  const int nw = A.nw, lane = threadIdx.x & 31;
+  const long long nl = (long long)A.nk * nw;
+  const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (k >= nl) return;
+  double acc[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) acc[m] = 0.0;
+  const bool pos = A.S[k] > 0.0;
+  const int kk = (int)(k / nw), kw = (int)(k - (long long)kk * nw);
+  if (pos) {
+    const int W = kw + 1, rows = kk / 2 + 1, da = 32 / W, dw = 32 % W;
+    int a = lane / W, iw = lane % W;
+    while (a < rows) {
+      const int b = kk - a;
+      if (!((a == 0 && iw == 0) || iw > ((a == b) ? kw / 2 : kw))) {
+        const double *hi = in + ((size_t)a * nw + iw) * M;
+        const double *hj = in + ((size_t)b * nw + kw - iw) * M;
+        double w = 1.0;
+        if (FORM != kIterSep) {
+          const int u = 2 * a - kk, v = 2 * iw - kw, au = u < 0 ? -u : u, av = v < 0 ? -v : v;
+          w = FORM == kIterTable ? A.G2[(size_t)au * nw + av] : A.EkSq[au] * A.EwSq[av];
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+          acc[m] = FORM == kIterSep ? fma(hi[m], hj[m], acc[m]) : fma(w, hi[m] * hj[m], acc[m]);
+      }
+      a += da;
+      iw += dw;
+      if (iw >= W) {
+        iw -= W;
+        ++a;
+      }
+    }
+    if (FORM == kIterMixed && kw >= 1 && kw < nw - 1) {
+      const int J = nw - 1 - kw, dj = 32 / J, dr = 32 % J;
+      int ia = lane / J, j = lane % J;
+      while (ia <= kk) {
+        const int jw = 1 + j, u = 2 * ia - kk;
+        const double w = A.EkSq[u < 0 ? -u : u] * A.EwSq[kw + 2 * jw];
+        const double *hi = in + ((size_t)ia * nw + kw + jw) * M;
+        const double *hj = in + ((size_t)(kk - ia) * nw + jw) * M;
+#pragma unroll
+        for (int m = 0; m < M; ++m) acc[m] = fma(w, hi[m] * hj[m], acc[m]);
+        ia += dj;
+        j += dr;
+        if (j >= J) {
+          j -= J;
+          ++ia;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < M; ++m)
+    for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
+  if (lane != 0) return;
+  double chg = 0.0;
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    double s = 0.0, q = 0.0, h = 0.0;
+    if (pos) {
+      s = A.scal[m] * (FORM == kIterSep ? A.b2[k] : 1.0) * acc[m];
+      if (s < 1.0) {
+        q = 1.0 / (1.0 - s);
+      } else {
+        atomicOr(&A.ctl->err[m], 1);
+      }
+      h = FORM == kIterSep ? (k == 0 ? 0.0 : A.a2[k] * q) : q;
+      const double h0 = in[k * M + m];
+      if (h != h0) chg = fmax(chg, fabs(h - h0) / fmax(fabs(h), fabs(h0)));
+      atomicMax(&A.ctl->maxb[it][m], (unsigned long long)__double_as_longlong(s));
+    }
+    out[k * M + m] = h;
+    A.sb2[m * nl + k] = s;
+    if (M == 1) A.q[k] = q;
+  }
+  if (chg > 0.0) atomicMax(&A.ctl->chg[it], (unsigned long long)__double_as_longlong(chg));
+}
+
+static bool iter_small(const srm3_plan *p, int M) {
+  const double T = 0.25 * p->nk * (p->nk + 1.0) * p->nw * (p->nw + 1.0);  // 2 x sum pairs
+  const double D = p->mixed ? 0.25 * p->nk * (p->nk + 1.0) * (p->nw - 1.0) * (p->nw - 2.0) : 0.0;
+  return (0.5 * T + D) * M <= kIterPairs && (!p->sep || p->env_e2);
+}
+
+static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, PassResult *r) {
+  const long long nl = (long long)p->nk * p->nw;
+  const int form = p->mixed ? kIterMixed : p->rec_sep ? kIterSep : kIterTable;
+  if (p->rec_sep && !p->sep && !p->rs_a2) {
+    SRM3_CUDA(dev_alloc(&p->rs_a2, nl * sizeof(double), st));
+    SRM3_CUDA(dev_alloc(&p->rs_b2, nl * sizeof(double), st));
+    k_gauss_sep<<<cdiv(nl, 256), 256, 0, st>>>(p->nk, p->nw, p->sigma_g * p->nk, p->sigma_g * p->nw,
+                                               p->rs_a2, p->rs_b2);
+    p->n_launch += 1;
+  }
+  char *blk = nullptr;
+  const size_t hb = (size_t)nl * M * sizeof(double);
+  SRM3_CUDA(dev_alloc((void **)&blk, 2 * hb + sizeof(IterCtl), st));
+  struct Guard {
+    char *b;
+    cudaStream_t st;
+    ~Guard() { dev_free(b, st); }
+  } guard{blk, st};
+  double *h[2] = {reinterpret_cast<double *>(blk), reinterpret_cast<double *>(blk + hb)};
+  IterArgs A;
+  A.nk = p->nk;
+  A.nw = p->nw;
+  A.S = p->S;
+  A.a2 = p->sep ? p->env_e2 : p->rs_a2;
+  A.b2 = p->sep ? p->env_b2 : p->rs_b2;
+  A.G2 = p->G2;
+  A.EkSq = p->EkSq;
+  A.EwSq = p->EwSq;
+  A.scal = p->scal;
+  A.sb2 = p->sb2;
+  A.q = p->qm;
+  A.ctl = reinterpret_cast<IterCtl *>(blk + 2 * hb);
+  A.tol = p->mixed ? kFpTol : 3e-16;
+  for (int m = 0; m < M; ++m) p->h_pinned[m] = x[m] * p->dkdw;
+  SRM3_CUDA(cudaMemcpyAsync(p->scal, p->h_pinned, M * sizeof(double), cudaMemcpyHostToDevice, st));
+  SRM3_CUDA(cudaEventRecord(t_ev[0], st));
+  IterCtl *hc = reinterpret_cast<IterCtl *>(reinterpret_cast<char *>(p->h_pinned) + kPinIterOff);
+  const double *q0 = p->q_warm ? p->qm : nullptr;
+  auto launch = [&](auto mc, auto fc) {
+    constexpr int Mc = decltype(mc)::value, F = decltype(fc)::value;
+    SRM3_CUDA(cudaMemsetAsync(A.ctl, 0, sizeof(IterCtl), st));
+    k_iter_init<Mc, F><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, q0, h[0]);
+    bool done = false;
+    for (int nit = 0; nit < kIterMax && !done;) {
+      const int upto = std::min(kIterMax, nit + (nit == 0 ? (q0 ? 7 : 12) : 6));
+      for (; nit < upto; ++nit) {
+        k_iter<Mc, F><<<cdiv(nl * 32, 256), 256, 0, st>>>(A, nit, h[nit & 1], h[(nit + 1) & 1]);
+        p->n_launch += 1;
+      }
+      SRM3_CUDA(cudaGetLastError());
+      SRM3_CUDA(cudaEventRecord(t_ev[1], st));
+      SRM3_CUDA(cudaMemcpyAsync(hc, A.ctl, sizeof(IterCtl), cudaMemcpyDeviceToHost, st));
+      SRM3_CUDA(cudaStreamSynchronize(st));
+      int last = 1;
+      for (; last < nit; ++last) {
+        double c;
+        std::memcpy(&c, &hc->chg[last], sizeof(c));
+        if (c <= A.tol) break;
+      }
+      done = last < nit;
+      last = std::min(last, nit - 1);
+      p->fp_iters = last + 1;
+      for (int m = 0; m < Mc; ++m) {
+        std::memcpy(&r[m].max_sb2, &hc->maxb[last][m], sizeof(double));
+        r[m].min_pure = 1.0 - r[m].max_sb2;
+        r[m].sumS = p->sumS < 0.0 ? p->h_pinned[kSumSlot] : p->sumS;
+        r[m].err = hc->err[m];
+        done = done || hc->err[m];
+      }
+    }
+    for (int m = 0; m < Mc; ++m)
+      if (!done) r[m].err = 1;  // no fixed point was reached
+    return SRM3_OK;
+  };
+  using std::integral_constant;
+  auto by_form = [&](auto mc) {
+    if (form == kIterMixed) return launch(mc, integral_constant<int, kIterMixed>{});
+    if (form == kIterSep) return launch(mc, integral_constant<int, kIterSep>{});
+    return launch(mc, integral_constant<int, kIterTable>{});
+  };
+  const int rc = M == 3 ? by_form(integral_constant<int, 3>{}) : by_form(integral_constant<int, 1>{});
+  if (rc) return rc;
+  if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];
+  float ms = 0.f;
+  SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
+  p->t_recursion_ms += ms;
+  p->t_rec64_ms += ms;
+  p->root_passes += 1;
+  return SRM3_OK;
+}
+
 static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M, bool fp64,
                           PassResult *r) {
+  if (fp64 && (M == 1 || M == 3) && iter_small(p, M)) {
+    if (p->w_deferred) {  // the W table, beside the pass
+      p->w_deferred = false;
+      if (int rcw = start_w_table(p, p->w_stream)) return rcw;
+    }
+    return run_pass_iter(p, st, x, M, r);
+  }
   if (int rc0 = setup_recursion(p, st)) return rc0;
   for (int m = 0; m < M; ++m) p->h_pinned[m] = x[m] * p->dkdw;
   SRM3_CUDA(cudaMemcpyAsync(p->scal, p->h_pinned, M * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -821,10 +1059,10 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
                                                      double *__restrict__ sb2,
                                                      double *__restrict__ q) {
   __shared__ double sX;
-  if (threadIdx.x < 32) {  // the first iteration whose change is within tol
+  if (threadIdx.x < 32) {  // the first iteration that was the last
     int first = nit;
-    for (int j = 1 + A.hold + threadIdx.x; j < nit; j += 32)
-      if (as_double(A.ctl->chg[j]) <= A.tol) {
+    for (int j = threadIdx.x; j < nit; j += 32)
+      if (solve_last(A, j)) {
         first = j;
         break;
       }
@@ -946,7 +1184,9 @@ static constexpr int kSolveMore = 5;
 // lattice's, and the root estimate the FP64 passes of FP64 plans start from
 // (their reach is 1e-5); the tables of FP32 plans (target met to 1e-9), in
 // double-float; those of separable bispectra, in FP64
-static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-11, kSolveF64 = 1e-12;
+static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-12, kSolveF64 = 3e-14;
+// the change at which a solve whose changes have stopped falling still counts
+static constexpr double kSolveAcceptDf = 1e-10, kSolveAcceptF64 = 3e-12;
 
 // The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
 // target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
@@ -1063,7 +1303,8 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   // iterations launched before the host looks, from how long they take (a
   // converged solve's later launches return at once): the damped ones from
   // scratch, from a coarser lattice's solution or from this lattice's own
-  const int first = from == p ? 6 : tol >= kSolveLoose ? 16 : from ? 19 : 20;
+  const int first = from == p ? (target > 0.0 ? 12 : 6) : tol >= kSolveLoose ? 16 : 21;
+  A.accept = std::max(tol, fp64 ? kSolveAcceptF64 : kSolveAcceptDf);
   do {
     const int upto = std::min(kSolveMaxIt, nit + (nit == 0 ? first : kSolveMore));
     for (; nit < upto; ++nit) {
@@ -1115,8 +1356,6 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
 // no q_k moves by more than kFpTol relative; they give up (the solve counts
 // as failed, as above the target) after kFpMaxIters, and a pass that meets
 // sum b_p^2 >= 1 fails at once.
-constexpr double kFpTol = 4e-16;
-constexpr int kFpMaxIters = 400;
 
 __global__ void k_q_init(long long n, const double *__restrict__ S, double *__restrict__ q) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1138,6 +1377,10 @@ __global__ void k_q_change(long long n, const double *__restrict__ S,
 // Solve the fixed point at x from the iterate in p->qm; r: the last pass
 // (r->err != 0: no solution was reached).
 static int solve_mixed(srm3_plan *p, cudaStream_t st, double x, PassResult *r) {
+  if (iter_small(p, 1)) {
+    p->q_warm = true;
+    return run_pass_iter(p, st, &x, 1, r);
+  }
   const long long nl = (long long)p->nk * p->nw;
   for (int it = 1; it <= kFpMaxIters; ++it) {
     k_rec_diff<<<cdiv(nl * 32, 256), 256, 0, st>>>(p->nk, p->nw, p->S, p->qm, p->EkSq, p->EwSq,
@@ -1242,9 +1485,60 @@ static int illinois(srm3_plan *p, cudaStream_t st, double target, double tol, in
 // the target (q >= 1), and at 0.9 (1 - target)^2 x0 it is below it (every q
 // <= 1/(1 - target) below the root); Illinois regula falsi between them,
 // each evaluation warm-started from the largest x found below the target.
+//
+// Where the whole-lattice solve applies (solve.cuh, on the signed omega axis),
+// FP32 plans take its tables, and FP64 plans start from its root and solution:
+// secant steps of a few warm iterations each.
 static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double tol) {
   const long long nl = (long long)p->nk * p->nw;
   PassResult r;
+  if (p->solve) {
+    SolveResult sr;
+    SRM3_CUDA(cudaEventRecord(t_ev[0], st));
+    int rc = solve_lattice(p, st, target, 0.0, p->sigma_g * p->nk, p->sigma_g * p->nw, false,
+                           p->precision == SRM3_FP32 ? kSolveDf : kSolveLoose, nullptr, 1, 1, &sr);
+    if (rc) return rc;
+    SRM3_CUDA(cudaEventRecord(t_ev[1], st));
+    SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
+    if (sr.no_pairs)
+      return fail(SRM3_ERR_BISECTION_FAILED, "no bispectral pairs: max_k sum_b2 is 0 for every eps");
+    if (sr.converged && !sr.err) {
+      float ms = 0.f;
+      SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
+      p->t_recursion_ms += ms;
+      p->t_rec32_ms += ms;
+      p->root_passes32 += 1;
+      double x = sr.x, xp = 0.0, fp = 0.0;
+      bool done = false;
+      r.max_sb2 = sr.max_sb2;
+      r.min_pure = 1.0 - sr.max_sb2;
+      r.sumS = p->sumS;
+      if (p->precision == SRM3_FP32) {
+        p->fp_iters = sr.its;
+        p->root_passes += 1;
+        done = true;
+      }
+      for (int it = 0; it < 8 && !done; ++it) {
+        if ((rc = solve_mixed(p, st, x, &r))) return rc;
+        if (r.err) break;
+        const double f = r.max_sb2 - target;
+        if ((done = std::fabs(f) <= tol)) break;
+        // the slope: the last two points', first that of s ~ x^2 at the target
+        const double slope = it > 0 && f != fp ? (f - fp) / (x - xp) : 2.0 * target / x;
+        if (!(slope > 0.0)) break;
+        xp = x;
+        fp = f;
+        x -= f / slope;
+      }
+      if (done) {
+        p->eps = std::sqrt(x);
+        p->max_sb2 = r.max_sb2;
+        p->min_pure = r.min_pure;
+        p->variance = 4.0 * p->dkdw * r.sumS;
+        return SRM3_OK;
+      }
+    }
+  }
   const double xt = 1e-20;
   p->qlo_x = -1.0;
   k_q_init<<<cdiv(nl, 256), 256, 0, st>>>(nl, p->S, p->qm);
@@ -1581,6 +1875,7 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc,
   SRM3_CUDA(dev_alloc(&c.sb2, kPlanes * nlc * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.scal, (8 + 4 * kPlanes) * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.err, (kPlanes + 1) * sizeof(int), st));
+  SRM3_CUDA(dev_alloc(&c.rec_max, kPlanes * sizeof(unsigned long long), st));
   SRM3_CUDA(dev_alloc(&c.EkSq, nkc * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&c.EkSq32, nkc * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&c.EwSq, 2 * nwc * sizeof(double), st));
@@ -1707,6 +2002,7 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
         return SRM3_OK;
       }
       xs = r.x;
+      p->q_warm = true;  // p->qm: its solution, where the direct iterations start
     } else {
       p->coarse_launches = p->coarse_passes = 0;
     }
@@ -2092,6 +2388,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
   SRM3_CUDA(dev_alloc(&p->EwSq, 2 * nw * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&p->scal, (8 + 4 * kPlanes) * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&p->err, (kPlanes + 1) * sizeof(int), st));
+  SRM3_CUDA(dev_alloc(&p->rec_max, kPlanes * sizeof(unsigned long long), st));
   SRM3_CUDA(cudaMemsetAsync(p->qm, 0, nl * sizeof(double), st));
   SRM3_CUDA(dev_alloc(&p->EkSq32, nk * sizeof(float), st));
   SRM3_CUDA(dev_alloc(&p->EwSq32, 2 * nw * sizeof(float), st));

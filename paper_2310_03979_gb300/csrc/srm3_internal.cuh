@@ -119,6 +119,7 @@ struct srm3_plan {
   // Eq. pure on the whole lattice by self-convolutions (solve.cuh) where the
   // envelope factors and the grid fits; the plan's tables come from it
   bool solve = false;
+  bool q_warm = false;          // qm holds a solution near the next pass's x
   // mixed-sign interactions: opposite-sheet pairs as well; Eq. pure then
   // a fixed point solved by iterations of (difference sums at the previous
   // iterate, level pass)

@@ -1,0 +1,65 @@
+"""Eq. pure on the whole lattice at once (FFT self-convolutions, the search for
+eps folded into the iteration) and the direct iterations of small FP64 plans:
+one-row and one-column lattices, lattices at and just past a power of two,
+targets from 0.05 to 0.95, sparse supports, the three kinds of envelope and
+mixed-sign interactions.  Tables and eps against the FP64 oracle (plain
+bisection) at the tolerances of tests/test_gpu_parity.py."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2310_03979_gb300 import srm3
+from paper_2310_03979_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+pow2 = lambda n: 1 << max(1, (n - 1).bit_length())  # noqa: E731
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("nk,nw,target,envelope,interactions,holes", [
+    (1, 9, 0.5, "gauss", "sum", 0), (9, 1, 0.5, "gauss", "sum", 0), (3, 2, 0.3, "gauss", "sum", 0),
+    (16, 16, 0.95, "gauss", "sum", 0), (17, 33, 0.05, "gauss", "sum", 0),
+    (40, 33, 0.6, "gauss", "sum", 3), (33, 65, 0.9, "gauss", "sum", 7),
+    (16, 17, 0.9, "separable", "sum", 0), (33, 16, 0.5, "sum", "sum", 0),
+    (9, 1, 0.4, "sum", "sum", 0), (20, 20, 0.7, "separable", "sum", 5),
+    (1, 9, 0.3, "gauss", "mixed", 0), (12, 11, 0.5, "gauss", "mixed", 0),
+    (9, 22, 0.6, "gauss", "mixed", 4),
+])
+def test_tables_and_eps_against_oracle(oracle_lib, precision, nk, nw, target, envelope,
+                                       interactions, holes):
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=pow2(max(2, nk)), nt=pow2(max(2, 2 * nw)),
+                              precision=precision, target=target),
+                 envelope=envelope, interactions=interactions)
+    S = oracle.kaimal_lorentzian(nk, nw, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    S[:, 0] = (S.max() or 1.0) / (1.0 + np.arange(nk))
+    if holes:
+        S.ravel()[::holes] = 0.0
+    env = oracle.Envelope("gauss", wl.sigma_g)
+    if envelope != "gauss":
+        ta, tb = wl.envelope_tables()
+        env = oracle.Envelope("separable", table=ta, table_b=tb)
+    mixed = interactions == "mixed"
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, target=target, env=env, mixed=mixed)
+    with srm3.Plan.create(wl, table=S) as p:
+        _, q, sb2 = p.tables()
+        info = p.info()
+    tol, rel = (1e-13, 1e-11) if precision == "fp64" else (1e-9, 2e-8)
+    assert info.eps == pytest.approx(op.eps, rel=rel)
+    assert abs(info.max_sum_b2 - target) <= tol
+    np.testing.assert_allclose(q, op.q, rtol=rel)
+    np.testing.assert_allclose(sb2, op.sum_b2, rtol=rel, atol=1e-15)
+
+
+def test_no_pairs_is_refused():
+    """A support without pairs has no eps: the error of the level search."""
+    wl = W.small_case(nk=8, nw=8, nx=8, nt=16)
+    S = np.zeros((8, 8))
+    S[7, 7] = 1.0
+    for precision in ("fp32", "fp64"):
+        with pytest.raises(srm3.SRM3Error) as ei:
+            srm3.Plan.create(wl, table=S, precision=precision)
+        assert ei.value.code == -4
