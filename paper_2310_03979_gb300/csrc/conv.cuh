@@ -103,24 +103,28 @@ struct ConvArgs {
   const void *twk, *tww;        // pass twiddles of lengths Nk, Nw
   double cb, sb;                // cos, sin of the biphase
   int row_lo, row_hi;           // lattice rows whose coefficients are written
+  int rows;                     // lattice rows per CTA of the row kernels
 };
 
 namespace {
 
-// Rows per CTA of the row passes: 64-thread CTAs (tx_tpt(Nw) threads a row;
-// one row of more than 64 threads for Nw > 1024).
-__host__ __device__ constexpr int conv_rows_per_cta(int log2Nw) {
-  return tx_tpt(1 << log2Nw) >= 64 ? 1 : 64 / tx_tpt(1 << log2Nw);
+// log2 of the values a thread holds of a length-2^l transform: 8, fewer for
+// the short transforms of small lattices, whose passes are bound by the latency
+// of a thread's own instructions, more for the longest, whose threads would not
+// fit in a CTA.  4 / 8 / 16 values everywhere measured, in us (pair sum with
+// phases): one sample of 32 x 32 19.4 / 22.4 / 31.7, 4 FP64 mixed ones of 29 x 12
+// 37 / 46 / 67; 64 samples of 256 x 512 2213 / 1931 / 2193, 16 of 512 x 1024 2589 /
+// 2561 / 2384, 64 separable ones of 256 x 512 907 / 624 / 662, 50 of 256 x 128
+// 192 / 139 / 180 (202 with separate phases and 16 values).
+__host__ __device__ constexpr int conv_lv(int l) { return l <= 6 ? 2 : l <= 12 ? 3 : 4; }
+__host__ __device__ constexpr int conv_tpt(int l) { return tx_tpt(1 << l, conv_lv(l)); }
+// Threads of a row CTA at most (64 unless one row takes more; whole warps, of
+// which A.rows rows are in use) and of a column CTA.
+__host__ __device__ constexpr int conv_row_threads(int lw) {
+  return conv_tpt(lw) >= 64 ? conv_tpt(lw) : 64;
 }
-__host__ __device__ constexpr int conv_row_threads(int log2Nw) {
-  return conv_rows_per_cta(log2Nw) * tx_tpt(1 << log2Nw);
-}
-// Threads of a column CTA at most: 512, or 256 for double-float, which wants
-// more registers than 512 threads leave it (one column of 8192 needs 512).
-template <typename T2>
-__host__ __device__ constexpr int conv_col_threads(int log2Nk) {
-  const int most = std::is_same<T2, df2>::value ? 256 : 512;
-  return tx_tpt(1 << log2Nk) > most ? tx_tpt(1 << log2Nk) : most;
+__host__ __device__ constexpr int conv_col_threads(int lk) {
+  return conv_tpt(lk) > 512 ? conv_tpt(lk) : 512;
 }
 
 template <typename T2>
@@ -179,10 +183,11 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
                                                                     const SeedChunk seeds) {
   using Y2 = typename ConvNum<T2>::Y2;
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nw = 1 << LW, tpt = tx_tpt(Nw), rb = conv_rows_per_cta(LW);
+  constexpr int Nw = 1 << LW, tpt = conv_tpt(LW), LV = conv_lv(LW);
+  const int rb = blockDim.x / tpt;  // rows that fit; A.rows of them are in use
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1), ss = blockIdx.y;
-  const int kk = blockIdx.x * rb + row, nw = A.nw;
-  const bool live = kk < A.nk;
+  const int kk = blockIdx.x * A.rows + row, nw = A.nw;
+  const bool live = row < A.rows && kk < A.nk;
   T2 *buf = reinterpret_cast<T2 *>(conv_smem) + row * (tx_len(Nw) + 1);
   // the row's phasors (and the other sheet's): up to Nw / 2 entries each
   Y2 *yr = reinterpret_cast<Y2 *>(reinterpret_cast<T2 *>(conv_smem) + rb * (tx_len(Nw) + 1)) +
@@ -221,7 +226,7 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
   auto dst = [&](int i, T2 v) {
     if (live) out[i] = v;
   };
-  stockham_passes<LW, 0, MIXED ? 0u : tx_mask_low_half<LW>()>(
+  stockham_passes<LW, 0, MIXED ? 0u : tx_mask_low_half<LW, LV>(), false, false, false, LV>(
       1, 0, tpt, jt, static_cast<const T2 *>(A.tww), buf, src, dst);
 }
 
@@ -232,12 +237,12 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
 // in Z ([ss][n_kappa][Nw]: the grid's rows past n_kappa are zero and not
 // stored).  Shared memory: colstride entries per column.
 template <int LK, typename T2>
-__global__ void __launch_bounds__(conv_col_threads<T2>(LK)) k_conv_cols(int nk, int Nw, int TC,
+__global__ void __launch_bounds__(conv_col_threads(LK)) k_conv_cols(int nk, int Nw, int TC,
                                                                         int colstride,
                                                                         const T2 *__restrict__ tw,
                                                                         T2 *__restrict__ Z) {
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nk = 1 << LK, tpt = tx_tpt(Nk);
+  constexpr int Nk = 1 << LK, tpt = conv_tpt(LK), LV = conv_lv(LK);
   const int c = threadIdx.x & (TC - 1), jt = threadIdx.x / TC, ss = blockIdx.y;
   T2 *col = reinterpret_cast<T2 *>(conv_smem) + c * colstride;
   T2 *base = Z + (size_t)ss * nk * Nw + blockIdx.x * TC + c;
@@ -249,7 +254,8 @@ __global__ void __launch_bounds__(conv_col_threads<T2>(LK)) k_conv_cols(int nk, 
     return v;
   };
   auto none = [](int, T2) {};
-  stockham_passes<LK, 0, tx_mask_low_half<LK>(), false, true>(1, 0, tpt, jt, tw, col, src1, none);
+  stockham_passes<LK, 0, tx_mask_low_half<LK, LV>(), false, true, false, LV>(1, 0, tpt, jt, tw, col,
+                                                                          src1, none);
   auto src2 = [&](int i) -> T2 {
     T2 v = col[sp16(i)];
     v = cmul(v, v);
@@ -259,7 +265,7 @@ __global__ void __launch_bounds__(conv_col_threads<T2>(LK)) k_conv_cols(int nk, 
   auto dst2 = [&](int kk, T2 v) {
     if (kk < nk) base[(size_t)kk * Nw] = v;
   };
-  stockham_passes<LK, 0, 0u, true, false, true>(1, 0, tpt, jt, tw, col, src2, dst2);
+  stockham_passes<LK, 0, 0u, true, false, true, LV>(1, 0, tpt, jt, tw, col, src2, dst2);
 }
 
 // Pass 3: lattice row kk of the twice-transformed grid, transformed along
@@ -273,10 +279,11 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_out(const ConvArg
   using Y2 = typename ConvNum<T2>::Y2;
   using T = decltype(Y2::x);
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nw = 1 << LW, tpt = tx_tpt(Nw), rb = conv_rows_per_cta(LW);
+  constexpr int Nw = 1 << LW, tpt = conv_tpt(LW), LV = conv_lv(LW);
+  const int rb = blockDim.x / tpt;  // rows that fit; A.rows of them are in use
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1), ss = blockIdx.y;
-  const int kk = A.row_lo + blockIdx.x * rb + row, nw = A.nw;
-  const bool live = kk < A.row_hi;
+  const int kk = A.row_lo + blockIdx.x * A.rows + row, nw = A.nw;
+  const bool live = row < A.rows && kk < A.row_hi;
   T2 *buf = reinterpret_cast<T2 *>(conv_smem) + row * (tx_len(Nw) + 1);
   const T2 *in = static_cast<const T2 *>(A.Z) + ((size_t)ss * A.nk + (live ? kk : 0)) * Nw;
   const Y2 *y = static_cast<const Y2 *>(A.y) + (size_t)ss * A.nk * nw;
@@ -345,7 +352,7 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_out(const ConvArg
     C[k] = o;
   };
   // the upper half of the outputs is never needed: n_omega <= Nw / 2
-  stockham_passes<LW, 0, 0u, false, false, true>(1, 0, tpt, jt,
+  stockham_passes<LW, 0, 0u, false, false, true, LV>(1, 0, tpt, jt,
                                                  static_cast<const T2 *>(A.tww), buf, src, dst);
 }
 

@@ -46,8 +46,8 @@ cudaError_t conv_prepare(int dev) {
 //
 // Which plans take it: every separable bispectrum, and the Gaussian envelope
 // with W recomputed at every size.  Both sides measured (GB300, FP32 plans,
-// pair sum with its phases): 256 x 512, 64 samples 44.4 -> 2.19 ms; 512 x
-// 1024, 16 samples 183 -> 2.4 ms; 32 spectra on lattices of 32..256 per axis
+// pair sum with its phases): 256 x 512, 64 samples 44.4 -> 1.93 ms; 512 x
+// 1024, 16 samples 183 -> 2.56 ms; 32 spectra on lattices of 32..256 per axis
 // in one captured batch 22.7 -> 4.0 ms; one sample on 32 x 32, with its field,
 // 60 -> 43 us.  FP64 plans: 90 x 117, 4 samples 1.64 -> 0.12 ms.  Against 64-bit
 // coefficients the FP32 fields' relative error went 1.9e-7 -> 1.8e-7 (2.1e-7
@@ -69,7 +69,13 @@ int conv_run(const ConvJob &j) {
   per = std::min(per, 16384);
   if (!j.dseeds) per = std::min(per, kMaxChunk);
   if (per < 1) return fail(SRM3_ERR_INVALID_ARG, "pair sum: workspace too small");
-  const int rb = conv_rows_per_cta(lw), rthreads = conv_row_threads(lw);
+  // rows per CTA: what 64 threads hold, fewer where that leaves SMs idle; whole warps
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
+  const int tpt = conv_tpt(lw), most = std::max(1, 64 / tpt);
+  const long long allrows = (long long)p->nk * 2 * per;
+  const int rows = (int)std::min<long long>(most, std::max<long long>(1, allrows / (4 * nsm)));
+  const int rthreads = (rows * tpt + 31) / 32 * 32, rb = rthreads / tpt;
   const int copies = p->mixed ? 2 : 1;
   const size_t stage = (size_t)rb * (tx_len(Nw) + 1) * sizeof(T2);
   const size_t srow = stage + (size_t)rb * copies * p->nw * sizeof(Y2);
@@ -81,7 +87,8 @@ int conv_run(const ConvJob &j) {
   };
   int TC = 16;
   while (TC > 1 && (TC > Nw || (size_t)TC * colstride(TC) * sizeof(T2) > 100 * 1024 ||
-                    TC * tx_tpt(Nk) > conv_col_threads<T2>(lk)))
+                    TC * conv_tpt(lk) > conv_col_threads(lk) ||
+                    (long long)(Nw / TC) * 2 * per < nsm))
     TC >>= 1;
   const int cs = colstride(TC);
   const size_t scol = (size_t)TC * cs * sizeof(T2);
@@ -115,11 +122,12 @@ int conv_run(const ConvJob &j) {
   A.ck_of = j.ck_of;
   A.dseeds = j.dseeds;
   A.twk = p->tw_conv;
-  A.tww = static_cast<const T2 *>(p->tw_conv) + tx_twlen(lk);
+  A.tww = static_cast<const T2 *>(p->tw_conv) + tx_twlen(lk, conv_lv(lk));
   A.cb = std::cos(p->beta);
   A.sb = std::sin(p->beta);
   A.row_lo = p->row_lo;
   A.row_hi = p->row_hi;
+  A.rows = rows;
   A.Z = j.work;
   SeedChunk sc;
   std::memset(&sc, 0, sizeof(sc));
@@ -132,7 +140,7 @@ int conv_run(const ConvJob &j) {
     cudaError_t err = cudaSuccess;
     conv_with_log2<1, 13>(lw, [&](auto c) {
       constexpr int L = decltype(c)::value;
-      const dim3 grid(conv_cdiv(p->nk, rb), 2 * ns);
+      const dim3 grid(conv_cdiv(p->nk, rows), 2 * ns);
       if constexpr (!f32) {
         if (p->mixed) {
           err = conv_prepare<k_conv_rows<L, T2, true>>(p->device);
@@ -151,14 +159,14 @@ int conv_run(const ConvJob &j) {
       constexpr int L = decltype(c)::value;
       err = conv_prepare<k_conv_cols<L, T2>>(p->device);
       if (err == cudaSuccess)
-        k_conv_cols<L, T2><<<dim3(Nw / TC, 2 * ns), TC * tx_tpt(1 << L), scol, j.stream>>>(
+        k_conv_cols<L, T2><<<dim3(Nw / TC, 2 * ns), TC * conv_tpt(L), scol, j.stream>>>(
             p->nk, Nw, TC, cs, static_cast<const T2 *>(A.twk), static_cast<T2 *>(A.Z));
     });
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "pair sum, columns");
     conv_with_log2<1, 13>(lw, [&](auto c) {
       constexpr int L = decltype(c)::value;
-      const dim3 grid(conv_cdiv(p->row_hi - p->row_lo, rb), 2 * ns);
+      const dim3 grid(conv_cdiv(p->row_hi - p->row_lo, rows), 2 * ns);
       if constexpr (!f32) {
         if (p->mixed) {
           err = conv_prepare<k_conv_out<L, T2, true>>(p->device);

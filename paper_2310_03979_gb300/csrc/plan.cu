@@ -14,6 +14,7 @@
 #include <numeric>
 #include <unordered_map>
 
+#include "conv.cuh"
 #include "recursion.cuh"
 #include "solve.cuh"
 #include "srm3_internal.cuh"
@@ -2599,20 +2600,21 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
     p->cNk = 1 << p->log2cNk;
     p->cNw = 1 << p->log2cNw;
     const int lk = p->log2cNk, lw = p->log2cNw;
-    const int ntwc = tx_twlen(lk) + tx_twlen(lw) + (1 << lw);
+    const int vk = conv_lv(lk), vw = conv_lv(lw);
+    const int ntwc = tx_twlen(lk, vk) + tx_twlen(lw, vw) + (1 << lw);
     const int nfac = 2 * nk + 3 * nw - 1, m = std::max(nk, 2 * nw - 1);
     const double sk = p->sigma_g * nk, sw = p->sigma_g * nw;
     SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(double2), st));
     if (!p->sep) SRM3_CUDA(dev_alloc(&p->conv_fac, (size_t)nfac * sizeof(double), st));
     if (!f32) {
-      k_tx_twiddles<double2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (double2 *)p->tw_conv);
+      k_tx_twiddles<double2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (double2 *)p->tw_conv, vk, vw);
       if (!p->sep)
         k_conv_factors<double><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw,
                                                              (double *)p->conv_fac);
     } else if (p->sep) {
-      k_tx_twiddles<float2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (float2 *)p->tw_conv);
+      k_tx_twiddles<float2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (float2 *)p->tw_conv, vk, vw);
     } else {
-      k_tx_twiddles<df2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (df2 *)p->tw_conv);
+      k_tx_twiddles<df2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (df2 *)p->tw_conv, vk, vw);
       k_conv_factors<df><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw, (df *)p->conv_fac);
     }
   }
