@@ -203,10 +203,7 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
   }
   __syncthreads();
   auto src = [&](int m) -> T2 {
-    T2 v;
-    v.x = 0;
-    v.y = 0;
-    if (!live) return v;
+    if (!live) return c_zero<T2>();
     int w = m;
     const Y2 *y = yr;
     if constexpr (MIXED) {
@@ -216,12 +213,10 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
       }
     }
     const int aw = w < 0 ? -w : w;
-    if (aw >= nw) return v;
+    if (aw >= nw) return c_zero<T2>();
     const Y2 yv = y[aw];
     const auto a = conv_a<T2>(A, kk, w);
-    v.x = conv_scale(yv.x, a);
-    v.y = conv_scale(yv.y, a);
-    return v;
+    return c_make<T2>(conv_scale(yv.x, a), conv_scale(yv.y, a));
   };
   auto dst = [&](int i, T2 v) {
     if (live) out[i] = v;
@@ -247,20 +242,14 @@ __global__ void __launch_bounds__(conv_col_threads(LK)) k_conv_cols(int nk, int 
   T2 *col = reinterpret_cast<T2 *>(conv_smem) + c * colstride;
   T2 *base = Z + (size_t)ss * nk * Nw + blockIdx.x * TC + c;
   auto src1 = [&](int kk) -> T2 {
-    T2 v;
-    v.x = 0;
-    v.y = 0;
-    if (kk < nk) v = base[(size_t)kk * Nw];
-    return v;
+    return kk < nk ? base[(size_t)kk * Nw] : c_zero<T2>();
   };
   auto none = [](int, T2) {};
   stockham_passes<LK, 0, tx_mask_low_half<LK, LV>(), false, true, false, LV>(1, 0, tpt, jt, tw, col,
                                                                           src1, none);
   auto src2 = [&](int i) -> T2 {
-    T2 v = col[sp16(i)];
-    v = cmul(v, v);
-    v.y = -v.y;
-    return v;
+    const T2 v = col[sp16(i)];
+    return c_conj(cmul(v, v));
   };
   auto dst2 = [&](int kk, T2 v) {
     if (kk < nk) base[(size_t)kk * Nw] = v;
@@ -293,36 +282,22 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_out(const ConvArg
   const float inv = 1.0f / ((float)A.Nk * (float)Nw);  // a power of two
   const T cb = (T)A.cb, sb = (T)A.sb;
   auto z_at = [&](int hk, int hw) -> T2 {
-    T2 z;
-    z.x = 0;
-    z.y = 0;
-    if (hk == 0 && hw == 0) return z;
+    if (hk == 0 && hw == 0) return c_zero<T2>();
     const Y2 yh = y[(size_t)hk * nw + hw];
     const F a = conv_a<T2>(A, hk, hw);
-    z.x = conv_scale(yh.x, a);
-    z.y = conv_scale(yh.y, a);
-    return z;
+    return c_make<T2>(conv_scale(yh.x, a), conv_scale(yh.y, a));
   };
   T2 *part = buf + tx_len(Nw);  // MIXED: the kw = 0 sum of the row, past the transform
   if constexpr (MIXED) {
     T2 *psum = reinterpret_cast<T2 *>(conv_smem) + rb * (tx_len(Nw) + 1) + row * tpt;
-    T2 s;
-    s.x = 0;
-    s.y = 0;
+    T2 s = c_zero<T2>();
     if (live)
-      for (int a = jt; a <= kk; a += tpt) {
-        const T2 t = cmul(z_at(a, 0), z_at(kk - a, 0));
-        s.x += t.x;
-        s.y += t.y;
-      }
+      for (int a = jt; a <= kk; a += tpt) s = c_add(s, cmul(z_at(a, 0), z_at(kk - a, 0)));
     psum[jt] = s;
     __syncthreads();
     if (jt == 0) {
       s = psum[0];
-      for (int j = 1; j < tpt; ++j) {
-        s.x += psum[j].x;
-        s.y += psum[j].y;
-      }
+      for (int j = 1; j < tpt; ++j) s = c_add(s, psum[j]);
       *part = s;
     }
     __syncthreads();
@@ -330,19 +305,15 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_out(const ConvArg
   auto src = [&](int i) -> T2 { return in[i]; };
   auto dst = [&](int kw, T2 cv) {
     if (!live || kw >= nw) return;
-    T2 t;
-    t.x = conv_pow2(cv.x, inv);
-    t.y = conv_pow2(-cv.y, inv);
+    T2 t = c_make<T2>(conv_pow2(c_re(cv), inv), conv_pow2(-c_im(cv), inv));
     if constexpr (MIXED) {
       if (kw == 0) t = *part;
     }
     if (((kk | kw) & 1) == 0) {  // the diagonal pair {k/2, k/2}
-      T2 z = z_at(kk >> 1, kw >> 1);
-      z = cmul(z, z);
-      t.x += z.x;
-      t.y += z.y;
+      const T2 z = z_at(kk >> 1, kw >> 1);
+      t = c_add(t, cmul(z, z));
     }
-    const T ar = (T)0.5 * conv_round(t.x), ai = (T)0.5 * conv_round(t.y);
+    const T ar = (T)0.5 * conv_round(c_re(t)), ai = (T)0.5 * conv_round(c_im(t));
     const size_t k = (size_t)kk * nw + kw;
     const Y2 yk = y[k];
     const T f = ck[k] * conv_round(conv_b<T2>(A, kk, kw)), P = Pk[k];

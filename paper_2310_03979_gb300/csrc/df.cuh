@@ -27,8 +27,11 @@ struct df {
   __host__ __device__ constexpr df(float h_, float l_) : h(h_), l(l_) {}
 };
 
+// A complex double-float: the high parts of its two components side by side,
+// then the low parts, so that a sum of two of them is eight packed operations
+// on pairs (f32x2: two FP32 operations per lane in one issue slot).
 struct __align__(16) df2 {
-  df x, y;
+  float2 h, l;
 };
 
 // a + b = s + e exactly
@@ -69,11 +72,116 @@ __device__ __forceinline__ df dot2(df a, df b, df c, df d) {
   return df(s, __fadd_rn(e, __fadd_rn(ep, eq)));
 }
 
-__device__ __forceinline__ df2 cmul(df2 a, df2 b) {
-  df2 r;
-  r.x = dot2(a.x, b.x, -a.y, b.y);
-  r.y = dot2(a.x, b.y, a.y, b.x);
+// Packed FP32 pairs.
+typedef unsigned long long pk2;
+__device__ __forceinline__ pk2 pk(float2 v) {
+  pk2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
   return r;
+}
+__device__ __forceinline__ float2 unpk(pk2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ pk2 pk_add(pk2 a, pk2 b) {
+  pk2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// b - a, as a * (-1) + b: one rounding either way
+__device__ __forceinline__ pk2 pk_rsub(pk2 a, pk2 b) {
+  pk2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(0xbf800000bf800000ull), "l"(b));
+  return r;
+}
+
+// The complex operations of the transforms, by type.
+template <typename T2>
+struct RealOf;
+template <>
+struct RealOf<float2> {
+  using type = float;
+};
+template <>
+struct RealOf<double2> {
+  using type = double;
+};
+template <>
+struct RealOf<df2> {
+  using type = df;
+};
+template <typename T2>
+__device__ __forceinline__ auto c_re(const T2 &v) {
+  return v.x;
+}
+template <typename T2>
+__device__ __forceinline__ auto c_im(const T2 &v) {
+  return v.y;
+}
+template <>
+__device__ __forceinline__ auto c_re<df2>(const df2 &v) {
+  return df(v.h.x, v.l.x);
+}
+template <>
+__device__ __forceinline__ auto c_im<df2>(const df2 &v) {
+  return df(v.h.y, v.l.y);
+}
+template <typename T2>
+__device__ __forceinline__ T2 c_make(typename RealOf<T2>::type re, typename RealOf<T2>::type im) {
+  T2 v;
+  v.x = re;
+  v.y = im;
+  return v;
+}
+template <>
+__device__ __forceinline__ df2 c_make<df2>(df re, df im) {
+  df2 v;
+  v.h = make_float2(re.h, im.h);
+  v.l = make_float2(re.l, im.l);
+  return v;
+}
+template <typename T2>
+__device__ __forceinline__ T2 c_zero() {
+  using F = typename RealOf<T2>::type;
+  return c_make<T2>(F(0), F(0));
+}
+template <typename T2>
+__device__ __forceinline__ T2 c_conj(const T2 &v) {
+  return c_make<T2>(c_re(v), -c_im(v));
+}
+template <typename T2>
+__device__ __forceinline__ T2 c_add(const T2 &a, const T2 &b) {
+  return c_make<T2>(c_re(a) + c_re(b), c_im(a) + c_im(b));
+}
+template <typename T2>
+__device__ __forceinline__ T2 c_sub(const T2 &a, const T2 &b) {
+  return c_make<T2>(c_re(a) - c_re(b), c_im(a) - c_im(b));
+}
+template <>
+__device__ __forceinline__ df2 c_add<df2>(const df2 &a, const df2 &b) {
+  const pk2 ah = pk(a.h), bh = pk(b.h);
+  const pk2 s = pk_add(ah, bh), v = pk_rsub(ah, s);
+  const pk2 e = pk_add(pk_rsub(pk_rsub(v, s), ah), pk_rsub(v, bh));
+  df2 r;
+  r.h = unpk(s);
+  r.l = unpk(pk_add(pk_add(pk(a.l), pk(b.l)), e));
+  return r;
+}
+template <>
+__device__ __forceinline__ df2 c_sub<df2>(const df2 &a, const df2 &b) {
+  const pk2 ah = pk(a.h), bh = pk(b.h);
+  const pk2 s = pk_rsub(bh, ah), v = pk_rsub(ah, s);
+  const pk2 e = pk_rsub(pk_add(bh, v), pk_rsub(pk_rsub(v, s), ah));
+  df2 r;
+  r.h = unpk(s);
+  r.l = unpk(pk_add(pk_rsub(pk(b.l), pk(a.l)), e));
+  return r;
+}
+
+__device__ __forceinline__ df2 cmul(df2 a, df2 b) {
+  const df ax = c_re(a), ay = c_im(a), bx = c_re(b), by = c_im(b);
+  return c_make<df2>(dot2(ax, bx, -ay, by), dot2(ax, by, ay, bx));
 }
 
 }  // namespace srm3

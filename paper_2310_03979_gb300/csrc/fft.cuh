@@ -6,6 +6,7 @@
 // it gets its own copy of the kernels.
 #pragma once
 
+#include <type_traits>
 #include <utility>
 
 #include "df.cuh"
@@ -148,37 +149,71 @@ __device__ __forceinline__ int brev(int m, int log2n) {
 // item, or 16/R items of radix R); log2 L splits into ceil(log2 L / 4)
 // passes of near-equal radix.  w_N = e^{+2 pi i / N}.
 
+// cos(pi / 8), sin(pi / 8), cos(pi / 4), and tan(pi / 8)
+constexpr double kC1 = 0.92387953251128675613, kS1 = 0.38268343236508977173;
+constexpr double kH = 0.70710678118654752440, kT1 = 0.41421356237309504880;
+
 // b * e^{2 pi i e / 16}, e in [0, 8) (e a constant after unrolling)
 template <typename T2>
 __device__ __forceinline__ T2 rot16(T2 b, int e) {
-  using T = decltype(b.x);
-  constexpr double c1 = 0.92387953251128675613;  // cos(pi / 8)
-  constexpr double s1 = 0.38268343236508977173;  // sin(pi / 8)
-  constexpr double h = 0.70710678118654752440;   // cos(pi / 4)
-  T2 r;
+  using T = typename RealOf<T2>::type;
+  const auto x = c_re(b), y = c_im(b);
   switch (e) {
     case 0:
       return b;
     case 2:
-      r.x = (T)h * (b.x - b.y);
-      r.y = (T)h * (b.x + b.y);
-      return r;
+      return c_make<T2>((T)kH * (x - y), (T)kH * (x + y));
     case 4:
-      r.x = -b.y;
-      r.y = b.x;
-      return r;
+      return c_make<T2>(-y, x);
     case 6:
-      r.x = -(T)h * (b.x + b.y);
-      r.y = (T)h * (b.x - b.y);
-      return r;
+      return c_make<T2>(-((T)kH * (x + y)), (T)kH * (x - y));
     default: {
-      const T c = e == 1 ? (T)c1 : e == 3 ? (T)s1 : e == 5 ? (T)-s1 : (T)-c1;
-      const T s = (e == 1 || e == 7) ? (T)s1 : (T)c1;
-      T2 w;
-      w.x = c;
-      w.y = s;
-      return cmul(b, w);
+      const T c = e == 1 ? (T)kC1 : e == 3 ? (T)kS1 : e == 5 ? (T)-kS1 : (T)-kC1;
+      const T s = (e == 1 || e == 7) ? (T)kS1 : (T)kC1;
+      return cmul(b, c_make<T2>(c, s));
     }
+  }
+}
+
+// The butterfly (a, b) <- (a + w b, a - w b), w = e^{2 pi i E / 16}.  In FP32
+// and FP64 the larger of |cos|, |sin| is taken out of the rotation and into
+// the sums, w b = f (u + i v) with one multiply-add each for u and v: six
+// multiply-adds instead of eight operations.
+template <int E, typename T2>
+__device__ __forceinline__ void bfly16(T2 &a, T2 &b) {
+  if constexpr (E == 0 || E == 4 || std::is_same<T2, df2>::value) {
+    const T2 t = rot16(b, E), x = a;
+    a = c_add(x, t);
+    b = c_sub(x, t);
+  } else {
+    using T = typename RealOf<T2>::type;
+    constexpr T t = (T)kT1, f = (T)(E % 4 == 2 ? kH : kC1);
+    const T x = b.x, y = b.y;
+    T u, v;
+    if constexpr (E == 1) {  // c (x - t y, y + t x)
+      u = fma(-t, y, x);
+      v = fma(t, x, y);
+    } else if constexpr (E == 2) {
+      u = x - y;
+      v = x + y;
+    } else if constexpr (E == 3) {  // s (t x - y, x + t y)
+      u = fma(t, x, -y);
+      v = fma(t, y, x);
+    } else if constexpr (E == 5) {  // s (-t x - y, x - t y)
+      u = fma(-t, x, -y);
+      v = fma(-t, y, x);
+    } else if constexpr (E == 6) {
+      u = -x - y;
+      v = x - y;
+    } else {  // c (-x - t y, t x - y)
+      u = fma(-t, y, -x);
+      v = fma(t, x, -y);
+    }
+    const T ax = a.x, ay = a.y;
+    a.x = fma(f, u, ax);
+    a.y = fma(f, v, ay);
+    b.x = fma(-f, u, ax);
+    b.y = fma(-f, v, ay);
   }
 }
 
@@ -188,45 +223,15 @@ struct Log2R {
 };
 
 // v[r] <- sum_s v[s] e^{2 pi i r s / R}: radix-2 decimation in time on the
-// bit-reversed copy, every index and twiddle a compile-time constant.
-template <int R, typename T2>
-__device__ __forceinline__ void dft_inv(T2 (&v)[R]) {
-  constexpr int B = Log2R<R>::v;
-  T2 a[R];
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    int rb = 0;
-#pragma unroll
-    for (int bit = 0; bit < B; ++bit) rb |= ((i >> bit) & 1) << (B - 1 - bit);
-    a[i] = v[rb];
-  }
-#pragma unroll
-  for (int st = 0; st < B; ++st) {
-    const int h = 1 << st;
-#pragma unroll
-    for (int g = 0; g < R; g += 2 * h)
-#pragma unroll
-      for (int j = 0; j < h; ++j) {
-        const T2 t = rot16(a[g + j + h], j * (8 >> st));  // w_{2h}^j
-        const T2 x = a[g + j];
-        a[g + j].x = x.x + t.x;
-        a[g + j].y = x.y + t.y;
-        a[g + j + h].x = x.x - t.x;
-        a[g + j + h].y = x.y - t.y;
-      }
-  }
-#pragma unroll
-  for (int i = 0; i < R; ++i) v[i] = a[i];
-}
-
-// The same DFT when some inputs are zero by construction: bit r of VMASK is
-// set when v[r] may be nonzero (the others must be zero).  Each butterfly
+// bit-reversed copy, every index and twiddle a compile-time constant.  Some
+// inputs may be zero by construction: bit r of VMASK is set when v[r] may be
+// nonzero (the others must be zero).  Each butterfly
 // of the decimation in time is resolved at compile time from the zero
 // pattern its stage inherits: both operands zero, skipped; the rotated one
 // zero, a copy (x +- 0 = x); the other zero, the rotated operand and its
-// negation (0 +- t = +-t); else computed as in dft_inv.  IEEE arithmetic does
-// not let the compiler drop the additions of zeros by itself.  The results
-// equal dft_inv's up to the sign of zero outputs.
+// negation (0 +- t = +-t); else computed.  IEEE arithmetic does not let the
+// compiler drop the additions of zeros by itself.  The results equal the
+// unmasked ones up to the sign of zero outputs.
 template <int R>
 __host__ __device__ constexpr unsigned dit_in_mask(unsigned vmask) {
   unsigned m = 0;
@@ -253,19 +258,13 @@ __device__ __forceinline__ void dit_bfly(T2 (&a)[R]) {
   constexpr int h = 1 << ST, j = B % h, i0 = (B / h) * 2 * h + j, i1 = i0 + h;
   constexpr bool n0 = (M >> i0) & 1u, n1 = (M >> i1) & 1u;
   if constexpr (n0 && n1) {
-    const T2 t = rot16(a[i1], j * (8 >> ST));
-    const T2 x = a[i0];
-    a[i0].x = x.x + t.x;
-    a[i0].y = x.y + t.y;
-    a[i1].x = x.x - t.x;
-    a[i1].y = x.y - t.y;
+    bfly16<j *(8 >> ST)>(a[i0], a[i1]);
   } else if constexpr (n0) {
     a[i1] = a[i0];
   } else if constexpr (n1) {
     const T2 t = rot16(a[i1], j * (8 >> ST));
     a[i0] = t;
-    a[i1].x = -t.x;
-    a[i1].y = -t.y;
+    a[i1] = c_make<T2>(-c_re(t), -c_im(t));
   }
 }
 template <int R, int ST, unsigned M, typename T2, int... Bs>
@@ -280,7 +279,7 @@ __device__ __forceinline__ void dit_stages(T2 (&a)[R]) {
   }
 }
 template <int R, unsigned VMASK, typename T2>
-__device__ __forceinline__ void dft_inv_masked(T2 (&v)[R]) {
+__device__ __forceinline__ void dft_inv(T2 (&v)[R]) {
   constexpr int B = Log2R<R>::v;
   T2 a[R];
 #pragma unroll
@@ -376,8 +375,7 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
           if ((VMASK >> r) & 1u) {
             v[it][r] = src(j + r * LR);
           } else {
-            v[it][r].x = 0;
-            v[it][r].y = 0;
+            v[it][r] = c_zero<T2>();
           }
         }
       } else {
@@ -394,10 +392,7 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
 #pragma unroll
         for (int r = 1; r < R; ++r) v[it][r] = cmul(v[it][r], w[r]);
       }
-      if constexpr (FIRST && VMASK != tx_in_mask(R, 0))
-        dft_inv_masked<R, VMASK>(v[it]);
-      else
-        dft_inv<R>(v[it]);
+      dft_inv<R, FIRST ? VMASK : tx_in_mask(R, 0)>(v[it]);
     }
   }
   if constexpr ((!FIRST || SRCSM) && (!LAST || DSTSM))
@@ -449,14 +444,40 @@ __device__ __forceinline__ void stockham_passes(int Ns, int toff, int tpt, int j
 // The first pass's mask for inputs at both ends of the spectrum (nz blocks
 // each, tx_in_mask) or at the low end only (the lower half of the blocks:
 // a zero-padded sequence of at most L/2 entries).
-template <int l>
+template <int l, int lv = 4>
 __host__ __device__ constexpr unsigned tx_mask_ends(int nz) {
-  return tx_in_mask(1 << tx_lr(l, 0), nz);
+  return tx_in_mask(1 << tx_lr(l, 0, lv), nz);
 }
 template <int l, int lv = 4>
 __host__ __device__ constexpr unsigned tx_mask_low_half() {
   return (1u << ((1 << tx_lr(l, 0, lv)) / 2)) - 1u;
 }
+
+// Nonzero input blocks of a stage's first pass (tx_in_mask): a length-2^l
+// transform whose inputs vanish except at the n indices of each end of the
+// spectrum (kk < nk or nx - kk < nk in x; m < nw or M - m < nw in t).  The
+// smallest of 1, 2, 4 blocks (of 2^l / R each, R the first radix) that
+// covers them, else 0 (all).  Pruned passes are compiled for FP32 and
+// transforms of 64 points or more.
+inline int tx_nz(int l, int n, bool fp32) {
+  if (!fp32 || l < 6) return 0;
+  const int R = 1 << tx_lr(l, 0), LR = (1 << l) / R;
+  for (int nz = 1; nz <= 4 && 2 * nz < R; nz *= 2)
+    if ((long long)nz * LR >= n) return nz;
+  return 0;
+}
+
+// log2 of the values a thread holds of a length-2^l output transform: 16 where
+// the first pass is pruned (its radix of 16 skips more of the zero blocks), else
+// 8, and 4 in short transforms, whose passes are bound by the latency of a
+// thread's own instructions.  Measured with 16 values / this rule, in us: 64
+// fields of 512 x 1024 206 / 165, 16 of 1024 x 2048 244 / 187, one FP64 64 x 64 35 /
+// 17, 16 FP64 512 x 1024 576 / 554; 50 of 1024 x 2048 from 256 x 128 (pruned)
+// 177, with 8 values 210.
+__host__ __device__ constexpr int out_lv(int l, int nz) {
+  return nz > 0 ? 4 : l <= 6 ? 2 : l <= 12 ? 3 : 4;
+}
+__host__ __device__ constexpr int out_tpt(int l, int nz) { return tx_tpt(1 << l, out_lv(l, nz)); }
 
 // Stage 1: TC columns m0 + c of one coefficient set per CTA (blockIdx.y =
 // set), thread (c, jt) = (t mod TC, t / TC); TC consecutive columns make the
@@ -470,7 +491,7 @@ __global__ void __launch_bounds__(512) k_tx_cols(int nk, int nw, int TC, int col
                                                   T2 *__restrict__ G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using T = decltype(T2::x);
-  constexpr int L = 1 << LOG2NX;
+  constexpr int L = 1 << LOG2NX, LV = out_lv(LOG2NX, NZ);
   const int n = blockIdx.y;
   const int c = threadIdx.x & (TC - 1), jt = threadIdx.x / TC;
   const int m = blockIdx.x * TC + c;
@@ -510,7 +531,8 @@ __global__ void __launch_bounds__(512) k_tx_cols(int nk, int nw, int TC, int col
   auto dst = [&](int i, T2 v) {
     if (live) Gn[(size_t)i * nw + m] = v;
   };
-  stockham_passes<LOG2NX, 0, tx_mask_ends<LOG2NX>(NZ)>(1, 0, tx_tpt(L), jt, twp, col, src, dst);
+  stockham_passes<LOG2NX, 0, tx_mask_ends<LOG2NX, LV>(NZ), false, false, false, LV>(
+      1, 0, out_tpt(LOG2NX, NZ), jt, twp, col, src, dst);
 }
 
 // Stage 2: RB rows mx of one set per CTA, thread (row, jt) = (t / tpt,
@@ -522,7 +544,7 @@ __global__ void __launch_bounds__(512) k_tx_rows(int nx, int nw, int rowstride,
                                                  const T2 *__restrict__ twp,
                                                  const T2 *__restrict__ twz, T *__restrict__ u) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int M = 1 << LOG2M, tpt = tx_tpt(M);
+  constexpr int M = 1 << LOG2M, tpt = out_tpt(LOG2M, NZ), LV = out_lv(LOG2M, NZ);
   const int n = blockIdx.y;
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1);
   const int rb = blockDim.x / tpt, mx = blockIdx.x * rb + row;
@@ -557,7 +579,8 @@ __global__ void __launch_bounds__(512) k_tx_rows(int nx, int nw, int rowstride,
   if constexpr (LOG2M == 0) {  // nt = 2: z[0] = Z[0]
     if (jt == 0) dst(0, src(0));
   } else {
-    stockham_passes<LOG2M, 0, tx_mask_ends<LOG2M>(NZ)>(1, 0, tpt, jt, twp, buf, src, dst);
+    stockham_passes<LOG2M, 0, tx_mask_ends<LOG2M, LV>(NZ), false, false, false, LV>(
+        1, 0, tpt, jt, twp, buf, src, dst);
   }
 }
 

@@ -334,8 +334,8 @@ __global__ void k_tx_twiddles(int lx, int lm, T2 *tw, int vx = 4, int vm = 4) {
   }
   double sn, cs;
   sincospi(2.0 * (double)num / (double)den, &sn, &cs);
-  tw[e].x = cs;
-  tw[e].y = sn;
+  using F = typename RealOf<T2>::type;
+  tw[e] = c_make<T2>((F)cs, (F)sn);
 }
 
 template <typename T2>
@@ -2621,7 +2621,9 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
   p->rowstride = nw + 2 * kPad;  // y row length, workspace or batch buffers
   SRM3_CUDA(dev_alloc(&p->Ek, nk * es, st));
   SRM3_CUDA(dev_alloc(&p->Ews, p->ew_len * es, st));
-  const int tw_n = tx_twlen(p->log2nx) + tx_twlen(p->log2nt - 1) + p->nt / 2;
+  const int ox = out_lv(p->log2nx, tx_nz(p->log2nx, nk, f32));
+  const int ot = out_lv(p->log2nt - 1, tx_nz(p->log2nt - 1, nw, f32));
+  const int tw_n = tx_twlen(p->log2nx, ox) + tx_twlen(p->log2nt - 1, ot) + p->nt / 2;
   SRM3_CUDA(dev_alloc(&p->tw, (size_t)tw_n * 2 * es, st));
   if (f32) {
     k_env<float><<<cdiv(nk, 256), 256, 0, st>>>(nk, 0, p->sigma_g * nk, (float *)p->Ek);
@@ -2636,13 +2638,13 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
                                                          (float *)p->Ewd);
     }
     k_tx_twiddles<float2><<<cdiv(tw_n, 256), 256, 0, st>>>(p->log2nx, p->log2nt - 1,
-                                                            (float2 *)p->tw);
+                                                            (float2 *)p->tw, ox, ot);
   } else {
     k_env<double><<<cdiv(nk, 256), 256, 0, st>>>(nk, 0, p->sigma_g * nk, (double *)p->Ek);
     k_env<double><<<cdiv(p->ew_len, 256), 256, 0, st>>>(p->ew_len, p->ew_off,
                                                        p->sigma_g * nw, (double *)p->Ews);
     k_tx_twiddles<double2><<<cdiv(tw_n, 256), 256, 0, st>>>(p->log2nx, p->log2nt - 1,
-                                                             (double2 *)p->tw);
+                                                             (double2 *)p->tw, ox, ot);
   }
   SRM3_CUDA(cudaGetLastError());
   return SRM3_OK;

@@ -171,7 +171,7 @@ __host__ __device__ constexpr int solve_col_threads(int lk) {
 // Rows: the iterate s (from g of the iteration before), h and its transform.
 template <int LM, typename T2>
 __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const SolveArgs A, int it) {
-  using F = decltype(T2::x);
+  using F = typename RealOf<T2>::type;
   if (solve_done(A, it)) return;
   extern __shared__ __align__(16) unsigned char solve_smem[];
   constexpr int M = 1 << LM, tpt = solve_tpt(LM), LV = solve_lv(LM);
@@ -202,10 +202,8 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const Solv
     return (solve_pos(A, k) && k != 0) ? solve_a2<F>(A, kk, w) * solve_q(s) : F(0.0);
   };
   auto src = [&](int m) -> T2 {
-    T2 v;
-    v.x = h_at(2 * m);
-    v.y = h_at(2 * m + 1);
-    return v;
+    const F re = h_at(2 * m);
+    return c_make<T2>(re, h_at(2 * m + 1));
   };
   auto dst = [&](int i, T2 v) {
     if (live) out[i] = v;
@@ -232,33 +230,22 @@ __global__ void __launch_bounds__(solve_col_threads(LK)) k_solve_cols(const Solv
   T2 *base = static_cast<T2 *>(A.Z) + f;
   const T2 *tw = static_cast<const T2 *>(A.twk);
   auto src1 = [&](int kk) -> T2 {
-    T2 v;
-    v.x = 0;
-    v.y = 0;
-    if (live && kk < nk) v = base[(size_t)kk * M];
-    return v;
+    return live && kk < nk ? base[(size_t)kk * M] : c_zero<T2>();
   };
   auto none = [](int, T2) {};
   stockham_passes<LK, 0, tx_mask_low_half<LK, LV>(), false, true, false, LV>(1, 0, tpt, jt, tw, col,
                                                                           src1, none);
-  T2 w1;  // 1 + e^{2 pi i f / M}; 0 at f = M / 2
-  w1.x = 0;
-  w1.y = 0;
+  using F = typename RealOf<T2>::type;
+  T2 w1 = c_zero<T2>();  // 1 + e^{2 pi i f / M}; 0 at f = M / 2
   if (live && p < M / 2) {
-    w1 = static_cast<const T2 *>(A.twz)[2 * p];
-    if (c >= TC && p > 0) w1.y = -w1.y;
-    w1.x = w1.x + decltype(w1.x)(1.0);
+    const T2 t = static_cast<const T2 *>(A.twz)[2 * p];
+    w1 = c_make<T2>(c_re(t) + F(1.0), c >= TC && p > 0 ? -c_im(t) : c_im(t));
   }
   auto src2 = [&](int i) -> T2 {  // conj V
     const T2 z = col[sp16(i)], y = other[sp16((Nk - i) & (Nk - 1))];
-    T2 o;  // -i (z - conj y) / 2
-    o.x = (z.y + y.y) * decltype(z.x)(0.5);
-    o.y = (y.x - z.x) * decltype(z.x)(0.5);
-    const T2 zz = cmul(z, z), oo = cmul(w1, cmul(o, o));
-    T2 v;
-    v.x = zz.x + oo.x;
-    v.y = -(zz.y + oo.y);
-    return v;
+    // -i (z - conj y) / 2
+    const T2 o = c_make<T2>((c_im(z) + c_im(y)) * F(0.5), (c_re(y) - c_re(z)) * F(0.5));
+    return c_conj(c_add(cmul(z, z), cmul(w1, cmul(o, o))));
   };
   auto dst2 = [&](int kk, T2 v) {
     if (live && kk < nk) base[(size_t)kk * M] = v;
@@ -271,7 +258,7 @@ __global__ void __launch_bounds__(solve_col_threads(LK)) k_solve_cols(const Solv
 // the row's omega = 0 pairs are summed directly.
 template <int LM, typename T2>
 __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_out(const SolveArgs A, int it) {
-  using F = decltype(T2::x);
+  using F = typename RealOf<T2>::type;
   if (solve_done(A, it)) return;
   extern __shared__ __align__(16) unsigned char solve_smem[];
   constexpr int M = 1 << LM, tpt = solve_tpt(LM), LV = solve_lv(LM);
@@ -316,8 +303,8 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_out(const Solve
   };
   auto src = [&](int i) -> T2 { return in[i]; };
   auto dst = [&](int m, T2 v) {
-    put(2 * m, v.x * half_inv);
-    put(2 * m + 1, -v.y * half_inv);
+    put(2 * m, c_re(v) * half_inv);
+    put(2 * m + 1, -c_im(v) * half_inv);
   };
   stockham_passes<LM, 0, 0u, false, false, true, LV>(1, 0, tpt, jt, static_cast<const T2 *>(A.twm),
                                                  buf, src, dst);

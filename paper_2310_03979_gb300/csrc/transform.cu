@@ -25,24 +25,32 @@ struct TxShape {
   size_t smem1, smem2;
 };
 
-TxShape tx_shape(const srm3_plan *p, size_t e2) {
+TxShape tx_shape(const srm3_plan *p, size_t e2, int n) {
   const size_t cap = 72 * 1024;
   const int wf = (int)(128 / e2);  // lanes of one shared-memory wavefront
   TxShape s{};
   const int L = p->nx, M = p->nt / 2;
+  const int tptx = out_tpt(p->log2nx, tx_nz(p->log2nx, p->nk, e2 == 8));
   int TC = 16;
   while (TC > 1 && TC / 2 >= p->nw) TC >>= 1;
   auto colstride = [&](int tc) {
     const int len = (tx_len(L) + wf - 1) / wf * wf;
     return len + (tc >= wf ? 1 : wf / tc);
   };
-  while (TC > 1 && ((size_t)TC * colstride(TC) * e2 > cap || TC * tx_tpt(L) > 512)) TC >>= 1;
+  int nsm = 0;  // narrower column groups where the wide ones leave SMs idle
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
+  while (TC > 1 && ((size_t)TC * colstride(TC) * e2 > cap || TC * tptx > 512 ||
+                    (TC > 4 && (long long)cdiv(p->nw, TC) * n < nsm)))
+    TC >>= 1;
   s.TC = TC;
   s.colstride = colstride(TC);
   s.smem1 = (size_t)TC * s.colstride * e2;
   s.rowstride = tx_len(M) + 1;
-  int rb = std::max(1, 64 / tx_tpt(M));
-  while (rb > 1 && ((size_t)rb * s.rowstride * e2 > cap || rb > p->nx)) rb >>= 1;
+  const int tpt = out_tpt(p->log2nt - 1, tx_nz(p->log2nt - 1, p->nw, e2 == 8));
+  int rb = std::max(1, 64 / tpt);
+  while (rb > 1 && ((size_t)rb * s.rowstride * e2 > cap || rb > p->nx ||
+                    (rb * tpt > 32 && (long long)(p->nx / rb) * n < nsm)))
+    rb >>= 1;
   s.rb = rb;
   s.smem2 = (size_t)rb * s.rowstride * e2;
   return s;
@@ -59,20 +67,6 @@ void with_log2(int v, F &&f) {
   }
 }
 
-// Nonzero input blocks of a stage's first pass (tx_in_mask): a length-2^l
-// transform whose inputs vanish except at the n indices of each end of the
-// spectrum (kk < nk or nx - kk < nk in x; m < nw or M - m < nw in t).  The
-// smallest of 1, 2, 4 blocks (of 2^l / R each, R the first radix) that
-// covers them, else 0 (all).  Pruned passes are compiled for FP32 and
-// transforms of 64 points or more.
-int tx_nz(int l, int n, bool fp32) {
-  if (!fp32 || l < 6) return 0;
-  const int R = 1 << tx_lr(l, 0), LR = (1 << l) / R;
-  for (int nz = 1; nz <= 4 && 2 * nz < R; nz *= 2)
-    if ((long long)nz * LR >= n) return nz;
-  return 0;
-}
-
 // f(integral_constant NZ) for NZ in {0, 1, 2, 4} equal to nz (0 alone when
 // the pruned forms are not compiled for this type and length).
 template <bool PRUNE, class F>
@@ -87,12 +81,16 @@ void with_nz(int nz, F &&f) {
 
 template <typename T, typename T2>
 int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2 *G) {
-  const TxShape s = tx_shape(p, sizeof(T2));
+  const TxShape s = tx_shape(p, sizeof(T2), n);
   const int lim = 200 * 1024;
-  const T2 *tw1 = (const T2 *)p->tw, *tw2 = tw1 + tx_twlen(p->log2nx);
-  const T2 *twz = tw2 + tx_twlen(p->log2nt - 1);
+  const T2 *tw1 = (const T2 *)p->tw, *tw2 = nullptr, *twz = nullptr;
   cudaError_t e = cudaSuccess;
   constexpr bool f32 = std::is_same<T, float>::value;
+  {
+    const int lx = p->log2nx, lt = p->log2nt - 1;
+    tw2 = tw1 + tx_twlen(lx, out_lv(lx, tx_nz(lx, p->nk, f32)));
+    twz = tw2 + tx_twlen(lt, out_lv(lt, tx_nz(lt, p->nw, f32)));
+  }
   with_log2<1, 13>(p->log2nx, [&](auto c) {
     constexpr int l = decltype(c)::value;
     with_nz<f32 && l >= 6>(tx_nz(l, p->nk, f32), [&](auto z) {
@@ -100,7 +98,7 @@ int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2
       e = cudaFuncSetAttribute(k_tx_cols<l, T2, nz>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                lim);
       if (e == cudaSuccess) {
-        k_tx_cols<l, T2, nz><<<dim3(cdiv(p->nw, s.TC), n), s.TC * tx_tpt(1 << l), s.smem1, st>>>(
+        k_tx_cols<l, T2, nz><<<dim3(cdiv(p->nw, s.TC), n), s.TC * out_tpt(l, nz), s.smem1, st>>>(
             p->nk, p->nw, s.TC, s.colstride, C, tw1, G);
         e = cudaGetLastError();
       }
@@ -114,7 +112,7 @@ int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2
       e = cudaFuncSetAttribute(k_tx_rows<l, T, T2, nz>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (e == cudaSuccess) {
-        k_tx_rows<l, T, T2, nz><<<dim3(p->nx / s.rb, n), s.rb * tx_tpt(1 << l), s.smem2, st>>>(
+        k_tx_rows<l, T, T2, nz><<<dim3(p->nx / s.rb, n), s.rb * out_tpt(l, nz), s.smem2, st>>>(
             p->nx, p->nw, s.rowstride, G, tw2, twz, out);
         e = cudaGetLastError();
       }
