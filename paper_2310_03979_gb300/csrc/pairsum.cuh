@@ -142,6 +142,15 @@ __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// a - b, as b * (-1) + a: one rounding either way
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+  return f2_fma(b, 0xbf800000bf800000ull, a);
+}
 __device__ __forceinline__ f32x2 f2_dup(float x) {
   f32x2 d;
   asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
@@ -323,40 +332,46 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
                                          const float4 *__restrict__ pb,
                                          const float2 *__restrict__ pw,
                                          const float2 *__restrict__ pe, int i0, int kw0,
-                                         f32x2 (&Txp)[packed::R], f32x2 (&Txm)[packed::R],
-                                         f32x2 (&Ty)[packed::R]) {
+                                         f32x2 (&Tx)[packed::R], f32x2 (&Ty)[packed::R]) {
   using namespace packed;
   // y_b rows by their offset m = v + U (NB - 1 - blk) from the lowest row any
   // block reads: every row keeps one name.
   ulonglong2 Bc[NV + U * (NB - 1)];
+  f32x2 Dc[NV + U * (NB - 1)];  // qx - qy
 #pragma unroll
   for (int blk = 0; blk < NB; ++blk) {
     if (i0 + blk * U > kw0 + R - 1) break;
-    ulonglong2 A[U];
+    f32x2 Ay[U], Am[U], As[U];  // py, px - py, px + py
 #pragma unroll
-    for (int uu = 0; uu < U; ++uu) A[uu] = lds_pair(pa + (blk * U + uu) * RS);
+    for (int uu = 0; uu < U; ++uu) {
+      const ulonglong2 v = lds_pair(pa + (blk * U + uu) * RS);
+      Ay[uu] = v.y;
+      Am[uu] = f2_sub(v.x, v.y);
+      As[uu] = f2_add(v.x, v.y);
+    }
     const int m0 = U * (NB - 1 - blk);
 #pragma unroll
     for (int v = (blk == 0 ? 0 : NV - U); v < NV; ++v) {
-      const int vv = blk == 0 ? v : v - (NV - U);  // rows not loaded yet
-      Bc[m0 + vv] = lds_pair(pb + (m0 + vv - U * (NB - 1)) * RS);
+      const int m = m0 + (blk == 0 ? v : v - (NV - U));  // rows not loaded yet
+      Bc[m] = lds_pair(pb + (m - U * (NB - 1)) * RS);
+      Dc[m] = f2_sub(Bc[m].x, Bc[m].y);
     }
-    const ulonglong2 *B = Bc + m0;
+    // one weighted product into the sums of output r
+    auto term = [&](int r, int uu, float wv) {
+      const int m = m0 + r - uu + U - 1;
+      const f32x2 w = f2_dup(wv), k = f2_mul(Ay[uu], Dc[m]);
+      Tx[r] = f2_fma(w, f2_fma(Am[uu], Bc[m].x, k), Tx[r]);
+      Ty[r] = f2_fma(w, f2_fma(As[uu], Bc[m].y, k), Ty[r]);
+    };
     if (TABLE) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const float4 w4 =
             *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(pw) + r * CH + blk * U);
-        const f32x2 w[U] = {f2_dup(w4.x), f2_dup(w4.y), f2_dup(w4.z), f2_dup(w4.w)};
-#pragma unroll
-        for (int uu = 0; uu < U; ++uu) {
-          const int v = r - uu + U - 1;
-          const f32x2 wpx = f2_mul(w[uu], A[uu].x), wpy = f2_mul(w[uu], A[uu].y);
-          Txp[r] = f2_fma(wpx, B[v].x, Txp[r]);
-          Txm[r] = f2_fma(wpy, B[v].y, Txm[r]);
-          Ty[r] = f2_fma(wpx, B[v].y, Ty[r]);
-          Ty[r] = f2_fma(wpy, B[v].x, Ty[r]);
-        }
+        term(r, 0, w4.x);
+        term(r, 1, w4.y);
+        term(r, 2, w4.z);
+        term(r, 3, w4.w);
       }
     } else {
       // the block's NE = 14 weights: three 16-byte loads and one 8-byte load
@@ -376,15 +391,7 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
 #pragma unroll
       for (int r = 0; r < R; ++r) {
 #pragma unroll
-        for (int uu = 0; uu < U; ++uu) {
-          const int v = r - uu + U - 1;
-          const f32x2 w = f2_dup(e[2 * uu - r + R - 1]);
-          const f32x2 wpx = f2_mul(w, A[uu].x), wpy = f2_mul(w, A[uu].y);
-          Txp[r] = f2_fma(wpx, B[v].x, Txp[r]);
-          Txm[r] = f2_fma(wpy, B[v].y, Txm[r]);
-          Ty[r] = f2_fma(wpx, B[v].y, Ty[r]);
-          Ty[r] = f2_fma(wpy, B[v].x, Ty[r]);
-        }
+        for (int uu = 0; uu < U; ++uu) term(r, uu, e[2 * uu - r + R - 1]);
       }
     }
   }
@@ -521,9 +528,9 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
     const bool tile_ok = kw0 < nw;
 #pragma unroll
     for (int j = 0; j < NK; ++j) kacc[j * NCT] = kcmp[j * NCT] = 0.f;
-    f32x2 Txp[R], Txm[R], Ty[R];
+    f32x2 Tx[R], Ty[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) Txp[r] = Txm[r] = Ty[r] = 0ull;
+    for (int r = 0; r < R; ++r) Tx[r] = Ty[r] = 0ull;
     int a = 0, c = 0;
     for (int item = 0; item < nitems; ++item, ++q) {
       const int stage = q & 1;
@@ -537,14 +544,14 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
         if (half) {
           const float4 *pa = sy + stage * STAGE_Y + hl * YROWS * (LANES / 2) + ln;
           const float4 *pb = pa + (CH + R * warp + CH - U) * (LANES / 2);
-          ps_chunk<false, LANES / 2>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
+          ps_chunk<false, LANES / 2>(pa, pb, pw, pe, i0, kw0, Tx, Ty);
         } else {
           const float4 *pa = sy + stage * STAGE_Y + lane;
           const float4 *pb = pa + (CH + R * warp + CH - U) * LANES;
           if (tab)
-            ps_chunk<true, LANES>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
+            ps_chunk<true, LANES>(pa, pb, pw, pe, i0, kw0, Tx, Ty);
           else
-            ps_chunk<false, LANES>(pa, pb, pw, pe, i0, kw0, Txp, Txm, Ty);
+            ps_chunk<false, LANES>(pa, pb, pw, pe, i0, kw0, Tx, Ty);
         }
       }
       mbar_arrive(&empty[stage]);
@@ -564,8 +571,8 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
         const float rowfac_odd = odd_live ? rw(2 * a + 1) : 0.0f;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const float2 xp = f2_split(Txp[r]), xm = f2_split(Txm[r]), yy = f2_split(Ty[r]);
-          float v[4] = {xp.x - xm.x, xp.y - xm.y, yy.x, yy.y};
+          const float2 xx = f2_split(Tx[r]), yy = f2_split(Ty[r]);
+          float v[4] = {xx.x, xx.y, yy.x, yy.y};
           if (live && ah == b) {
             const int kw = kw0 + r;
             if ((kw & 1) == 0 && kw < nw) {
@@ -614,7 +621,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
               }
             }
           }
-          Txp[r] = Txm[r] = Ty[r] = 0ull;
+          Tx[r] = Ty[r] = 0ull;
         }
       }
       if (++c == nch) {
