@@ -522,17 +522,129 @@ struct srm3_batch {
   bool capturing = false;         // inside srm3_batch_capture
   int max_ctas = 0;               // cap on the pair sum's CTAs (0: all resident)
   cudaEvent_t ps_ev[2] = {nullptr, nullptr};
+  // Self-convolution work that shares no buffer, each shape group and each
+  // plan on its own workspace a branch {group or -1, plan, lane}: lane 0 is the
+  // batch stream, lane l the stream side[l - 1], forked from and joined to it
+  struct Branch {
+    int group, plan, lane;
+  };
+  std::vector<Branch> branches;
+  std::vector<char> conv;  // plans sampled by the self-convolution, as they were at creation
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> joined;
+  cudaEvent_t forked = nullptr;
   long long dev_bytes = 0;        // device memory the batch allocated itself
 };
 
 using namespace srm3;
 
-// The launch sequence of one batch run on the batch stream.
+// The branches of a batch dealt to its lanes, the costliest first, each to the
+// lane with the least work so far.  A branch of a small lattice is a few launches
+// of a few dozen CTAs one after the other; side by side they fill the SMs.  32
+// spectra on 16 lattices of 32..256 per axis, captured: 3.07 -> 2.46 ms.
+static constexpr int kBatchLanes = 8;
+
+static int plan_branches(srm3_batch *b) {
+  struct Cost {
+    double c;
+    int group, plan;
+  };
+  std::vector<Cost> v;
+  auto cost = [](const srm3_plan *p, int n) { return (double)p->cNk * p->cNw * n; };
+  for (size_t g = 0; g < b->groups.size(); ++g) {
+    const int i = b->groups[g].members[0];
+    if (b->conv[i])
+      v.push_back({cost(b->plans[i], b->groups[g].total), (int)g, i});
+  }
+  for (size_t i = 0; i < b->plans.size(); ++i)
+    if (b->group_of[i] < 0 && b->conv[i])
+      v.push_back({cost(b->plans[i], b->counts[i]), -1, (int)i});
+  std::stable_sort(v.begin(), v.end(), [](const Cost &x, const Cost &y) { return x.c > y.c; });
+  const int lanes = std::min<int>(kBatchLanes, (int)v.size());
+  std::vector<double> load(std::max(lanes, 1), 0.0);
+  for (const Cost &x : v) {
+    const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    load[l] += x.c;
+    b->branches.push_back({x.group, x.plan, l});
+  }
+  if (lanes < 2) return SRM3_OK;
+  int prio = 0;  // the batch stream's
+  SRM3_CUDA(cudaStreamGetPriority(b->stream, &prio));
+  SRM3_CUDA(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
+  for (int l = 1; l < lanes; ++l) {
+    cudaStream_t st = nullptr;
+    cudaEvent_t ev = nullptr;
+    SRM3_CUDA(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, prio));
+    b->side.push_back(st);
+    SRM3_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    b->joined.push_back(ev);
+  }
+  return SRM3_OK;
+}
+
+// Phases, self-convolution and coefficients of a branch.
+static int branch_coeffs(srm3_batch *b, const srm3_batch::Branch &br, cudaStream_t st) {
+  srm3_plan *p = b->plans[br.plan];
+  const uint64_t *dseeds = b->dseeds + b->dev_off[br.plan];
+  if (br.group < 0) return conv_on(p, st, nullptr, dseeds, b->counts[br.plan], p->C);
+  const srm3_batch::Group &g = b->groups[br.group];
+  ConvJob j;
+  std::memset(&j, 0, sizeof(j));
+  j.plan = p;
+  j.stream = st;
+  j.n = g.total;
+  j.dseeds = dseeds;
+  j.sqq_of = (const void *const *)g.sqq_of;
+  j.pk_of = (const void *const *)g.pk_of;
+  j.ck_of = (const void *const *)g.ck_of;
+  j.work = g.y;
+  j.work_bytes = g.ybytes;
+  j.C = g.C;
+  return conv_sample(j);
+}
+
+// The fields of a shape group's members.
+static int group_fields(srm3_batch *b, const srm3_batch::Group &g, cudaStream_t st) {
+  for (size_t m = 0; m < g.members.size(); ++m) {
+    const int i = g.members[m];
+    srm3_plan *p = b->plans[i];
+    const char *C = (const char *)g.C + (size_t)2 * g.sample_off[m] * p->nk * p->nw *
+                                            sizeof(float2);
+    if (int rc = transform_on(p, st, C, b->counts[i], b->outs[i], g.H)) return rc;
+  }
+  return SRM3_OK;
+}
+static int branch_fields(srm3_batch *b, const srm3_batch::Branch &br, cudaStream_t st) {
+  if (br.group >= 0) return group_fields(b, b->groups[br.group], st);
+  srm3_plan *p = b->plans[br.plan];
+  return transform_on(p, st, p->C, b->counts[br.plan], b->outs[br.plan], p->H);
+}
+
+// The launch sequence of one batch run on the batch stream (and its lanes).
 static int batch_launch(srm3_batch *b) {
   int rc;
   const unsigned evf = b->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
+  // with the pair sum timed, everything on the batch stream, the pair sums first
+  const bool lanes = !b->timing && !b->side.empty();
+  if (lanes) {
+    SRM3_CUDA(cudaEventRecord(b->forked, b->stream));
+    for (cudaStream_t st : b->side) SRM3_CUDA(cudaStreamWaitEvent(st, b->forked, 0));
+    rc = SRM3_OK;
+    for (const auto &br : b->branches) {
+      if (br.lane == 0) continue;
+      const cudaStream_t st = b->side[br.lane - 1];
+      if (!rc) rc = branch_coeffs(b, br, st);
+      if (!rc) rc = branch_fields(b, br, st);
+    }
+    for (size_t l = 0; l < b->side.size(); ++l)
+      SRM3_CUDA(cudaEventRecord(b->joined[l], b->side[l]));
+    if (rc) {  // the lanes come back to the batch stream all the same
+      for (cudaEvent_t ev : b->joined) SRM3_CUDA(cudaStreamWaitEvent(b->stream, ev, 0));
+      return rc;
+    }
+  }
   for (auto &g : b->groups) {
-    if (conv_now(b->plans[g.members[0]])) continue;
+    if (b->conv[g.members[0]]) continue;
     SRM3_CUDA(cudaMemsetAsync(g.y, 0, g.ybytes, b->stream));
     for (size_t m = 0; m < g.members.size(); ++m) {
       const int i = g.members[m];
@@ -542,28 +654,14 @@ static int batch_launch(srm3_batch *b) {
     }
   }
   for (size_t i = 0; i < b->plans.size(); ++i)
-    if (b->group_of[i] < 0 && !conv_now(b->plans[i]) &&
+    if (b->group_of[i] < 0 && !b->conv[i] &&
         (rc = phases_on(b->plans[i], b->stream, nullptr, b->dseeds + b->dev_off[i],
                         b->counts[i], nullptr)))
       return rc;
   // in a capture the events must be external nodes of the graph
   if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[0], b->stream, evf));
-  for (auto &g : b->groups) {  // phases, self-convolution and coefficients of a shape group
-    if (!conv_now(b->plans[g.members[0]])) continue;
-    ConvJob j;
-    std::memset(&j, 0, sizeof(j));
-    j.plan = b->plans[g.members[0]];
-    j.stream = b->stream;
-    j.n = g.total;
-    j.dseeds = b->dseeds + b->dev_off[g.members[0]];
-    j.sqq_of = (const void *const *)g.sqq_of;
-    j.pk_of = (const void *const *)g.pk_of;
-    j.ck_of = (const void *const *)g.ck_of;
-    j.work = g.y;
-    j.work_bytes = g.ybytes;
-    j.C = g.C;
-    if ((rc = conv_sample(j))) return rc;
-  }
+  for (const auto &br : b->branches)
+    if ((!lanes || br.lane == 0) && (rc = branch_coeffs(b, br, b->stream))) return rc;
   if (b->nunits > 0) {
     PsDesc none;
     std::memset(static_cast<void *>(&none), 0, sizeof(none));
@@ -575,11 +673,8 @@ static int batch_launch(srm3_batch *b) {
   }
   for (size_t i = 0; i < b->plans.size(); ++i) {
     srm3_plan *p = b->plans[i];
-    if (b->group_of[i] >= 0) continue;
-    if (conv_now(p)) {
-      if ((rc = conv_on(p, b->stream, nullptr, b->dseeds + b->dev_off[i], b->counts[i], p->C)))
-        return rc;
-    } else if (p->mixed && p->precision == SRM3_FP32) {  // its difference pairs, after its sum pairs
+    if (b->group_of[i] >= 0 || b->conv[i]) continue;
+    if (p->mixed && p->precision == SRM3_FP32) {  // its difference pairs, after its sum pairs
       if ((rc = launch_pairsum_f32_diff(p, b->stream, b->counts[i], p->C))) return rc;
     } else if (p->precision == SRM3_FP64 &&
                (rc = pairsum_f64_on(p, b->stream, b->counts[i], p->C))) {
@@ -587,19 +682,18 @@ static int batch_launch(srm3_batch *b) {
     }
   }
   if (b->timing) SRM3_CUDA(cudaEventRecordWithFlags(b->ps_ev[1], b->stream, evf));
+  for (const auto &br : b->branches)
+    if ((!lanes || br.lane == 0) && (rc = branch_fields(b, br, b->stream))) return rc;
   for (auto &g : b->groups)
-    for (size_t m = 0; m < g.members.size(); ++m) {
-      const int i = g.members[m];
-      srm3_plan *p = b->plans[i];
-      const char *C = (const char *)g.C + (size_t)2 * g.sample_off[m] * p->nk * p->nw *
-                                              sizeof(float2);
-      if ((rc = transform_on(p, b->stream, C, b->counts[i], b->outs[i], g.H))) return rc;
-    }
-  for (size_t i = 0; i < b->plans.size(); ++i)
-    if (b->group_of[i] < 0 &&
-        (rc = transform_on(b->plans[i], b->stream, b->plans[i]->C, b->counts[i], b->outs[i],
-                           b->plans[i]->H)))
+    if (!b->conv[g.members[0]] && (rc = group_fields(b, g, b->stream))) return rc;
+  for (size_t i = 0; i < b->plans.size(); ++i) {
+    srm3_plan *p = b->plans[i];
+    if (b->group_of[i] < 0 && !b->conv[i] &&
+        (rc = transform_on(p, b->stream, p->C, b->counts[i], b->outs[i], p->H)))
       return rc;
+  }
+  if (lanes)
+    for (cudaEvent_t ev : b->joined) SRM3_CUDA(cudaStreamWaitEvent(b->stream, ev, 0));
   return SRM3_OK;
 }
 
@@ -607,6 +701,7 @@ static int batch_launch(srm3_batch *b) {
 // that creating and freeing batches never waits for work on other streams.
 static void batch_free(srm3_batch *b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
+  for (cudaStream_t st : b->side) cudaStreamSynchronize(st);
   if (b->holds_refs)
     for (size_t i = 0; i < b->plans.size(); ++i)
       if (b->group_of[i] < 0) --b->plans[i]->batch_refs;
@@ -614,6 +709,9 @@ static void batch_free(srm3_batch *b) {
   if (b->graph) cudaGraphDestroy(b->graph);
   for (cudaEvent_t e : b->ps_ev)
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : b->joined) cudaEventDestroy(e);
+  if (b->forked) cudaEventDestroy(b->forked);
+  for (cudaStream_t st : b->side) cudaStreamDestroy(st);
   for (auto &g : b->groups)
     for (void *q : {g.y, g.y0, g.C, g.H, (void *)g.sqq_of})
       if (q) cudaFreeAsync(q, b->stream);
@@ -913,6 +1011,7 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
   for (int i = 0; i < m; ++i) {
     srm3_plan *p = plans[i];
     b->plans.push_back(p);
+    b->conv.push_back(conv_now(p));
     b->counts.push_back(counts[i]);
     b->outs.push_back(outs[i]);
     b->seed_off.push_back(b->total);
@@ -1037,6 +1136,7 @@ SRM3_API int srm3_batch_create(srm3_plan *const *plans, const int32_t *counts,
   e = cudaMallocAsync(&b->dseeds, sizeof(uint64_t) * b->total, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMallocAsync(batch seeds)"));
+  if ((rc = plan_branches(b))) return bail(rc);
   b->hseeds.resize(b->total);
   for (int i = 0; i < m; ++i)  // plans whose own workspace the batch uses
     if (b->group_of[i] < 0) ++b->plans[i]->batch_refs;

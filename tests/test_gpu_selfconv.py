@@ -69,3 +69,35 @@ def test_samples_do_not_depend_on_the_scratch(precision, interactions, n):
         C = p.coeffs(list(range(1, n + 1)))
         for j in (0, 41, 42, n - 1):
             assert torch.equal(C[j], p.coeffs([j + 1])[0])
+
+
+@pytest.mark.parametrize("captured,timed", [(False, False), (True, False), (False, True)])
+def test_batch_lanes_match_plans_alone(captured, timed):
+    """More lattices than a batch has lanes, of every kind side by side (shape
+    groups, FP64, mixed, a plan of the O(N^2) pair sum): each plan's fields
+    are those of the plan alone, also when run again with other seeds."""
+    wls = [_case(nk, nw, "fp32") for nk, nw in
+           [(8, 8), (16, 8), (8, 16), (33, 20), (64, 40), (20, 64), (12, 12), (40, 9), (9, 40), (64, 40)]]
+    wls += [_case(16, 16, "fp64"), _case(12, 9, "fp32", interactions="mixed"),
+            _case(20, 24, "fp32", sigma_g=0.1)]
+    wls[-4] = replace(wls[-4], U=25.0)
+    plans = [srm3.Plan.create(w, storage="recompute") for w in wls]
+    counts = [1 + i % 5 for i in range(len(wls))]
+    outs = [torch.empty((c, w.n_x, w.n_t), device="cuda",
+                        dtype=torch.float64 if w.precision == "fp64" else torch.float32)
+            for c, w in zip(counts, wls)]
+    batch = srm3.Batch(plans, counts, outs)
+    batch.enable_timing(timed)
+    if captured:
+        batch.capture()
+    for base in (3, 5000):
+        seeds = [np.arange(base + 100 * i, base + 100 * i + c, dtype=np.uint64)
+                 for i, c in enumerate(counts)]
+        batch.run(np.concatenate(seeds))
+        batch.sync()
+        got = [o.clone() for o in outs]
+        for p, s, g in zip(plans, seeds, got):
+            assert torch.equal(p.sample(s), g)
+    batch.destroy()
+    for p in plans:
+        p.destroy()
