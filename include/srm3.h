@@ -485,8 +485,8 @@ int64_t srm3_batch_pair_terms(const srm3_batch *b);
  * the caller's output buffers are not included. */
 int64_t srm3_batch_device_bytes(const srm3_batch *b);
 
-/* Cap the batch's FP32 pair-sum launch at max_ctas CTAs (0: as many as are
- * resident, the default).  The launch is persistent and otherwise fills
+/* Cap the batch's FP32 pair-sum launch at max_ctas CTAs, counted as halves of
+ * an SM (0: as many as are resident, the default).  The launch is persistent and otherwise fills
  * every SM; a cap leaves room for work on other streams to run beside it
  * (a serving loop keeps short requests moving this way).  Set it before
  * srm3_batch_capture for graph replays. */

@@ -85,27 +85,40 @@ __global__ void __launch_bounds__(256) k_pairsum_f64(
 // arithmetic.
 //
 // Work unit: a super-tile of 32 outputs kws0..kws0+31 of lattice row kk for
-// one group of 64 sheet-samples.  Units are ordered by decreasing cost and
-// dealt to the resident CTAs in a snake order; a CTA walks its units one
-// after another.  Every lane carries two sheet-samples, stored pair-planar
+// one sample group of 64 sheet-samples.  Units are ordered by decreasing cost
+// and dealt to the warp groups of the resident CTAs in a snake order; a group
+// walks its units one after another.  Every lane carries two sheet-samples, stored pair-planar
 // as {x0, x1, y0, y1} (the layout k_phases writes for FP32 plans), so that
 // fma.rn.f32x2 / mul.rn.f32x2 act on both samples at once.
 //
-// Warps 0-3 compute: warp w owns the 8-output tile kw0 = kws0 + 8w.  Per row
+// Groups.  One CTA per SM holds three independent groups of four compute warps,
+// each with its own two stages, and a warpgroup of producers, one warp per
+// group.  What bounds the kernel is the packed FP32 pipe, and the warps that
+// keep it fed: with two groups per SM (CTAs of four compute warps and a
+// producer) it was 59 % active, each scheduler waiting on the latencies of two
+// warps.  Three need 12 x 32 x 168 registers, all of an SM's, so the producers
+// hand theirs over (setmaxnreg: 152 for a compute thread, 56 for a producer, 512
+// threads of 128 at launch) and the Kahan sums, 32 KB a group, moved from shared
+// to local memory (touched once per row pair).  256 x 512, 64 samples, stored W:
+// 64.6 -> 59.0 ms.  Without producers (the last warp done with a stage refilling
+// it, three CTAs per SM) it took 75.7 ms.
+//
+// Compute warp w of a group owns the 8-output tile kw0 = kws0 + 8w.  Per row
 // pair (a, b = kk - a) a thread forms, for r < 8,
 //   T_r = sum_iw w(r, iw) y_a[iw] y_b[kw0 + r - iw]
 // in blocks of 4 iw: 4 values of y_a and a window of 11 values of y_b serve 32
-// (r, iw) products; 7 of the 11 carry over to the next block.  A product is
-// w*p*q with the minus sign of the complex product kept in a third
-// accumulator:
-//   Tx+ += (w px) qx,  Tx- += (w py) qy,  Ty += (w px) qy + (w py) qx,
-// six packed instructions for two pair-terms.  Terms with iw > kw read zero
+// (r, iw) products; 7 of the 11 carry over to the next block.  The complex
+// product takes three multiplications,
+//   k = py (qx - qy),  Tx += w ((px - py) qx + k),  Ty += w ((px + py) qy + k),
+// five packed instructions for two pair-terms (and a difference per row of
+// y_b, two sums per row of y_a), against six with (w px), (w py) and four
+// products: 68.9 -> 64.6 ms.  Terms with iw > kw read zero
 // padding; the centre row a = b runs the full range and is halved with its
 // diagonal added back, T = (T_full + w y_{kw/2}^2) / 2.  Row partials are
-// merged once per row pair into Kahan-compensated FP32 sums kept in shared
+// merged once per row pair into Kahan-compensated FP32 sums kept in local
 // memory.
 //
-// Warp 4 produces: the omega range [0, kws0 + 31] of each row pair is
+// A group's producer: the omega range [0, kws0 + 31] of each row pair is
 // walked in chunks of 16, and for each chunk one lane stages the 16 y_a rows
 // and 48 y_b rows (47 used) of the group with four TMA tile loads of 16 rows
 // x 512 bytes through a 2-D tensor map over y (rows outside the lattice read
@@ -116,10 +129,10 @@ __global__ void __launch_bounds__(256) k_pairsum_f64(
 // cost 3 % of the launch), four weights per 16-byte load on the compute side,
 // each paired with itself (w, w) in registers for the packed products --
 // half the shared-memory loads of storing the pairs, worth 4 % of the launch;
-// otherwise the chunk's
-// 64-entry window of the omega envelope table Ew is bulk-copied, w =
-// Ew[2 iw - kw], each weight paired with itself in registers as above, with the kappa factor Ek[kk - 2a] applied
-// per row pair and c_k at the end.
+// otherwise the chunk's 64-entry window of the omega envelope table Ew is
+// bulk-copied, w = Ew[2 iw - kw], each weight paired with itself in registers
+// as above, with the kappa factor Ek[kk - 2a] applied per row pair and c_k at
+// the end.
 // Half-group mode (at most 32 sheet-samples, W recomputed): the lanes of a
 // group would be half empty, so each half-warp takes one of two row pairs
 // (a = 2i, 2i + 1) of a work item, on 256-byte rows staged by eight tile
@@ -128,9 +141,9 @@ __global__ void __launch_bounds__(256) k_pairsum_f64(
 // order as the full form, so a sample's result does not depend on how many
 // samples share its launch.
 // The compute warps release a stage through a second mbarrier.  Every wait
-// is bounded: past kWaitCycles the waiter raises the CTA's abort flag and
-// the error word, all warps leave their loops, and the producer first waits
-// (bounded again) for the copies it has in flight.
+// is bounded: past kWaitCycles the waiter raises the group's abort flag and
+// the error word, the group's warps leave their loops, and its producer first
+// waits (bounded again) for the copies it has in flight.
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 d;
@@ -178,36 +191,54 @@ constexpr long long kWaitCycles = 4000000000LL;  // about 2 s at 2 GHz
 static_assert(kTileU == CH && kTileR == R, "W table chunks: one 512-byte span per tile");
 static_assert(NB * U == CH && (NE % 2) == 0 && CH == BOX_ROWS, "block shape");
 
-// Tile shape of the FP32 pair sum: NC compute warps, each one 8-wide output
-// tile, make one super-tile of SW = 8 NC outputs (a work unit with one
-// sample group).  NC = 4 (32-wide) suits long rows; NC = 2 (16-wide) halves
-// the triangle of work across a super-tile's warps in the last chunks of
-// every row pair (the low tiles of a super-tile need fewer omega values), at
-// the cost of staging 48 rows per chunk for two warps instead of 64 for four.
-// The sums of an output and their order do not depend on NC: a warp walks
-// the same chunks and register blocks of its tile either way.
+// Tile shape of the FP32 pair sum: NC warps, each one 8-wide output tile, make
+// one super-tile of SW = 8 NC outputs (a work unit with one sample group).
+// NC = 4 (32-wide) suits long rows; NC = 2 (16-wide) halves the triangle of
+// work across a super-tile's warps in the last chunks of every row pair (the
+// low tiles of a super-tile need fewer omega values), at the cost of staging
+// 48 rows per chunk for two warps instead of 64 for four.  The sums of an
+// output and their order do not depend on NC: a warp walks the same chunks and
+// register blocks of its tile either way.
 template <int NC_>
 struct Shape {
   static constexpr int NC = NC_;                    // compute warps = tiles per super-tile
-  static constexpr int NCT = 32 * NC;               // compute threads
-  static constexpr int NT = NCT + 32;               // plus the producer warp
+  static constexpr int NCT = 32 * NC;               // compute threads of a group
+  static constexpr int NG = NC == 4 ? 3 : 4;        // groups per CTA
+  static constexpr int NT = NG * NCT + 128;         // threads of a CTA: and a warpgroup of producers
+  static constexpr int NTD = NCT + 32;              // difference pairs: one group, one producer
   static constexpr int SW = NC * R;                 // super-tile width
   static constexpr int YB_ROWS = CH + SW - 1;       // y_b rows per chunk
   static constexpr int YB_BOXES = (YB_ROWS + BOX_ROWS - 1) / BOX_ROWS;
   static constexpr int YROWS = CH + YB_BOXES * BOX_ROWS;  // staged rows per chunk
   static constexpr int STAGE_Y = YROWS * LANES;     // float4 per stage
-  static constexpr int STAGE_W = NC * R * CH;       // float2 slots per stage (W: the first half)
-  static constexpr int CTAS_PER_SM = NC == 4 ? 2 : 3;  // the launch bounds' residency
+  static constexpr int STAGE_W = NC * R * CH;       // floats per stage: W or the envelope window
   static_assert(2 * (CH - 1) + SW <= EWIN && EWIN <= STAGE_W, "envelope window of a chunk");
   static_assert(kPad >= SW + CH + 1, "staged rows stay inside the zero padding of y");
 };
+
+// Control words of a group, at the start of its shared memory.
+struct Ctl {
+  unsigned long long full[2], empty[2];
+  int abort;
+};
+constexpr int kCtlBytes = 128;
+static_assert(sizeof(Ctl) <= kCtlBytes, "control words");
 }  // namespace packed
 
 template <int NC>
-inline size_t pairsum_f32p_smem() {
+__host__ __device__ constexpr size_t ps_group_smem() {
   using namespace packed;
   using S = Shape<NC>;
-  return 128 + (size_t)2 * S::STAGE_Y * sizeof(float4) + (size_t)2 * S::STAGE_W * sizeof(float2) +
+  return kCtlBytes + (size_t)2 * S::STAGE_Y * sizeof(float4) + (size_t)2 * S::STAGE_W * sizeof(float);
+}
+template <int NC>
+inline size_t pairsum_f32p_smem() {
+  return packed::Shape<NC>::NG * ps_group_smem<NC>();
+}
+inline size_t pairsum_f32d_smem() {
+  using namespace packed;
+  using S = Shape<4>;
+  return kCtlBytes + (size_t)2 * S::STAGE_Y * sizeof(float4) + (size_t)2 * EWIN * sizeof(float) +
          (size_t)2 * NK * S::NCT * sizeof(float);
 }
 
@@ -330,8 +361,8 @@ __device__ __forceinline__ int4 ps_get_unit(int u, const PsDesc &d0,
 template <bool TABLE, int RS>
 __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
                                          const float4 *__restrict__ pb,
-                                         const float2 *__restrict__ pw,
-                                         const float2 *__restrict__ pe, int i0, int kw0,
+                                         const float *__restrict__ pw,
+                                         const float *__restrict__ pe, int i0, int kw0,
                                          f32x2 (&Tx)[packed::R], f32x2 (&Ty)[packed::R]) {
   using namespace packed;
   // y_b rows by their offset m = v + U (NB - 1 - blk) from the lowest row any
@@ -366,8 +397,7 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
     if (TABLE) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const float4 w4 =
-            *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(pw) + r * CH + blk * U);
+        const float4 w4 = *reinterpret_cast<const float4 *>(pw + r * CH + blk * U);
         term(r, 0, w4.x);
         term(r, 1, w4.y);
         term(r, 2, w4.z);
@@ -375,7 +405,7 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
       }
     } else {
       // the block's NE = 14 weights: three 16-byte loads and one 8-byte load
-      const float *pef = reinterpret_cast<const float *>(pe) + 8 * blk;
+      const float *pef = pe + 8 * blk;
       float e[NE];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
@@ -403,37 +433,43 @@ __device__ __forceinline__ void ps_chunk(const float4 *__restrict__ pa,
 // alone (every descriptor has half = 0); MIXED = true also takes half-mode
 // descriptors.
 template <bool MIXED, int NCW>
-__global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CTAS_PER_SM)
+__global__ void __launch_bounds__(packed::Shape<NCW>::NT, 1)
     k_pairsum_f32p(const __grid_constant__ PsDesc d0, const PsDesc *__restrict__ descs,
                    const int4 *__restrict__ units, int nunits, int *__restrict__ err) {
   using namespace packed;
   using S = Shape<NCW>;
-  constexpr int NC = S::NC, NCT = S::NCT, SW = S::SW, YB_BOXES = S::YB_BOXES, YROWS = S::YROWS;
-  constexpr int STAGE_Y = S::STAGE_Y, STAGE_W = S::STAGE_W;
+  constexpr int NC = S::NC, NCT = S::NCT, NG = S::NG, SW = S::SW, YB_BOXES = S::YB_BOXES;
+  constexpr int YROWS = S::YROWS, STAGE_Y = S::STAGE_Y, STAGE_W = S::STAGE_W;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  unsigned long long *full = reinterpret_cast<unsigned long long *>(smem_raw);  // [2]
-  unsigned long long *empty = full + 2;                                         // [2]
-  volatile int *abort = reinterpret_cast<volatile int *>(full + 4);
-  float4 *sy = reinterpret_cast<float4 *>(smem_raw + 128);    // [2][STAGE_Y]
-  float2 *sw = reinterpret_cast<float2 *>(sy + 2 * STAGE_Y);  // [2][STAGE_W] (W or envelope)
-  float *kst = reinterpret_cast<float *>(sw + 2 * STAGE_W);   // [2 NK][NCT]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) {
-    mbar_init(&full[0], 32);
-    mbar_init(&full[1], 32);
-    mbar_init(&empty[0], NCT);
-    mbar_init(&empty[1], NCT);
-    *abort = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const bool producer = tid >= NG * NCT;
+  // the group, and the warp's tile in it; its units are those of virtual CTA
+  // vc: consecutive (equally costly) units go to different SMs
+  const int wg = producer ? (tid - NG * NCT) >> 5 : tid / NCT, warp = (tid >> 5) % NC;
+  const int vc = wg * gridDim.x + blockIdx.x, nvc = NG * gridDim.x;
+  unsigned char *gs = smem_raw + (wg < NG ? wg : 0) * ps_group_smem<NCW>();
+  Ctl *ctl = reinterpret_cast<Ctl *>(gs);
+  volatile int *abort = &ctl->abort;
+  float4 *sy = reinterpret_cast<float4 *>(gs + kCtlBytes);   // [2][STAGE_Y]
+  float *sw = reinterpret_cast<float *>(sy + 2 * STAGE_Y);   // [2][STAGE_W] (W or envelope)
+  if (producer && wg < NG && lane == 0) {
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(&ctl->full[j], 32);
+      mbar_init(&ctl->empty[j], NCT);
+    }
+    ctl->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
 
-  if (warp == NC) {
-    // ---------------- producer ----------------
+  if (producer) {
+    // ---------------- producers ----------------
+    if constexpr (NCW == 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (wg >= NG) return;
     unsigned q = 0;
     bool ok = true;
     for (int k = 0; ok; ++k) {
-      const int u = ps_unit_id(k, blockIdx.x, gridDim.x);
+      const int u = ps_unit_id(k, vc, nvc);
       if (u >= nunits) break;
       const int4 un = ps_get_unit(u, d0, units);
       const PsDesc &d = descs ? descs[un.x] : d0;
@@ -445,7 +481,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
       int a = 0, c = 0;
       for (int item = 0; item < nitems; ++item, ++q) {
         const int stage = q & 1;
-        if (q >= 2 && !mbar_wait(&empty[stage], ((q >> 1) & 1) ^ 1, abort, err)) {
+        if (q >= 2 && !mbar_wait(&ctl->empty[stage], ((q >> 1) & 1) ^ 1, abort, err)) {
           ok = false;
           break;
         }
@@ -462,7 +498,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
           const unsigned tx = YROWS * ROW_BYTES +
                               (tab ? ntile * R * CH * (unsigned)sizeof(float)
                                    : EWIN * (unsigned)sizeof(float));
-          mbar_expect_tx(&full[stage], tx);
+          mbar_expect_tx(&ctl->full[stage], tx);
           // one row pair (full rows), or two in half mode (half rows each; a
           // second row pair past the centre repeats the first and is
           // weighted 0 by the compute warps)
@@ -470,29 +506,29 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
             const int ah = half ? min(2 * a + h, kk / 2) : a, bh = kk - ah;
             const int rw = half ? LANES / 2 : LANES;  // float4 per staged row
             float4 *dst = sy + stage * STAGE_Y + h * YROWS * (LANES / 2);
-            tma_load_2d(dst, &d.ymap, x, ah * rs + kPad + i0, &full[stage]);
+            tma_load_2d(dst, &d.ymap, x, ah * rs + kPad + i0, &ctl->full[stage]);
             const int jrow = bh * rs + kPad + kws0 - i0 - CH + 1;
 #pragma unroll
             for (int j = 0; j < YB_BOXES; ++j)
               tma_load_2d(dst + (CH + BOX_ROWS * j) * rw, &d.ymap, x, jrow + BOX_ROWS * j,
-                          &full[stage]);
+                          &ctl->full[stage]);
           }
           if (!tab) {
             bulk_g2s(sw + stage * STAGE_W, d.Ew + d.ew_off + 2 * i0 - kws0 - (SW - 1),
-                     EWIN * sizeof(float), &full[stage]);
+                     EWIN * sizeof(float), &ctl->full[stage]);
           } else {
             for (int t = 0; t < NC; ++t) {  // the tiles counted above
               const int k0 = kws0 + R * t;
               const int ncht = ((k0 + R + kTileU - 1) / kTileU) * kTileU / CH;
               if (k0 >= d.nw || c >= ncht) continue;
               const long long base = d.toff[kk * d.ntw + k0 / R];
-              bulk_g2s(reinterpret_cast<float *>(sw + stage * STAGE_W) + t * R * CH,
+              bulk_g2s(sw + stage * STAGE_W + t * R * CH,
                        d.W + base + ((long long)a * ncht + c) * R * CH,
-                       R * CH * (unsigned)sizeof(float), &full[stage]);
+                       R * CH * (unsigned)sizeof(float), &ctl->full[stage]);
             }
           }
         }
-        mbar_arrive(&full[stage]);
+        mbar_arrive(&ctl->full[stage]);
         if (++c == nch) {
           c = 0;
           ++a;
@@ -502,7 +538,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
     if (!ok) {  // leave no bulk copy in flight: wait (bounded) for the last two stages
       for (unsigned j = (q >= 2 ? q - 2 : 0); j < q; ++j) {
         const long long t0 = clock64();
-        while (!mbar_try_wait(&full[j & 1], (j >> 1) & 1) && clock64() - t0 < kWaitCycles) {
+        while (!mbar_try_wait(&ctl->full[j & 1], (j >> 1) & 1) && clock64() - t0 < kWaitCycles) {
         }
       }
     }
@@ -510,10 +546,16 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
   }
 
   // ---------------- compute warps ----------------
-  float *kacc = kst + tid, *kcmp = kst + NK * NCT + tid;
+  if constexpr (NCW == 4) asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
+  // Kahan sums and compensations of the tile, in local memory (a pointer the
+  // compiler cannot see through keeps them out of the registers)
+  float4 kst[2 * R];
+  float4 *kacc = kst;
+  asm volatile("" : "+l"(kacc));
+  float4 *kcmp = kacc + R;
   unsigned q = 0;
   for (int k = 0;; ++k) {
-    const int u = ps_unit_id(k, blockIdx.x, gridDim.x);
+    const int u = ps_unit_id(k, vc, nvc);
     if (u >= nunits) break;
     const int4 un = ps_get_unit(u, d0, units);
     const PsDesc &d = descs ? descs[un.x] : d0;
@@ -527,20 +569,18 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
     const size_t SP = (size_t)d.SSpad / 2;  // float4 per lattice entry
     const bool tile_ok = kw0 < nw;
 #pragma unroll
-    for (int j = 0; j < NK; ++j) kacc[j * NCT] = kcmp[j * NCT] = 0.f;
+    for (int r = 0; r < R; ++r) kacc[r] = kcmp[r] = make_float4(0.f, 0.f, 0.f, 0.f);
     f32x2 Tx[R], Ty[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) Tx[r] = Ty[r] = 0ull;
     int a = 0, c = 0;
     for (int item = 0; item < nitems; ++item, ++q) {
       const int stage = q & 1;
-      if (!mbar_wait(&full[stage], (q >> 1) & 1, abort, err)) return;
+      if (!mbar_wait(&ctl->full[stage], (q >> 1) & 1, abort, err)) return;
       const int i0 = c * CH;
       if (tile_ok) {
-        const float2 *pw = reinterpret_cast<const float2 *>(
-            reinterpret_cast<const float *>(sw + stage * STAGE_W) + warp * R * CH);
-        const float2 *pe = reinterpret_cast<const float2 *>(
-            reinterpret_cast<const float *>(sw + stage * STAGE_W) + (SW - R) - R * warp);
+        const float *pw = sw + stage * STAGE_W + warp * R * CH;
+        const float *pe = sw + stage * STAGE_W + (SW - R) - R * warp;
         if (half) {
           const float4 *pa = sy + stage * STAGE_Y + hl * YROWS * (LANES / 2) + ln;
           const float4 *pb = pa + (CH + R * warp + CH - U) * (LANES / 2);
@@ -554,7 +594,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
             ps_chunk<false, LANES>(pa, pb, pw, pe, i0, kw0, Tx, Ty);
         }
       }
-      mbar_arrive(&empty[stage]);
+      mbar_arrive(&ctl->empty[stage]);
       if (tile_ok && c == nch - 1) {  // row pair complete: centre-row halving and merge
         // Half mode: lanes 16-31 hand the odd row pair's terms to lanes 0-15,
         // which merge both row pairs in order -- the same sums, in the same
@@ -602,24 +642,21 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
 #pragma unroll
           for (int j = 0; j < 4; ++j) vo[j] = half ? __shfl_down_sync(0xffffffffu, v[j], 16) : 0.f;
           if (hl == 0) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {  // Kahan: s += rowfac v with compensation
-              float &s_ = kacc[(4 * r + j) * NCT], &cp = kcmp[(4 * r + j) * NCT];
-              const float s0 = s_, yv = fmaf(rowfac, v[j], -cp);
-              const float tt = s0 + yv;
-              cp = (tt - s0) - yv;
-              s_ = tt;
-            }
-            if (odd_live) {
+            float4 s4 = kacc[r], c4 = kcmp[r];
+            float *s_ = &s4.x, *cp = &c4.x;
+            auto add = [&](float fac, const float *t) {  // Kahan: s += fac t with compensation
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                float &s_ = kacc[(4 * r + j) * NCT], &cp = kcmp[(4 * r + j) * NCT];
-                const float s0 = s_, yv = fmaf(rowfac_odd, vo[j], -cp);
+                const float s0 = s_[j], yv = fmaf(fac, t[j], -cp[j]);
                 const float tt = s0 + yv;
-                cp = (tt - s0) - yv;
-                s_ = tt;
+                cp[j] = (tt - s0) - yv;
+                s_[j] = tt;
               }
-            }
+            };
+            add(rowfac, v);
+            if (odd_live) add(rowfac_odd, vo);
+            kacc[r] = s4;
+            kcmp[r] = c4;
           }
           Tx[r] = Ty[r] = 0ull;
         }
@@ -643,6 +680,7 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
       const float4 yk4 =
           d.y[((size_t)kk * d.rowstride + kPad + kw) * SP + (size_t)grp * LANES + ln];
       const float cf = ck[kidx];  // the pair factor (the table holds the envelopes alone)
+      const float4 s4 = kacc[r], c4 = kcmp[r];
       const float P = Pk[kidx];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -650,8 +688,8 @@ __global__ void __launch_bounds__(packed::Shape<NCW>::NT, packed::Shape<NCW>::CT
         if (ss >= d.SS) break;
         const float2 yk = (kidx == 0) ? d.y0[ss] : (h ? make_float2(yk4.y, yk4.w)
                                                        : make_float2(yk4.x, yk4.z));
-        const float ar = kacc[(4 * r + h) * NCT] - kcmp[(4 * r + h) * NCT];
-        const float ai = kacc[(4 * r + 2 + h) * NCT] - kcmp[(4 * r + 2 + h) * NCT];
+        const float ar = h ? s4.y - c4.y : s4.x - c4.x;
+        const float ai = h ? s4.w - c4.w : s4.z - c4.z;
         float2 out;
         out.x = fmaf(P, yk.x, __fmul_rn(cf, __fsub_rn(__fmul_rn(ar, d.cb), __fmul_rn(ai, d.sb))));
         out.y = fmaf(P, yk.y, __fmul_rn(cf, __fadd_rn(__fmul_rn(ar, d.sb), __fmul_rn(ai, d.cb))));
@@ -743,18 +781,18 @@ __device__ __forceinline__ void ps_chunk_diff(const float4 *__restrict__ pb,
   }
 }
 
-__global__ void __launch_bounds__(packed::Shape<4>::NT, 2) k_pairsum_f32d(
+__global__ void __launch_bounds__(packed::Shape<4>::NTD, 2) k_pairsum_f32d(
     const __grid_constant__ PsDiffDesc d, int nunits, int *__restrict__ err) {
   using namespace packed;
   using S = Shape<4>;
   constexpr int NC = S::NC, NCT = S::NCT, YB_BOXES = S::YB_BOXES, YROWS = S::YROWS;
-  constexpr int STAGE_Y = S::STAGE_Y, STAGE_W = S::STAGE_W;
+  constexpr int STAGE_Y = S::STAGE_Y, STAGE_W = EWIN;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned long long *full = reinterpret_cast<unsigned long long *>(smem_raw);  // [2]
   unsigned long long *empty = full + 2;                                         // [2]
   volatile int *abort = reinterpret_cast<volatile int *>(full + 4);
   float4 *sy = reinterpret_cast<float4 *>(smem_raw + 128);    // [2][STAGE_Y]
-  float2 *sw = reinterpret_cast<float2 *>(sy + 2 * STAGE_Y);  // [2][STAGE_W] (envelope)
+  float *sw = reinterpret_cast<float *>(sy + 2 * STAGE_Y);    // [2][STAGE_W] (envelope)
   float *kst = reinterpret_cast<float *>(sw + 2 * STAGE_W);   // [2 NK][NCT]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -844,7 +882,7 @@ __global__ void __launch_bounds__(packed::Shape<4>::NT, 2) k_pairsum_f32d(
       if (tile_ok) {
         const float4 *pb = sy + stage * STAGE_Y + lane;
         const float4 *pa = pb + (CH + R * warp) * LANES;
-        const float *pe = reinterpret_cast<const float *>(sw + stage * STAGE_W) + R * warp;
+        const float *pe = sw + stage * STAGE_W + R * warp;
         ps_chunk_diff<LANES>(pb, pa, pe, c * CH, kw0, nw, Txp, Txm, Ty);
       }
       mbar_arrive(&empty[stage]);

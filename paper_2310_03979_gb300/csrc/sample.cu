@@ -265,8 +265,11 @@ static int launch_pairsum_f32_nc(srm3_plan *p, cudaStream_t st, const PsDesc &d0
     if (per_sm < 1) return fail(SRM3_ERR_NOT_SUPPORTED, "FP32 pair sum does not fit on an SM");
     ctas = nsm * per_sm;
   }
-  int grid = std::min(nunits, ctas);
-  if (max_ctas > 0) grid = std::min(grid, max_ctas);
+  constexpr int NG = packed::Shape<NC>::NG;
+  int grid = std::min(cdiv(nunits, NG), ctas);
+  // the cap counts halves of an SM, so that a cap of one per SM leaves half the
+  // SMs (a CTA takes a whole one) to other streams
+  if (max_ctas > 0) grid = std::min(grid, cdiv(max_ctas, 2));
   if (grid == 0) return SRM3_OK;
   if (mixed)
     k_pairsum_f32p<true, NC><<<grid, NT, smem, st>>>(d0, descs, units, nunits, p->ps_err);
@@ -318,7 +321,7 @@ static int launch_pairsum_f32_diff(srm3_plan *p, cudaStream_t st, int n, void *C
   d.G = sp / (2 * packed::LANES);
   d.cb = (float)std::cos(p->beta);
   d.sb = (float)std::sin(p->beta);
-  const size_t smem = pairsum_f32p_smem<4>();
+  const size_t smem = pairsum_f32d_smem();
   SRM3_CUDA(cudaFuncSetAttribute(k_pairsum_f32d, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
   SRM3_CUDA(cudaFuncSetAttribute(k_pairsum_f32d, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -326,13 +329,13 @@ static int launch_pairsum_f32_diff(srm3_plan *p, cudaStream_t st, int n, void *C
   int nsm = 0, per_sm = 0;
   SRM3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device));
   SRM3_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairsum_f32d,
-                                                          packed::Shape<4>::NT,
+                                                          packed::Shape<4>::NTD,
                                                           smem));
   if (per_sm < 1) return fail(SRM3_ERR_NOT_SUPPORTED, "difference pair sum does not fit on an SM");
   const int nunits = p->nsuper_d * d.G;
   const int grid = std::min(nunits, nsm * per_sm);
   if (grid == 0) return SRM3_OK;
-  k_pairsum_f32d<<<grid, packed::Shape<4>::NT, smem, st>>>(d, nunits, p->ps_err);
+  k_pairsum_f32d<<<grid, packed::Shape<4>::NTD, smem, st>>>(d, nunits, p->ps_err);
   SRM3_CUDA(cudaGetLastError());
   return SRM3_OK;
 }
