@@ -123,8 +123,19 @@ __host__ __device__ constexpr int conv_tpt(int l) { return tx_tpt(1 << l, conv_l
 __host__ __device__ constexpr int conv_row_threads(int lw) {
   return conv_tpt(lw) >= 64 ? conv_tpt(lw) : 64;
 }
+// The column pass holds its CTAs to 64 registers a thread, 1024 threads per SM:
+// with the 68 that lengths past 512 took, one CTA of 512 was all an SM held, its
+// loads, transforms and stores one after the other.  Up to length 512 the CTAs
+// are of 256 threads, so that four of them overlap.  512 threads without the
+// limit / with it / 256 threads with it, ms: 16 samples of 512 x 1024 2.60 / 2.31 /
+// 2.34, 256 x 512 plan and 64 samples 3.58 / 3.54 / 3.52, 32 uneven spectra 2.46 /
+// 2.46 / 2.39; with the two as here 2.31, 3.51 and 2.39.  (Length 4096 would
+// spill.)
 __host__ __device__ constexpr int conv_col_threads(int lk) {
-  return conv_tpt(lk) > 512 ? conv_tpt(lk) : 512;
+  return conv_tpt(lk) > 512 ? conv_tpt(lk) : lk <= 9 ? 256 : 512;
+}
+__host__ __device__ constexpr int conv_col_ctas(int lk) {
+  return lk <= 11 ? 1024 / conv_col_threads(lk) : 1;
 }
 
 template <typename T2>
@@ -232,10 +243,9 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
 // in Z ([ss][n_kappa][Nw]: the grid's rows past n_kappa are zero and not
 // stored).  Shared memory: colstride entries per column.
 template <int LK, typename T2>
-__global__ void __launch_bounds__(conv_col_threads(LK)) k_conv_cols(int nk, int Nw, int TC,
-                                                                        int colstride,
-                                                                        const T2 *__restrict__ tw,
-                                                                        T2 *__restrict__ Z) {
+__global__ void __launch_bounds__(conv_col_threads(LK), conv_col_ctas(LK))
+    k_conv_cols(int nk, int Nw, int TC, int colstride, const T2 *__restrict__ tw,
+                T2 *__restrict__ Z) {
   extern __shared__ __align__(16) unsigned char conv_smem[];
   constexpr int Nk = 1 << LK, tpt = conv_tpt(LK), LV = conv_lv(LK);
   const int c = threadIdx.x & (TC - 1), jt = threadIdx.x / TC, ss = blockIdx.y;
