@@ -168,10 +168,19 @@ __host__ __device__ constexpr int solve_col_threads(int lk) {
   return 2 * solve_tpt(lk) > 256 ? 2 * solve_tpt(lk) : 256;
 }
 
+// The kernels of an iteration are launched as programmatic dependents
+// (solve_launch.cuh): the next one's CTAs are placed while this one runs and wait
+// here until it has completed and its writes are visible.
+__device__ __forceinline__ void solve_turn() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Rows: the iterate s (from g of the iteration before), h and its transform.
 template <int LM, typename T2>
 __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const SolveArgs A, int it) {
   using F = typename RealOf<T2>::type;
+  solve_turn();
   if (solve_done(A, it)) return;
   extern __shared__ __align__(16) unsigned char solve_smem[];
   constexpr int M = 1 << LM, tpt = solve_tpt(LM), LV = solve_lv(LM);
@@ -217,6 +226,7 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const Solv
 template <int LK, typename T2>
 __global__ void __launch_bounds__(solve_col_threads(LK)) k_solve_cols(const SolveArgs A, int it,
                                                                       int TC, int colstride) {
+  solve_turn();
   if (solve_done(A, it)) return;
   extern __shared__ __align__(16) unsigned char solve_smem[];
   constexpr int Nk = 1 << LK, tpt = solve_tpt(LK), LV = solve_lv(LK);
@@ -259,6 +269,7 @@ __global__ void __launch_bounds__(solve_col_threads(LK)) k_solve_cols(const Solv
 template <int LM, typename T2>
 __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_out(const SolveArgs A, int it) {
   using F = typename RealOf<T2>::type;
+  solve_turn();
   if (solve_done(A, it)) return;
   extern __shared__ __align__(16) unsigned char solve_smem[];
   constexpr int M = 1 << LM, tpt = solve_tpt(LM), LV = solve_lv(LM);

@@ -37,6 +37,28 @@ cudaError_t solve_prepare(int dev) {
   return e;
 }
 
+// A launch whose CTAs may be placed before the kernel ahead of it in the stream
+// has completed (its kernels wait for that themselves, solve_turn), where it has
+// at most one CTA per SM: early CTAs of larger launches settle unevenly on the
+// SMs.  Without / with / with this rule: 32 x 32 FP64 plan and sample 913 / 822 /
+// 817 us, 40 x 70 mixed with 16 samples 1028 / 867 / 864 us, 256 x 512 with 64
+// samples 3514 / 3617 / 3424 us.
+template <class... P, class... Q>
+cudaError_t solve_launch(void (*k)(P...), int nsm, int grid, int threads, size_t smem,
+                         cudaStream_t st, Q... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = grid <= nsm ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 // Column pairs per CTA: two where that still leaves two CTAs per SM, else one
 // (a pass is short: the spread over the SMs counts for more than the width of
 // its 16- or 32-byte accesses, which stay in L2).
@@ -63,7 +85,7 @@ int solve_iterate(SolveArgs A, int it, int device, int nsm, cudaStream_t st) {
   solve_with_log2<1, 12>(lm, [&](auto c) {
     constexpr int L = decltype(c)::value;
     err = solve_prepare<k_solve_rows<L, T2>>(device);
-    if (err == cudaSuccess) k_solve_rows<L, T2><<<rows, rthreads, srow, st>>>(A, it);
+    if (err == cudaSuccess) err = solve_launch(k_solve_rows<L, T2>, nsm, rows, rthreads, srow, st, A, it);
   });
   if (err == cudaSuccess) err = cudaGetLastError();
   if (err != cudaSuccess) return cuda_fail(err, "whole-lattice solve, rows");
@@ -71,15 +93,15 @@ int solve_iterate(SolveArgs A, int it, int device, int nsm, cudaStream_t st) {
     constexpr int L = decltype(c)::value;
     err = solve_prepare<k_solve_cols<L, T2>>(device);
     if (err == cudaSuccess)
-      k_solve_cols<L, T2>
-          <<<(pairs + TC - 1) / TC, 2 * TC * solve_tpt(L), scol, st>>>(A, it, TC, cs);
+      err = solve_launch(k_solve_cols<L, T2>, nsm, (pairs + TC - 1) / TC, 2 * TC * solve_tpt(L), scol, st,
+                         A, it, TC, cs);
   });
   if (err == cudaSuccess) err = cudaGetLastError();
   if (err != cudaSuccess) return cuda_fail(err, "whole-lattice solve, columns");
   solve_with_log2<1, 12>(lm, [&](auto c) {
     constexpr int L = decltype(c)::value;
     err = solve_prepare<k_solve_out<L, T2>>(device);
-    if (err == cudaSuccess) k_solve_out<L, T2><<<rows, rthreads, sout, st>>>(A, it);
+    if (err == cudaSuccess) err = solve_launch(k_solve_out<L, T2>, nsm, rows, rthreads, sout, st, A, it);
   });
   if (err == cudaSuccess) err = cudaGetLastError();
   if (err != cudaSuccess) return cuda_fail(err, "whole-lattice solve, output rows");
