@@ -5,17 +5,16 @@
 //
 // One pass over the values per call, HBM-bound: every CTA of a fixed grid
 // walks 16-byte vectors in a grid-stride loop, four vectors per thread per
-// step.  Power sums of d = u - shift go to FP64 per thread; FP32 input is
-// summed in FP32 over the 16 values of a step first (one FP64 add per power
-// per step: the FP64 pipe of this part is far narrower than its FP32 pipe),
-// FP64 input in FP64 throughout.  Bins are b = floor((u - lo) * (nbins /
-// (hi - lo))) in the input's precision, each operation rounded once; b < 0
-// counts below, b >= nbins (or a NaN) above, as two extra slots of the
-// shared histogram, so that every value costs one shared atomic and no
-// branch.  Per-CTA shared histograms merge into the global one with integer
-// atomics; the per-CTA power sums go to a partials array, added in a fixed
-// order of runs.  The same values given in the same calls yield
-// bit-identical results.
+// step.  FP32 input is summed in FP32 over the 16 values of a step, and those
+// sums of the powers of d = u - shift in double-float per thread (StatAcc), FP64
+// input in FP64 throughout; the threads' sums meet in FP64.  Bins are b =
+// floor((u - lo) * (nbins / (hi - lo))) in the input's precision, each operation
+// rounded once; b < 0 counts below, b >= nbins (or a NaN) above, as two extra
+// slots of the shared histogram, so that every value costs one shared atomic
+// and no branch (32 copies of the histogram, one per lane, measured the same).
+// Per-CTA shared histograms merge into the global one with integer atomics;
+// the per-CTA power sums go to a partials array, added in a fixed order of
+// runs.  The same values given in the same calls yield bit-identical results.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,6 +22,7 @@
 #include <vector>
 
 #include "srm3.h"
+#include "df.cuh"
 #include "srm3_internal.cuh"
 
 struct srm3_stats {
@@ -30,16 +30,22 @@ struct srm3_stats {
   double lo = 0.0, hi = 1.0, shift = 0.0;
   int grid = 0;
   double count = 0.0;
-  double *acc = nullptr;                 // [4] running power sums
+  // one block: [4] running power sums and the count of CTAs done (0 between
+  // calls), then the bins, below, above
+  double *acc = nullptr;
   double *part = nullptr;                // [grid][4] per-CTA sums of one call
-  unsigned long long *hist = nullptr;    // [nbins + 2]: bins, below, above
+  unsigned long long *hist = nullptr;    // acc + 5
 };
 
 namespace srm3 {
 namespace {
 
 constexpr int kStatThreads = 256;
-constexpr int kStatVec = 4;  // vectors per thread per step
+constexpr int kStatVec = 4;   // vectors per thread per step
+constexpr int kStatCtas = 4;  // CTAs per SM (2 or 3 with the next step's loads ahead: the same)
+
+// The accumulator's block: 4 sums, the CTA count, bins, below, above.
+size_t stat_bytes(int nbins) { return (5 + (size_t)nbins + 2) * 8; }
 
 template <typename T>
 struct StatVec;
@@ -70,6 +76,54 @@ __device__ __forceinline__ int stat_slot(T u, T lo, T scale, int nbins) {
   return t < (T)0 ? nbins : (t < (T)nbins ? (int)t : nbins + 1);
 }
 
+// A thread's running power sums over its steps.  FP64 input: FP64.  FP32 input:
+// double-float (a two-sum of the high part, its error in the low part: 48
+// bits, against the 24 of a step's own sum), as four FP64 additions and
+// conversions a step kept this part's FP64 pipe (2 lanes per SM and clock) busy
+// for most of the pass.  1.05e8 values, reset and read included: 159 -> 132 us
+// (121 us with the CTAs' sums merged by the last CTA in place of a launch, and one
+// block for sums and bins).  What a float could not hold, or infinities and
+// NaN, goes on in FP64.
+template <typename T>
+struct StatAcc {
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  __device__ __forceinline__ void add(T s1, T s2, T s3, T s4) {
+    a[0] += (double)s1;
+    a[1] += (double)s2;
+    a[2] += (double)s3;
+    a[3] += (double)s4;
+  }
+  __device__ __forceinline__ void flush() {}
+};
+template <>
+struct StatAcc<float> {
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+  __device__ __forceinline__ void flush() {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      a[p] += (double)h[p] + (double)l[p];
+      h[p] = l[p] = 0.f;
+    }
+  }
+  __device__ __forceinline__ void add(float s1, float s2, float s3, float s4) {
+    const float s[4] = {s1, s2, s3, s4};
+    // the fourth powers bound the others (|d|^p <= 1 + d^4)
+    if (!(s4 < 1e37f) || !(h[3] < 1e37f)) {
+      flush();
+#pragma unroll
+      for (int p = 0; p < 4; ++p) a[p] += (double)s[p];
+      return;
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      float e;
+      h[p] = two_sum(h[p], s[p], e);
+      l[p] = __fadd_rn(l[p], e);
+    }
+  }
+};
+
 // One value into the running FP32 (or FP64) power sums and the histogram.
 template <typename T>
 __device__ __forceinline__ void stat_one(T val, T sh, T lo, T scale, int nbins,
@@ -83,9 +137,10 @@ __device__ __forceinline__ void stat_one(T val, T sh, T lo, T scale, int nbins,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kStatThreads) k_stats(const T *__restrict__ u, long long count,
+__global__ void __launch_bounds__(kStatThreads, kStatCtas) k_stats(const T *__restrict__ u, long long count,
                                                         T lo, T scale, int nbins, double shift,
                                                         double *__restrict__ part,
+                                                        double *__restrict__ acc_out,
                                                         unsigned long long *__restrict__ hist) {
   using SV = StatVec<T>;
   using V = typename SV::V;
@@ -98,7 +153,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const T *__restrict__ u,
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const V *uv = reinterpret_cast<const V *>(u);
   const T sh = (T)shift;
-  double a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
+  StatAcc<T> acc;
   // steps whose kStatVec vectors all exist, without per-value checks
   const long long full = nv / (nth * kStatVec) * (nth * kStatVec);
   for (long long v0 = tid; v0 < full; v0 += nth * kStatVec) {
@@ -111,10 +166,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const T *__restrict__ u,
 #pragma unroll
       for (int i = 0; i < SV::N; ++i)
         stat_one<T>(SV::at(x[j], i), sh, lo, scale, nbins, sh_hist, s1, s2, s3, s4);
-    a1 += (double)s1;
-    a2 += (double)s2;
-    a3 += (double)s3;
-    a4 += (double)s4;
+    acc.add(s1, s2, s3, s4);
   }
   // the last partial step: one vector at a time
   for (long long v = full + tid; v < nv; v += nth) {
@@ -123,24 +175,19 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const T *__restrict__ u,
 #pragma unroll
     for (int i = 0; i < SV::N; ++i)
       stat_one<T>(SV::at(x, i), sh, lo, scale, nbins, sh_hist, s1, s2, s3, s4);
-    a1 += (double)s1;
-    a2 += (double)s2;
-    a3 += (double)s3;
-    a4 += (double)s4;
+    acc.add(s1, s2, s3, s4);
   }
   // the count % N trailing values: block 0, thread 0, in index order
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (long long e = nv * SV::N; e < count; ++e) {
       T s1 = 0, s2 = 0, s3 = 0, s4 = 0;
       stat_one<T>(u[e], sh, lo, scale, nbins, sh_hist, s1, s2, s3, s4);
-      a1 += (double)s1;
-      a2 += (double)s2;
-      a3 += (double)s3;
-      a4 += (double)s4;
+      acc.add(s1, s2, s3, s4);
     }
   }
   // CTA reduction in a fixed order: butterflies within warps, then warps in order
-  double a[4] = {a1, a2, a3, a4};
+  acc.flush();
+  double *a = acc.a;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
     for (int o = 16; o > 0; o >>= 1) a[p] += __shfl_xor_sync(0xffffffffu, a[p], o);
@@ -157,25 +204,28 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const T *__restrict__ u,
   }
   for (int b = threadIdx.x; b < nbins + 2; b += blockDim.x)
     if (sh_hist[b]) atomicAdd(hist + b, (unsigned long long)sh_hist[b]);
-}
-
-// acc[p] += sum over CTAs in a fixed order: thread t sums power t & 3 over
-// the t >> 2-th contiguous run of CTAs, then thread p < 4 adds the runs in
-// order.
-constexpr int kMergeThreads = 256;
-__global__ void __launch_bounds__(kMergeThreads) k_stats_merge(const double *__restrict__ part,
-                                                               int grid, double *__restrict__ acc) {
-  __shared__ double run[kMergeThreads];
-  const int t = threadIdx.x, p = t & 3, r = t >> 2, nr = kMergeThreads / 4;
-  const int per = (grid + nr - 1) / nr, c0 = r * per, c1 = min(grid, c0 + per);
+  // the last CTA to get here adds all CTAs' sums, in a fixed order: thread t sums
+  // power t & 3 over the t >> 2-th contiguous run of CTAs, then thread p < 4
+  // adds the runs in order
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0)
+    last = atomicInc(reinterpret_cast<unsigned int *>(acc_out + 4), gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  __shared__ double run[kStatThreads];
+  const int t = threadIdx.x, p = t & 3, r = t >> 2, nr = kStatThreads / 4;
+  const int grid = gridDim.x, per = (grid + nr - 1) / nr, c0 = r * per, c1 = min(grid, c0 + per);
   double s = 0.0;
-  for (int c = c0; c < c1; ++c) s += part[(size_t)c * 4 + p];
+  for (int c = c0; c < c1; ++c) s += __ldcg(part + (size_t)c * 4 + p);
   run[t] = s;
   __syncthreads();
   if (t < 4) {
     double tot = 0.0;
     for (int q = 0; q < nr; ++q) tot += run[4 * q + t];
-    acc[t] += tot;
+    acc_out[t] += tot;
   }
 }
 
@@ -200,17 +250,16 @@ SRM3_API int srm3_stats_create(int32_t nbins, double lo, double hi, double shift
   s->lo = lo;
   s->hi = hi;
   s->shift = shift;
-  s->grid = 4 * nsm;
-  cudaError_t e = cudaMalloc(&s->acc, 4 * sizeof(double));
+  s->grid = kStatCtas * nsm;
+  cudaError_t e = cudaMalloc(&s->acc, stat_bytes(nbins));
   if (e == cudaSuccess) e = cudaMalloc(&s->part, (size_t)s->grid * 4 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->hist, (size_t)(nbins + 2) * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemset(s->acc, 0, 4 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemset(s->hist, 0, (size_t)(nbins + 2) * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(s->acc, 0, stat_bytes(nbins));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     srm3_stats_destroy(s);
     return cuda_fail(e, "srm3_stats_create");
   }
+  s->hist = reinterpret_cast<unsigned long long *>(s->acc + 5);
   *out = s;
   return SRM3_OK;
 }
@@ -233,16 +282,14 @@ SRM3_API int srm3_stats_add(srm3_stats *s, const void *u, int32_t precision, int
                                    (int)smem));
     k_stats<float><<<s->grid, kStatThreads, smem, st>>>(
         static_cast<const float *>(u), count, (float)s->lo, (float)scale, s->nbins, s->shift,
-        s->part, s->hist);
+        s->part, s->acc, s->hist);
   } else {
     SRM3_CUDA(cudaFuncSetAttribute(k_stats<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)smem));
     k_stats<double><<<s->grid, kStatThreads, smem, st>>>(
         static_cast<const double *>(u), count, s->lo, scale, s->nbins, s->shift, s->part,
-        s->hist);
+        s->acc, s->hist);
   }
-  SRM3_CUDA(cudaGetLastError());
-  k_stats_merge<<<1, kMergeThreads, 0, st>>>(s->part, s->grid, s->acc);
   SRM3_CUDA(cudaGetLastError());
   s->count += (double)count;
   return SRM3_OK;
@@ -251,19 +298,19 @@ SRM3_API int srm3_stats_add(srm3_stats *s, const void *u, int32_t precision, int
 SRM3_API int srm3_stats_read(srm3_stats *s, void *stream, srm3_stats_result *r, uint64_t *hist) {
   if (!s || !r) return fail(SRM3_ERR_INVALID_ARG, "stats and result must be non-NULL");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  double acc[4];
-  std::vector<unsigned long long> h((size_t)s->nbins + 2);
-  SRM3_CUDA(cudaMemcpyAsync(acc, s->acc, sizeof(acc), cudaMemcpyDeviceToHost, st));
-  SRM3_CUDA(cudaMemcpyAsync(h.data(), s->hist, h.size() * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, st));
+  std::vector<unsigned long long> blk(stat_bytes(s->nbins) / 8);
+  SRM3_CUDA(cudaMemcpyAsync(blk.data(), s->acc, stat_bytes(s->nbins), cudaMemcpyDeviceToHost, st));
   SRM3_CUDA(cudaStreamSynchronize(st));
+  double acc[4];
+  std::memcpy(acc, blk.data(), sizeof(acc));
+  const unsigned long long *h = blk.data() + 5;
   std::memset(r, 0, sizeof(*r));
   const double n = s->count;
   r->count = n;
   for (int p = 0; p < 4; ++p) r->power_sum[p] = acc[p];
   r->below = h[s->nbins];
   r->above = h[s->nbins + 1];
-  if (hist) std::memcpy(hist, h.data(), (size_t)s->nbins * sizeof(uint64_t));
+  if (hist) std::memcpy(hist, h, (size_t)s->nbins * sizeof(uint64_t));
   if (n > 0) {
     // central moments about the mean from the moments about the shift
     const double m1 = acc[0] / n, e2 = acc[1] / n, e3 = acc[2] / n, e4 = acc[3] / n;
@@ -281,8 +328,7 @@ SRM3_API int srm3_stats_read(srm3_stats *s, void *stream, srm3_stats_result *r, 
 SRM3_API int srm3_stats_reset(srm3_stats *s, void *stream) {
   if (!s) return fail(SRM3_ERR_INVALID_ARG, "stats is NULL");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  SRM3_CUDA(cudaMemsetAsync(s->acc, 0, 4 * sizeof(double), st));
-  SRM3_CUDA(cudaMemsetAsync(s->hist, 0, ((size_t)s->nbins + 2) * sizeof(unsigned long long), st));
+  SRM3_CUDA(cudaMemsetAsync(s->acc, 0, stat_bytes(s->nbins), st));
   s->count = 0.0;
   return SRM3_OK;
 }
@@ -291,6 +337,5 @@ SRM3_API void srm3_stats_destroy(srm3_stats *s) {
   if (!s) return;
   if (s->acc) cudaFree(s->acc);
   if (s->part) cudaFree(s->part);
-  if (s->hist) cudaFree(s->hist);
   delete s;
 }

@@ -132,3 +132,29 @@ def test_sampled_fields_stats_and_skewness(envelope):
     assert abs(s - exact) < 5 * se, (s, exact, se)
     v, sev = np.mean(vars_), np.std(vars_, ddof=1) / math.sqrt(groups)
     assert abs(v - var) < 5 * sev, (v, var, sev)
+
+
+@pytest.mark.parametrize("big", [0.0, 3.0e9, 4.0e18, float("inf"), float("nan")])
+def test_stats_sums_past_the_range_of_a_float(big):
+    """FP32 sums leave double-float where a float's range ends (d^4 near and
+    past 3.4e38 in a step of 16 values), and infinities and NaN pass through
+    as they do in FP64.  Tolerance: 2e-6 of sum |u|^p where a step's own FP32
+    sum stays finite, as for ordinary values."""
+    n = 4 * 152 * 4 * 256 * 16 + 11  # several steps per thread, ragged
+    u = torch.randn(n, generator=torch.Generator().manual_seed(5)).cuda()
+    if big != 0.0:
+        u[17] = big
+        u[n - 3] = big
+    with srm3.Stats(100, -5, 5) as st:
+        st.add(u)
+        r = st.read()
+    d = u.double()
+    for p in range(4):
+        exact = float((d ** (p + 1)).sum())
+        got = r["power_sum"][p]
+        if not math.isfinite(exact):
+            assert math.isnan(got) if math.isnan(exact) else got == exact
+        elif big ** (p + 1) < 1e38:
+            assert abs(got - exact) <= 2e-6 * float((d.abs() ** (p + 1)).sum())
+        else:  # the step's own FP32 sum overflows, as it always did
+            assert got == math.inf
