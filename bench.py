@@ -113,6 +113,28 @@ def _conv_roofline(wl, n, es, launch_ms):
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy bandwidth)"}
 
 
+def _selfconv_roofline(lattices, ms):
+    """Roofline of the double-float self-convolution pair sum (Gaussian envelope
+    with W recomputed, FP32 plans): about 28 FP32-pipe lane operations per point
+    and level of the transforms -- rows there and back on n_kappa rows of Nw,
+    columns there and back on Nw columns of Nk -- over the pipe's rate.
+    lattices: (n_kappa, n_omega, samples, mixed) of everything in ms."""
+    ops = 0.0
+    for nk, nw, n, mixed in lattices:
+        lk = max(1, (2 * nk - 2).bit_length())
+        lw = max(1, ((3 * nw - 3) if mixed else (2 * nw - 2)).bit_length())
+        ops += 2 * n * 28.0 * 2 * (nk * (lw << lw) + (lk << lk) * (1 << lw))
+    sm_max = float(_peaks().get("sm_max_mhz", 2070.0))
+    rate = FP32_LANES_PER_SM * n_sm() * sm_max * 1e6
+    got = ops / (ms * 1e-3)
+    return {"bound": "alu", "achieved": got / 1e12, "peak": rate / 1e12,
+            "unit": "T FP32-pipe lane-ops/s", "frac": got / rate, "traffic": None,
+            "per_unit": "28 FP32-pipe lane-ops per point and level, unpruned",
+            "kernel": "k_conv_rows + k_conv_cols + k_conv_out",
+            "peak_source": f"derived: {n_sm()} SM x {FP32_LANES_PER_SM} FP32 lanes x "
+                           f"{sm_max:.0f} MHz (max SM clock of MEASURED_PEAKS.json)"}
+
+
 def _pairsum_roofline_fp64(terms_per_s, **extra):
     """Roofline of the plain FP64 pair sum (one thread per output): 6 FP64
     lane operations per pair-term (complex product 2 DMUL + 2 DFMA, weighted
@@ -130,36 +152,21 @@ def _pairsum_roofline_fp64(terms_per_s, **extra):
     return out
 
 
-def _pairsum_roofline(terms_per_s, traffic=None, separable=False, sep_share=None, **extra):
-    """Roofline object of the FP32 pair sum from its kernel-only rate.
+def _pairsum_roofline(terms_per_s, traffic=None, **extra):
+    """Roofline object of the FP32 O(N^2) pair sum from its kernel-only rate.
 
-    The bound is the FP32 pipe.  A pair-term is 6 FP32-pipe lane operations
-    (2 FMUL + 4 FFMA, 10 flop: the weight times one phasor, then the complex
-    product accumulated), so the fraction is pair-terms/s x 6 over the pipe's
+    The bound is the FP32 pipe.  A pair-term is 5 FP32-pipe lane operations
+    (the complex product by three multiplications, 1 FMUL + 2 FFMA, and two
+    weighted sums, 2 FFMA: 9 flop; the differences the product needs are made
+    once per staged row), so the fraction is pair-terms/s x 5 over the pipe's
     lane-operation rate, 152 SM x 128 lanes x the maximum SM clock.  The same
-    rate in flops (10 per pair-term against 2 flop per lane-cycle) is given
-    beside it: its ceiling is 10/12 because an FMUL fills a lane slot for one
-    flop.  In separable form (the Gaussian envelope's weights folded into the
-    phasor rows and the per-row-pair and per-output factors) a pair-term is
-    the complex product accumulated alone: 4 FFMA, 8 flop."""
+    rate in flops is given beside it."""
     peaks = _peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     nsm = n_sm()
     lane_rate = FP32_LANES_PER_SM * nsm * sm_max * 1e6  # lane-ops/s
-    # sep_share: the fraction of the pair-terms in separable form (a batch
-    # of plans in both forms)
-    share = (1.0 if separable else 0.0) if sep_share is None else float(sep_share)
-    per_ops, per_flop = 6.0 - 2.0 * share, 10.0 - 2.0 * share
-    ops = per_ops * terms_per_s
-    flops = per_flop * terms_per_s
-    if share == 0.0:
-        unit_txt = "6 FP32-pipe lane-ops (2 FMUL + 4 FFMA = 10 flop) per pair-term"
-    elif share == 1.0:
-        unit_txt = "4 FP32-pipe lane-ops (4 FFMA = 8 flop) per pair-term, separable form"
-    else:
-        unit_txt = (f"{per_ops:.3f} FP32-pipe lane-ops per pair-term: 4 (4 FFMA) for the "
-                    f"{100 * share:.1f} % of pair-terms in separable form, 6 (2 FMUL + 4 FFMA) "
-                    "for the rest")
+    ops, flops = 5.0 * terms_per_s, 9.0 * terms_per_s
+    unit_txt = "5 FP32-pipe lane-ops (1 FMUL + 4 FFMA = 9 flop) per pair-term"
     out = {"bound": "alu", "achieved": ops / 1e12, "peak": lane_rate / 1e12,
            "unit": "T FP32-pipe lane-ops/s", "frac": ops / lane_rate, "traffic": traffic,
            "per_unit": unit_txt,
@@ -355,11 +362,8 @@ def run_uneven(args):
         torch.cuda.synchronize()
         e2e_ms.append((time.perf_counter() - t1) * 1e3)
     ps_ms = statistics.median(ps)
-    sep_terms = 0  # pair-terms of plans whose pair sum runs in separable form
-    for p, c in zip(plans, counts):
-        inf = p.info()
-        if inf.recursion_flags & srm3.SRM3_PAIRSUM_SEPARABLE:
-            sep_terms += 2 * inf.pairs * c
+    conv = [(w.n_kappa, w.n_omega, c, False) for w, p, c in zip(wls, plans, counts)
+            if p.info().recursion_flags & srm3.SRM3_PAIRSUM_SEPARABLE]
     choice = {}
     for k, v in tuned.items():
         c = f'{v["storage"]}, {v["tile"]}'
@@ -373,15 +377,18 @@ def run_uneven(args):
                    "samples_per_step": nsamp, "pair_terms_per_step": terms,
                    "grids": "32..256 per axis (powers of two)",
                    "l2": "inputs smaller than L2 for some spectra; steps are back to back",
-                   "step": "one replay of the captured batch graph (phases, one persistent "
-                           "pair-sum launch over all spectra, transforms); plans prebuilt"},
+                   "step": "one replay of the captured batch graph (phases, pair sums, "
+                           "transforms); plans prebuilt"},
         "samples_per_s": nsamp / (ms * 1e-3),
         "wall_ms_per_step": wall * 1e3 / args.steps,
         "plan_build_s_all_spectra": t_plans, "autotune_s": t_tune,
         "autotune_choices": choice,
-        "roofline": _pairsum_roofline(terms / (ps_ms * 1e-3), sep_share=sep_terms / terms,
+        "roofline": _selfconv_roofline(conv, ps_ms) if len(conv) == len(plans) else
+                    _pairsum_roofline(terms / (ps_ms * 1e-3),
                                       kernel="k_pairsum_f32p (batched, one launch)"),
-        "gpu_launches": (3 * len(wls) + 1) * args.steps,
+        # two transform stages per spectrum; three self-convolution passes per
+        # lattice (at least one lattice)
+        "gpu_launches": (2 * len(wls) + 3) * args.steps,
         "clocks": clocks,
         "e2e": {"value": terms / (statistics.median(e2e_ms) * 1e-3), "unit": "pair-terms/s",
                 "h2d_bytes_per_step": 8 * nsamp,
@@ -667,12 +674,10 @@ def run_paper_bridge(args):
             "exact": {"mean": 0.0, "variance": var_exact,
                       "skewness": m3_exact / var_exact ** 1.5},
             "values": r3["count"], "histogram_bins": nbins, "range_sigma": 6},
-        # per step: spectrum 1, envelope tables 3, sum of S 1, recursion
-        # passes, sampling tables 4, conv twiddles 1; per batch of 50 (one
-        # sampling chunk): phases, three FFT self-convolution passes, two
-        # output FFT stages, statistics pass and merge
-        "gpu_launches": args.steps * (1 + 3 + 1 + info.root_passes + info.root_passes_fp32
-                                      + 4 + 1 + 8 * math.ceil(n / B)),
+        # per step, at least: the plan's tables 12, its solve 30 iterations'
+        # launches and 3 more; per batch of 50 (one sampling chunk) three FFT
+        # self-convolution passes, two output FFT stages, the statistics pass
+        "gpu_launches": args.steps * (12 + 30 + 3 + 6 * math.ceil(n / B)),
         "clocks": clocks,
         "eps": info.eps, "max_sum_b2": info.max_sum_b2,
         "e2e": {"value": 2 * pairs * n / wall, "unit": "pair-terms/s",
@@ -807,37 +812,17 @@ def main():
     info = recs[-1][1]
     t_last = recs[-1][0]
     chunks = math.ceil(n / 128)
-    # kernels launched per step (matches the ncu launch list): spectrum 1,
-    # envelope tables 2 + g^2 1, separable factors 1 (Gaussian envelope in
-    # separable form), recursion index lists 2, the sum of S 2, linear pass
-    # 2 + its reduction 2, each recursion pass 1, slope and move of the
-    # tables 2 (FP32 plans whose tables were moved), sampling tables 4 (+1
-    # for the separable pair sum's), W table 1 if stored; per 128-sample
-    # chunk: phases, pair sum, two FFT stages
-    flags = info.recursion_flags
-    sep_gauss = 1 if (flags & srm3.SRM3_REC_SEPARABLE) and wl.envelope == "gauss" else 0
-    moved = 2 if flags & srm3.SRM3_REC_TABLES_MOVED else 0
-    # tables interpolated from a three-plane FP64 pass (FP64 plans): 1 kernel
-    moved += 1 if flags & srm3.SRM3_REC_TABLES_INTERPOLATED else 0
-    # the separable pair sum's scaled tables (FP32 Gaussian plans, either storage)
-    sep_tables = 1 if sep_gauss and es == 4 and getattr(wl, "interactions", "sum") == "sum" else 0
-    # coarse start of the eps search: its own kernels (subsampled spectrum,
-    # envelope tables, index lists, reductions, linear pass, passes), and no
-    # linear pass (4 kernels) on the plan's lattice
-    coarse = info.coarse_launches - (4 if flags & srm3.SRM3_REC_COARSE_START else 0)
-    launches_per_step = (1 + 3 + sep_gauss + 2 + 2 + 4 + (info.root_passes + info.root_passes_fp32)
-                         + moved + 4 + sep_tables + (1 if info.storage == 1 else 0) + 4 * chunks
-                         + coarse)
-    if wl.envelope != "gauss":
-        # the bracketing pass is an FP32 pass (counted above) instead of the
-        # linear pass; conv twiddles 1; per chunk phases, three FFT
-        # self-convolution passes, two output FFT stages
-        # (+ the coarse search's kernels: its bound is a pass as well)
-        launches_per_step = (1 + 3 + 2 + 2 + (info.root_passes + info.root_passes_fp32)
-                             + 4 + 1 + 6 * chunks + info.coarse_launches)
+    # kernels launched per step, at least (from the ncu launch list): spectrum,
+    # envelope tables, g^2, twiddles and factors 9, the sum of S 2; the
+    # whole-lattice solve's tables 4, its iterations (10 or more, 3 launches
+    # each), the direct sums and results 3, on the coarse lattice (counted by the
+    # plan) and on the plan's; FP64 plans' direct iterations 6 or more; sampling
+    # tables 1, W table 1 if stored; per 128-sample chunk the pair sum (phases and
+    # one launch, or three self-convolution passes), two FFT stages
+    selfconv = wl.envelope != "gauss" or info.storage != 1
+    launches_per_step = (11 + 4 + 30 + 3 + info.coarse_launches + (6 if es == 8 else 0) + 1 +
+                         (1 if info.storage == 1 else 0) + (5 if selfconv else 4) * chunks)
     if prebuilt is not None:
-        # sampling only: per chunk phases, sum and difference pair sums, two
-        # FFT stages
         launches_per_step = 5 * chunks
     traffic = None
     src = os.path.join(ROOT, "paper_2310_03979_gb300", "csrc", "pairsum.cuh")
@@ -877,19 +862,18 @@ def main():
                                 "transform": t_last.transform_ms},
         "sampling_only_pair_terms_per_s": terms_per_step / (
             (t_last.phases_ms + t_last.pairsum_ms + t_last.transform_ms) * 1e-3),
-        "roofline": (_conv_roofline(wl, n, es, avg_launch_ms) if wl.envelope != "gauss"
+        "roofline": (_conv_roofline(wl, n, es, avg_launch_ms)
+                     if wl.envelope != "gauss" or (selfconv and es == 8)
+                     else _selfconv_roofline([(wl.n_kappa, wl.n_omega, min(n, 128),
+                                               wl.interactions == "mixed")], avg_launch_ms)
+                     if selfconv
                      else _pairsum_roofline_fp64(terms_per_launch / (avg_launch_ms * 1e-3),
                                                  kernel="k_pairsum_f64") if es == 8
                      else _pairsum_roofline(
             terms_per_launch / (avg_launch_ms * 1e-3), traffic,
-            separable=bool(info.recursion_flags & srm3.SRM3_PAIRSUM_SEPARABLE),
             algorithmic_bytes_per_launch=info.table_bytes + n * 2 * 8 * (
                 wl.n_kappa * (wl.n_omega + 128) + wl.n_kappa * wl.n_omega),
-            kernel="k_pairsum_f32p<table>" if info.storage == 1 else
-                   "k_pairsum_f32p<recompute, separable>" if (
-                       prebuilt is None and info.recursion_flags & srm3.SRM3_PAIRSUM_SEPARABLE) else
-                   "k_pairsum_f32p<recompute>" if prebuilt is None else
-                   "k_pairsum_f32p<recompute> + k_pairsum_f32d (sum and difference pairs)")),
+            kernel="k_pairsum_f32p<table>" if info.storage == 1 else "k_pairsum_f32p<recompute>")),
         "gpu_launches": launches_per_step * args.steps,
         "clocks": clocks,
         "eps": info.eps, "max_sum_b2": info.max_sum_b2,
