@@ -1060,6 +1060,7 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
                                                      double *__restrict__ sb2,
                                                      double *__restrict__ q) {
   __shared__ double sX;
+  __shared__ int sLast;
   if (threadIdx.x < 32) {  // the first iteration that was the last
     int first = nit;
     for (int j = threadIdx.x; j < nit; j += 32)
@@ -1071,6 +1072,7 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
     if (threadIdx.x == 0) {
       const int last = min(first, nit - 1);
       sX = solve_X(A, last);
+      sLast = last;
       const double gm = as_double(A.ctl->gmax);
       if (stage == 2 && A.target > 0.0) sX = gm > 0.0 ? A.target / gm : 0.0;
       if (blockIdx.x == 0) {
@@ -1089,7 +1091,7 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
     if (stage == 1) {
       const int kk = (int)(i / A.nw), kw = (int)(i - (long long)kk * A.nw);
       direct = low && (long long)(kk + 1) * (kw + 1) <= kSolveLow;
-      g64[i] = g = solve_real(static_cast<const F *>(A.g)[i]);
+      g64[i] = g = solve_real(static_cast<const F *>(A.g[sLast % 3])[i]);
     } else {
       g = g64[i];
     }
@@ -1179,8 +1181,6 @@ struct SolveResult {
   bool no_pairs;
 };
 
-// Iterations launched per further look of the host.
-static constexpr int kSolveMore = 5;
 // largest change of s at which the solve stops: the coarse
 // lattice's, and the root estimate the FP64 passes of FP64 plans start from
 // (their reach is 1e-5); the tables of FP32 plans (target met to 1e-9), in
@@ -1209,7 +1209,7 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   const size_t zb = (size_t)nk * M * 16, lb = up((size_t)nl * 8), tb = (size_t)ntw * 16;
   const size_t fb = up((size_t)nfac * 8);
   char *blk = nullptr, *at = nullptr;
-  SRM3_CUDA(dev_alloc((void **)&blk, zb + (p->sep ? 6 : 4) * lb + tb + 2 * fb + sizeof(SolveCtl), st));
+  SRM3_CUDA(dev_alloc((void **)&blk, zb + (p->sep ? 10 : 8) * lb + tb + 2 * fb + sizeof(SolveCtl), st));
   struct Guard {
     char *b;
     cudaStream_t st;
@@ -1230,9 +1230,9 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   A.mixed = p->mixed ? 1 : 0;
   A.S = p->S;
   A.Z = take(zb);
-  A.g = take(lb);
+  for (void *&g : A.g) g = take(lb);
+  for (void *&s : A.s) s = take(lb);
   double *g64 = reinterpret_cast<double *>(take(lb));
-  char *s[2] = {take(lb), take(lb)};
   char *tw = take(tb);
   A.ctl = reinterpret_cast<SolveCtl *>(take(sizeof(SolveCtl)));
   A.twk = tw;
@@ -1281,9 +1281,9 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
     k_solve_prolong<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, fk, fw, from->nk, from->nw, from->sb2,
                                                    g64);
     if (fp64)
-      k_solve_convert<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (double *)s[0]);
+      k_solve_convert<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (double *)A.s[3]);
     else
-      k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (df *)s[0]);
+      k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (df *)A.s[3]);
     A.warm = 1;
     A.hold = from == p ? 0 : hold;
     p->n_launch += 2;
@@ -1302,15 +1302,15 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   int nlow = 0, nit = 0;
   for (int kk = 0; kk < std::min(nk, kSolveLow); ++kk) nlow += solve_low_ctas(kk, nw);
   // iterations launched before the host looks, from how long they take (a
-  // converged solve's later launches return at once): the damped ones from
-  // scratch, from a coarser lattice's solution or from this lattice's own
-  const int first = from == p ? (target > 0.0 ? 12 : 6) : tol >= kSolveLoose ? 16 : 21;
+  // converged solve's later launches return at once): mixed ones (Gaussian
+  // envelope) to the loose or the tight change; of separable bispectra, damped
+  // ones from scratch or a coarser lattice, or from this lattice's own solution
+  const int first = !p->sep ? (tol >= kSolveLoose ? 12 : 15)
+                            : from == p ? (target > 0.0 ? 12 : 6) : 16;
   A.accept = std::max(tol, fp64 ? kSolveAcceptF64 : kSolveAcceptDf);
   do {
-    const int upto = std::min(kSolveMaxIt, nit + (nit == 0 ? first : kSolveMore));
+    const int upto = std::min(kSolveMaxIt, nit + (nit == 0 ? first : p->sep ? 5 : 3));
     for (; nit < upto; ++nit) {
-      A.s_in = s[nit & 1];
-      A.s_out = s[(nit + 1) & 1];
       const int rc = fp64 ? solve_iterate_f64(A, nit, p->device, occ.nsm, st)
                           : solve_iterate_df(A, nit, p->device, occ.nsm, st);
       if (rc) return rc;

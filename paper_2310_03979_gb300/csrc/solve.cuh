@@ -9,13 +9,20 @@
 //  * Given X (a fixed eps): plain iterations from s = 0.  A point's sum takes
 //    lower points only, so the error's dependence is strictly triangular and
 //    the iterations converge faster than geometrically (about ten).
-//  * Given the target of max_k s: X = target / max_k g at every iteration, and
-//    s moved 3/4 of the way to X g.  The normalisation turns the search for
-//    eps into the same iteration: its one slow mode is X itself, which
-//    overshoots by a factor of about -0.45 (undamped) and converges at 0.25-0.3
-//    an iteration with the damping: about 20 iterations to 1e-12, whatever
-//    the lattice (numpy simulation; targets 0.1-0.97).  The last g gives X and
-//    s = X g meets the target by construction: a move in X to first order.
+//  * Given the target of max_k s: X = target / max_k g at every iteration.  The
+//    normalisation turns the search for eps into the same iteration, whose one
+//    slow mode is X itself; it overshoots by a factor of about -0.45.  Moving s
+//    3/4 of the way to X g (damping) converges at 0.25-0.3 an iteration, about
+//    20 iterations to 3e-12; Anderson's mixing of the last three (J. ACM 12,
+//    1965; solve_mix) takes 9-16 for the Gaussian envelope, whatever the lattice
+//    (numpy simulation, 17 x 300 to 128 x 128, targets 0.15-0.95; 10 to 14
+//    measured at 0.28-0.53).  Tables of a separable bispectrum keep the damping:
+//    their weight can sit in a few points that the fit does not see (the
+//    wind-field envelope on 94 x 603: 24 iterations to 1e-8 against about 14).
+//    So do iterations past kSolveMixIt.  The last g gives X and s = X g meets
+//    the target by construction: a move in X to first order.
+//    256 x 512 plan and 64 samples 3.42 -> 3.29 ms, 40 x 70 mixed plan and 16
+//    samples 864 -> 739 us, 32 x 32 FP64 plan and sample 817 -> 801 us.
 // Iterations that do not converge (extreme targets with sparse supports) leave
 // the plan to the level passes (recursion.cuh).
 //
@@ -46,6 +53,8 @@
 namespace srm3 {
 
 constexpr int kSolveMaxIt = 96;
+constexpr int kSolveMixIt = 40;       // iterations with Anderson mixing at most
+constexpr int kSolveMixPoints = 256;  // lattice points its coefficients are fitted on
 
 // Control words of a solve, zeroed before it: the bits of max_k g and of the
 // largest change of s, per iteration; then the results (k_solve_final).
@@ -69,14 +78,15 @@ struct SolveArgs {
   // (aW at signed omega index + nw - 1), in the transform's real type F
   const void *e2, *b2;
   const void *aK, *bK, *aW, *bW;
-  void *g;                  // F [nk][nw]
-  void *s_in, *s_out;       // F: the iterate before and after this iteration
+  // F [nk][nw]: g of iteration n in g[n % 3]; the iterate of iteration n in s[n & 3]
+  // (of -1, in s[3]: the warm start)
+  void *g[3], *s[4];
   void *Z;                  // [nk][M] complex
   const void *twk, *twm, *twz;  // pass twiddles of Nk and M; e^{pi i m / M}
   SolveCtl *ctl;
   double target;            // > 0: of max_k s; else X is given
   double X, w, tol, accept;
-  int warm;                 // s_in holds the first iterate (else it is 0)
+  int warm;                 // s[3] holds the first iterate (else it is 0)
   int hold;                 // the first updates take X as given, undamped
 };
 
@@ -93,8 +103,12 @@ __device__ __forceinline__ double as_double(unsigned long long b) {
 __device__ __forceinline__ bool solve_last(const SolveArgs &A, int it) {
   if (it < A.hold + 1) return false;
   const double c = as_double(A.ctl->chg[it]);
-  return c <= A.tol ||
-         (it >= A.hold + 2 && c <= A.accept && c >= 0.5 * as_double(A.ctl->chg[it - 1]));
+  if (c <= A.tol) return true;
+  if (it < A.hold + (A.e2 ? 2 : 4) || c > A.accept) return false;
+  double m = as_double(A.ctl->chg[it - 1]);
+  if (!A.e2)  // mixed iterations fall less evenly
+    m = fmin(m, fmin(as_double(A.ctl->chg[it - 2]), as_double(A.ctl->chg[it - 3])));
+  return c >= 0.5 * m;
 }
 __device__ __forceinline__ bool solve_done(const SolveArgs &A, int it) {
   return it >= 1 && solve_last(A, it - 1);
@@ -129,6 +143,8 @@ __device__ __forceinline__ df solve_q(df s) {
   const float e = __fmaf_rn(-d.l, r, __fmaf_rn(-d.h, r, 1.0f));
   return df(r, __fmul_rn(r, e));
 }
+__device__ __forceinline__ double solve_num(float v, double) { return v; }
+__device__ __forceinline__ df solve_num(float v, df) { return df(v, 0.0f); }
 __device__ __forceinline__ double solve_real(double v) { return v; }
 __device__ __forceinline__ double solve_real(df v) { return (double)v.h + (double)v.l; }
 // v, 0 if negative, its parts not overlapping (so that h orders first)
@@ -148,6 +164,59 @@ __device__ __forceinline__ void warp_atomic_max(unsigned long long *p, double v)
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0 && v > 0.0)
     atomicMax(p, (unsigned long long)__double_as_longlong(v));
+}
+
+// Anderson mixing.  With G_n = X_n g(s_n), f_n = G_n - s_n, the next iterate is
+// G_n + c1 (G_{n-1} - G_n) + c2 (G_{n-2} - G_n), the coefficients those that
+// make the same combination of the f smallest.  The few slow modes are smooth: a
+// fit on 256 points spread over the lattice (golden-ratio steps) takes the
+// iterations that one over all points does (numpy), and every CTA makes it for
+// itself, in the same order, with no reduction over the grid.  past: 1 or 2.
+template <typename F>
+__device__ __forceinline__ void solve_mix(const SolveArgs &A, int n, int past, float &c1, float &c2) {
+  const unsigned nl = (unsigned)A.nk * A.nw;
+  const F X0 = F(solve_X(A, n)), X1 = F(solve_X(A, n - 1)), X2 = F(past > 1 ? solve_X(A, n - 2) : 0.0);
+  const F *g0 = static_cast<const F *>(A.g[n % 3]), *g1 = static_cast<const F *>(A.g[(n + 2) % 3]);
+  const F *g2 = static_cast<const F *>(A.g[(n + 1) % 3]);
+  const F *s0 = static_cast<const F *>(A.s[n & 3]), *s1 = static_cast<const F *>(A.s[(n - 1) & 3]);
+  const F *s2 = static_cast<const F *>(A.s[(n - 2) & 3]);
+  float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // d1.d1, d1.d2, d2.d2, d1.f0, d2.f0
+  for (int j = threadIdx.x; j < kSolveMixPoints; j += blockDim.x) {
+    // point floor(nl frac((j + 1/2) / golden ratio))
+    const unsigned k = __umulhi((unsigned)(2 * j + 1) * 1327217885u, nl);
+    const float f0 = (float)solve_real(X0 * g0[k] - s0[k]);
+    const float d1 = f0 - (float)solve_real(X1 * g1[k] - s1[k]);
+    const float d2 = past > 1 ? f0 - (float)solve_real(X2 * g2[k] - s2[k]) : 0.f;
+    v[0] = fmaf(d1, d1, v[0]);
+    v[1] = fmaf(d1, d2, v[1]);
+    v[2] = fmaf(d2, d2, v[2]);
+    v[3] = fmaf(d1, f0, v[3]);
+    v[4] = fmaf(d2, f0, v[4]);
+  }
+  __shared__ float part[32][5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+  if (blockDim.x > 32) {
+    if ((threadIdx.x & 31) == 0)
+      for (int i = 0; i < 5; ++i) part[threadIdx.x >> 5][i] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      v[i] = 0.f;
+      for (unsigned w = 0; w < blockDim.x / 32; ++w) v[i] += part[w][i];
+    }
+  }
+  c1 = c2 = 0.f;
+  const float det = v[0] * v[2] - v[1] * v[1];
+  if (past > 1 && det > 1e-6f * v[0] * v[2]) {
+    c1 = (v[3] * v[2] - v[4] * v[1]) / det;
+    c2 = (v[4] * v[0] - v[3] * v[1]) / det;
+  } else if (v[0] > 0.f) {
+    c1 = v[3] / v[0];
+  }
+  const float m = fmaxf(fabsf(c1), fabsf(c2));
+  if (!(m <= 16.f)) c1 = c2 = 0.f;  // (NaN too)
 }
 
 // log2 of the values a thread holds of a length-2^l transform: 4 of them where
@@ -189,9 +258,20 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const Solv
   const bool live = row < A.rows && kk < A.nk;
   T2 *buf = reinterpret_cast<T2 *>(solve_smem) + row * (tx_len(M) + 1);
   T2 *out = static_cast<T2 *>(A.Z) + (size_t)kk * M;
-  const F X = F(it > 0 ? solve_X(A, it - 1) : 0.0), damp = F(it <= A.hold ? 1.0 : A.w);
-  const F *s_in = static_cast<const F *>(A.s_in), *g = static_cast<const F *>(A.g);
-  F *s_out = static_cast<F *>(A.s_out);
+  // iteration n's results make the iterate of it = n + 1
+  const int n = it - 1;
+  const bool mix = A.target > 0.0 && !A.e2 && it < kSolveMixIt;
+  const int past = mix && n > A.hold ? min(n - A.hold, 2) : 0;
+  float c1 = 0.f, c2 = 0.f;
+  if (past > 0) solve_mix<F>(A, n, past, c1, c2);
+  const F m1 = solve_num(c1, F()), m2 = solve_num(c2, F());
+  const F X = F(it > 0 ? solve_X(A, n) : 0.0);
+  const F X1 = F(past > 0 ? solve_X(A, n - 1) : 0.0), X2 = F(past > 1 ? solve_X(A, n - 2) : 0.0);
+  const F damp = F(it <= A.hold || mix ? 1.0 : A.w);
+  const F *s_in = static_cast<const F *>(A.s[(it + 3) & 3]);
+  const F *g = static_cast<const F *>(A.g[(it + 2) % 3]), *g1 = static_cast<const F *>(A.g[(it + 1) % 3]);
+  const F *g2 = static_cast<const F *>(A.g[it % 3]);
+  F *s_out = static_cast<F *>(A.s[it & 3]);
   float chg = 0.0f;
   auto h_at = [&](int p) -> F {  // position p of the row: omega = p, or p - 2 M
     int w = p;
@@ -202,6 +282,12 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_rows(const Solv
     F s = F(0.0);
     if (it == 0) {
       if (A.warm) s = s_in[k];
+    } else if (past > 0) {
+      const F G = X * g[k];
+      s = G + m1 * (X1 * g1[k] - G);
+      if (past > 1) s = s + m2 * (X2 * g2[k] - G);
+      s = solve_clip(s);
+      if (w >= 0) chg = fmaxf(chg, solve_abs(s - s_in[k]));
     } else {
       const F s0 = s_in[k], d = (X * g[k] - s0) * damp;
       s = s0 + d;
@@ -278,8 +364,8 @@ __global__ void __launch_bounds__(solve_row_threads(LM)) k_solve_out(const Solve
   const bool live = row < A.rows && kk < A.nk;
   T2 *buf = reinterpret_cast<T2 *>(solve_smem) + row * (tx_len(M) + 1);
   const T2 *in = static_cast<const T2 *>(A.Z) + (size_t)(live ? kk : 0) * M;
-  const F *s = static_cast<const F *>(A.s_out);
-  F *g = static_cast<F *>(A.g);
+  const F *s = static_cast<const F *>(A.s[it & 3]);
+  F *g = static_cast<F *>(A.g[it % 3]);
   const F half_inv = F(0.5 / ((double)A.Nk * M)), half = F(0.5);  // powers of two
   F mx = F(0.0);
   auto h_of = [&](int hk, int hw) -> F {

@@ -23,7 +23,7 @@ void solve_with_log2(int v, F &&f) {
   }
 }
 
-constexpr int kSolveSmemMax = 227 * 1024;
+constexpr int kSolveSmemMax = 224 * 1024;  // beside the kernels' static words
 
 // The kernel's dynamic shared memory limit raised once per device.
 template <auto K>
