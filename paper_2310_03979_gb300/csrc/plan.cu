@@ -1177,6 +1177,7 @@ int solve_iterate_f64(const SolveArgs &A, int it, int device, int nsm, cudaStrea
 struct SolveResult {
   bool converged;
   double x, max_sb2;  // eps^2, max_k sum_b2
+  double change;      // of the last iteration
   int its, err;
   bool no_pairs;
 };
@@ -1188,6 +1189,12 @@ struct SolveResult {
 static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-12, kSolveF64 = 3e-14;
 // the change at which a solve whose changes have stopped falling still counts
 static constexpr double kSolveAcceptDf = 1e-10, kSolveAcceptF64 = 3e-12;
+// and of FP64 plans' tables (separable bispectra): where the transform's
+// rounding keeps the sums moving by more (the wind-field envelope on 486 x 202:
+// 9e-13; tables up to 8 times further off than the level pass's) they come from
+// the level pass, from the solve's root: 42.5 -> 20.8 ms there, 33.4 -> 16.0 on 94 x
+// 603, where the solve alone took about 2
+static constexpr double kSolveExact = 1e-13;
 
 // The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
 // target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
@@ -1332,6 +1339,7 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   r->x = h->X / p->dkdw;
   std::memcpy(&r->max_sb2, &h->max_sb2, sizeof(double));
   r->its = h->last;
+  std::memcpy(&r->change, &h->chg[h->last], sizeof(double));
   r->err = h->err;
   r->no_pairs = h->maxg[0] == 0 && target > 0.0;
   return SRM3_OK;
@@ -1986,7 +1994,7 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
       p->t_recursion_ms += ms;
       p->t_rec32_ms += ms - p->t_coarse_ms;
       p->coarse_start = xc > 0.0 && std::fabs(xc - r.x) <= kCoarseWindow * r.x;
-      if (tables) {
+      if (tables && (p->precision == SRM3_FP32 || r.change <= kSolveExact)) {
         p->root_passes32 += 1;  // the solve, and its tables in FP64
         p->root_passes += 1;
         p->eps = std::sqrt(r.x);
@@ -2027,7 +2035,11 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
     rc = wide_search(p, st, target, s);
     if (rc) return rc;
   }
-  double x32 = xs, slope32 = 0.0;
+  // a separable bispectrum's level passes: the bulk's form first (three planes
+  // at once only without its FFT form)
+  if (xs > 0.0 && p->sep && !iter_small(p, 3) && (rc = setup_recursion(p, st))) return rc;
+  // (from the solve: about d ln max sum_b2 / d ln x = 1.5, its slow mode's gain)
+  double x32 = xs, slope32 = xs > 0.0 ? 1.5 * target / xs : 0.0;
   const bool hi_ok = xs > 0.0 || root_fp32(s, &x32, &slope32);
 
   // Loose targets (FP32 plans, tol >= kShiftTol): the slope in x of every
@@ -2522,7 +2534,9 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
         rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr);
       if (rc) return rc;
       // a solve that met sum_b2 >= 1 leaves the verdict to the level pass
-      if ((done = sr.converged && !sr.err)) {
+      done = sr.converged && !sr.err &&
+             (p->precision == SRM3_FP32 || sr.change <= kSolveExact);
+      if (done) {
         r.max_sb2 = sr.max_sb2;
         r.min_pure = 1.0 - sr.max_sb2;
         r.sumS = p->sumS;

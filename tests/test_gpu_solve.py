@@ -63,3 +63,21 @@ def test_no_pairs_is_refused():
         with pytest.raises(srm3.SRM3Error) as ei:
             srm3.Plan.create(wl, table=S, precision=precision)
         assert ei.value.code == -4
+
+
+@pytest.mark.parametrize("nk,nw", [(486, 202), (60, 44), (12, 9)])
+def test_fp64_separable_tables_keep_fp64_accuracy(oracle_lib, nk, nw):
+    """FP64 plans of the wind-field envelope, whose sums span the widest range:
+    where the transform's rounding keeps the solve's sums moving the tables come
+    from the level pass.  Against the oracle's tables at the plan's eps: 5e-13 of
+    max sum_b2 (an accepted last change of 1e-13, converging at 0.3 or better,
+    leaves 1.5e-13; as much again for eps, and room for the level pass's sums)."""
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=512, nt=512, precision="fp64"), envelope="sum")
+    with srm3.Plan.create(wl) as p:
+        S, q, sb2 = p.tables()
+        info = p.info()
+    assert abs(info.max_sum_b2 - wl.target) <= 1e-12
+    ta, tb = wl.envelope_tables()
+    ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps,
+                           env=oracle.Envelope("separable", table=ta, table_b=tb))
+    assert np.abs(sb2 - ref.sum_b2).max() <= 5e-13 * ref.sum_b2.max()
