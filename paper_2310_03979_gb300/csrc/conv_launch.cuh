@@ -46,10 +46,10 @@ cudaError_t conv_prepare(int dev) {
 //
 // Which plans take it: every separable bispectrum, and the Gaussian envelope
 // with W recomputed at every size.  Both sides measured (GB300, FP32 plans,
-// pair sum with its phases): 256 x 512, 64 samples 44.4 -> 1.93 ms; 512 x
-// 1024, 16 samples 183 -> 2.56 ms; 32 spectra on lattices of 32..256 per axis
-// in one captured batch 22.7 -> 4.0 ms; one sample on 32 x 32, with its field,
-// 60 -> 43 us.  FP64 plans: 90 x 117, 4 samples 1.64 -> 0.12 ms.  Against 64-bit
+// pair sum with its phases): 256 x 512, 64 samples 44.4 -> 1.74 ms; 512 x
+// 1024, 16 samples 183 -> 2.13 ms; 32 spectra on lattices of 32..256 per axis
+// in one captured batch 22.7 -> 2.4 ms; one sample on 32 x 32, with its field,
+// 60 -> 26 us.  FP64 plans: 90 x 117, 4 samples 1.64 -> 0.10 ms.  Against 64-bit
 // coefficients the FP32 fields' relative error went 1.9e-7 -> 1.8e-7 (2.1e-7
 // -> 1.9e-7 on 512 x 1024), the FP64 coefficients' stayed at 6.6e-15.
 //

@@ -2464,7 +2464,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     if (p->mixed) p->storage = SRM3_STORAGE_RECOMPUTE;  // the table holds sum pairs only
     if (p->storage == SRM3_STORAGE_AUTO && p->conv) {
       // W recomputed by the self-convolution is the faster one at every size
-      // (conv_launch.cuh; 256 x 512, 64 samples: 2.2 ms against 69 ms with the
+      // (conv_launch.cuh; 256 x 512, 64 samples: 1.7 ms against 59 ms with the
       // stored table, whose build and memory it saves too)
       p->storage = SRM3_STORAGE_RECOMPUTE;
     }
