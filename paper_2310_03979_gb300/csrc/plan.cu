@@ -1194,7 +1194,7 @@ static constexpr double kSolveAcceptDf = 1e-10, kSolveAcceptF64 = 3e-12;
 // 9e-13; tables up to 8 times further off than the level pass's) they come from
 // the level pass, from the solve's root: 42.5 -> 20.8 ms there, 33.4 -> 16.0 on 94 x
 // 603, where the solve alone took about 2
-static constexpr double kSolveExact = 1e-13;
+static constexpr double kSolveExact = kSolveF64;
 
 // The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
 // target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
