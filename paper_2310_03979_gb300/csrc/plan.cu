@@ -1338,6 +1338,7 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   r->converged = h->converged != 0 && h->X >= 0.0 && std::isfinite(h->X);
   r->x = h->X / p->dkdw;
   std::memcpy(&r->max_sb2, &h->max_sb2, sizeof(double));
+  r->converged = r->converged && r->max_sb2 < kSolveTop;
   r->its = h->last;
   std::memcpy(&r->change, &h->chg[h->last], sizeof(double));
   r->err = h->err;
@@ -1495,7 +1496,7 @@ static int illinois(srm3_plan *p, cudaStream_t st, double target, double tol, in
 static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double tol) {
   const long long nl = (long long)p->nk * p->nw;
   PassResult r;
-  if (p->solve) {
+  if (p->solve && target < kSolveTop) {
     SolveResult sr;
     SRM3_CUDA(cudaEventRecord(t_ev[0], st));
     int rc = solve_lattice(p, st, target, 0.0, p->sigma_g * p->nk, p->sigma_g * p->nw, false,
@@ -1962,7 +1963,7 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
   s.pts.push_back({0.0, -target});
   p->coarse_start = false;
   double xs = -1.0;  // the root, from the whole-lattice solve
-  if (p->solve) {
+  if (p->solve && target < kSolveTop) {
     if (p->w_deferred) {  // the W table beside it
       p->w_deferred = false;
       if ((rc = start_w_table(p, p->w_stream))) return rc;
@@ -2533,7 +2534,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
       if (!rc && sr.converged && !sr.err)
         rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr);
       if (rc) return rc;
-      // a solve that met sum_b2 >= 1 leaves the verdict to the level pass
+      // a solve that met sums of 1 or close to it leaves the verdict to the level pass
       done = sr.converged && !sr.err &&
              (p->precision == SRM3_FP32 || sr.change <= kSolveExact);
       if (done) {

@@ -23,8 +23,9 @@
 //    the target by construction: a move in X to first order.
 //    256 x 512 plan and 64 samples 3.42 -> 3.29 ms, 40 x 70 mixed plan and 16
 //    samples 864 -> 739 us, 32 x 32 FP64 plan and sample 817 -> 801 us.
-// Iterations that do not converge (extreme targets with sparse supports) leave
-// the plan to the level passes (recursion.cuh).
+// Iterations that do not converge (extreme targets with sparse supports), and
+// sums close to 1 (kSolveTop), leave the plan to the level passes
+// (recursion.cuh).
 //
 // The convolution.  h is real: its omega axis is packed two to a complex
 // entry, z(m) = h(2m) + i h(2m + 1), on a zero-padded nk x M grid (M = Nw / 2,
@@ -55,6 +56,11 @@ namespace srm3 {
 constexpr int kSolveMaxIt = 96;
 constexpr int kSolveMixIt = 40;       // iterations with Anderson mixing at most
 constexpr int kSolveMixPoints = 256;  // lattice points its coefficients are fitted on
+// An iterate's s enters q as min(s, kSolveClip).  Points above it at the fixed
+// point would feed others a q too small: a solve counts only where every s ends
+// below kSolveTop (the margin is far above the rounding of s), and targets from
+// there on go to the level passes at once.
+constexpr double kSolveClip = 0.99, kSolveTop = 0.9899;
 
 // Control words of a solve, zeroed before it: the bits of max_k g and of the
 // largest change of s, per iteration; then the results (k_solve_final).
@@ -135,10 +141,11 @@ __device__ __forceinline__ F solve_b2(const SolveArgs &A, int kk, int kw) {
 // The per-point arithmetic stays in the transform's type: an FP64 operation
 // takes a warp 16 cycles of its SM's FP64 pipe, and the first form of these
 // kernels, with s, g and h in FP64, spent 25 us a launch on a 32 x 32 lattice.
-// q from s: 1/(1 - s), s kept below 0.99 while the iterations are on their way.
-__device__ __forceinline__ double solve_q(double s) { return 1.0 / (1.0 - fmin(s, 0.99)); }
+// q from s: 1/(1 - s), s kept below kSolveClip while the iterations are on their
+// way; a fixed point that reaches it is not Eq. pure's (kSolveTop).
+__device__ __forceinline__ double solve_q(double s) { return 1.0 / (1.0 - fmin(s, kSolveClip)); }
 __device__ __forceinline__ df solve_q(df s) {
-  const df d = s.h < 0.99f ? df(1.0f, 0.0f) - s : df(0.01);
+  const df d = s.h < (float)kSolveClip ? df(1.0f, 0.0f) - s : df(1.0 - kSolveClip);
   const float r = __frcp_rn(d.h);  // one Newton step on it: error r (1 - d r)^2
   const float e = __fmaf_rn(-d.l, r, __fmaf_rn(-d.h, r, 1.0f));
   return df(r, __fmul_rn(r, e));

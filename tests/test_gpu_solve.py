@@ -81,3 +81,63 @@ def test_fp64_separable_tables_keep_fp64_accuracy(oracle_lib, nk, nw):
     ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps,
                            env=oracle.Envelope("separable", table=ta, table_b=tb))
     assert np.abs(sb2 - ref.sum_b2).max() <= 5e-13 * ref.sum_b2.max()
+
+
+class _Tables:
+    """A workload with separable tables of its own."""
+    envelope = "separable"
+
+    def __init__(self, wl, a):
+        self._wl, self._a = wl, a
+
+    def __getattr__(self, name):
+        return getattr(self._wl, name)
+
+    def envelope_tables(self):
+        return self._a, None
+
+
+# Sums close to 1, where 1/(1 - s) must not be cut off.  Tolerances: a rounding of
+# a sum (1e-14) reaches a dependent sum times q^2 = 1/(1 - s)^2, and FP32 plans
+# move their tables to the root to first order (1e-9 of it); a cut-off q = 100
+# is off by tens of per cent and its dependents by 1e-6 and more.
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("nk,nw,peak", [(128, 96, 0.992), (32, 32, 0.992)])
+def test_fixed_eps_with_sums_close_to_one(oracle_lib, precision, nk, nw, peak):
+    """A separable bispectrum at a given eps: points above 0.99 feed others."""
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=pow2(nk), nt=pow2(2 * nw), precision=precision),
+                 envelope="separable")
+    S = oracle.kaimal_lorentzian(nk, nw, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    env = oracle.Envelope("separable", table=wl.envelope_tables()[0])
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, target=peak, env=env)
+    with srm3.Plan.create(wl, table=S, eps=op.eps) as p:
+        _, q, sb2 = p.tables()
+    np.testing.assert_allclose(q, op.q, rtol=1e-8)
+    np.testing.assert_allclose(sb2, op.sum_b2, atol=1e-9)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("kind", ["separable", "gauss", "mixed"])
+@pytest.mark.parametrize("target", [0.992, 0.995])
+def test_targets_close_to_one_on_sparse_supports(oracle_lib, precision, kind, target):
+    """The largest sum feeds other points: tables at the plan's eps."""
+    mixed = kind == "mixed"
+    if kind == "separable":
+        wl = W.small_case(nk=1, nw=6, nx=2, nt=16, precision=precision, target=target)
+        S = np.ones((1, 6))
+        a = np.sqrt(np.array([[0.0, 1.0, 1.0, 0.004, 0.0, 0.15]]))
+        wl, env = _Tables(wl, a), oracle.Envelope("separable", table=a)
+    else:
+        wl = replace(W.small_case(nk=20, nw=20, nx=32, nt=64, precision=precision, target=target),
+                     interactions="mixed" if mixed else "sum")
+        S = oracle.kaimal_lorentzian(20, 20, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+        S[:, 0] = S.max() / (1.0 + np.arange(20))
+        S[np.random.default_rng(5).random(S.shape) < 0.5] = 0.0
+        env = oracle.Envelope("gauss", wl.sigma_g)
+    with srm3.Plan.create(wl, table=S) as p:
+        _, q, sb2 = p.tables()
+        info = p.info()
+    assert abs(info.max_sum_b2 - target) <= 1e-9
+    ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps, env=env, mixed=mixed)
+    np.testing.assert_allclose(sb2, ref.sum_b2, atol=1e-6 if kind != "mixed" else 1e-9)
+    np.testing.assert_allclose(q, ref.q, rtol=1e-5 if kind != "mixed" else 1e-6)
