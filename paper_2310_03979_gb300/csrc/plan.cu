@@ -1052,6 +1052,8 @@ __global__ void k_solve_convert(long long n, const double *__restrict__ in, F *_
 // with the maximum and the solve's outcome in ctl.  Stage 1: g from the
 // iterations (F), kept in FP64 in g64, X theirs; gmax over the points that
 // k_solve_low leaves.  Stage 2: g64, X from gmax where the target is given.
+// hmax, bmax (stage 1) and h2 (stage 2) say what the transforms' rounding is
+// relative to (kSolveSpread).
 constexpr int kSolveLow = 2048;
 
 template <typename F>
@@ -1084,12 +1086,13 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
   }
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double v = 0.0, g = 0.0;
+  double v = 0.0, g = 0.0, hm = 0.0, bm = 0.0;
+  unsigned long long h2 = 0;
   bool direct = false;
   if (i < n) {
     const bool pos = A.S[i] > 0.0;
+    const int kk = (int)(i / A.nw), kw = (int)(i - (long long)kk * A.nw);
     if (stage == 1) {
-      const int kk = (int)(i / A.nw), kw = (int)(i - (long long)kk * A.nw);
       direct = low && (long long)(kk + 1) * (kw + 1) <= kSolveLow;
       g64[i] = g = solve_real(static_cast<const F *>(A.g[sLast % 3])[i]);
     } else {
@@ -1099,11 +1102,48 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
     sb2[i] = v;
     q[i] = pos && v < 1.0 ? 1.0 / (1.0 - v) : 0.0;
     if (stage == 2 && !(v < 1.0)) atomicOr(&A.ctl->err, 1);
+    if (pos && i > 0) {  // both signs of omega
+      hm = solve_real(solve_a2<F>(A, kk, kw)) * q[i];
+      const double hn = A.mixed && kw > 0 ? solve_real(solve_a2<F>(A, kk, -kw)) * q[i] : 0.0;
+      if (stage == 1) {
+        hm = fmax(hm, hn);
+        bm = solve_real(solve_b2<F>(A, kk, kw));
+      } else {
+        const double r = 1.0 / as_double(A.ctl->hmax), a = hm * r, b = hn * r;
+        h2 = (unsigned long long)(fmin(a * a + b * b, 4.0) * (1.0 / kSolveH2Unit));
+      }
+    }
   }
-  if (stage == 1)
-    warp_atomic_max(&A.ctl->gmax, direct ? 0.0 : g);
-  else
-    warp_atomic_max(&A.ctl->max_sb2, v);
+  // one atomic per CTA and word
+  double m[3] = {stage == 1 ? (direct ? 0.0 : g) : v, hm, bm};
+  for (int o = 16; o > 0; o >>= 1) {
+    h2 += __shfl_xor_sync(0xffffffffu, h2, o);
+    for (double &w : m) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+  }
+  __shared__ double sm[8][3];
+  __shared__ unsigned long long sh2[8];
+  const int wp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    for (int j = 0; j < 3; ++j) sm[wp][j] = m[j];
+    sh2[wp] = h2;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 8; ++w) {
+    for (int j = 0; j < 3; ++j) m[j] = fmax(m[j], sm[w][j]);
+    h2 += sh2[w];
+  }
+  auto put = [](unsigned long long *p, double w) {
+    if (w > 0.0) atomicMax(p, (unsigned long long)__double_as_longlong(w));
+  };
+  if (stage == 1) {
+    put(&A.ctl->gmax, m[0]);
+    put(&A.ctl->hmax, m[1]);
+    put(&A.ctl->bmax, m[2]);
+  } else {
+    put(&A.ctl->max_sb2, m[0]);
+    if (h2) atomicAdd(&A.ctl->h2, h2);
+  }
 }
 
 // g of the points with few pairs, (kk + 1)(kw + 1) <= kSolveLow, summed
@@ -1179,7 +1219,7 @@ struct SolveResult {
   double x, max_sb2;  // eps^2, max_k sum_b2
   double change;      // of the last iteration
   int its, err;
-  bool no_pairs;
+  bool no_pairs;  // none, or so weak that the sums may be the transforms' rounding
 };
 
 // largest change of s at which the solve stops: the coarse
@@ -1338,11 +1378,17 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   r->converged = h->converged != 0 && h->X >= 0.0 && std::isfinite(h->X);
   r->x = h->X / p->dkdw;
   std::memcpy(&r->max_sb2, &h->max_sb2, sizeof(double));
-  r->converged = r->converged && r->max_sb2 < kSolveTop;
+  double gm, hm, bm;
+  std::memcpy(&gm, &h->gmax, sizeof(gm));
+  std::memcpy(&hm, &h->hmax, sizeof(hm));
+  std::memcpy(&bm, &h->bmax, sizeof(bm));
+  const double spread = bm * hm * hm * ((double)h->h2 * kSolveH2Unit);
+  r->no_pairs = !(h->X * spread <= (p->sep ? kSolveSpreadSep : kSolveSpread)) ||
+                (target > 0.0 && !(gm > 0.0));
+  r->converged = r->converged && r->max_sb2 < kSolveTop && !r->no_pairs;
   r->its = h->last;
   std::memcpy(&r->change, &h->chg[h->last], sizeof(double));
   r->err = h->err;
-  r->no_pairs = h->maxg[0] == 0 && target > 0.0;
   return SRM3_OK;
 }
 
@@ -1504,8 +1550,6 @@ static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double t
     if (rc) return rc;
     SRM3_CUDA(cudaEventRecord(t_ev[1], st));
     SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
-    if (sr.no_pairs)
-      return fail(SRM3_ERR_BISECTION_FAILED, "no bispectral pairs: max_k sum_b2 is 0 for every eps");
     if (sr.converged && !sr.err) {
       float ms = 0.f;
       SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
@@ -1989,8 +2033,6 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
     SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
     float ms = 0.f;
     SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
-    if (r.no_pairs)
-      return fail(SRM3_ERR_BISECTION_FAILED, "no bispectral pairs: max_k sum_b2 is 0 for every eps");
     if (r.converged && !r.err) {
       p->t_recursion_ms += ms;
       p->t_rec32_ms += ms - p->t_coarse_ms;

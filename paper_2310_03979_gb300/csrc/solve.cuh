@@ -61,6 +61,16 @@ constexpr int kSolveMixPoints = 256;  // lattice points its coefficients are fit
 // below kSolveTop (the margin is far above the rounding of s), and targets from
 // there on go to the level passes at once.
 constexpr double kSolveClip = 0.99, kSolveTop = 0.9899;
+// A transform's rounding is relative to sum h^2 (the largest sum there can be, by
+// Cauchy and Schwarz), times b_k^2 at a point.  Supports whose pairs are few or
+// weak, or that have none, can leave max_k g anywhere below that, down to the
+// rounding itself.  A solve counts where X max b^2 sum h^2 stays below kSolveSpread
+// (double-float, Gaussian envelope: 3e4 at most on full lattices and on ones with
+// nine of ten points empty, sigma_g >= 0.2237) or kSolveSpreadSep (separable
+// tables, finished in FP64: 3 times the number of points); where X comes from
+// rounding alone it is 2^36 and above.
+constexpr double kSolveSpread = 0x1p22, kSolveSpreadSep = 0x1p26;
+constexpr double kSolveH2Unit = 0x1p-24;
 
 // Control words of a solve, zeroed before it: the bits of max_k g and of the
 // largest change of s, per iteration; then the results (k_solve_final).
@@ -70,6 +80,8 @@ struct SolveCtl {
   double X;                    // eps^2 dk dw
   unsigned long long gmax;     // bits: max_k g, the directly summed points' included
   unsigned long long max_sb2;  // bits
+  unsigned long long hmax, bmax;  // bits: max h and max b_k^2 where S > 0
+  unsigned long long h2;       // sum of (h / hmax)^2, in units of kSolveH2Unit
   int last;                    // the iteration g is from
   int converged;
   int err;                     // some sum_b2 >= 1

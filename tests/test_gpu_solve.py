@@ -65,6 +65,50 @@ def test_no_pairs_is_refused():
         assert ei.value.code == -4
 
 
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("interactions", ["sum", "mixed"])
+@pytest.mark.parametrize("n,support", [
+    (8, [(4, 6), (6, 3)]), (8, [(4, 2), (5, 1), (7, 2)]), (8, [(4, 3), (6, 2), (6, 5), (7, 6)]),
+    (256, "upper half"),
+])
+def test_no_pairs_is_refused_whatever_the_rounding(precision, interactions, n, support):
+    """Supports of several points, no two of which sum to a third: the
+    transforms' rounding is not a pair sum."""
+    S = np.zeros((n, n))
+    if isinstance(support, str):
+        if interactions == "mixed":
+            pytest.skip("points of one half have difference pairs")
+        r = np.random.default_rng(2)
+        S[r.integers(n // 2 + 1, n, 500), r.integers(n // 2 + 1, n, 500)] = 1.0
+    else:
+        for k in support:
+            S[k] = 1.0
+    wl = replace(W.small_case(nk=n, nw=n, nx=n, nt=2 * n, precision=precision),
+                 interactions=interactions)
+    with pytest.raises(srm3.SRM3Error) as ei:
+        srm3.Plan.create(wl, table=S)
+    assert ei.value.code == -4
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_weak_pairs_among_many_points(oracle_lib, precision):
+    """200 points with no pairs among them and one that has pairs with them, of
+    weight 2e-7 and less: far below the largest sums the transforms could hold."""
+    S = np.zeros((64, 64))
+    r = np.random.default_rng(4)
+    S[r.integers(43, 64, 200), r.integers(53, 64, 200)] = 1.0
+    S[1, 1] = S[40, 50] = S[41, 51] = 1.0
+    wl = W.small_case(nk=64, nw=64, nx=64, nt=128, precision=precision)
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, target=wl.target)
+    with srm3.Plan.create(wl, table=S) as p:
+        _, q, sb2 = p.tables()
+        info = p.info()
+    rel = 1e-11 if precision == "fp64" else 2e-8
+    assert info.eps == pytest.approx(op.eps, rel=rel)
+    np.testing.assert_allclose(sb2, op.sum_b2, rtol=rel, atol=1e-15)
+    np.testing.assert_allclose(q, op.q, rtol=rel)
+
+
 @pytest.mark.parametrize("nk,nw", [(486, 202), (60, 44), (12, 9)])
 def test_fp64_separable_tables_keep_fp64_accuracy(oracle_lib, nk, nw):
     """FP64 plans of the wind-field envelope, whose sums span the widest range:
