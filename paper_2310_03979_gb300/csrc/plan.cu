@@ -698,6 +698,12 @@ constexpr int kFpMaxIters = 400;
 // Mixed interactions add their difference pairs (whose q are not lower
 // points': the iterations then converge geometrically, as the alternating
 // ones do).
+//
+// Sums close to 1 take more steps: ones that have not converged by the time a
+// level pass would have taken (iter_most) leave this and the plan's later passes
+// to it (128 x 96 with max sum_b2 = 0.999: 2.6 ms a pass by iterations, 1.5 ms by
+// levels), mixed ones after kIterMax steps to the alternating iterations, which
+// go on from their q.
 constexpr double kIterPairs = 4e7;
 
 enum { kIterTable = 0, kIterSep = 1, kIterMixed = 2 };
@@ -808,13 +814,27 @@ __global__ void __launch_bounds__(256) k_iter(const IterArgs A, int it, const do
   if (chg > 0.0) atomicMax(&A.ctl->chg[it], (unsigned long long)__double_as_longlong(chg));
 }
 
-static bool iter_small(const srm3_plan *p, int M) {
+static double iter_products(const srm3_plan *p, int M) {
   const double T = 0.25 * p->nk * (p->nk + 1.0) * p->nw * (p->nw + 1.0);  // 2 x sum pairs
   const double D = p->mixed ? 0.25 * p->nk * (p->nk + 1.0) * (p->nw - 1.0) * (p->nw - 2.0) : 0.0;
-  return (0.5 * T + D) * M <= kIterPairs && (!p->sep || p->env_e2);
+  return (0.5 * T + D) * M;
+}
+static bool iter_small(const srm3_plan *p, int M) {
+  return !p->iter_off && iter_products(p, M) <= kIterPairs && (!p->sep || p->env_e2);
+}
+// Steps a pass may take: the time of the levels, 6 us each, in steps of 4 us and the
+// products; at least the first look's.
+static int iter_most(const srm3_plan *p, int M, int first) {
+  if (p->mixed) return kIterMax;
+  const double step = 4.0 + iter_products(p, M) / 0.35e6, pass = 6.0 * (p->nk + p->nw - 1);
+  return std::max(first, (int)std::min<double>(kIterMax, pass / step));
 }
 
-static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, PassResult *r) {
+// *reached: whether r holds a verdict, the fixed point of every plane or, of a
+// single one started from q = 1, whose iterates only grow, a sum of 1 or more (a
+// mixed plan's also from its warm start, as in the alternating iterations).
+static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, PassResult *r,
+                         bool *reached) {
   const long long nl = (long long)p->nk * p->nw;
   const int form = p->mixed ? kIterMixed : p->rec_sep ? kIterSep : kIterTable;
   if (p->rec_sep && !p->sep && !p->rs_a2) {
@@ -852,13 +872,16 @@ static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, 
   SRM3_CUDA(cudaEventRecord(t_ev[0], st));
   IterCtl *hc = reinterpret_cast<IterCtl *>(reinterpret_cast<char *>(p->h_pinned) + kPinIterOff);
   const double *q0 = p->q_warm ? p->qm : nullptr;
+  bool any_err = false;
   auto launch = [&](auto mc, auto fc) {
     constexpr int Mc = decltype(mc)::value, F = decltype(fc)::value;
     SRM3_CUDA(cudaMemsetAsync(A.ctl, 0, sizeof(IterCtl), st));
     k_iter_init<Mc, F><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, q0, h[0]);
+    const int look = q0 ? 7 : 12, most = iter_most(p, M, look);
     bool done = false;
-    for (int nit = 0; nit < kIterMax && !done;) {
-      const int upto = std::min(kIterMax, nit + (nit == 0 ? (q0 ? 7 : 12) : 6));
+    any_err = false;
+    for (int nit = 0; nit < most && !done && !any_err;) {
+      const int upto = std::min(most, nit + (nit == 0 ? look : 6));
       for (; nit < upto; ++nit) {
         k_iter<Mc, F><<<cdiv(nl * 32, 256), 256, 0, st>>>(A, nit, h[nit & 1], h[(nit + 1) & 1]);
         p->n_launch += 1;
@@ -881,11 +904,10 @@ static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, 
         r[m].min_pure = 1.0 - r[m].max_sb2;
         r[m].sumS = p->sumS < 0.0 ? p->h_pinned[kSumSlot] : p->sumS;
         r[m].err = hc->err[m];
-        done = done || hc->err[m];
+        any_err = any_err || hc->err[m];
       }
     }
-    for (int m = 0; m < Mc; ++m)
-      if (!done) r[m].err = 1;  // no fixed point was reached
+    *reached = (done && !any_err) || (any_err && M == 1 && (!q0 || p->mixed));
     return SRM3_OK;
   };
   using std::integral_constant;
@@ -894,16 +916,28 @@ static int run_pass_iter(srm3_plan *p, cudaStream_t st, const double *x, int M, 
     if (form == kIterSep) return launch(mc, integral_constant<int, kIterSep>{});
     return launch(mc, integral_constant<int, kIterTable>{});
   };
-  const int rc = M == 3 ? by_form(integral_constant<int, 3>{}) : by_form(integral_constant<int, 1>{});
+  auto run = [&]() {
+    return M == 3 ? by_form(integral_constant<int, 3>{}) : by_form(integral_constant<int, 1>{});
+  };
+  int rc = run();
+  if (!rc && any_err && M == 1 && !*reached) {  // a warm start's overshoot decides nothing
+    q0 = nullptr;
+    rc = run();
+  }
   if (rc) return rc;
+  p->iter_off = p->iter_off || !*reached;
   if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];
   float ms = 0.f;
   SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
   p->t_recursion_ms += ms;
   p->t_rec64_ms += ms;
-  p->root_passes += 1;
+  if (*reached) p->root_passes += 1;
   return SRM3_OK;
 }
+
+// Three FP64 planes at once need the direct form of the bulk: r[].err of
+// kPassNone says that no pass was run.
+constexpr int kPassNone = -1;
 
 static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M, bool fp64,
                           PassResult *r) {
@@ -912,9 +946,15 @@ static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M,
       p->w_deferred = false;
       if (int rcw = start_w_table(p, p->w_stream)) return rcw;
     }
-    return run_pass_iter(p, st, x, M, r);
+    bool reached = false;
+    const int rci = run_pass_iter(p, st, x, M, r, &reached);
+    if (rci || reached) return rci;
   }
   if (int rc0 = setup_recursion(p, st)) return rc0;
+  if (fp64 && M == 3 && p->rec_fft) {  // (known since setup_recursion)
+    for (int m = 0; m < M; ++m) r[m].err = kPassNone;
+    return SRM3_OK;
+  }
   for (int m = 0; m < M; ++m) p->h_pinned[m] = x[m] * p->dkdw;
   SRM3_CUDA(cudaMemcpyAsync(p->scal, p->h_pinned, M * sizeof(double), cudaMemcpyHostToDevice, st));
   SRM3_CUDA(cudaMemsetAsync(p->err, 0, (kPlanes + 1) * sizeof(int), st));
@@ -934,7 +974,7 @@ static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M,
   A.S = p->S;
   if (fp64 && M != 1 && M != 3)
     return fail(SRM3_ERR_INVALID_ARG, "FP64 recursion pass takes one or three planes");
-  if (fp64 && M == 3 && (p->rec_fft || p->mixed))
+  if (fp64 && M == 3 && p->mixed)
     return fail(SRM3_ERR_INVALID_ARG, "three-plane FP64 pass: direct bulk, sum pairs only");
   if (!fp64 && M != kPlanes && (M != kWindowPlanes || p->rec_fft))
     return fail(SRM3_ERR_INVALID_ARG, "FP32 recursion pass: 8 planes, or 4 with the direct bulk");
@@ -986,7 +1026,7 @@ static int run_pass_multi(srm3_plan *p, cudaStream_t st, const double *x, int M,
   SRM3_CUDA(cudaMemcpyAsync(p->h_err, p->err, (kPlanes + 1) * sizeof(int), cudaMemcpyDeviceToHost,
                             st));
   SRM3_CUDA(cudaStreamSynchronize(st));
-  if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];  // copied by setup_recursion
+  if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];  // copied by start_sum_S
   float ms = 0.f;
   SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
   p->t_recursion_ms += ms;
@@ -1427,12 +1467,16 @@ __global__ void k_q_change(long long n, const double *__restrict__ S,
 // Solve the fixed point at x from the iterate in p->qm; r: the last pass
 // (r->err != 0: no solution was reached).
 static int solve_mixed(srm3_plan *p, cudaStream_t st, double x, PassResult *r) {
+  int it = 1;
   if (iter_small(p, 1)) {
     p->q_warm = true;
-    return run_pass_iter(p, st, &x, 1, r);
+    bool reached = false;
+    const int rc = run_pass_iter(p, st, &x, 1, r, &reached);
+    if (rc || reached) return rc;
+    it += p->fp_iters;
   }
   const long long nl = (long long)p->nk * p->nw;
-  for (int it = 1; it <= kFpMaxIters; ++it) {
+  for (; it <= kFpMaxIters; ++it) {
     k_rec_diff<<<cdiv(nl * 32, 256), 256, 0, st>>>(p->nk, p->nw, p->S, p->qm, p->EkSq, p->EwSq,
                                                     p->Dsum);
     SRM3_CUDA(cudaGetLastError());
@@ -1452,6 +1496,7 @@ static int solve_mixed(srm3_plan *p, cudaStream_t st, double x, PassResult *r) {
     std::memcpy(&ch, &bits, sizeof(ch));
     if (it >= 2 && ch <= kFpTol) return SRM3_OK;
   }
+  p->fp_iters = kFpMaxIters;
   r->err = 1;  // no convergence: treated as an infeasible x
   return SRM3_OK;
 }
@@ -2179,9 +2224,9 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
     PassResult r3[3];
     rc = run_pass_multi(p, st, x3, 3, true, r3);
     if (rc) return rc;
-    bool ok3 = true;
+    bool ok3 = r3[0].err != kPassNone;
     double f3[3];
-    for (int m = 0; m < 3; ++m) {
+    for (int m = 0; m < 3 && r3[0].err != kPassNone; ++m) {
       if (r3[m].err) {
         ok3 = false;
         b.xhi = std::min(b.xhi, x3[m]);

@@ -120,6 +120,7 @@ struct srm3_plan {
   // envelope factors and the grid fits; the plan's tables come from it
   bool solve = false;
   bool q_warm = false;          // qm holds a solution near the next pass's x
+  bool iter_off = false;        // direct iterations were too slow: level passes
   // mixed-sign interactions: opposite-sheet pairs as well; Eq. pure then
   // a fixed point solved by iterations of (difference sums at the previous
   // iterate, level pass)

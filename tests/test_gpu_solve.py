@@ -185,3 +185,17 @@ def test_targets_close_to_one_on_sparse_supports(oracle_lib, precision, kind, ta
     ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps, env=env, mixed=mixed)
     np.testing.assert_allclose(sb2, ref.sum_b2, atol=1e-6 if kind != "mixed" else 1e-9)
     np.testing.assert_allclose(q, ref.q, rtol=1e-5 if kind != "mixed" else 1e-6)
+
+
+def test_mixed_fixed_point_reached_slowly(oracle_lib):
+    """An eps 1e-7 below the largest that has a fixed point: 225 direct iterations
+    (numpy), more than the small lattice's pass takes by itself.  Tolerance: there
+    q moves by 1/sqrt(1e-7) of a relative change of the sums, 1e-15 each."""
+    wl = replace(W.small_case(nk=4, nw=6, nx=4, nt=16, precision="fp64"), interactions="mixed")
+    S = oracle.kaimal_lorentzian(4, 6, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    eps = 1.1686150240765587
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=eps, mixed=True)
+    with srm3.Plan.create(wl, table=S, eps=eps) as p:
+        _, q, sb2 = p.tables()
+        assert p.info().fixed_point_iterations > 96
+    np.testing.assert_allclose(sb2, op.sum_b2, atol=1e-8)
