@@ -623,29 +623,18 @@ static int branch_fields(srm3_batch *b, const srm3_batch::Branch &br, cudaStream
   return transform_on(p, st, p->C, b->counts[br.plan], b->outs[br.plan], p->H);
 }
 
-// The launch sequence of one batch run on the batch stream (and its lanes).
-static int batch_launch(srm3_batch *b) {
+// The launch sequence of one batch run on the batch stream (and, with lanes, on
+// the streams beside it, which batch_launch has forked and joins).
+static int batch_work(srm3_batch *b, bool lanes) {
   int rc;
   const unsigned evf = b->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-  // with the pair sum timed, everything on the batch stream, the pair sums first
-  const bool lanes = !b->timing && !b->side.empty();
-  if (lanes) {
-    SRM3_CUDA(cudaEventRecord(b->forked, b->stream));
-    for (cudaStream_t st : b->side) SRM3_CUDA(cudaStreamWaitEvent(st, b->forked, 0));
-    rc = SRM3_OK;
+  if (lanes)
     for (const auto &br : b->branches) {
       if (br.lane == 0) continue;
       const cudaStream_t st = b->side[br.lane - 1];
-      if (!rc) rc = branch_coeffs(b, br, st);
-      if (!rc) rc = branch_fields(b, br, st);
+      if ((rc = branch_coeffs(b, br, st))) return rc;
+      if ((rc = branch_fields(b, br, st))) return rc;
     }
-    for (size_t l = 0; l < b->side.size(); ++l)
-      SRM3_CUDA(cudaEventRecord(b->joined[l], b->side[l]));
-    if (rc) {  // the lanes come back to the batch stream all the same
-      for (cudaEvent_t ev : b->joined) SRM3_CUDA(cudaStreamWaitEvent(b->stream, ev, 0));
-      return rc;
-    }
-  }
   for (auto &g : b->groups) {
     if (b->conv[g.members[0]]) continue;
     SRM3_CUDA(cudaMemsetAsync(g.y, 0, g.ybytes, b->stream));
@@ -695,9 +684,25 @@ static int batch_launch(srm3_batch *b) {
         (rc = transform_on(p, b->stream, p->C, b->counts[i], b->outs[i], p->H)))
       return rc;
   }
-  if (lanes)
-    for (cudaEvent_t ev : b->joined) SRM3_CUDA(cudaStreamWaitEvent(b->stream, ev, 0));
   return SRM3_OK;
+}
+
+static int batch_launch(srm3_batch *b) {
+  // with the pair sum timed, everything on the batch stream, the pair sums first
+  const bool lanes = !b->timing && !b->side.empty();
+  if (!lanes) return batch_work(b, false);
+  cudaError_t e = cudaEventRecord(b->forked, b->stream);
+  for (cudaStream_t st : b->side)
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->forked, 0);
+  int rc = e == cudaSuccess ? batch_work(b, true) : cuda_fail(e, "batch lanes, fork");
+  // every lane comes back to the batch stream, whatever was enqueued before a
+  // failure: a later run, or the freeing of the buffers, must not overtake it
+  for (size_t l = 0; l < b->side.size(); ++l) {
+    cudaError_t ej = cudaEventRecord(b->joined[l], b->side[l]);
+    if (ej == cudaSuccess) ej = cudaStreamWaitEvent(b->stream, b->joined[l], 0);
+    if (ej != cudaSuccess && !rc) rc = cuda_fail(ej, "batch lanes, join");
+  }
+  return rc;
 }
 
 // Device buffers of a batch are stream-ordered allocations on its stream, so
