@@ -136,7 +136,8 @@ enum srm3_storage {
     SRM3_STORAGE_TABLE = 1,    /* W streamed from an HBM table (FP32 only) */
     SRM3_STORAGE_RECOMPUTE = 2, /* W rebuilt from envelope factors in-kernel */
     SRM3_STORAGE_TUNED = 3      /* the storage srm3_autotune chose for this lattice
-                                   shape in this process, else as AUTO */
+                                   shape and form of the pair sum in this process,
+                                   else as AUTO */
 };
 
 typedef struct srm3_grid {
@@ -401,9 +402,12 @@ int srm3_get_timings(srm3_plan *plan, srm3_timings *t, int reset);
  * the plan's workspace), keeps the fastest -- building the W table when a
  * table form wins and the plan has none (if it fits the plan's table
  * budget), freeing it when recomputation wins -- and records the choice for
- * the plan's (n_kappa, n_omega) in this process: plans created later with
- * that lattice take the tile (the coefficients do not depend on it), and
- * those created with SRM3_STORAGE_TUNED the storage too.  Synchronous.
+ * the plan's device, (n_kappa, n_omega) and form of the pair sum with W
+ * recomputed (self-convolution or O(N^2), which sigma_g decides) in this
+ * process: plans created later with these take the tile (the coefficients do
+ * not depend on it), and those created with SRM3_STORAGE_TUNED the storage
+ * too.  The self-convolution has no tiles: it is timed once, and recompute_ms_w16
+ * repeats recompute_ms_w32.  Synchronous.
  * Errors: INVALID_ARG (n outside 1..128), NOT_SUPPORTED (FP64 plan, mixed
  * or separable plan), OUT_OF_MEMORY, CUDA. */
 typedef struct srm3_tune_result {

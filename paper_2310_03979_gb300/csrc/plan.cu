@@ -2545,7 +2545,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
   } wguard{&wst};
   if (p->precision == SRM3_FP32 && !p->sep) {
     int tuned_nc = 4;
-    const int tuned = tune_cache_lookup(nk, nw, &tuned_nc);
+    const int tuned = tune_cache_lookup(p, &tuned_nc);
     if (tuned >= 0) p->ps_nc = tuned_nc;  // the tuned tile (results do not depend on it)
     if (p->storage == SRM3_STORAGE_TUNED)  // the autotuner's storage for this lattice
       p->storage = tuned >= 0 ? tuned : SRM3_STORAGE_AUTO;

@@ -2,6 +2,7 @@
 // the O(N^2) pair sum that assembles the coefficients C^s_k (FFT form,
 // Sec. 4.3), and the hand-written 2-D inverse FFT to u(x,t).
 #include <algorithm>
+#include <array>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -462,21 +463,26 @@ static size_t elem1(const srm3_plan *p) {
   return p->precision == SRM3_FP32 ? sizeof(float) : sizeof(double);
 }
 
-// Autotuner choices per lattice shape, process-wide: (storage, compute warps).
+// Autotuner choices, process-wide: (storage, compute warps) per device, lattice
+// shape and form of the pair sum with W recomputed (the self-convolution of a wide
+// Gaussian envelope is the faster storage where the O(N^2) form of a narrow one
+// is not: 1.7 ms and 59 ms on 256 x 512).
 static std::mutex g_tune_mu;
-static std::map<std::pair<int, int>, std::pair<int, int>> g_tune;
+using TuneKey = std::array<int, 4>;
+static std::map<TuneKey, std::pair<int, int>> g_tune;
+static TuneKey tune_key(const srm3_plan *p) { return {p->device, p->nk, p->nw, p->conv ? 1 : 0}; }
 
-int tune_cache_lookup(int nk, int nw, int *nc) {
+int tune_cache_lookup(const srm3_plan *p, int *nc) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  auto it = g_tune.find({nk, nw});
+  auto it = g_tune.find(tune_key(p));
   if (it == g_tune.end()) return -1;
-  if (nc) *nc = it->second.second;
+  *nc = it->second.second;
   return it->second.first;
 }
 
-void tune_cache_store(int nk, int nw, int storage, int nc) {
+void tune_cache_store(const srm3_plan *p, int storage, int nc) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  g_tune[{nk, nw}] = {storage, nc};
+  g_tune[tune_key(p)] = {storage, nc};
 }
 
 }  // namespace srm3
@@ -909,12 +915,15 @@ SRM3_API int srm3_autotune(srm3_plan *plan, int n, srm3_tune_result *res) {
     return SRM3_OK;
   };
   // every (storage, tile) the plan can take: the stored table when it exists,
-  // W recomputed; 32- and 16-wide tiles
+  // W recomputed; 32- and 16-wide tiles (the self-convolution has none: timed once)
   double t[2][2] = {{-1.0, -1.0}, {-1.0, -1.0}};  // [storage: table, recompute][tile]
   for (int v = 0; v < 2 && !rc; ++v) {
     const int nc = v == 0 ? 4 : 2;
     if (plan->W) rc = time_one(SRM3_STORAGE_TABLE, nc, &t[0][v]);
-    if (!rc) rc = time_one(SRM3_STORAGE_RECOMPUTE, nc, &t[1][v]);
+    if (v == 1 && plan->conv)
+      t[1][1] = t[1][0];
+    else if (!rc)
+      rc = time_one(SRM3_STORAGE_RECOMPUTE, nc, &t[1][v]);
   }
   cudaEventDestroy(ev[0]);
   cudaEventDestroy(ev[1]);
@@ -940,7 +949,7 @@ SRM3_API int srm3_autotune(srm3_plan *plan, int n, srm3_tune_result *res) {
     plan->W = nullptr;
     plan->table_bytes = 0.0;
   }
-  tune_cache_store(plan->nk, plan->nw, choice, nc);
+  tune_cache_store(plan, choice, nc);
   res->table_ms = std::min(t[0][0] < 0 ? 1e30 : t[0][0], t[0][1] < 0 ? 1e30 : t[0][1]);
   if (res->table_ms >= 1e30) res->table_ms = -1.0;
   res->recompute_ms = std::min(t[1][0], t[1][1]);

@@ -290,10 +290,11 @@ int conv_run_f64(const ConvJob &j);
 int conv_run_df(const ConvJob &j);
 int build_w_table(srm3_plan *p, cudaStream_t st);
 int ensure_tiles(srm3_plan *p, cudaStream_t st);
-// autotuner choices per lattice shape (process-wide): storage (or -1 when
-// the shape was never tuned) and the pair-sum tile's compute warps
-int tune_cache_lookup(int nk, int nw, int *nc = nullptr);
-void tune_cache_store(int nk, int nw, int storage, int nc);
+// autotuner choices per device, lattice shape and form of the pair sum
+// (process-wide): storage (or -1 when it was never tuned) and the pair-sum
+// tile's compute warps
+int tune_cache_lookup(const srm3_plan *p, int *nc);
+void tune_cache_store(const srm3_plan *p, int storage, int nc);
 // tile-shape index of nc compute warps (4 -> 0, 2 -> 1)
 inline int tile_index(int nc) { return nc == 4 ? 0 : 1; }
 }  // namespace srm3

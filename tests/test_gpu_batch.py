@@ -102,6 +102,22 @@ def test_autotune_chooses_a_storage_and_tuned_plans_use_it():
             srm3.autotune(d.handle, 2)
 
 
+def test_autotune_choice_stays_with_the_form_of_the_pair_sum():
+    """sigma_g = 0.25 takes the self-convolution, 0.1 the O(N^2) pair sum: what one
+    is tuned to says nothing about the other."""
+    import dataclasses
+    wl = W.small_case(nk=128, nw=192, nx=128, nt=512, precision="fp32")
+    with srm3.Plan.create(wl, storage="recompute") as p:
+        r = srm3.autotune(p.handle, 64)
+        assert r.recompute_ms_w16 == r.recompute_ms_w32 and r.tile_width == 32
+        assert r.storage == srm3.SRM3_STORAGE_RECOMPUTE  # 1e10 pair-terms with the table
+    narrow = dataclasses.replace(wl, sigma_g=0.1)
+    with srm3.Plan.create(narrow, storage="tuned") as q:  # never tuned: as "auto"
+        assert q.info().storage == srm3.SRM3_STORAGE_TABLE
+    with srm3.Plan.create(wl, storage="tuned") as q:
+        assert q.info().storage == srm3.SRM3_STORAGE_RECOMPUTE
+
+
 def test_uneven_batch_spectra_against_oracle(oracle_lib):
     """The uneven-batch workload's own spectra (seed 4, the benchmark's draw):
     its smallest lattices, autotuned storage as in the benchmark, through one
