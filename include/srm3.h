@@ -213,11 +213,15 @@ typedef struct srm3_info {
     double table_bytes;      /* bytes of the W table (0 when recomputed) */
     double plan_ms;          /* wall time of srm3_plan_create */
     int64_t pairs;           /* sum_k |Pi(k)| over the plan's rows */
-    int32_t root_passes;     /* FP64 recursion passes of the build */
+    int32_t root_passes;     /* evaluations of Eq. pure that the tables come from or
+                                that were made on the way to them in FP64: recursion
+                                passes, and 1 for a whole-lattice solve whose
+                                own tables the plan keeps (bit 5 below) */
     int32_t storage;         /* storage actually chosen */
     int32_t precision;
     int32_t tile_r;          /* outputs per thread along omega (FP32 path) */
-    int32_t root_passes_fp32;/* FP32 recursion passes used to locate eps */
+    int32_t root_passes_fp32;/* FP32 recursion passes used to locate eps, and 1 for
+                                a whole-lattice solve that located it */
     int32_t interactions;    /* enum srm3_interactions */
     int32_t fixed_point_iterations; /* MIXED: iterations of the final solve */
     int64_t diff_pairs;      /* MIXED: difference pairs of one sheet, sum over k
@@ -235,30 +239,36 @@ typedef struct srm3_info {
                                 separable form, g^2(i,j) = a_i^2 a_j^2 b_k^2 on the
                                 pairs of k (the separable kind, or the Gaussian
                                 envelope split on i + j = k, Sec. 4.1 Eq. pure);
-                                bit 1 (SRM3_REC_TABLES_MOVED): the tables are those
-                                of the FP64 pass at the FP32 root estimate, moved to
-                                the final eps to first order (FP32 plans);
+                                bit 1 (SRM3_REC_TABLES_MOVED): the tables (FP32 plans,
+                                Gaussian envelope) are not those of an FP64 pass at
+                                the final eps: with bit 5 they are the whole-lattice
+                                solve's, else those of the FP64 pass at the FP32
+                                root estimate, moved to the final eps to first order;
                                 bit 2 (SRM3_PAIRSUM_SEPARABLE): the FP32 pair sum
                                 runs in separable form, g = a_i a_j b_k, as a
                                 self-convolution of a y (W recomputed, Gaussian
                                 envelope, Sec. 4.3);
                                 bit 3 (SRM3_REC_COARSE_START): the eps search
                                 started from the root of the same search on a
-                                coarser lattice (coarse_fk, coarse_fw below) and
-                                one FP32 pass on this lattice bracketed it (no
-                                linear bound on this lattice);
+                                coarser lattice (coarse_fk, coarse_fw below), which
+                                one FP32 pass on this lattice bracketed or, with
+                                bit 5, the whole-lattice solve confirmed;
                                 bit 4 (SRM3_REC_TABLES_INTERPOLATED): the tables
                                 are those of one FP64 pass at three eps^2 values
                                 x32 (1 +- 2e-6) around the FP32 root, taken per
                                 point at the final eps^2 by the quadratic through
-                                the three (FP64 plans) */
+                                the three (FP64 plans);
+                                bit 5 (SRM3_REC_LATTICE_SOLVE): Eq. pure was solved on
+                                the whole lattice at once (envelopes that factor
+                                on i + j = k), which gave the tables or, where FP64
+                                passes followed, their eps and first iterate */
     int32_t coarse_fk, coarse_fw; /* the coarse lattice of the eps search takes
                                 every coarse_fk-th kappa and coarse_fw-th omega
                                 point of this one (1, 1: no coarse search; plans
                                 with a target, sum interactions and at least
                                 65536 points, either envelope kind) */
     int32_t coarse_launches;  /* kernels the coarse search launched */
-    int32_t coarse_passes;    /* its FP32 recursion passes */
+    int32_t coarse_passes;    /* its FP32 recursion passes, 1 for a solve */
 } srm3_info;
 
 #define SRM3_REC_SEPARABLE 1
@@ -266,6 +276,7 @@ typedef struct srm3_info {
 #define SRM3_PAIRSUM_SEPARABLE 4
 #define SRM3_REC_COARSE_START 8
 #define SRM3_REC_TABLES_INTERPOLATED 16
+#define SRM3_REC_LATTICE_SOLVE 32
 
 int srm3_plan_info(const srm3_plan *plan, srm3_info *info);
 
@@ -369,7 +380,8 @@ int srm3_field_from_coeffs_noalloc(srm3_plan *plan, const void *C, int n, void *
  * recorded); the sampling stages accumulate over srm3_sample /
  * srm3_sample_host / srm3_coeffs calls made while timing is enabled. */
 typedef struct srm3_timings {
-    double recursion_ms;   /* sum over all recursion passes of the build */
+    double recursion_ms;   /* Eq. pure: all recursion passes and whole-lattice
+                              solves of the build */
     double table_ms;       /* W-table build */
     double phases_ms;      /* Philox phase kernels */
     double pairsum_ms;     /* pair-sum kernels (the dominant stage) */
@@ -377,10 +389,12 @@ typedef struct srm3_timings {
     int32_t recursion_passes;
     int32_t pairsum_launches;
     int64_t pair_terms;    /* pair-terms issued by the timed pair-sum launches */
-    double recursion_fp32_ms;  /* part of recursion_ms spent in FP32 search passes */
-    double recursion_fp64_ms;  /* part of recursion_ms spent in FP64 passes */
+    double recursion_fp32_ms;  /* part of recursion_ms spent in FP32 search passes
+                                  and whole-lattice solves in double-float */
+    double recursion_fp64_ms;  /* part of recursion_ms spent in FP64 passes and the
+                                  solves that finish tables beyond double-float */
     int32_t recursion_passes_fp32;
-    int32_t recursion_passes_coarse; /* FP32 passes of the coarse eps search */
+    int32_t recursion_passes_coarse; /* FP32 passes of the coarse eps search (1: solve) */
     double coarse_ms;      /* the coarse eps search, its tables included (its
                               passes are also part of recursion_ms) */
 } srm3_timings;

@@ -406,7 +406,7 @@ struct PassResult {
   int err;
 };
 
-static thread_local cudaEvent_t t_ev[2] = {nullptr, nullptr};
+static thread_local cudaEvent_t t_ev[3] = {nullptr, nullptr, nullptr};
 
 static constexpr int kPlanes = 8;  // eps values per FP32 search pass
 // eps values of the FP32 pass over the window around the coarse-lattice root
@@ -1601,6 +1601,7 @@ static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double t
       p->t_recursion_ms += ms;
       p->t_rec32_ms += ms;
       p->root_passes32 += 1;
+      p->lattice_solve = true;
       double x = sr.x, xp = 0.0, fp = 0.0;
       bool done = false;
       r.max_sb2 = sr.max_sb2;
@@ -2058,6 +2059,7 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
       if ((rc = start_w_table(p, p->w_stream))) return rc;
     }
     const bool tables = p->precision == SRM3_FP32 || p->sep;  // not only the root
+    bool finish = false;  // a second solve, timed from t_ev[2]
     SolveResult r;
     std::memset(&r, 0, sizeof(r));
     auto run = [&](const srm3_plan *from, int fk, int fw) {
@@ -2065,8 +2067,10 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
       const bool f64 = p->sep;  // separable bispectra: finished in FP64
       int rc1 = solve_lattice(p, st, target, from ? from->eps * from->eps : 0.0, sk, sw, false,
                               tables && !f64 ? kSolveDf : kSolveLoose, from, fk, fw, &r);
-      if (!rc1 && f64 && r.converged)
+      if (!rc1 && f64 && r.converged) {
+        if (cudaEventRecord(t_ev[2], st) == cudaSuccess) finish = true;
         rc1 = solve_lattice(p, st, target, 0.0, sk, sw, true, kSolveF64, p, 1, 1, &r);
+      }
       return rc1;
     };
     const std::function<int(const srm3_plan *, int, int)> warm = run;
@@ -2076,14 +2080,17 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
     if (!r.converged && (rc = run(nullptr, 1, 1))) return rc;
     SRM3_CUDA(cudaEventRecord(t_ev[1], st));
     SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
-    float ms = 0.f;
+    float ms = 0.f, ms64 = 0.f;
     SRM3_CUDA(cudaEventElapsedTime(&ms, t_ev[0], t_ev[1]));
+    if (finish) SRM3_CUDA(cudaEventElapsedTime(&ms64, t_ev[2], t_ev[1]));
+    p->t_recursion_ms += ms;
+    p->t_rec32_ms += ms - ms64 - p->t_coarse_ms;
+    p->t_rec64_ms += ms64;
     if (r.converged && !r.err) {
-      p->t_recursion_ms += ms;
-      p->t_rec32_ms += ms - p->t_coarse_ms;
+      p->lattice_solve = true;
+      p->root_passes32 += 1;
       p->coarse_start = xc > 0.0 && std::fabs(xc - r.x) <= kCoarseWindow * r.x;
       if (tables && (p->precision == SRM3_FP32 || r.change <= kSolveExact)) {
-        p->root_passes32 += 1;  // the solve, and its tables in FP64
         p->root_passes += 1;
         p->eps = std::sqrt(r.x);
         p->max_sb2 = r.max_sb2;
@@ -2456,15 +2463,15 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
   const size_t nl = (size_t)nk * nw;
   cudaStream_t st;
   SRM3_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-  SRM3_CUDA(cudaEventCreate(&t_ev[0]));
-  SRM3_CUDA(cudaEventCreate(&t_ev[1]));
+  for (cudaEvent_t &e : t_ev) SRM3_CUDA(cudaEventCreate(&e));
   struct StreamGuard {
     cudaStream_t s;
     ~StreamGuard() {
       cudaStreamDestroy(s);
-      cudaEventDestroy(t_ev[0]);
-      cudaEventDestroy(t_ev[1]);
-      t_ev[0] = t_ev[1] = nullptr;
+      for (cudaEvent_t &e : t_ev) {
+        if (e) cudaEventDestroy(e);
+        e = nullptr;
+      }
     }
   } guard{st};
 
@@ -2617,10 +2624,21 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
     if (p->sep && p->solve) {
       SolveResult sr;
       const double x = bs->eps * bs->eps;
+      float ms32 = 0.f, ms64 = 0.f;
+      SRM3_CUDA(cudaEventRecord(t_ev[0], st));
       rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, false, kSolveLoose, nullptr, 1, 1, &sr);
-      if (!rc && sr.converged && !sr.err)
-        rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr);
       if (rc) return rc;
+      SRM3_CUDA(cudaEventRecord(t_ev[1], st));
+      if (sr.converged && !sr.err &&
+          (rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr)))
+        return rc;
+      SRM3_CUDA(cudaEventRecord(t_ev[2], st));
+      SRM3_CUDA(cudaEventSynchronize(t_ev[2]));
+      SRM3_CUDA(cudaEventElapsedTime(&ms32, t_ev[0], t_ev[1]));
+      SRM3_CUDA(cudaEventElapsedTime(&ms64, t_ev[1], t_ev[2]));
+      p->t_recursion_ms += ms32 + ms64;
+      p->t_rec32_ms += ms32;
+      p->t_rec64_ms += ms64;
       // a solve that met sums of 1 or close to it leaves the verdict to the level pass
       done = sr.converged && !sr.err &&
              (p->precision == SRM3_FP32 || sr.change <= kSolveExact);
@@ -2630,6 +2648,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
         r.sumS = p->sumS;
         r.err = 0;
         p->root_passes += 1;
+        p->lattice_solve = true;
       }
     }
     if (!done && (rc = run_pass(p, st, bs->eps * bs->eps, true, &r))) return rc;
@@ -3014,7 +3033,8 @@ SRM3_API int srm3_plan_info(const srm3_plan *plan, srm3_info *info) {
                           (plan->eps_interp ? SRM3_REC_TABLES_INTERPOLATED : 0) |
                           (conv_now(plan) && !plan->sep && plan->precision == SRM3_FP32
                                ? SRM3_PAIRSUM_SEPARABLE : 0) |
-                          (plan->coarse_start ? SRM3_REC_COARSE_START : 0);
+                          (plan->coarse_start ? SRM3_REC_COARSE_START : 0) |
+                          (plan->lattice_solve ? SRM3_REC_LATTICE_SOLVE : 0);
   info->coarse_fk = plan->coarse_fk;
   info->coarse_fw = plan->coarse_fw;
   info->coarse_launches = plan->coarse_launches;

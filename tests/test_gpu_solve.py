@@ -199,3 +199,33 @@ def test_mixed_fixed_point_reached_slowly(oracle_lib):
         _, q, sb2 = p.tables()
         assert p.info().fixed_point_iterations > 96
     np.testing.assert_allclose(sb2, op.sum_b2, atol=1e-8)
+
+
+def _timings(p):
+    return srm3.get_timings(p.handle)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_info_says_where_the_tables_come_from(precision):
+    """The whole-lattice solve has a flag of its own, counts as one search pass and,
+    where the plan keeps its tables, as one evaluation of them; its time is in
+    the passes' times.  Level passes (a target close to 1, a narrow envelope)
+    report no solve."""
+    wl = W.small_case(nk=40, nw=30, nx=64, nt=64, precision=precision)
+    with srm3.Plan.create(wl) as p:
+        i, t = p.info(), _timings(p)
+        assert i.recursion_flags & srm3.SRM3_REC_LATTICE_SOLVE
+        assert (i.root_passes_fp32, i.root_passes) == (1, 1)
+        assert t.recursion_fp32_ms > 0 and (t.recursion_fp64_ms > 0) == (precision == "fp64")
+    sep = replace(wl, envelope="separable")
+    for eps in (None, 0.5):
+        with srm3.Plan.create(sep, eps=eps) as p:
+            i, t = p.info(), _timings(p)
+            assert i.recursion_flags & srm3.SRM3_REC_LATTICE_SOLVE
+            assert not i.recursion_flags & srm3.SRM3_REC_TABLES_MOVED
+            assert i.root_passes_fp32 == (eps is None)
+            assert t.recursion_fp32_ms > 0 and t.recursion_fp64_ms > 0
+            assert t.recursion_ms == pytest.approx(t.recursion_fp32_ms + t.recursion_fp64_ms, rel=1e-3)
+    for narrow in (replace(wl, target=0.995), replace(wl, sigma_g=0.15)):
+        with srm3.Plan.create(narrow) as p:
+            assert not p.info().recursion_flags & srm3.SRM3_REC_LATTICE_SOLVE
