@@ -44,24 +44,6 @@ int scratch_address(int dev, void **addr) {
   return SRM3_OK;
 }
 
-// Makes `dev` current for the lifetime of the guard and restores the
-// caller's device afterwards.
-struct DeviceGuard {
-  int prev = -1;
-  bool switched = false;
-  int enter(int dev) {
-    SRM3_CUDA(cudaGetDevice(&prev));
-    if (prev != dev) {
-      SRM3_CUDA(cudaSetDevice(dev));
-      switched = true;
-    }
-    return SRM3_OK;
-  }
-  ~DeviceGuard() {
-    if (switched) cudaSetDevice(prev);
-  }
-};
-
 // The transform of n sets in groups whose x-stage columns fit the scratch, by
 // the launch sequence of srm3_field_from_coeffs (transform_on) with the
 // scratch in place of the plan workspace.

@@ -3212,6 +3212,8 @@ SRM3_API int srm3_plan_tables(const srm3_plan *plan, double *S, double *q, doubl
   if (!plan) return fail(SRM3_ERR_INVALID_ARG, "plan is NULL");
   const size_t nl = (size_t)plan->nk * plan->nw, b = nl * sizeof(double);
   const cudaStream_t st = plan->stream;
+  DeviceGuard guard;  // the events, the kernel and the block of this call are the plan's device's
+  if (int rc = guard.enter(plan->device)) return rc;
   SRM3_CUDA(cudaStreamSynchronize(st));
   TabSpan span[3];
   int n = 0;

@@ -271,6 +271,23 @@ int stage_end(srm3_plan *p, int rec);
 int collect_timings(srm3_plan *p);
 int check_pairsum_error(srm3_plan *p);
 int sspad_for(int chunk);
+// Makes `dev` current for the lifetime of the guard and restores the
+// caller's device afterwards.
+struct DeviceGuard {
+  int prev = -1;
+  bool switched = false;
+  int enter(int dev) {
+    SRM3_CUDA(cudaGetDevice(&prev));
+    if (prev != dev) {
+      SRM3_CUDA(cudaSetDevice(dev));
+      switched = true;
+    }
+    return SRM3_OK;
+  }
+  ~DeviceGuard() {
+    if (switched) cudaSetDevice(prev);
+  }
+};
 // The pair sum of n samples as an FFT self-convolution (conv_launch.cuh):
 // phases, convolution and coefficients into C ([2 n][nk][nw], the rows of the
 // plan), on a stream.  Seeds from the host array (passed by value) or from
