@@ -1276,6 +1276,22 @@ static constexpr double kSolveAcceptDf = 1e-10, kSolveAcceptF64 = 3e-12;
 // 603, where the solve alone took about 2
 static constexpr double kSolveExact = kSolveF64;
 
+// Whether the last eight changes of nit iterations got no closer than half the
+// ones before: targets that the iterations do not reach ("separable" tables from
+// about 0.95 on small and 0.985 on larger lattices) are left to the level passes
+// after 24 of them or so, not after kSolveMaxIt.
+static bool solve_stalled(const SolveCtl *h, int nit) {
+  if (nit < 24) return false;
+  double m[2] = {INFINITY, INFINITY};
+  for (int it = 4; it < nit; ++it) {
+    double c;
+    std::memcpy(&c, &h->chg[it], sizeof(c));
+    double &b = m[it >= nit - 8];
+    b = std::min(b, c);
+  }
+  return !(m[1] < 0.5 * m[0]);
+}
+
 // The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
 // target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
 // widths in lattice units.  from: a solved coarser plan (every fk-th, fw-th
@@ -1413,7 +1429,7 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
     SRM3_CUDA(cudaMemcpyAsync(h, A.ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
     SRM3_CUDA(cudaStreamSynchronize(st));
     if (p->sumS < 0.0) p->sumS = p->h_pinned[kSumSlot];  // copied by start_sum_S
-  } while (!h->converged && nit < kSolveMaxIt);
+  } while (!h->converged && nit < kSolveMaxIt && !solve_stalled(h, nit));
   p->n_launch += 1 + 3 * nit + 2 + low;
   r->converged = h->converged != 0 && h->X >= 0.0 && std::isfinite(h->X);
   r->x = h->X / p->dkdw;
