@@ -27,7 +27,8 @@
 // against e^16 with c in the middle of the lattice).  A transform's rounding
 // is relative to its largest values, so b_k is what it costs an output: the
 // FP32 plans run it in double-float (df.cuh), whose 2^-46 leaves every output
-// far below the FP32 rounding of y, FP64 plans in FP64.
+// far below the FP32 rounding of y, FP64 plans in triple-float (tf.cuh), which
+// leaves the rounding of the outputs alone.
 //
 // Mixed-sign interactions (Gaussian envelope): on the axis of signed omega
 // the sheet's own y sits at +omega and the other sheet's at -omega (omega >=
@@ -68,6 +69,11 @@ struct ConvNum<df2> {
   using F = df;
   using Y2 = float2;
 };
+template <>
+struct ConvNum<tf2> {
+  using F = tf;
+  using Y2 = double2;
+};
 
 __device__ __forceinline__ float conv_scale(float y, float a) { return y * a; }
 __device__ __forceinline__ double conv_scale(double y, double a) { return y * a; }
@@ -75,12 +81,17 @@ __device__ __forceinline__ df conv_scale(float y, df a) {  // the exact product,
   const float p = __fmul_rn(y, a.h);
   return df(p, __fmaf_rn(y, a.l, __fmaf_rn(y, a.h, -p)));
 }
+__device__ __forceinline__ tf conv_scale(double y, tf a) { return tf(y) * a; }
 __device__ __forceinline__ float conv_round(float v) { return v; }
 __device__ __forceinline__ double conv_round(double v) { return v; }
 __device__ __forceinline__ float conv_round(df v) { return v.h + v.l; }
+__device__ __forceinline__ double conv_round(tf v) { return (double)v.h + ((double)v.m + (double)v.l); }
 template <typename F>
 __device__ __forceinline__ F conv_pow2(F v, float s) { return v * (F)s; }
 __device__ __forceinline__ df conv_pow2(df v, float s) { return df(v.h * s, v.l * s); }
+__device__ __forceinline__ tf conv_pow2(tf v, float s) { return tf(v.h * s, v.m * s, v.l * s); }
+// the phasor rows of a row kernel follow its transforms, 16-byte aligned
+__host__ __device__ constexpr size_t conv_align(size_t b) { return (b + 15) / 16 * 16; }
 
 }  // namespace
 
@@ -115,13 +126,22 @@ namespace {
 // phases): one sample of 32 x 32 19.4 / 22.4 / 31.7, 4 FP64 mixed ones of 29 x 12
 // 37 / 46 / 67; 64 samples of 256 x 512 2213 / 1931 / 2193, 16 of 512 x 1024 2589 /
 // 2561 / 2384, 64 separable ones of 256 x 512 907 / 624 / 662, 50 of 256 x 128
-// 192 / 139 / 180 (202 with separate phases and 16 values).
-__host__ __device__ constexpr int conv_lv(int l) { return l <= 6 ? 2 : l <= 12 ? 3 : 4; }
-__host__ __device__ constexpr int conv_tpt(int l) { return tx_tpt(1 << l, conv_lv(l)); }
+// 192 / 139 / 180 (202 with separate phases and 16 values).  Triple-floats: 4,
+// whose passes hold 64 registers or so and need no rotations within.
+template <typename T2>
+__host__ __device__ constexpr int conv_lv(int l) {
+  return l <= 6 || sizeof(T2) == 24 ? 2 : l <= 12 ? 3 : 4;
+}
+// log2 of the longest transform: a row or column has to fit in shared memory.
+template <typename T2>
+constexpr int kConvMaxLog2 = sizeof(T2) == 24 ? 12 : 13;
+template <typename T2>
+__host__ __device__ constexpr int conv_tpt(int l) { return tx_tpt(1 << l, conv_lv<T2>(l)); }
 // Threads of a row CTA at most (64 unless one row takes more; whole warps, of
 // which A.rows rows are in use) and of a column CTA.
+template <typename T2>
 __host__ __device__ constexpr int conv_row_threads(int lw) {
-  return conv_tpt(lw) >= 64 ? conv_tpt(lw) : 64;
+  return conv_tpt<T2>(lw) >= 64 ? conv_tpt<T2>(lw) : 64;
 }
 // The column pass holds its CTAs to 64 registers a thread, 1024 threads per SM:
 // with the 68 that lengths past 512 took, one CTA of 512 was all an SM held, its
@@ -131,11 +151,14 @@ __host__ __device__ constexpr int conv_row_threads(int lw) {
 // 2.34, 256 x 512 plan and 64 samples 3.58 / 3.54 / 3.52, 32 uneven spectra 2.46 /
 // 2.46 / 2.39; with the two as here 2.31, 3.51 and 2.39.  (Length 4096 would
 // spill.)
+template <typename T2>
 __host__ __device__ constexpr int conv_col_threads(int lk) {
-  return conv_tpt(lk) > 512 ? conv_tpt(lk) : lk <= 9 ? 256 : 512;
+  return conv_tpt<T2>(lk) > 512 ? conv_tpt<T2>(lk) : lk <= 9 ? 256 : 512;
 }
+// (Triple-floats: no limit but the CTA's own.)
+template <typename T2>
 __host__ __device__ constexpr int conv_col_ctas(int lk) {
-  return lk <= 11 ? 1024 / conv_col_threads(lk) : 1;
+  return lk <= 11 && sizeof(T2) != 24 ? 1024 / conv_col_threads<T2>(lk) : 1;
 }
 
 template <typename T2>
@@ -190,18 +213,18 @@ __device__ __forceinline__ void conv_phases(const ConvArgs &A, uint64_t seed, in
 // transformed; rb rows of one sheet-sample per CTA (blockIdx.y = ss).
 // Threads of rows past n_kappa take part in the barriers only.
 template <int LW, typename T2, bool MIXED>
-__global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvArgs A,
+__global__ void __launch_bounds__(conv_row_threads<T2>(LW)) k_conv_rows(const ConvArgs A,
                                                                     const SeedChunk seeds) {
   using Y2 = typename ConvNum<T2>::Y2;
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nw = 1 << LW, tpt = conv_tpt(LW), LV = conv_lv(LW);
+  constexpr int Nw = 1 << LW, tpt = conv_tpt<T2>(LW), LV = conv_lv<T2>(LW);
   const int rb = blockDim.x / tpt;  // rows that fit; A.rows of them are in use
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1), ss = blockIdx.y;
   const int kk = blockIdx.x * A.rows + row, nw = A.nw;
   const bool live = row < A.rows && kk < A.nk;
   T2 *buf = reinterpret_cast<T2 *>(conv_smem) + row * (tx_len(Nw) + 1);
   // the row's phasors (and the other sheet's): up to Nw / 2 entries each
-  Y2 *yr = reinterpret_cast<Y2 *>(reinterpret_cast<T2 *>(conv_smem) + rb * (tx_len(Nw) + 1)) +
+  Y2 *yr = reinterpret_cast<Y2 *>(conv_smem + conv_align(rb * (tx_len(Nw) + 1) * sizeof(T2))) +
            (size_t)row * (MIXED ? 2 : 1) * nw;
   T2 *out = static_cast<T2 *>(A.Z) + ((size_t)ss * A.nk + kk) * Nw;
   if (live) {
@@ -243,11 +266,11 @@ __global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_rows(const ConvAr
 // in Z ([ss][n_kappa][Nw]: the grid's rows past n_kappa are zero and not
 // stored).  Shared memory: colstride entries per column.
 template <int LK, typename T2>
-__global__ void __launch_bounds__(conv_col_threads(LK), conv_col_ctas(LK))
+__global__ void __launch_bounds__(conv_col_threads<T2>(LK), conv_col_ctas<T2>(LK))
     k_conv_cols(int nk, int Nw, int TC, int colstride, const T2 *__restrict__ tw,
                 T2 *__restrict__ Z) {
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nk = 1 << LK, tpt = conv_tpt(LK), LV = conv_lv(LK);
+  constexpr int Nk = 1 << LK, tpt = conv_tpt<T2>(LK), LV = conv_lv<T2>(LK);
   const int c = threadIdx.x & (TC - 1), jt = threadIdx.x / TC, ss = blockIdx.y;
   T2 *col = reinterpret_cast<T2 *>(conv_smem) + c * colstride;
   T2 *base = Z + (size_t)ss * nk * Nw + blockIdx.x * TC + c;
@@ -273,12 +296,12 @@ __global__ void __launch_bounds__(conv_col_threads(LK), conv_col_ctas(LK))
 // as in the O(N^2) pair sums:
 //   C_k = P_k y_k + c_k e^{i beta} b_k ((z * z)_k + [k even] z_{k/2}^2) / 2.
 template <int LW, typename T2, bool MIXED>
-__global__ void __launch_bounds__(conv_row_threads(LW)) k_conv_out(const ConvArgs A) {
+__global__ void __launch_bounds__(conv_row_threads<T2>(LW)) k_conv_out(const ConvArgs A) {
   using F = typename ConvNum<T2>::F;
   using Y2 = typename ConvNum<T2>::Y2;
   using T = decltype(Y2::x);
   extern __shared__ __align__(16) unsigned char conv_smem[];
-  constexpr int Nw = 1 << LW, tpt = conv_tpt(LW), LV = conv_lv(LW);
+  constexpr int Nw = 1 << LW, tpt = conv_tpt<T2>(LW), LV = conv_lv<T2>(LW);
   const int rb = blockDim.x / tpt;  // rows that fit; A.rows of them are in use
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1), ss = blockIdx.y;
   const int kk = A.row_lo + blockIdx.x * A.rows + row, nw = A.nw;

@@ -1,4 +1,4 @@
-// conv_f64.cu - the self-convolution pair sum in FP64 (FP64 plans).
+// conv_f64.cu - the self-convolution pair sum in FP64 (separable bispectra of FP64 plans).
 #include "conv_launch.cuh"
 
 namespace srm3 {

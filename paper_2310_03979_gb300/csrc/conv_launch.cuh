@@ -49,9 +49,12 @@ cudaError_t conv_prepare(int dev) {
 // pair sum with its phases): 256 x 512, 64 samples 44.4 -> 1.74 ms; 512 x
 // 1024, 16 samples 183 -> 2.13 ms; 32 spectra on lattices of 32..256 per axis
 // in one captured batch 22.7 -> 2.4 ms; one sample on 32 x 32, with its field,
-// 60 -> 26 us.  FP64 plans: 90 x 117, 4 samples 1.64 -> 0.10 ms.  Against 64-bit
-// coefficients the FP32 fields' relative error went 1.9e-7 -> 1.8e-7 (2.1e-7
-// -> 1.9e-7 on 512 x 1024), the FP64 coefficients' stayed at 6.6e-15.
+// 60 -> 26 us.  FP64 plans: 90 x 117, 4 samples 1.64 -> 0.070 ms (in FP64 0.097 ms).
+// Against 64-bit coefficients the FP32 fields' relative error went 1.9e-7 -> 1.8e-7
+// (2.1e-7 -> 1.9e-7 on 512 x 1024).  FP64 coefficients against the oracle's, direct
+// sums / triple-float / FP64 transforms: 90 x 117 2.96e-16 / 2.96e-16 / 9.6e-16,
+// sigma_g = 0.2237 2.91e-16 / 2.90e-16 / 1.9e-15, 24 x 37 mixed 2.98e-16 / 2.93e-16 /
+// 4.3e-16 in the norm.
 //
 // What bounds it: the FP32 pipe.  A point and level of a transform costs ~28
 // FP32 operations in double-float (2 two-sums of 8 per sum, 32 a complex
@@ -72,22 +75,23 @@ int conv_run(const ConvJob &j) {
   // rows per CTA: what 64 threads hold, fewer where that leaves SMs idle; whole warps
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
-  const int tpt = conv_tpt(lw), most = std::max(1, 64 / tpt);
+  const int tpt = conv_tpt<T2>(lw), most = std::max(1, 64 / tpt);
   const long long allrows = (long long)p->nk * 2 * per;
   const int rows = (int)std::min<long long>(most, std::max<long long>(1, allrows / (4 * nsm)));
   const int rthreads = (rows * tpt + 31) / 32 * 32, rb = rthreads / tpt;
   const int copies = p->mixed ? 2 : 1;
   const size_t stage = (size_t)rb * (tx_len(Nw) + 1) * sizeof(T2);
-  const size_t srow = stage + (size_t)rb * copies * p->nw * sizeof(Y2);
+  const size_t srow = conv_align(stage) + (size_t)rb * copies * p->nw * sizeof(Y2);
   const size_t sout = stage + (p->mixed ? (size_t)rthreads * sizeof(T2) : 0);
-  const int wf = (int)(128 / sizeof(T2));  // lanes of one shared-memory wavefront
+  // lanes of one shared-memory wavefront (triple-floats: of their 32-byte spacing)
+  const int wf = sizeof(T2) == 24 ? 4 : (int)(128 / sizeof(T2));
   auto colstride = [&](int tc) {
     const int len = (tx_len(Nk) + wf - 1) / wf * wf;
     return len + (tc >= wf ? 1 : wf / tc);
   };
   int TC = 16;
   while (TC > 1 && (TC > Nw || (size_t)TC * colstride(TC) * sizeof(T2) > 100 * 1024 ||
-                    TC * conv_tpt(lk) > conv_col_threads(lk) ||
+                    TC * conv_tpt<T2>(lk) > conv_col_threads<T2>(lk) ||
                     (long long)(Nw / TC) * 2 * per < nsm))
     TC >>= 1;
   const int cs = colstride(TC);
@@ -103,6 +107,7 @@ int conv_run(const ConvJob &j) {
   A.Nw = Nw;
   A.mixed = p->mixed ? 1 : 0;
   constexpr bool f32 = std::is_same<T2, float2>::value;
+  constexpr bool gauss = !kPlainNum<T2>;  // the others: separable bispectra alone
   if (p->sep) {
     A.e = f32 ? (const void *)p->env_e32 : (const void *)p->env_e;
     A.eb = f32 ? (const void *)p->env_b32 : (const void *)p->env_b;
@@ -122,7 +127,7 @@ int conv_run(const ConvJob &j) {
   A.ck_of = j.ck_of;
   A.dseeds = j.dseeds;
   A.twk = p->tw_conv;
-  A.tww = static_cast<const T2 *>(p->tw_conv) + tx_twlen(lk, conv_lv(lk));
+  A.tww = static_cast<const T2 *>(p->tw_conv) + tx_twlen(lk, conv_lv<T2>(lk));
   A.cb = std::cos(p->beta);
   A.sb = std::sin(p->beta);
   A.row_lo = p->row_lo;
@@ -138,10 +143,10 @@ int conv_run(const ConvJob &j) {
     A.C = static_cast<char *>(j.C) + 2 * n0 * yrow;
     if (!j.dseeds) std::memcpy(sc.s, j.seeds + n0, sizeof(uint64_t) * ns);
     cudaError_t err = cudaSuccess;
-    conv_with_log2<1, 13>(lw, [&](auto c) {
+    conv_with_log2<1, kConvMaxLog2<T2>>(lw, [&](auto c) {
       constexpr int L = decltype(c)::value;
       const dim3 grid(conv_cdiv(p->nk, rows), 2 * ns);
-      if constexpr (!f32) {
+      if constexpr (gauss) {
         if (p->mixed) {
           err = conv_prepare<k_conv_rows<L, T2, true>>(p->device);
           if (err == cudaSuccess)
@@ -155,19 +160,19 @@ int conv_run(const ConvJob &j) {
     });
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "pair sum, rows");
-    conv_with_log2<1, 13>(lk, [&](auto c) {
+    conv_with_log2<1, kConvMaxLog2<T2>>(lk, [&](auto c) {
       constexpr int L = decltype(c)::value;
       err = conv_prepare<k_conv_cols<L, T2>>(p->device);
       if (err == cudaSuccess)
-        k_conv_cols<L, T2><<<dim3(Nw / TC, 2 * ns), TC * conv_tpt(L), scol, j.stream>>>(
+        k_conv_cols<L, T2><<<dim3(Nw / TC, 2 * ns), TC * conv_tpt<T2>(L), scol, j.stream>>>(
             p->nk, Nw, TC, cs, static_cast<const T2 *>(A.twk), static_cast<T2 *>(A.Z));
     });
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "pair sum, columns");
-    conv_with_log2<1, 13>(lw, [&](auto c) {
+    conv_with_log2<1, kConvMaxLog2<T2>>(lw, [&](auto c) {
       constexpr int L = decltype(c)::value;
       const dim3 grid(conv_cdiv(p->row_hi - p->row_lo, rows), 2 * ns);
-      if constexpr (!f32) {
+      if constexpr (gauss) {
         if (p->mixed) {
           err = conv_prepare<k_conv_out<L, T2, true>>(p->device);
           if (err == cudaSuccess) k_conv_out<L, T2, true><<<grid, rthreads, sout, j.stream>>>(A);

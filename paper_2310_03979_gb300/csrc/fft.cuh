@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "df.cuh"
+#include "tf.cuh"
 #include "srm3_internal.cuh"
 
 namespace srm3 {
@@ -152,6 +153,21 @@ __device__ __forceinline__ int brev(int m, int log2n) {
 // cos(pi / 8), sin(pi / 8), cos(pi / 4), and tan(pi / 8)
 constexpr double kC1 = 0.92387953251128675613, kS1 = 0.38268343236508977173;
 constexpr double kH = 0.70710678118654752440, kT1 = 0.41421356237309504880;
+// what kC1, kS1 and kH leave of their numbers
+constexpr double kC1l = 1.7645047084336677e-17, kS1l = -1.0050772696461588e-17;
+constexpr double kHl = -4.833646656726457e-17;
+
+// One number of the machine, or several (df, tf).
+template <typename T2>
+constexpr bool kPlainNum = std::is_floating_point<typename RealOf<T2>::type>::value;
+
+template <typename T>
+__device__ __forceinline__ T rot_const(double v, double rest) {
+  if constexpr (std::is_same<T, tf>::value)
+    return tf(v, rest);
+  else
+    return (T)v;
+}
 
 // b * e^{2 pi i e / 16}, e in [0, 8) (e a constant after unrolling)
 template <typename T2>
@@ -161,15 +177,20 @@ __device__ __forceinline__ T2 rot16(T2 b, int e) {
   switch (e) {
     case 0:
       return b;
-    case 2:
-      return c_make<T2>((T)kH * (x - y), (T)kH * (x + y));
+    case 2: {
+      const T h = rot_const<T>(kH, kHl);
+      return c_make<T2>(h * (x - y), h * (x + y));
+    }
     case 4:
       return c_make<T2>(-y, x);
-    case 6:
-      return c_make<T2>(-((T)kH * (x + y)), (T)kH * (x - y));
+    case 6: {
+      const T h = rot_const<T>(kH, kHl);
+      return c_make<T2>(-(h * (x + y)), h * (x - y));
+    }
     default: {
-      const T c = e == 1 ? (T)kC1 : e == 3 ? (T)kS1 : e == 5 ? (T)-kS1 : (T)-kC1;
-      const T s = (e == 1 || e == 7) ? (T)kS1 : (T)kC1;
+      const T c1 = rot_const<T>(kC1, kC1l), s1 = rot_const<T>(kS1, kS1l);
+      const T c = e == 1 ? c1 : e == 3 ? s1 : e == 5 ? -s1 : -c1;
+      const T s = (e == 1 || e == 7) ? s1 : c1;
       return cmul(b, c_make<T2>(c, s));
     }
   }
@@ -181,7 +202,7 @@ __device__ __forceinline__ T2 rot16(T2 b, int e) {
 // multiply-adds instead of eight operations.
 template <int E, typename T2>
 __device__ __forceinline__ void bfly16(T2 &a, T2 &b) {
-  if constexpr (E == 0 || E == 4 || std::is_same<T2, df2>::value) {
+  if constexpr (E == 0 || E == 4 || !kPlainNum<T2>) {
     const T2 t = rot16(b, E), x = a;
     a = c_add(x, t);
     b = c_sub(x, t);
@@ -327,8 +348,8 @@ __device__ __forceinline__ int sp16(int i) { return i + (i >> 4); }
 __host__ __device__ constexpr int tx_len(int L) { return L + (L >> 4); }
 __host__ __device__ constexpr int tx_tpt(int L, int lv = 4) { return L >> lv > 0 ? L >> lv : 1; }
 
-// The R twiddles of one item (16-byte loads; the tables start 16-byte aligned
-// and every run is an even number of entries).
+// The R twiddles of one item (16-byte loads: the tables start 16-byte aligned
+// and every run is an even number of entries; 8-byte ones of triple-floats).
 template <int R, typename T2>
 __device__ __forceinline__ void load_tw(const T2 *__restrict__ p, T2 (&w)[R]) {
   if constexpr (sizeof(T2) == 8) {
@@ -340,6 +361,14 @@ __device__ __forceinline__ void load_tw(const T2 *__restrict__ p, T2 (&w)[R]) {
       w[2 * i].y = t.y;
       w[2 * i + 1].x = t.z;
       w[2 * i + 1].y = t.w;
+    }
+  } else if constexpr (sizeof(T2) == 24) {
+    const float2 *q = reinterpret_cast<const float2 *>(p);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      w[i].h = __ldg(q + 3 * i);
+      w[i].m = __ldg(q + 3 * i + 1);
+      w[i].l = __ldg(q + 3 * i + 2);
     }
   } else {
     const float4 *q = reinterpret_cast<const float4 *>(p);  // one 16-byte entry each

@@ -271,27 +271,77 @@ __global__ void k_sampling_tables(int n, double dkdw, double eps,
   ck[k] = (T)(pos ? 2.0 * eps * dkdw * sqrt(s) : 0.0);
 }
 
+// Tables of triple-float transforms.  They are worth more than FP64's 53 bits, and
+// FP32 operations take a thread a few cycles where FP64 ones take tens: formed in
+// double-double they added 70 us to the plan of a 32 x 32 lattice.
+
+// e^x, |x| < 60: x = k ln 2 + 16 r, the Taylor series of e^r (|r| < 0.022: eleven
+// terms), squared four times.
+__device__ __forceinline__ tf tf_exp(tf x) {
+  const tf ln2(0.6931471805599453, 2.3190468138462996e-17);
+  const float k = rintf(x.h * 1.44269504f);
+  tf r = x - tf(k, 0.f, 0.f) * ln2;
+  r = tf(r.h * 0.0625f, r.m * 0.0625f, r.l * 0.0625f);
+  tf s(1.0);
+#pragma unroll
+  for (int n = 11; n >= 1; --n) s = tf(1.0) + r * (s * tf(1.0 / n));
+  for (int n = 0; n < 4; ++n) s = s * s;
+  const float p = ldexpf(1.0f, (int)k);
+  return tf(s.h * p, s.m * p, s.l * p);
+}
+
+// 1 / s^2 to twice FP64's precision, as a triple-float (host).
+static tf inv_square(double s) {
+  const double q = 1.0 / s, ql = std::fma(-q, s, 1.0) / s, p = q * q;
+  return tf(p, std::fma(q, q, -p) + 2.0 * q * ql);
+}
+
+// e^{f (ic / s)^2} in the real type of a transform, f a power of two; is2 =
+// 1 / s^2.  (ic is a multiple of 1/4 below 2^14: its square is exact.)
+template <typename F>
+__device__ __forceinline__ F gauss_factor(double ic, double s, tf is2, double f) {
+  if constexpr (std::is_same<F, tf>::value) {
+    return tf_exp(tf(f * (ic * ic)) * is2);
+  } else {
+    const double u = ic / s;
+    return (F)exp(f * (u * u));
+  }
+}
+
+// cos and sin of 2 pi num / den, den a power of two: Newton's step for w^den = 1
+// from the values rounded to FP64.
+__device__ __forceinline__ tf2 tf_root(long long num, long long den) {
+  double sn, cs;
+  sincospi(2.0 * (double)num / (double)den, &sn, &cs);
+  while (den > 1 && !(num & 1)) {
+    num >>= 1;
+    den >>= 1;
+  }
+  tf2 w = c_make<tf2>(tf(cs), tf(sn));
+  if (den <= 4) return w;  // exact
+  const tf2 w0 = w;
+  for (long long m = den; m > 1; m >>= 1) w = cmul(w, w);
+  const tf re = c_re(w), im = c_im(w);
+  const float inv = 1.0f / (float)den;
+  const float dr = (__fadd_rn(re.h, -1.0f) + re.m + re.l) * inv, di = (im.h + im.m + im.l) * inv;
+  return c_sub(w0, cmul(w0, c_make<tf2>(tf(dr, 0.f, 0.f), tf(di, 0.f, 0.f))));
+}
+
 // The factors of the Gaussian envelope for the self-convolution (conv.cuh):
 // per axis a = exp(-((i - c)/s)^2) and b = exp(1/2 ((k - 2c)/s)^2), c = (n -
 // 1)/4, the omega axis of a over the signed indices -(nw - 1) .. nw - 1.
 template <typename F>
-__global__ void k_conv_factors(int nk, int nw, double sk, double sw, F *__restrict__ fac) {
+__global__ void k_conv_factors(int nk, int nw, double sk, double sw, tf isk, tf isw,
+                               F *__restrict__ fac) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   F *aK = fac, *bK = fac + nk, *aW = fac + 2 * nk, *bW = aW + 2 * nw - 1;
   const double ck = 0.25 * (nk - 1), cw = 0.25 * (nw - 1);
   if (i < nk) {
-    const double u = (i - ck) / sk, v = (i - 2.0 * ck) / sk;
-    aK[i] = (F)exp(-u * u);
-    bK[i] = (F)exp(0.5 * v * v);
+    aK[i] = gauss_factor<F>(i - ck, sk, isk, -1.0);
+    bK[i] = gauss_factor<F>(i - 2.0 * ck, sk, isk, 0.5);
   }
-  if (i < 2 * nw - 1) {
-    const double u = (i - (nw - 1) - cw) / sw;
-    aW[i] = (F)exp(-u * u);
-  }
-  if (i < nw) {
-    const double v = (i - 2.0 * cw) / sw;
-    bW[i] = (F)exp(0.5 * v * v);
-  }
+  if (i < 2 * nw - 1) aW[i] = gauss_factor<F>(i - (nw - 1) - cw, sw, isw, -1.0);
+  if (i < nw) bW[i] = gauss_factor<F>(i - 2.0 * cw, sw, isw, 0.5);
 }
 
 template <typename T>
@@ -332,10 +382,14 @@ __global__ void k_tx_twiddles(int lx, int lm, T2 *tw, int vx = 4, int vm = 4) {
       ns *= R;
     }
   }
-  double sn, cs;
-  sincospi(2.0 * (double)num / (double)den, &sn, &cs);
   using F = typename RealOf<T2>::type;
-  tw[e] = c_make<T2>((F)cs, (F)sn);
+  if constexpr (std::is_same<F, tf>::value) {
+    tw[e] = tf_root(num, den);
+  } else {
+    double sn, cs;
+    sincospi(2.0 * (double)num / (double)den, &sn, &cs);
+    tw[e] = c_make<T2>((F)cs, (F)sn);
+  }
 }
 
 template <typename T2>
@@ -2731,22 +2785,26 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
     p->cNk = 1 << p->log2cNk;
     p->cNw = 1 << p->log2cNw;
     const int lk = p->log2cNk, lw = p->log2cNw;
-    const int vk = conv_lv(lk), vw = conv_lv(lw);
+    const bool tri = !f32 && !p->sep;  // in triple-float
+    const int vk = tri ? conv_lv<tf2>(lk) : conv_lv<df2>(lk);
+    const int vw = tri ? conv_lv<tf2>(lw) : conv_lv<df2>(lw);
     const int ntwc = tx_twlen(lk, vk) + tx_twlen(lw, vw) + (1 << lw);
     const int nfac = 2 * nk + 3 * nw - 1, m = std::max(nk, 2 * nw - 1);
     const double sk = p->sigma_g * nk, sw = p->sigma_g * nw;
-    SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(double2), st));
-    if (!p->sep) SRM3_CUDA(dev_alloc(&p->conv_fac, (size_t)nfac * sizeof(double), st));
-    if (!f32) {
+    SRM3_CUDA(dev_alloc(&p->tw_conv, (size_t)ntwc * sizeof(tf2), st));
+    if (!p->sep) SRM3_CUDA(dev_alloc(&p->conv_fac, (size_t)nfac * sizeof(tf), st));
+    if (tri) {
+      k_tx_twiddles<tf2><<<cdiv(ntwc, 64), 64, 0, st>>>(lk, lw, (tf2 *)p->tw_conv, vk, vw);
+      k_conv_factors<tf><<<cdiv(m, 64), 64, 0, st>>>(nk, nw, sk, sw, inv_square(sk), inv_square(sw),
+                                                     (tf *)p->conv_fac);
+    } else if (!f32) {
       k_tx_twiddles<double2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (double2 *)p->tw_conv, vk, vw);
-      if (!p->sep)
-        k_conv_factors<double><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw,
-                                                             (double *)p->conv_fac);
     } else if (p->sep) {
       k_tx_twiddles<float2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (float2 *)p->tw_conv, vk, vw);
     } else {
       k_tx_twiddles<df2><<<cdiv(ntwc, 256), 256, 0, st>>>(lk, lw, (df2 *)p->tw_conv, vk, vw);
-      k_conv_factors<df><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw, (df *)p->conv_fac);
+      k_conv_factors<df><<<cdiv(m, 256), 256, 0, st>>>(nk, nw, sk, sw, tf(0.0), tf(0.0),
+                                                       (df *)p->conv_fac);
     }
   }
   p->rowstride = nw + 2 * kPad;  // y row length, workspace or batch buffers
@@ -2988,10 +3046,12 @@ SRM3_API int srm3_plan_create(const srm3_spectrum *spectrum, const srm3_bispectr
     // the pair sum as a self-convolution: its factors centred at a quarter
     // of the lattice, b reaches exp(E / 8), which the transform's rounding is
     // multiplied by (e^5 at the limit: 1e-12 of an output in double-float);
-    // one padded row and column of the grid have to fit in shared memory
+    // one padded row and column of the grid have to fit in shared memory (of
+    // triple-floats, FP64 plans: 4096 points)
     const int padw = p->mixed ? 3 * g.n_omega - 2 : 2 * g.n_omega - 1;
+    const int most = p->precision == SRM3_FP64 && !p->sep ? kMaxFft / 2 : kMaxFft;
     p->solve = (p->sep || E <= kSepExpMax) && 2 * g.n_kappa - 1 <= kMaxFft / 2 && padw <= kMaxFft;
-    p->conv = p->sep || (E <= kSepExpMax && 2 * g.n_kappa - 1 <= kMaxFft && padw <= kMaxFft);
+    p->conv = p->sep || (E <= kSepExpMax && 2 * g.n_kappa - 1 <= most && padw <= most);
   }
   p->beta = bispectrum->beta;
   p->table_budget = g.table_budget_bytes > 0 ? g.table_budget_bytes : 64.0 * (1ull << 30);

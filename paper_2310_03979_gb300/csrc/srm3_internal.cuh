@@ -307,6 +307,7 @@ struct ConvJob {
 int conv_run_f32(const ConvJob &j);
 int conv_run_f64(const ConvJob &j);
 int conv_run_df(const ConvJob &j);
+int conv_run_tf(const ConvJob &j);
 int build_w_table(srm3_plan *p, cudaStream_t st);
 int ensure_tiles(srm3_plan *p, cudaStream_t st);
 // autotuner choices per device, lattice shape and form of the pair sum
@@ -338,6 +339,6 @@ inline size_t y_bytes(const srm3_plan *p, int sp) {
 }
 inline int conv_sample(const srm3::ConvJob &j) {
   const srm3_plan *p = j.plan;
-  if (p->precision == SRM3_FP64) return srm3::conv_run_f64(j);
+  if (p->precision == SRM3_FP64) return p->sep ? srm3::conv_run_f64(j) : srm3::conv_run_tf(j);
   return p->sep ? srm3::conv_run_f32(j) : srm3::conv_run_df(j);
 }

@@ -101,3 +101,25 @@ def test_batch_lanes_match_plans_alone(captured, timed):
     batch.destroy()
     for p in plans:
         p.destroy()
+
+
+@pytest.mark.parametrize("nk,nw,sigma_g,interactions", [
+    (90, 117, 0.25, "sum"), (90, 117, 0.2237, "sum"), (64, 65, 0.3, "sum"), (1, 50, 0.25, "sum"),
+    (40, 33, 0.5, "mixed"), (20, 70, 0.2237, "mixed"),
+])
+def test_fp64_coefficients_keep_the_rounding_of_direct_sums(oracle_lib, nk, nw, sigma_g,
+                                                            interactions):
+    """FP64 coefficients as close to the oracle's as directly summed pairs are: 3e-16
+    in the norm, the rounding of the phasors, tables and outputs of both sides.
+    A transform in FP64, whose rounding is relative to its largest values and
+    multiplied by the envelope's factor, leaves 8e-16 to 2e-15."""
+    wl = _case(nk, nw, "fp64", sigma_g, 0.0, interactions)
+    S = oracle.kaimal_lorentzian(nk, nw, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    S[:, 0] = S.max() / (1.0 + np.arange(nk))
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, target=0.5, mixed=interactions == "mixed",
+                          env=oracle.Envelope("gauss", sigma_g))
+    with srm3.Plan.create(wl, table=S, eps=op.eps) as p:
+        C = _cplx(p.coeffs([1, 2, 3]))
+    for i in range(3):
+        ref = op.coeffs(i + 1)
+        assert np.linalg.norm(C[i] - ref) <= 5e-16 * np.linalg.norm(ref)
