@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsrm3.so")
 SOURCES = ["plan.cu", "sample.cu", "transform.cu", "conv_f32.cu", "conv_f64.cu",
-           "conv_df.cu", "conv_tf.cu", "solve_df.cu", "solve_f64.cu", "noalloc.cu", "stats.cu"]
+           "conv_df.cu", "conv_tf.cu", "solve_df.cu", "solve_tf.cu", "noalloc.cu", "stats.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

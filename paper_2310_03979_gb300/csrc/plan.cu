@@ -1110,35 +1110,29 @@ static int run_pass(srm3_plan *p, cudaStream_t st, double x, bool fp64, PassResu
 // The squared envelope factors per axis, centred at a quarter of the lattice
 // (k_conv_factors, squared), in FP64 and in the transform's type.
 template <typename F>
-__global__ void k_solve_factors(int nk, int nw, double sk, double sw, double *__restrict__ fac,
-                                F *__restrict__ ffac) {
+__global__ void k_solve_factors(int nk, int nw, double sk, double sw, tf isk, tf isw,
+                                double *__restrict__ fac, F *__restrict__ ffac) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int oa = 2 * nk, ob = 2 * nk + 2 * nw - 1;  // aK, bK, aW, bW
   const double ck = 0.25 * (nk - 1), cw = 0.25 * (nw - 1);
-  auto put = [&](int j, double v) {
-    fac[j] = v;
-    ffac[j] = F(v);
+  auto put = [&](int j, double ic, double sg, tf isg, double f) {
+    fac[j] = gauss_factor<double>(ic, sg, isg, f);
+    ffac[j] = std::is_same<F, tf>::value ? gauss_factor<F>(ic, sg, isg, f) : F(fac[j]);
   };
   if (i < nk) {
-    const double u = (i - ck) / sk, v = (i - 2.0 * ck) / sk;
-    put(i, exp(-2.0 * u * u));
-    put(nk + i, exp(v * v));
+    put(i, i - ck, sk, isk, -2.0);
+    put(nk + i, i - 2.0 * ck, sk, isk, 1.0);
   }
-  if (i < 2 * nw - 1) {
-    const double u = (i - (nw - 1) - cw) / sw;
-    put(oa + i, exp(-2.0 * u * u));
-  }
-  if (i < nw) {
-    const double v = (i - 2.0 * cw) / sw;
-    put(ob + i, exp(v * v));
-  }
+  if (i < 2 * nw - 1) put(oa + i, i - (nw - 1) - cw, sw, isw, -2.0);
+  if (i < nw) put(ob + i, i - 2.0 * cw, sw, isw, 1.0);
 }
 
-// n doubles in the transform's type.
+// n doubles times a power of two in the transform's type.
 template <typename F>
-__global__ void k_solve_convert(long long n, const double *__restrict__ in, F *__restrict__ out) {
+__global__ void k_solve_convert(long long n, double scale, const double *__restrict__ in,
+                                F *__restrict__ out) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = F(in[i]);
+  if (i < n) out[i] = F(in[i] * scale);
 }
 
 // sum_b2 = X g and q = 1/(1 - sum_b2) (0 where S = 0 or sum_b2 >= 1, which
@@ -1244,7 +1238,8 @@ __global__ void __launch_bounds__(256) k_solve_final(long long n, const SolveArg
 // directly in FP64 from the solve's q: their sums are small, and a
 // transform's rounding is not relative to them.  One warp per point, up to 8
 // points of a lattice row per CTA (solve_low_ctas); e2, b2: the separable tables
-// in FP64, or NULL and fac the Gaussian envelope's.  256 x 512: 20 M products.
+// in FP64, with the scales of the transform's copies, or NULL and fac the Gaussian
+// envelope's.  256 x 512: 20 M products.
 __host__ __device__ inline int solve_low_ctas(int kk, int nw) {
   const int n = kSolveLow / (kk + 1) < nw ? kSolveLow / (kk + 1) : nw;
   return (n + 7) / 8;
@@ -1252,7 +1247,8 @@ __host__ __device__ inline int solve_low_ctas(int kk, int nw) {
 
 __global__ void __launch_bounds__(256) k_solve_low(const SolveArgs A,
                                                    const double *__restrict__ e2,
-                                                   const double *__restrict__ b2,
+                                                   const double *__restrict__ b2, double se,
+                                                   double sb,
                                                    const double *__restrict__ fac,
                                                    const double *__restrict__ q,
                                                    double *__restrict__ g64) {
@@ -1270,7 +1266,7 @@ __global__ void __launch_bounds__(256) k_solve_low(const SolveArgs A,
     const int b = kk - a, jw = kw - iw;
     if (!((a == 0 && iw == 0) || iw > ((a == b) ? kw / 2 : kw))) {
       const size_t i = (size_t)a * nw + iw, jj = (size_t)b * nw + jw;
-      const double w = e2 ? e2[i] * e2[jj] : (aK[a] * aW[iw]) * (aK[b] * aW[jw]);
+      const double w = e2 ? (e2[i] * se) * (e2[jj] * se) : (aK[a] * aW[iw]) * (aK[b] * aW[jw]);
       t = fma(w, q[i] * q[jj], t);
     }
     a += da;
@@ -1282,7 +1278,7 @@ __global__ void __launch_bounds__(256) k_solve_low(const SolveArgs A,
   }
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   const size_t k = (size_t)kk * nw + kw;
-  const double g = A.S[k] > 0.0 ? (b2 ? b2[k] : bK[kk] * bW[kw]) * t : 0.0;
+  const double g = A.S[k] > 0.0 ? (b2 ? b2[k] * sb : bK[kk] * bW[kw]) * t : 0.0;
   if (lane == 0) {
     g64[k] = g;
     if (g > 0.0) atomicMax(&A.ctl->gmax, (unsigned long long)__double_as_longlong(g));
@@ -1306,7 +1302,7 @@ __global__ void k_solve_prolong(int nk, int nw, int fk, int fw, int nkc, int nwc
 }
 
 int solve_iterate_df(const SolveArgs &A, int it, int device, int nsm, cudaStream_t st);
-int solve_iterate_f64(const SolveArgs &A, int it, int device, int nsm, cudaStream_t st);
+int solve_iterate_tf(const SolveArgs &A, int it, int device, int nsm, cudaStream_t st);
 
 struct SolveResult {
   bool converged;
@@ -1316,19 +1312,16 @@ struct SolveResult {
   bool no_pairs;  // none, or so weak that the sums may be the transforms' rounding
 };
 
-// largest change of s at which the solve stops: the coarse
-// lattice's, and the root estimate the FP64 passes of FP64 plans start from
-// (their reach is 1e-5); the tables of FP32 plans (target met to 1e-9), in
-// double-float; those of separable bispectra, in FP64
-static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-12, kSolveF64 = 3e-14;
-// the change at which a solve whose changes have stopped falling still counts
-static constexpr double kSolveAcceptDf = 1e-10, kSolveAcceptF64 = 3e-12;
-// and of FP64 plans' tables (separable bispectra): where the transform's
-// rounding keeps the sums moving by more (the wind-field envelope on 486 x 202:
-// 9e-13; tables up to 8 times further off than the level pass's) they come from
-// the level pass, from the solve's root: 42.5 -> 20.8 ms there, 33.4 -> 16.0 on 94 x
-// 603, where the solve alone took about 2
-static constexpr double kSolveExact = kSolveF64;
+// largest change of s at which the solve stops: the coarse lattice's, and the root
+// estimate the FP64 passes of FP64 plans start from (their reach is 1e-5); in
+// double-float, the tables of FP32 plans with the Gaussian envelope (target met to
+// 1e-9); in triple-float, tables that were those of FP64 passes (at a given eps the
+// changes fall ever faster)
+static constexpr double kSolveLoose = 1e-8, kSolveDf = 3e-12, kSolveTf = 4e-16, kSolveTfEps = 1e-15;
+// the change at which a solve whose changes have stopped falling still counts; of
+// a triple-float one FP64's rounding of the sums: where they move by more the tables
+// come from the level pass, from the solve's root
+static constexpr double kSolveAcceptDf = 1e-10, kSolveExact = 2e-15;
 
 // Whether the last eight changes of nit iterations got no closer than half the
 // ones before: targets that the iterations do not reach ("separable" tables from
@@ -1349,9 +1342,10 @@ static bool solve_stalled(const SolveCtl *h, int nit) {
 // The tables of Eq. pure into p->sb2 (plane 0) and p->qm: at max_k sum_b2 =
 // target, or for target <= 0 at eps^2 = x.  sk, sw: the Gaussian envelope's
 // widths in lattice units.  from: a solved coarser plan (every fk-th, fw-th
-// point) to start from, or NULL.
+// point, or p itself) to start from, or NULL.  fine: in triple-float.  Separable
+// tables are taken relative to the powers of two at their maxima.
 static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x, double sk,
-                         double sw, bool fp64, double tol, const srm3_plan *from, int fk, int fw,
+                         double sw, bool fine, double tol, const srm3_plan *from, int fk, int fw,
                          SolveResult *r) {
   const int hold = 3;
   const int nk = p->nk, nw = p->nw;
@@ -1363,10 +1357,12 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   const int vk = solve_lv(lk), vm = solve_lv(lm);
   const int ntw = tx_twlen(lk, vk) + tx_twlen(lm, vm) + M;
   auto up = [](size_t b) { return (b + 15) / 16 * 16; };
-  const size_t zb = (size_t)nk * M * 16, lb = up((size_t)nl * 8), tb = (size_t)ntw * 16;
-  const size_t fb = up((size_t)nfac * 8);
+  const size_t cs = fine ? sizeof(tf2) : sizeof(df2), es = fine ? sizeof(tf) : sizeof(df);
+  const size_t zb = (size_t)nk * M * cs, lb = up((size_t)nl * es), gb = up((size_t)nl * 8);
+  const size_t tb = up((size_t)ntw * cs), db = up((size_t)nfac * 8), fb = up((size_t)nfac * es);
   char *blk = nullptr, *at = nullptr;
-  SRM3_CUDA(dev_alloc((void **)&blk, zb + (p->sep ? 10 : 8) * lb + tb + 2 * fb + sizeof(SolveCtl), st));
+  SRM3_CUDA(dev_alloc((void **)&blk,
+                      up(zb) + (p->sep ? 9 : 7) * lb + gb + tb + db + fb + sizeof(SolveCtl), st));
   struct Guard {
     char *b;
     cudaStream_t st;
@@ -1386,61 +1382,64 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   A.M = M;
   A.mixed = p->mixed ? 1 : 0;
   A.S = p->S;
-  A.Z = take(zb);
+  A.Z = take(up(zb));
   for (void *&g : A.g) g = take(lb);
   for (void *&s : A.s) s = take(lb);
-  double *g64 = reinterpret_cast<double *>(take(lb));
+  double *g64 = reinterpret_cast<double *>(take(gb));
   char *tw = take(tb);
   A.ctl = reinterpret_cast<SolveCtl *>(take(sizeof(SolveCtl)));
   A.twk = tw;
-  A.twm = tw + (size_t)tx_twlen(lk, vk) * 16;
-  A.twz = tw + (size_t)(tx_twlen(lk, vk) + tx_twlen(lm, vm)) * 16;
+  A.twm = tw + (size_t)tx_twlen(lk, vk) * cs;
+  A.twz = tw + (size_t)(tx_twlen(lk, vk) + tx_twlen(lm, vm)) * cs;
   SRM3_CUDA(cudaMemsetAsync(A.ctl, 0, sizeof(SolveCtl), st));
-  double *fac = nullptr;
+  double *fac = nullptr, scale[2] = {1.0, 1.0};
+  int unit = 0;  // g is formed in units of 2^unit
   if (p->sep) {
     const double *t[2] = {p->env_e2, p->env_b2};
     const void *c[2];
     for (int j = 0; j < 2; ++j) {
       char *o = take(lb);
-      if (fp64) {
-        c[j] = t[j];
-      } else {
-        k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, t[j], reinterpret_cast<df *>(o));
-        c[j] = o;
-        p->n_launch += 1;
-      }
+      scale[j] = std::ldexp(1.0, -p->sep_exp[j]);
+      if (fine)
+        k_solve_convert<tf><<<cdiv(nl, 256), 256, 0, st>>>(nl, scale[j], t[j], (tf *)o);
+      else
+        k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, scale[j], t[j], (df *)o);
+      c[j] = o;
+      p->n_launch += 1;
     }
     A.e2 = c[0];
     A.b2 = c[1];
+    unit = 2 * p->sep_exp[0] + p->sep_exp[1];
   } else {
-    fac = reinterpret_cast<double *>(take(fb));
-    char *f = fp64 ? reinterpret_cast<char *>(fac) : take(fb);
-    const int m = cdiv(std::max(nk, 2 * nw - 1), 256);
-    if (fp64)
-      k_solve_factors<double><<<m, 256, 0, st>>>(nk, nw, sk, sw, fac, fac);
+    fac = reinterpret_cast<double *>(take(db));
+    char *f = take(fb);
+    const int m = cdiv(std::max(nk, 2 * nw - 1), 64);
+    const tf isk = inv_square(sk), isw = inv_square(sw);
+    if (fine)
+      k_solve_factors<tf><<<m, 64, 0, st>>>(nk, nw, sk, sw, isk, isw, fac, (tf *)f);
     else
-      k_solve_factors<df><<<m, 256, 0, st>>>(nk, nw, sk, sw, fac, reinterpret_cast<df *>(f));
+      k_solve_factors<df><<<m, 64, 0, st>>>(nk, nw, sk, sw, isk, isw, fac, (df *)f);
     p->n_launch += 1;
     A.aK = f;
-    A.bK = f + (size_t)nk * 8;
-    A.aW = f + (size_t)2 * nk * 8;
-    A.bW = f + (size_t)(2 * nk + 2 * nw - 1) * 8;
+    A.bK = f + (size_t)nk * es;
+    A.aW = f + (size_t)2 * nk * es;
+    A.bW = f + (size_t)(2 * nk + 2 * nw - 1) * es;
   }
-  if (fp64)
-    k_tx_twiddles<double2><<<cdiv(ntw, 256), 256, 0, st>>>(lk, lm, (double2 *)tw, vk, vm);
+  if (fine)
+    k_tx_twiddles<tf2><<<cdiv(ntw, 64), 64, 0, st>>>(lk, lm, (tf2 *)tw, vk, vm);
   else
     k_tx_twiddles<df2><<<cdiv(ntw, 256), 256, 0, st>>>(lk, lm, (df2 *)tw, vk, vm);
   A.target = target;
-  A.X = x * p->dkdw;
+  A.X = std::ldexp(x * p->dkdw, unit);
   A.w = target > 0.0 ? 0.75 : 1.0;
   A.tol = tol;
   if (from) {
     k_solve_prolong<<<cdiv(nl, 256), 256, 0, st>>>(nk, nw, fk, fw, from->nk, from->nw, from->sb2,
                                                    g64);
-    if (fp64)
-      k_solve_convert<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (double *)A.s[3]);
+    if (fine)
+      k_solve_convert<tf><<<cdiv(nl, 256), 256, 0, st>>>(nl, 1.0, g64, (tf *)A.s[3]);
     else
-      k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, g64, (df *)A.s[3]);
+      k_solve_convert<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, 1.0, g64, (df *)A.s[3]);
     A.warm = 1;
     A.hold = from == p ? 0 : hold;
     p->n_launch += 2;
@@ -1449,10 +1448,12 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   RecOccupancy occ;
   if (int rc = rec_occupancy(p->device, &occ)) return rc;
   SolveCtl *h = reinterpret_cast<SolveCtl *>(reinterpret_cast<char *>(p->h_pinned) + kPinCtlOff);
-  const int low = p->mixed ? 0 : 1;  // (with difference pairs no point has few)
+  // direct sums: not with difference pairs (no point has few), nor for the first
+  // iterate of a triple-float solve (59 us on 256 x 128)
+  const int low = p->mixed || (p->sep && !fine) ? 0 : 1;
   auto final = [&](int nit, int stage) {
-    if (fp64)
-      k_solve_final<double><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, nit, stage, low, g64, p->sb2, p->qm);
+    if (fine)
+      k_solve_final<tf><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, nit, stage, low, g64, p->sb2, p->qm);
     else
       k_solve_final<df><<<cdiv(nl, 256), 256, 0, st>>>(nl, A, nit, stage, low, g64, p->sb2, p->qm);
   };
@@ -1462,13 +1463,13 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   // converged solve's later launches return at once): mixed ones (Gaussian
   // envelope) to the loose or the tight change; of separable bispectra, damped
   // ones from scratch or a coarser lattice, or from this lattice's own solution
-  const int first = !p->sep ? (tol >= kSolveLoose ? 12 : 15)
-                            : from == p ? (target > 0.0 ? 12 : 6) : 16;
-  A.accept = std::max(tol, fp64 ? kSolveAcceptF64 : kSolveAcceptDf);
+  const int first = !p->sep ? (tol >= kSolveLoose ? 12 : from == p ? 9 : 15)
+                            : from == p ? 12 : 16;
+  A.accept = std::max(tol, fine ? kSolveExact : kSolveAcceptDf);
   do {
     const int upto = std::min(kSolveMaxIt, nit + (nit == 0 ? first : p->sep ? 5 : 3));
     for (; nit < upto; ++nit) {
-      const int rc = fp64 ? solve_iterate_f64(A, nit, p->device, occ.nsm, st)
+      const int rc = fine ? solve_iterate_tf(A, nit, p->device, occ.nsm, st)
                           : solve_iterate_df(A, nit, p->device, occ.nsm, st);
       if (rc) return rc;
     }
@@ -1477,7 +1478,8 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
     final(nit, 1);
     if (low)
       k_solve_low<<<nlow, 256, 0, st>>>(
-          A, p->sep ? p->env_e2 : nullptr, p->sep ? p->env_b2 : nullptr, fac, p->qm, g64);
+          A, p->sep ? p->env_e2 : nullptr, p->sep ? p->env_b2 : nullptr, scale[0], scale[1], fac,
+          p->qm, g64);
     final(nit, 2);
     SRM3_CUDA(cudaGetLastError());
     SRM3_CUDA(cudaMemcpyAsync(h, A.ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
@@ -1486,7 +1488,7 @@ static int solve_lattice(srm3_plan *p, cudaStream_t st, double target, double x,
   } while (!h->converged && nit < kSolveMaxIt && !solve_stalled(h, nit));
   p->n_launch += 1 + 3 * nit + 2 + low;
   r->converged = h->converged != 0 && h->X >= 0.0 && std::isfinite(h->X);
-  r->x = h->X / p->dkdw;
+  r->x = std::ldexp(h->X, -unit) / p->dkdw;
   std::memcpy(&r->max_sb2, &h->max_sb2, sizeof(double));
   double gm, hm, bm;
   std::memcpy(&gm, &h->gmax, sizeof(gm));
@@ -2005,6 +2007,7 @@ static int coarse_root(srm3_plan *p, cudaStream_t st, double target, double *xc,
   c.rec_sep = p->rec_sep;
   c.sep = p->sep;
   c.sigma_g = p->sigma_g;
+  std::copy(p->sep_exp, p->sep_exp + 2, c.sep_exp);
   c.solve = p->solve;
   c.h_pinned = p->h_pinned;
   c.h_err = p->h_err;
@@ -2134,12 +2137,12 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
     std::memset(&r, 0, sizeof(r));
     auto run = [&](const srm3_plan *from, int fk, int fw) {
       const double sk = p->sigma_g * p->nk, sw = p->sigma_g * p->nw;
-      const bool f64 = p->sep;  // separable bispectra: finished in FP64
+      const bool f64 = p->sep;  // separable bispectra: to FP64's accuracy
       int rc1 = solve_lattice(p, st, target, from ? from->eps * from->eps : 0.0, sk, sw, false,
                               tables && !f64 ? kSolveDf : kSolveLoose, from, fk, fw, &r);
       if (!rc1 && f64 && r.converged) {
         if (cudaEventRecord(t_ev[2], st) == cudaSuccess) finish = true;
-        rc1 = solve_lattice(p, st, target, 0.0, sk, sw, true, kSolveF64, p, 1, 1, &r);
+        rc1 = solve_lattice(p, st, target, 0.0, sk, sw, true, kSolveTf, p, 1, 1, &r);
       }
       return rc1;
     };
@@ -2160,7 +2163,7 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
       p->lattice_solve = true;
       p->root_passes32 += 1;
       p->coarse_start = xc > 0.0 && std::fabs(xc - r.x) <= kCoarseWindow * r.x;
-      if (tables && (p->precision == SRM3_FP32 || r.change <= kSolveExact)) {
+      if (tables && (!p->sep || r.change <= kSolveExact)) {
         p->root_passes += 1;
         p->eps = std::sqrt(r.x);
         p->max_sb2 = r.max_sb2;
@@ -2700,7 +2703,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
       if (rc) return rc;
       SRM3_CUDA(cudaEventRecord(t_ev[1], st));
       if (sr.converged && !sr.err &&
-          (rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveF64, p, 1, 1, &sr)))
+          (rc = solve_lattice(p, st, 0.0, x, 0.0, 0.0, true, kSolveTfEps, p, 1, 1, &sr)))
         return rc;
       SRM3_CUDA(cudaEventRecord(t_ev[2], st));
       SRM3_CUDA(cudaEventSynchronize(t_ev[2]));
@@ -2710,8 +2713,7 @@ int build_plan(srm3_plan *p, const srm3_spectrum *sp, const srm3_bispectrum *bs)
       p->t_rec32_ms += ms32;
       p->t_rec64_ms += ms64;
       // a solve that met sums of 1 or close to it leaves the verdict to the level pass
-      done = sr.converged && !sr.err &&
-             (p->precision == SRM3_FP32 || sr.change <= kSolveExact);
+      done = sr.converged && !sr.err && sr.change <= kSolveExact;
       if (done) {
         r.max_sb2 = sr.max_sb2;
         r.min_pure = 1.0 - sr.max_sb2;
@@ -2979,16 +2981,22 @@ SRM3_API int srm3_plan_create(const srm3_spectrum *spectrum, const srm3_bispectr
   } else {
     return fail(SRM3_ERR_INVALID_ARG, "unknown spectrum kind");
   }
+  double env_max[2] = {0.0, 0.0};
   if (bispectrum->kind == SRM3_BISPECTRUM_GAUSS_ENVELOPE) {
     if (!(bispectrum->sigma_g > 0.0)) return fail(SRM3_ERR_INVALID_ARG, "sigma_g must be > 0");
   } else if (bispectrum->kind == SRM3_BISPECTRUM_SEPARABLE) {
     if (!bispectrum->env_table) return fail(SRM3_ERR_INVALID_ARG, "env_table is NULL");
-    for (const double *t : {bispectrum->env_table, bispectrum->env_table_b}) {
+    const double *t2[2] = {bispectrum->env_table, bispectrum->env_table_b};
+    for (int j = 0; j < 2; ++j) {
+      const double *t = t2[j];
       if (!t) continue;
-      for (size_t i = 0; i < (size_t)g.n_kappa * g.n_omega; ++i)
+      for (size_t i = 0; i < (size_t)g.n_kappa * g.n_omega; ++i) {
         if (!(t[i] >= 0.0) || !std::isfinite(t[i]))
           return fail(SRM3_ERR_INVALID_ARG, "env_table and env_table_b must be finite and >= 0");
+        env_max[j] = std::max(env_max[j], t[i]);
+      }
     }
+    if (!t2[1]) env_max[1] = env_max[0];
   } else {
     return fail(SRM3_ERR_INVALID_ARG, "unknown bispectrum kind");
   }
@@ -3052,6 +3060,10 @@ SRM3_API int srm3_plan_create(const srm3_spectrum *spectrum, const srm3_bispectr
     const int most = p->precision == SRM3_FP64 && !p->sep ? kMaxFft / 2 : kMaxFft;
     p->solve = (p->sep || E <= kSepExpMax) && 2 * g.n_kappa - 1 <= kMaxFft / 2 && padw <= kMaxFft;
     p->conv = p->sep || (E <= kSepExpMax && 2 * g.n_kappa - 1 <= most && padw <= most);
+  }
+  for (int j = 0; j < 2 && p->sep; ++j) {
+    std::frexp(env_max[j], &p->sep_exp[j]);
+    p->sep_exp[j] *= 2;
   }
   p->beta = bispectrum->beta;
   p->table_budget = g.table_budget_bytes > 0 ? g.table_budget_bytes : 64.0 * (1ull << 30);

@@ -43,9 +43,12 @@
 // largest pair sums, and a point multiplies it by b_k^2 / b^2 there: for the
 // Gaussian envelope, centred at a quarter of the lattice as in conv.cuh, at
 // most e^{E/4} (e^8 for sigma_g = 0.25) at the lattice's corners.  In
-// double-float (the search of FP32 and FP64 plans) s is good to ~1e-11 there and
-// 1e-14 in the middle, in FP64 (separable bispectra) to ~1e-13.  The points
-// with few pairs, whose sums are small, are summed directly at the end
+// double-float (the search, and the tables of FP32 plans with the Gaussian
+// envelope) s is good to ~1e-11 there and 1e-14 in the middle; where tables were
+// those of FP64 passes the solve finishes in triple-float, whose rounding is below
+// FP64's everywhere.  (In FP64, which takes the FP64 pipe longer, the sums of the
+// wind-field envelope were off by 2.7e-14 on 256 x 128, and by 9e-13 on 486 x 202.)
+// The points with few pairs, whose sums are small, are summed directly at the end
 // (k_solve_low), which keeps them accurate relative to themselves.
 #pragma once
 
@@ -67,8 +70,8 @@ constexpr double kSolveClip = 0.99, kSolveTop = 0.9899;
 // rounding itself.  A solve counts where X max b^2 sum h^2 stays below kSolveSpread
 // (double-float, Gaussian envelope: 3e4 at most on full lattices and on ones with
 // nine of ten points empty, sigma_g >= 0.2237) or kSolveSpreadSep (separable
-// tables, finished in FP64: 3 times the number of points); where X comes from
-// rounding alone it is 2^36 and above.
+// tables, finished in triple-float: 3 times the number of points); where X comes
+// from rounding alone it is 2^36 and above.
 constexpr double kSolveSpread = 0x1p22, kSolveSpreadSep = 0x1p26;
 constexpr double kSolveH2Unit = 0x1p-24;
 
@@ -115,9 +118,9 @@ __device__ __forceinline__ double as_double(unsigned long long b) {
 }
 // Whether iteration it was the last that counts: its change within tol, or
 // within accept and no longer falling (the transform's rounding: it keeps the
-// sums of some bispectra moving by a few 1e-13 in FP64 and 1e-11 in
-// double-float, at points of large b_k^2, which are summed directly at the
-// end).  The words of skipped iterations stay 0.
+// sums of some bispectra moving by a few 1e-11 in double-float, at points of large
+// b_k^2, which are summed directly at the end).  The words of skipped iterations
+// stay 0.
 __device__ __forceinline__ bool solve_last(const SolveArgs &A, int it) {
   if (it < A.hold + 1) return false;
   const double c = as_double(A.ctl->chg[it]);
@@ -155,29 +158,44 @@ __device__ __forceinline__ F solve_b2(const SolveArgs &A, int kk, int kw) {
 // kernels, with s, g and h in FP64, spent 25 us a launch on a 32 x 32 lattice.
 // q from s: 1/(1 - s), s kept below kSolveClip while the iterations are on their
 // way; a fixed point that reaches it is not Eq. pure's (kSolveTop).
-__device__ __forceinline__ double solve_q(double s) { return 1.0 / (1.0 - fmin(s, kSolveClip)); }
 __device__ __forceinline__ df solve_q(df s) {
   const df d = s.h < (float)kSolveClip ? df(1.0f, 0.0f) - s : df(1.0 - kSolveClip);
   const float r = __frcp_rn(d.h);  // one Newton step on it: error r (1 - d r)^2
   const float e = __fmaf_rn(-d.l, r, __fmaf_rn(-d.h, r, 1.0f));
   return df(r, __fmul_rn(r, e));
 }
-__device__ __forceinline__ double solve_num(float v, double) { return v; }
+__device__ __forceinline__ tf solve_q(tf s) {
+  const tf one(1.0f, 0.0f, 0.0f), d = s.h < (float)kSolveClip ? one - s : tf(1.0 - kSolveClip);
+  const tf r0(__frcp_rn(d.h), 0.0f, 0.0f);  // two Newton steps
+  const tf r1 = r0 + r0 * (one - d * r0);
+  return r1 + r1 * (one - d * r1);
+}
 __device__ __forceinline__ df solve_num(float v, df) { return df(v, 0.0f); }
-__device__ __forceinline__ double solve_real(double v) { return v; }
+__device__ __forceinline__ tf solve_num(float v, tf) { return tf(v, 0.0f, 0.0f); }
 __device__ __forceinline__ double solve_real(df v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double solve_real(tf v) {
+  return (double)v.h + ((double)v.m + (double)v.l);
+}
 // v, 0 if negative, its parts not overlapping (so that h orders first)
-__device__ __forceinline__ double solve_clip(double v) { return v < 0.0 ? 0.0 : v; }
 __device__ __forceinline__ df solve_clip(df v) {
   const float h = __fadd_rn(v.h, v.l), l = __fsub_rn(v.l, __fsub_rn(h, v.h));
   return h > 0.0f ? df(h, l) : df(0.0f, 0.0f);
 }
-__device__ __forceinline__ double solve_max(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ tf solve_clip(tf v) {
+  float t, e, m, l;
+  t = two_sum(v.m, v.l, e);
+  const float h = two_sum(v.h, t, m);
+  m = two_sum(m, e, l);
+  return h > 0.0f ? tf(h, m, l) : tf(0.0f, 0.0f, 0.0f);
+}
 __device__ __forceinline__ df solve_max(df a, df b) {
   return (b.h > a.h || (b.h == a.h && b.l > a.l)) ? b : a;
 }
-__device__ __forceinline__ float solve_abs(double v) { return (float)fabs(v); }
+__device__ __forceinline__ tf solve_max(tf a, tf b) {
+  return (b.h > a.h || (b.h == a.h && (b.m > a.m || (b.m == a.m && b.l > a.l)))) ? b : a;
+}
 __device__ __forceinline__ float solve_abs(df v) { return fabsf(v.h + v.l); }
+__device__ __forceinline__ float solve_abs(tf v) { return fabsf(v.h + (v.m + v.l)); }
 
 __device__ __forceinline__ void warp_atomic_max(unsigned long long *p, double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));

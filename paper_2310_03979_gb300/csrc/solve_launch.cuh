@@ -1,6 +1,6 @@
 // solve_launch.cuh - one iteration of the whole-lattice solve of Eq. pure
 // (kernels in solve.cuh) for one number type; one translation unit per type
-// instantiates it (solve_df.cu, solve_f64.cu).
+// instantiates it (solve_df.cu, solve_tf.cu).
 #pragma once
 
 #include <algorithm>
@@ -72,8 +72,8 @@ int solve_iterate(SolveArgs A, int it, int device, int nsm, cudaStream_t st) {
   A.rows = std::min(most, std::max(1, (A.nk + nsm - 1) / nsm));
   const int rthreads = (A.rows * tpt + 31) / 32 * 32, rb = rthreads / tpt;
   const size_t srow = (size_t)rb * (tx_len(A.M) + 1) * sizeof(T2);
-  const size_t sout = srow + (A.mixed ? (size_t)rthreads * 8 : 0);
-  const int wf = (int)(128 / sizeof(T2));
+  const size_t sout = srow + (A.mixed ? (size_t)rthreads * sizeof(typename RealOf<T2>::type) : 0);
+  const int wf = sizeof(T2) == 24 ? 4 : (int)(128 / sizeof(T2));
   const int pairs = A.M / 2 + 1;
   int TC = 2;
   while (TC > 1 && ((pairs + TC - 1) / TC < 2 * nsm || 2 * TC * solve_tpt(lk) > solve_col_threads(lk)))

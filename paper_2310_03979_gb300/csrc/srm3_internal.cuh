@@ -119,6 +119,7 @@ struct srm3_plan {
   // Eq. pure on the whole lattice by self-convolutions (solve.cuh) where the
   // envelope factors and the grid fits; the plan's tables come from it
   bool solve = false;
+  int sep_exp[2] = {0, 0};      // separable tables: powers of two at the maxima of a^2, b^2
   bool q_warm = false;          // qm holds a solution near the next pass's x
   bool iter_off = false;        // direct iterations were too slow: level passes
   // mixed-sign interactions: opposite-sheet pairs as well; Eq. pure then

@@ -229,3 +229,33 @@ def test_info_says_where_the_tables_come_from(precision):
     for narrow in (replace(wl, target=0.995), replace(wl, sigma_g=0.15)):
         with srm3.Plan.create(narrow) as p:
             assert not p.info().recursion_flags & srm3.SRM3_REC_LATTICE_SOLVE
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("nk,nw,envelope,eps", [(256, 128, "sum", 50.0), (94, 603, "sum", 63.0),
+                                                (128, 256, "separable", 1.5)])
+def test_separable_tables_at_a_given_eps_keep_fp64_rounding(oracle_lib, precision, nk, nw, envelope,
+                                                           eps):
+    """Tables of either precision's plans are FP64's.  Level passes are 1e-15 to 3e-15
+    from the oracle here (a sum of some 1e4 pairs, rounded in another order)."""
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=512, nt=2048, precision=precision), envelope=envelope)
+    ta, tb = wl.envelope_tables()
+    with srm3.Plan.create(wl, eps=eps) as p:
+        S, q, sb2 = p.tables()
+    ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=eps,
+                           env=oracle.Envelope("separable", table=ta, table_b=tb))
+    assert 0.01 < ref.sum_b2.max() < 0.5
+    assert np.abs(sb2 - ref.sum_b2).max() <= 5e-15
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e-9, 1e9, 1e25])
+def test_separable_tables_of_any_magnitude(oracle_lib, scale):
+    """Tables far outside FP32's range: eps alone answers for their magnitude."""
+    wl = replace(W.small_case(nk=24, nw=20), envelope="separable")
+    S = oracle.kaimal_lorentzian(24, 20, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    with srm3.Plan.create(wl, table=S) as p:
+        one = p.tables()[2]
+        eps = p.info().eps
+    with srm3.Plan.create(_Tables(wl, scale * wl.envelope_table()), table=S) as p:
+        np.testing.assert_allclose(p.tables()[2], one, rtol=1e-12, atol=1e-18)
+        assert p.info().eps == pytest.approx(eps / scale ** 3, rel=1e-12)
