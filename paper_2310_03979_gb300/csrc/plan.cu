@@ -1653,9 +1653,14 @@ static int illinois(srm3_plan *p, cudaStream_t st, double target, double tol, in
 // <= 1/(1 - target) below the root); Illinois regula falsi between them,
 // each evaluation warm-started from the largest x found below the target.
 //
-// Where the whole-lattice solve applies (solve.cuh, on the signed omega axis),
-// FP32 plans take its tables, and FP64 plans start from its root and solution:
-// secant steps of a few warm iterations each.
+// Where the whole-lattice solve applies (solve.cuh, on the signed omega axis), the
+// search starts from its root and solution: secant steps of a few warm iterations
+// each (FP32 plans: one, which makes the tables FP64's fixed point).  On lattices
+// past kIterFinish FP32 plans take the tables of a triple-float solve instead (plan
+// and all, the steps / the solve, ms: 24 x 37 0.84 / 1.25, 40 x 70 1.23 / 1.32, 100 x 90
+// 3.4 / 1.3).
+constexpr double kIterFinish = 4e6;  // products of an iteration
+
 static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double tol) {
   const long long nl = (long long)p->nk * p->nw;
   PassResult r;
@@ -1679,10 +1684,25 @@ static int find_eps_mixed(srm3_plan *p, cudaStream_t st, double target, double t
       r.max_sb2 = sr.max_sb2;
       r.min_pure = 1.0 - sr.max_sb2;
       r.sumS = p->sumS;
-      if (p->precision == SRM3_FP32) {
-        p->fp_iters = sr.its;
-        p->root_passes += 1;
-        done = true;
+      if (p->precision == SRM3_FP32 && iter_products(p, 1) > kIterFinish) {
+        float ms64 = 0.f;
+        SRM3_CUDA(cudaEventRecord(t_ev[0], st));
+        if ((rc = solve_lattice(p, st, target, 0.0, p->sigma_g * p->nk, p->sigma_g * p->nw, true,
+                                kSolveTf, p, 1, 1, &sr)))
+          return rc;
+        SRM3_CUDA(cudaEventRecord(t_ev[1], st));
+        SRM3_CUDA(cudaEventSynchronize(t_ev[1]));
+        SRM3_CUDA(cudaEventElapsedTime(&ms64, t_ev[0], t_ev[1]));
+        p->t_recursion_ms += ms64;
+        p->t_rec64_ms += ms64;
+        if (sr.converged && !sr.err && sr.change <= kSolveExact) {
+          x = sr.x;
+          r.max_sb2 = sr.max_sb2;
+          r.min_pure = 1.0 - sr.max_sb2;
+          p->fp_iters = sr.its;
+          p->root_passes += 1;
+          done = true;
+        }
       }
       for (int it = 0; it < 8 && !done; ++it) {
         if ((rc = solve_mixed(p, st, x, &r))) return rc;

@@ -259,3 +259,16 @@ def test_separable_tables_of_any_magnitude(oracle_lib, scale):
     with srm3.Plan.create(_Tables(wl, scale * wl.envelope_table()), table=S) as p:
         np.testing.assert_allclose(p.tables()[2], one, rtol=1e-12, atol=1e-18)
         assert p.info().eps == pytest.approx(eps / scale ** 3, rel=1e-12)
+
+
+@pytest.mark.parametrize("nk,nw", [(12, 11), (40, 70), (100, 90)])
+def test_fp32_mixed_tables_are_the_fp64_fixed_point(oracle_lib, nk, nw):
+    """Tables of FP32 plans with mixed interactions at their own eps: FP64's fixed
+    point, as those of FP64 plans (some 1e4 pairs a sum, iterated: 1e-14)."""
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=pow2(nk), nt=pow2(2 * nw)), interactions="mixed")
+    with srm3.Plan.create(wl) as p:
+        S, q, sb2 = p.tables()
+        info = p.info()
+    assert abs(info.max_sum_b2 - wl.target) <= 1e-9
+    ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps, mixed=True)
+    assert np.abs(sb2 - ref.sum_b2).max() <= 3e-14
