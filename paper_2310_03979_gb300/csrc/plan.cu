@@ -2145,6 +2145,8 @@ static int find_eps(srm3_plan *p, cudaStream_t st, double target, double tol) {
   Search32 s;
   s.pts.push_back({0.0, -target});
   p->coarse_start = false;
+  // sums close to 1 take the direct iterations 30 steps and more
+  if (target >= kSolveTop) p->iter_off = iter_most(p, 1, 0) < 48;
   double xs = -1.0;  // the root, from the whole-lattice solve
   if (p->solve && target < kSolveTop) {
     if (p->w_deferred) {  // the W table beside it
