@@ -6,7 +6,7 @@
 // One pass over the values per call, HBM-bound: every CTA of a fixed grid
 // walks 16-byte vectors in a grid-stride loop, four vectors per thread per
 // step.  FP32 input is summed in FP32 over the 16 values of a step, and those
-// sums of the powers of d = u - shift in double-float per thread (StatAcc), FP64
+// sums of the powers of d = u - shift in triple-float per thread (StatAcc), FP64
 // input in FP64 throughout; the threads' sums meet in FP64.  Bins are b =
 // floor((u - lo) * (nbins / (hi - lo))) in the input's precision, each operation
 // rounded once; b < 0 counts below, b >= nbins (or a NaN) above, as two extra
@@ -77,8 +77,8 @@ __device__ __forceinline__ int stat_slot(T u, T lo, T scale, int nbins) {
 }
 
 // A thread's running power sums over its steps.  FP64 input: FP64.  FP32 input:
-// double-float (a two-sum of the high part, its error in the low part: 48
-// bits, against the 24 of a step's own sum), as four FP64 additions and
+// three FP32 numbers (two-sums of the first and the second, their errors in the
+// next: 72 bits, more than FP64's 53), as four FP64 additions and
 // conversions a step kept this part's FP64 pipe (2 lanes per SM and clock) busy
 // for most of the pass.  1.05e8 values, reset and read included: 159 -> 132 us
 // (121 us with the CTAs' sums merged by the last CTA in place of a launch, and one
@@ -98,12 +98,12 @@ struct StatAcc {
 template <>
 struct StatAcc<float> {
   double a[4] = {0.0, 0.0, 0.0, 0.0};
-  float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+  float h[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
   __device__ __forceinline__ void flush() {
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-      a[p] += (double)h[p] + (double)l[p];
-      h[p] = l[p] = 0.f;
+      a[p] += (double)h[p] + ((double)m[p] + (double)l[p]);
+      h[p] = m[p] = l[p] = 0.f;
     }
   }
   __device__ __forceinline__ void add(float s1, float s2, float s3, float s4) {
@@ -117,9 +117,10 @@ struct StatAcc<float> {
     }
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-      float e;
+      float e, f;
       h[p] = two_sum(h[p], s[p], e);
-      l[p] = __fadd_rn(l[p], e);
+      m[p] = two_sum(m[p], e, f);
+      l[p] = __fadd_rn(l[p], f);
     }
   }
 };

@@ -158,3 +158,18 @@ def test_stats_sums_past_the_range_of_a_float(big):
             assert abs(got - exact) <= 2e-6 * float((d.abs() ** (p + 1)).sum())
         else:  # the step's own FP32 sum overflows, as it always did
             assert got == math.inf
+
+
+def test_running_sums_keep_fp64_precision():
+    """One thread's steps hold 2^25, 1/2 + 2^-24 and 2^-27 (a step takes four 16-byte
+    vectors of each of 1024 threads per SM), all other values are zero: the sum
+    spans FP64's 53 bits and is exact in them."""
+    nth = 4 * 256 * torch.cuda.get_device_properties(0).multi_processor_count
+    u = torch.zeros(3 * 16 * nth, dtype=torch.float32, device="cuda")
+    parts = (2.0 ** 25, 0.5 + 2.0 ** -24, 2.0 ** -27)
+    for k, v in enumerate(parts):
+        u[16 * nth * k] = v
+    with srm3.Stats(8, -1.0, 1.0) as st:
+        st.add(u)
+        res = st.read()
+    assert res["power_sum"][0] == sum(parts)
