@@ -29,6 +29,18 @@ __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
   return r;
 }
 
+// The same with each component rounded once or so: the error of one product goes
+// into the sum (Kahan's difference of products).
+template <typename T2>
+__device__ __forceinline__ T2 cmul_acc(T2 a, T2 b) {
+  using T = decltype(a.x);
+  const T p = a.y * b.y, q = a.y * b.x;
+  T2 r;
+  r.x = fma(a.x, b.x, -p) + fma(-a.y, b.y, p);
+  r.y = fma(a.x, b.y, q) + fma(a.y, b.x, -q);
+  return r;
+}
+
 // One radix-2 butterfly: (a, b) <- (a + w b, a - w b).
 template <typename T2>
 __device__ __forceinline__ void bfly(T2 &a, T2 &b, T2 w) {
@@ -419,7 +431,17 @@ __device__ __forceinline__ void stockham_pass(int L, int Ns, int tpt, int jt,
         T2 w[R];
         load_tw<R>(twp + (j & (Ns - 1)) * R, w);
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[it][r] = cmul(v[it][r], w[r]);
+        for (int r = 1; r < R; ++r) {
+          if constexpr (kPlainNum<T2>) {
+            // passes of small radix multiply by more twiddles: rounded once, they
+            // leave no more than plans of radix 16 do
+            if (L <= (sizeof(T2) == 16 ? 256 : 64)) {
+              v[it][r] = cmul_acc(v[it][r], w[r]);
+              continue;
+            }
+          }
+          v[it][r] = cmul(v[it][r], w[r]);
+        }
       }
       dft_inv<R, FIRST ? VMASK : tx_in_mask(R, 0)>(v[it]);
     }
@@ -497,16 +519,20 @@ inline int tx_nz(int l, int n, bool fp32) {
 }
 
 // log2 of the values a thread holds of a length-2^l output transform: 16 where
-// the first pass is pruned (its radix of 16 skips more of the zero blocks), else
-// 8, and 4 in short transforms, whose passes are bound by the latency of a
-// thread's own instructions.  Measured with 16 values / this rule, in us: 64
+// the first pass is pruned (its radix of 16 skips more of the zero blocks) and in
+// FP64 ones past 512 (a pass fewer, and its roundings), else 8 (4 up to length 16):
+// short transforms' passes are bound by the latency of a thread's own instructions.
+// (4 up to length 64 took a pass more, whose roundings showed: fields of 64 x 64
+// off by 1.23e-7 of their norm against 1.21e-7.)  Measured with 16 values / this rule, in us: 64
 // fields of 512 x 1024 206 / 165, 16 of 1024 x 2048 244 / 187, one FP64 64 x 64 35 /
 // 17, 16 FP64 512 x 1024 576 / 554; 50 of 1024 x 2048 from 256 x 128 (pruned)
 // 177, with 8 values 210.
-__host__ __device__ constexpr int out_lv(int l, int nz) {
-  return nz > 0 ? 4 : l <= 6 ? 2 : l <= 12 ? 3 : 4;
+__host__ __device__ constexpr int out_lv(int l, int nz, bool fp64) {
+  return nz > 0 ? 4 : l <= 4 ? 2 : l <= (fp64 ? 9 : 12) ? 3 : 4;
 }
-__host__ __device__ constexpr int out_tpt(int l, int nz) { return tx_tpt(1 << l, out_lv(l, nz)); }
+__host__ __device__ constexpr int out_tpt(int l, int nz, bool fp64) {
+  return tx_tpt(1 << l, out_lv(l, nz, fp64));
+}
 
 // Stage 1: TC columns m0 + c of one coefficient set per CTA (blockIdx.y =
 // set), thread (c, jt) = (t mod TC, t / TC); TC consecutive columns make the
@@ -520,7 +546,7 @@ __global__ void __launch_bounds__(512) k_tx_cols(int nk, int nw, int TC, int col
                                                   T2 *__restrict__ G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using T = decltype(T2::x);
-  constexpr int L = 1 << LOG2NX, LV = out_lv(LOG2NX, NZ);
+  constexpr int L = 1 << LOG2NX, LV = out_lv(LOG2NX, NZ, sizeof(T2) == 16);
   const int n = blockIdx.y;
   const int c = threadIdx.x & (TC - 1), jt = threadIdx.x / TC;
   const int m = blockIdx.x * TC + c;
@@ -561,7 +587,7 @@ __global__ void __launch_bounds__(512) k_tx_cols(int nk, int nw, int TC, int col
     if (live) Gn[(size_t)i * nw + m] = v;
   };
   stockham_passes<LOG2NX, 0, tx_mask_ends<LOG2NX, LV>(NZ), false, false, false, LV>(
-      1, 0, out_tpt(LOG2NX, NZ), jt, twp, col, src, dst);
+      1, 0, out_tpt(LOG2NX, NZ, sizeof(T2) == 16), jt, twp, col, src, dst);
 }
 
 // Stage 2: RB rows mx of one set per CTA, thread (row, jt) = (t / tpt,
@@ -573,7 +599,8 @@ __global__ void __launch_bounds__(512) k_tx_rows(int nx, int nw, int rowstride,
                                                  const T2 *__restrict__ twp,
                                                  const T2 *__restrict__ twz, T *__restrict__ u) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int M = 1 << LOG2M, tpt = out_tpt(LOG2M, NZ), LV = out_lv(LOG2M, NZ);
+  constexpr int M = 1 << LOG2M, tpt = out_tpt(LOG2M, NZ, sizeof(T2) == 16),
+                LV = out_lv(LOG2M, NZ, sizeof(T2) == 16);
   const int n = blockIdx.y;
   const int row = threadIdx.x / tpt, jt = threadIdx.x & (tpt - 1);
   const int rb = blockDim.x / tpt, mx = blockIdx.x * rb + row;

@@ -2834,8 +2834,8 @@ int prepare_shape_tables(srm3_plan *p, cudaStream_t st) {
   p->rowstride = nw + 2 * kPad;  // y row length, workspace or batch buffers
   SRM3_CUDA(dev_alloc(&p->Ek, nk * es, st));
   SRM3_CUDA(dev_alloc(&p->Ews, p->ew_len * es, st));
-  const int ox = out_lv(p->log2nx, tx_nz(p->log2nx, nk, f32));
-  const int ot = out_lv(p->log2nt - 1, tx_nz(p->log2nt - 1, nw, f32));
+  const int ox = out_lv(p->log2nx, tx_nz(p->log2nx, nk, f32), !f32);
+  const int ot = out_lv(p->log2nt - 1, tx_nz(p->log2nt - 1, nw, f32), !f32);
   const int tw_n = tx_twlen(p->log2nx, ox) + tx_twlen(p->log2nt - 1, ot) + p->nt / 2;
   SRM3_CUDA(dev_alloc(&p->tw, (size_t)tw_n * 2 * es, st));
   if (f32) {

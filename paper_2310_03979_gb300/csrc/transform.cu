@@ -30,7 +30,7 @@ TxShape tx_shape(const srm3_plan *p, size_t e2, int n) {
   const int wf = (int)(128 / e2);  // lanes of one shared-memory wavefront
   TxShape s{};
   const int L = p->nx, M = p->nt / 2;
-  const int tptx = out_tpt(p->log2nx, tx_nz(p->log2nx, p->nk, e2 == 8));
+  const int tptx = out_tpt(p->log2nx, tx_nz(p->log2nx, p->nk, e2 == 8), e2 == 16);
   int TC = 16;
   while (TC > 1 && TC / 2 >= p->nw) TC >>= 1;
   auto colstride = [&](int tc) {
@@ -46,7 +46,7 @@ TxShape tx_shape(const srm3_plan *p, size_t e2, int n) {
   s.colstride = colstride(TC);
   s.smem1 = (size_t)TC * s.colstride * e2;
   s.rowstride = tx_len(M) + 1;
-  const int tpt = out_tpt(p->log2nt - 1, tx_nz(p->log2nt - 1, p->nw, e2 == 8));
+  const int tpt = out_tpt(p->log2nt - 1, tx_nz(p->log2nt - 1, p->nw, e2 == 8), e2 == 16);
   int rb = std::max(1, 64 / tpt);
   while (rb > 1 && ((size_t)rb * s.rowstride * e2 > cap || rb > p->nx ||
                     (rb * tpt > 32 && (long long)(p->nx / rb) * n < nsm)))
@@ -88,8 +88,8 @@ int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2
   constexpr bool f32 = std::is_same<T, float>::value;
   {
     const int lx = p->log2nx, lt = p->log2nt - 1;
-    tw2 = tw1 + tx_twlen(lx, out_lv(lx, tx_nz(lx, p->nk, f32)));
-    twz = tw2 + tx_twlen(lt, out_lv(lt, tx_nz(lt, p->nw, f32)));
+    tw2 = tw1 + tx_twlen(lx, out_lv(lx, tx_nz(lx, p->nk, f32), !f32));
+    twz = tw2 + tx_twlen(lt, out_lv(lt, tx_nz(lt, p->nw, f32), !f32));
   }
   with_log2<1, 13>(p->log2nx, [&](auto c) {
     constexpr int l = decltype(c)::value;
@@ -98,7 +98,7 @@ int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2
       e = cudaFuncSetAttribute(k_tx_cols<l, T2, nz>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                lim);
       if (e == cudaSuccess) {
-        k_tx_cols<l, T2, nz><<<dim3(cdiv(p->nw, s.TC), n), s.TC * out_tpt(l, nz), s.smem1, st>>>(
+        k_tx_cols<l, T2, nz><<<dim3(cdiv(p->nw, s.TC), n), s.TC * out_tpt(l, nz, !f32), s.smem1, st>>>(
             p->nk, p->nw, s.TC, s.colstride, C, tw1, G);
         e = cudaGetLastError();
       }
@@ -112,7 +112,7 @@ int transform_impl(srm3_plan *p, cudaStream_t st, const T2 *C, int n, T *out, T2
       e = cudaFuncSetAttribute(k_tx_rows<l, T, T2, nz>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (e == cudaSuccess) {
-        k_tx_rows<l, T, T2, nz><<<dim3(p->nx / s.rb, n), s.rb * out_tpt(l, nz), s.smem2, st>>>(
+        k_tx_rows<l, T, T2, nz><<<dim3(p->nx / s.rb, n), s.rb * out_tpt(l, nz, !f32), s.smem2, st>>>(
             p->nx, p->nw, s.rowstride, G, tw2, twz, out);
         e = cudaGetLastError();
       }

@@ -358,3 +358,34 @@ def test_sample_host_matches_device(oracle_lib):
         host = torch.empty((2, 16, 64), dtype=torch.float32).pin_memory()
         srm3.sample_host(p.handle, [7, 8], 2, host.data_ptr())
     np.testing.assert_array_equal(host.numpy(), dev)
+
+
+# Root mean square errors of the fields against extended precision, relative to the
+# field's: those of transforms by passes of radix 16 and 8 (measured, the mean of
+# six random coefficient sets).  Plans with more passes must not exceed them.
+@pytest.mark.parametrize("precision,nk,nw,nx,nt,bound", [
+    ("fp32", 32, 32, 64, 64, 1.2090e-7), ("fp32", 24, 37, 64, 128, 1.1985e-7),
+    ("fp64", 32, 32, 64, 64, 2.1955e-16), ("fp64", 24, 37, 64, 128, 2.2942e-16),
+])
+def test_short_transforms_round_no_more_than_long_radix_passes(precision, nk, nw, nx, nt, bound):
+    ld = np.longdouble
+    pi = ld("3.14159265358979323846264338327950288")
+
+    def cis(n, k):
+        a = 2 * pi * (np.outer(np.arange(n), np.arange(k)) % n).astype(ld) / ld(n)
+        return np.cos(a) + 1j * np.sin(a)
+
+    ex, et = cis(nx, nk), cis(nt, nw)
+    wl = W.small_case(nk=nk, nw=nw, nx=nx, nt=nt, precision=precision)
+    err = []
+    with srm3.Plan.create(wl, eps=1e-3) as p:
+        for seed in range(6):
+            g = torch.Generator().manual_seed(seed)
+            C = torch.randn((1, 2, nk, nw, 2), generator=g, dtype=torch.float64)
+            C = C.to(torch.float32 if precision == "fp32" else torch.float64)
+            u = p.field_from_coeffs(C.cuda()).cpu().numpy()[0].astype(ld)
+            c = C.numpy()[0].astype(np.float64)
+            z = c[..., 0].astype(ld) + 1j * c[..., 1].astype(ld)
+            ref = (ex @ z[0] @ et.T + ex @ z[1] @ et.conj().T).real
+            err.append(float(np.sqrt(((u - ref) ** 2).sum() / (ref ** 2).sum())))
+    assert np.mean(err) <= bound
