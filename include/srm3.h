@@ -497,26 +497,30 @@ int64_t srm3_batch_pair_terms(const srm3_batch *b);
  * them from one plan, on an n_kappa x n_omega lattice with n_t-point rows,
  * y + y0 = (n_kappa (n_omega + 128) + 1) P 8 bytes (P = 2 T sheet-samples
  * rounded up to a multiple of 64), C = 2 T n_kappa n_omega 8, H = m n_kappa
- * n_t 8 and 16 T of factor pointers; plus 8 bytes of seed per sample, the
+ * n_t 8 and 24 T of factor pointers; plus 8 bytes of seed per sample, the
  * plan descriptors and 16 bytes per work unit.  Plans outside shape groups
  * sample on their own workspace, which their srm3_info.device_bytes counts;
  * the caller's output buffers are not included. */
 int64_t srm3_batch_device_bytes(const srm3_batch *b);
 
-/* Cap the batch's FP32 pair-sum launch at max_ctas CTAs, counted as halves of
- * an SM (0: as many as are resident, the default).  The launch is persistent and otherwise fills
- * every SM; a cap leaves room for work on other streams to run beside it
- * (a serving loop keeps short requests moving this way).  Set it before
+/* Cap the batch's FP32 pair sums at max_ctas CTAs, counted as halves of an SM
+ * (0: as many as are resident, the default), so that work on other streams runs
+ * beside a large batch (a serving loop keeps short requests moving this way).
+ * The persistent O(N^2) launch, which otherwise fills every SM, takes that many;
+ * self-convolutions run on the batch stream alone, in launches of as few samples
+ * as those halves hold at a time, one at least: other streams wait for one such
+ * launch, not for the batch.  Results do not depend on it.  Set it before
  * srm3_batch_capture for graph replays. */
 int srm3_batch_set_max_ctas(srm3_batch *b, int max_ctas);
 
-/* on != 0: record CUDA events around the batch's FP32 pair-sum launch in
- * later runs (set it before srm3_batch_capture for graph replays: the
- * events become event-record nodes of the graph). */
+/* on != 0: record CUDA events around the batch's pair sums in later runs, which
+ * then take the batch stream alone, one after another (set it before
+ * srm3_batch_capture for graph replays: the events become event-record nodes of
+ * the graph). */
 int srm3_batch_enable_timing(srm3_batch *b, int on);
 
-/* Duration of the pair-sum launch of the last run, in ms (waits for it);
- * 0 when timing is off or the batch has no FP32 plan. */
+/* Duration of the pair sums of the last run, in ms (waits for them); 0 when timing
+ * is off. */
 int srm3_batch_pairsum_ms(srm3_batch *b, double *ms);
 
 /* Free the batch (not its plans).  NULL is a no-op.  No run may be in flight. */

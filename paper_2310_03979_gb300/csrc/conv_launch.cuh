@@ -76,6 +76,10 @@ int conv_run(const ConvJob &j) {
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
   const int tpt = conv_tpt<T2>(lw), most = std::max(1, 64 / tpt);
+  if (j.max_ctas > 0) {
+    const long long threads = 2LL * p->nk * tpt;  // of one sample's rows
+    per = (int)std::min<long long>(per, std::max<long long>(1, 1024LL * j.max_ctas / threads));
+  }
   const long long allrows = (long long)p->nk * 2 * per;
   const int rows = (int)std::min<long long>(most, std::max<long long>(1, allrows / (4 * nsm)));
   const int rthreads = (rows * tpt + 31) / 32 * 32, rb = rthreads / tpt;

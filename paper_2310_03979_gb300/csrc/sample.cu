@@ -366,7 +366,7 @@ int run_pairsum(srm3_plan *p, int n, void *C_out) {
 
 // The self-convolution of n samples in the plan's workspace.
 static int conv_on(srm3_plan *p, cudaStream_t st, const uint64_t *seeds, const uint64_t *dseeds,
-                   int n, void *C_out) {
+                   int n, void *C_out, int max_ctas = 0) {
   ConvJob j;
   std::memset(&j, 0, sizeof(j));
   j.plan = p;
@@ -377,6 +377,7 @@ static int conv_on(srm3_plan *p, cudaStream_t st, const uint64_t *seeds, const u
   j.work = p->y;
   j.work_bytes = y_bytes(p, sspad_for(p->ws_chunk));
   j.C = C_out;
+  j.max_ctas = max_ctas;
   return conv_sample(j);
 }
 
@@ -529,7 +530,7 @@ struct srm3_batch {
   bool holds_refs = false;        // the plans' batch_refs were raised
   bool timing = false;            // events around the pair-sum launch
   bool capturing = false;         // inside srm3_batch_capture
-  int max_ctas = 0;               // cap on the pair sum's CTAs (0: all resident)
+  int max_ctas = 0;               // cap on the pair sums' CTAs (0: all resident)
   cudaEvent_t ps_ev[2] = {nullptr, nullptr};
   // Self-convolution work that shares no buffer, each shape group and each
   // plan on its own workspace a branch {group or -1, plan, lane}: lane 0 is the
@@ -595,7 +596,8 @@ static int plan_branches(srm3_batch *b) {
 static int branch_coeffs(srm3_batch *b, const srm3_batch::Branch &br, cudaStream_t st) {
   srm3_plan *p = b->plans[br.plan];
   const uint64_t *dseeds = b->dseeds + b->dev_off[br.plan];
-  if (br.group < 0) return conv_on(p, st, nullptr, dseeds, b->counts[br.plan], p->C);
+  if (br.group < 0)
+    return conv_on(p, st, nullptr, dseeds, b->counts[br.plan], p->C, b->max_ctas);
   const srm3_batch::Group &g = b->groups[br.group];
   ConvJob j;
   std::memset(&j, 0, sizeof(j));
@@ -609,6 +611,7 @@ static int branch_coeffs(srm3_batch *b, const srm3_batch::Branch &br, cudaStream
   j.work = g.y;
   j.work_bytes = g.ybytes;
   j.C = g.C;
+  j.max_ctas = b->max_ctas;
   return conv_sample(j);
 }
 
@@ -694,8 +697,9 @@ static int batch_work(srm3_batch *b, bool lanes) {
 }
 
 static int batch_launch(srm3_batch *b) {
-  // with the pair sum timed, everything on the batch stream, the pair sums first
-  const bool lanes = !b->timing && !b->side.empty();
+  // with the pair sum timed, everything on the batch stream, the pair sums first;
+  // a capped batch keeps to that stream too
+  const bool lanes = !b->timing && !b->side.empty() && b->max_ctas == 0;
   if (!lanes) return batch_work(b, false);
   cudaError_t e = cudaEventRecord(b->forked, b->stream);
   for (cudaStream_t st : b->side)

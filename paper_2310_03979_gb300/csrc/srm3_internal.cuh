@@ -294,7 +294,9 @@ struct DeviceGuard {
 // plan), on a stream.  Seeds from the host array (passed by value) or from
 // device memory; with sqq_of, pk_of, ck_of (device, per sample) the samples
 // take those factors instead of the plan's.  work: device scratch, at least
-// one sample's grid rows and phasors.
+// one sample's grid rows and phasors.  With max_ctas a launch's row CTAs are no
+// more than that many halves of an SM hold at a time (or one sample's): work on
+// other streams waits for one such launch, not for the whole batch's.
 struct ConvJob {
   const srm3_plan *plan;
   cudaStream_t stream;
@@ -304,6 +306,7 @@ struct ConvJob {
   void *work;
   size_t work_bytes;
   void *C;
+  int max_ctas;  // > 0: launches of few enough samples (srm3_batch_set_max_ctas)
 };
 int conv_run_f32(const ConvJob &j);
 int conv_run_f64(const ConvJob &j);

@@ -123,3 +123,32 @@ def test_fp64_coefficients_keep_the_rounding_of_direct_sums(oracle_lib, nk, nw, 
     for i in range(3):
         ref = op.coeffs(i + 1)
         assert np.linalg.norm(C[i] - ref) <= 5e-16 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_capped_batch_runs_in_small_launches_with_the_same_fields(captured):
+    """A cap of one CTA leaves launches of one sample each, on the batch stream alone;
+    the fields are the uncapped batch's, bit for bit."""
+    wls = [_case(64, 40, "fp32"), replace(_case(64, 40, "fp32"), U=25.0), _case(20, 64, "fp32"),
+           _case(12, 9, "fp32", interactions="mixed"), _case(16, 16, "fp64")]
+    plans = [srm3.Plan.create(w, storage="recompute") for w in wls]
+    counts = [5, 2, 3, 4, 2]
+    outs = [torch.empty((c, w.n_x, w.n_t), device="cuda",
+                        dtype=torch.float64 if w.precision == "fp64" else torch.float32)
+            for c, w in zip(counts, wls)]
+    seeds = np.arange(7, 7 + sum(counts), dtype=np.uint64)
+    got = []
+    for cap in (0, 1):
+        with srm3.Batch(plans, counts, outs) as batch:
+            batch.set_max_ctas(cap)
+            if captured:
+                batch.capture()
+            for o in outs:
+                o.fill_(float("nan"))
+            batch.run(seeds)
+            batch.sync()
+            got.append([o.clone() for o in outs])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    for p in plans:
+        p.destroy()
