@@ -152,3 +152,21 @@ def test_capped_batch_runs_in_small_launches_with_the_same_fields(captured):
         assert torch.equal(a, b)
     for p in plans:
         p.destroy()
+
+
+@pytest.mark.parametrize("nk,nw,interactions", [(1, 2048, "sum"), (1, 2049, "sum"), (2048, 1, "sum"),
+                                                (2049, 1, "sum"), (1, 1366, "mixed"),
+                                                (1, 1367, "mixed")])
+def test_fp64_coefficients_at_the_longest_transforms(oracle_lib, nk, nw, interactions):
+    """Triple-float rows and columns reach 4096 points; the next lattice takes the
+    direct sums."""
+    wl = _case(nk, nw, "fp64", 0.25, 0.3, interactions)
+    S = oracle.kaimal_lorentzian(nk, nw, wl.kappa_u, wl.omega_u, wl.U, wl.z)
+    S[:, 0] = 1.0 / (1.0 + np.arange(nk))
+    mixed = interactions == "mixed"
+    op = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=0.02, beta=0.3, mixed=mixed)
+    with srm3.Plan.create(wl, table=S, eps=0.02) as p:
+        C = _cplx(p.coeffs([5, 6]))
+    for i in range(2):
+        ref = op.coeffs(5 + i)
+        assert np.abs(C[i] - ref).max() <= TOL["fp64"] * np.abs(ref).max()

@@ -272,3 +272,19 @@ def test_fp32_mixed_tables_are_the_fp64_fixed_point(oracle_lib, nk, nw):
     assert abs(info.max_sum_b2 - wl.target) <= 1e-9
     ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps, mixed=True)
     assert np.abs(sb2 - ref.sum_b2).max() <= 3e-14
+
+
+@pytest.mark.parametrize("nk,nw", [(2, 4096), (2048, 2), (2049, 2), (1025, 3), (3, 2049)])
+def test_separable_tables_at_the_longest_transforms(oracle_lib, nk, nw):
+    """The solve's transforms at 4096 points and just past 2048, and the level pass
+    beyond: the tables of an FP32 plan against the oracle (some 1e3 pairs a sum)."""
+    wl = replace(W.small_case(nk=nk, nw=nw, nx=pow2(nk), nt=pow2(2 * nw)), envelope="separable")
+    ta, _ = wl.envelope_tables()
+    S = np.ones((nk, nw))
+    with srm3.Plan.create(wl, table=S) as p:
+        _, q, sb2 = p.tables()
+        info = p.info()
+    assert bool(info.recursion_flags & srm3.SRM3_REC_LATTICE_SOLVE) == (nk <= 2048)
+    ref = oracle.make_plan(S, wl.kappa_u, wl.omega_u, eps=info.eps,
+                           env=oracle.Envelope("separable", table=ta))
+    assert np.abs(sb2 - ref.sum_b2).max() <= 1e-13 * max(1.0, ref.q.max() ** 2)
