@@ -820,7 +820,8 @@ def main():
     # envelope tables, g^2, twiddles and factors 9, the sum of S 2; the
     # whole-lattice solve's tables 4, its iterations (10 or more, 3 launches
     # each), the direct sums and results 3, on the coarse lattice (counted by the
-    # plan) and on the plan's; FP64 plans' direct iterations 6 or more; sampling
+    # plan) and on the plan's (a triple-float finish not counted); FP64 plans' direct
+    # iterations 6 or more; sampling
     # tables 1, W table 1 if stored; per 128-sample chunk the pair sum (phases and
     # one launch, or three self-convolution passes), two FFT stages
     selfconv = wl.envelope != "gauss" or info.storage != 1
@@ -846,11 +847,10 @@ def main():
                    "storage": "table" if info.storage == 1 else "recompute",
                    "precision": wl.precision, "l2": "inputs larger than L2 (W table "
                    f"{info.table_bytes / 1e9:.1f} GB, y {n * 2 * 8 * wl.n_kappa * (wl.n_omega + 128) / 1e6:.0f} MB)",
-                   "step": ("plan build (spectrum, FP64 recursion + eps search, W table) + "
+                   "step": ("plan build (spectrum, eps search and tables of Eq. pure, W table) + "
                             f"{n}-sample batch") if prebuilt is None else
                            (f"{n}-sample batch on a plan built beforehand (mixed interactions: "
-                            f"{prebuilt_ms:.0f} ms to build, the FP64 fixed point of Eq. pure "
-                            "solved for every eps of the search)"),
+                            f"{prebuilt_ms:.1f} ms to build)"),
                    "interactions": wl.interactions},
         "samples_per_s": n * world / (ms_per_step * 1e-3),
         "wall_ms_per_step": wall * 1e3 / args.steps,
@@ -866,10 +866,10 @@ def main():
                                 "transform": t_last.transform_ms},
         "sampling_only_pair_terms_per_s": terms_per_step / (
             (t_last.phases_ms + t_last.pairsum_ms + t_last.transform_ms) * 1e-3),
-        "roofline": (_conv_roofline(wl, n, es, avg_launch_ms)
-                     if wl.envelope != "gauss" or (selfconv and es == 8)
+        "roofline": (_conv_roofline(wl, n, es, avg_launch_ms) if wl.envelope != "gauss"
                      else _selfconv_roofline([(wl.n_kappa, wl.n_omega, min(n, 128),
-                                               wl.interactions == "mixed")], avg_launch_ms)
+                                               wl.interactions == "mixed")], avg_launch_ms,
+                                             fp64=es == 8)
                      if selfconv
                      else _pairsum_roofline_fp64(terms_per_launch / (avg_launch_ms * 1e-3),
                                                  kernel="k_pairsum_f64") if es == 8
