@@ -113,23 +113,30 @@ def _conv_roofline(wl, n, es, launch_ms):
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy bandwidth)"}
 
 
-def _selfconv_roofline(lattices, ms):
-    """Roofline of the double-float self-convolution pair sum (Gaussian envelope
-    with W recomputed, FP32 plans): about 28 FP32-pipe lane operations per point
-    and level of the transforms -- rows there and back on n_kappa rows of Nw,
-    columns there and back on Nw columns of Nk -- over the pipe's rate.
+def _selfconv_roofline(lattices, ms, fp64=False):
+    """Roofline of the self-convolution pair sum of the Gaussian envelope (W
+    recomputed): FP32-pipe lane operations per point and level of the transforms,
+    28 in double-float (FP32 plans: 8 a sum, 32 a complex product) and 95 in
+    triple-float (FP64 plans, radix 4: 21 a sum, 142 a complex product), over the
+    pipe's rate.  Rows there and back on n_kappa rows of Nw, columns there and
+    back on Nw columns of Nk; a transform whose upper half of inputs is zero
+    takes a level less (not the rows of mixed interactions), one whose upper half
+    of outputs is dropped half a level less.
     lattices: (n_kappa, n_omega, samples, mixed) of everything in ms."""
-    ops = 0.0
+    ops, per = 0.0, 95.0 if fp64 else 28.0
     for nk, nw, n, mixed in lattices:
         lk = max(1, (2 * nk - 2).bit_length())
         lw = max(1, ((3 * nw - 3) if mixed else (2 * nw - 2)).bit_length())
-        ops += 2 * n * 28.0 * 2 * (nk * (lw << lw) + (lk << lk) * (1 << lw))
+        rows = nk * (2 * lw - (0.5 if mixed else 1.5))
+        cols = (1 << lk) * (2 * lk - 1.5)
+        ops += 2 * n * per * (rows + cols) * (1 << lw)
     sm_max = float(_peaks().get("sm_max_mhz", 2070.0))
     rate = FP32_LANES_PER_SM * n_sm() * sm_max * 1e6
     got = ops / (ms * 1e-3)
     return {"bound": "alu", "achieved": got / 1e12, "peak": rate / 1e12,
             "unit": "T FP32-pipe lane-ops/s", "frac": got / rate, "traffic": None,
-            "per_unit": "28 FP32-pipe lane-ops per point and level, unpruned",
+            "per_unit": f"{per:.0f} FP32-pipe lane-ops per point and level, levels of zero "
+                        "inputs and dropped outputs left out",
             "kernel": "k_conv_rows + k_conv_cols + k_conv_out",
             "peak_source": f"derived: {n_sm()} SM x {FP32_LANES_PER_SM} FP32 lanes x "
                            f"{sm_max:.0f} MHz (max SM clock of MEASURED_PEAKS.json)"}
