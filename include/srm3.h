@@ -78,8 +78,9 @@ typedef struct srm3_spectrum {
  * instead of the O(N^2) pair sum (Sec. 4.3 FFT form; any storage setting is
  * ignored).  The Gaussian envelope factors on the pairs of k as well, since
  * (i-j)^2 = 2 (i-c)^2 + 2 (j-c)^2 - (k-2c)^2: with W recomputed it takes the
- * same form, in an arithmetic that leaves FP32 plans FP32 accuracy, unless
- * sigma_g is so small (below about 0.22) that the factors' range is too wide. */
+ * same form, in an arithmetic that leaves plans the accuracy of their precision,
+ * unless sigma_g is so small (below about 0.22) that the factors' range is too
+ * wide, or (FP64) a padded axis exceeds 4096 points. */
 enum srm3_bispectrum_kind {
     SRM3_BISPECTRUM_GAUSS_ENVELOPE = 0,
     SRM3_BISPECTRUM_SEPARABLE = 1
@@ -127,7 +128,9 @@ typedef struct srm3_bispectrum {
 
 enum srm3_precision {
     SRM3_FP32 = 0, /* tiled FP32 pair sum with compensated merge, FP32 FFT */
-    SRM3_FP64 = 1  /* plain FP64 pair sum (one warp per k and sheet-sample), FP64 FFT */
+    SRM3_FP64 = 1  /* FP64 phases, tables and FFT; the pair sum as a self-convolution
+                      beyond FP64's precision where the envelope takes that form, else
+                      the plain FP64 one (one warp per k and sheet-sample) */
 };
 enum srm3_storage {
     SRM3_STORAGE_AUTO = 0,     /* the fastest: recompute where the pair sum is a

@@ -123,7 +123,7 @@ namespace {
 // the short transforms of small lattices, whose passes are bound by the latency
 // of a thread's own instructions, more for the longest, whose threads would not
 // fit in a CTA.  4 / 8 / 16 values everywhere measured, in us (pair sum with
-// phases): one sample of 32 x 32 19.4 / 22.4 / 31.7, 4 FP64 mixed ones of 29 x 12
+// phases): one sample of 32 x 32 19.4 / 22.4 / 31.7, 4 mixed ones of 29 x 12 in FP64
 // 37 / 46 / 67; 64 samples of 256 x 512 2213 / 1931 / 2193, 16 of 512 x 1024 2589 /
 // 2561 / 2384, 64 separable ones of 256 x 512 907 / 624 / 662, 50 of 256 x 128
 // 192 / 139 / 180 (202 with separate phases and 16 values).  Triple-floats: 4,

@@ -9,8 +9,8 @@ its stream slots is free: all admitted requests go into one batch
 spectra of one lattice shape share the lanes of the pair sum.  Requests
 are light or heavy by the pair-terms of one sample (heavy above
 `heavy_terms`); each class has its own queue and stream slots, and a heavy
-batch's persistent pair sum is capped at one CTA per SM so that light
-batches run beside it instead of queueing behind it.  Batches admitted
+batch's pair sums are capped at half of every SM (srm3_batch_set_max_ctas) so that
+light batches run beside it instead of queueing behind it.  Batches admitted
 while others run overlap with them on the device.  A request's latency runs
 from its arrival to the completion of its batch.
 
